@@ -1,4 +1,4 @@
-"""ctypes binding of ``libmdraft.so`` — argument marshalling only.
+"""Binding of ``libmdraft.so`` — argument marshalling only (the per-layer calls through the extension ``_host``, the rest ctypes).
 
 Every function here has the name of the C entry point it calls (see
 ``include/mdraft.h``) and does nothing but turn torch tensors into pointers,
@@ -71,11 +71,16 @@ class _Ucb(C.Structure):
 
 
 _lib = None
+_host = None   # csrc/host.cpp
+
+# entry points whose arguments csrc/host.cpp marshals, in the order of its table
+_HOST_CALLS = ("mdraft_conv_scan_prefill", "mdraft_conv_scan_prefill_noalloc", "mdraft_tree_step", "mdraft_tree_step_proj",
+               "mdraft_state_commit", "mdraft_ssd_prefill", "mdraft_ssd_tree_step")
 
 
 def load_library(path: Optional[str] = None):
     """Load the CUDA library; raises if it has not been built (there is no other code path)."""
-    global _lib
+    global _lib, _host
     if _lib is not None and path is None:
         return _lib
     p = path or LIB_PATH
@@ -125,9 +130,21 @@ def load_library(path: Optional[str] = None):
     lib.mdraft_ssd_tree_step.argtypes = [C.POINTER(_SsdLayer), C.POINTER(_Cache), i32,
                                          vp, i64, vp, i64, vp, i64, vp, i64, vp, i64, vp, i64,
                                          i32, vp, vp, i32, C.POINTER(i32), vp, vp]
+    # The calls that are issued once per layer go through the extension, which is given the addresses of this library.
+    if _host is None:
+        try:
+            from . import _host as ext
+        except ImportError as e:
+            raise ImportError(f"{_HERE}/_host.so cannot be loaded ({e}): build it with `python -m paper_2506_01206_b200.build`") from e
+        _host = ext
+    lib.entry = _host.table([C.cast(getattr(lib, n), C.c_void_p).value for n in _HOST_CALLS])
     if path is None:
         _lib = lib
     return lib
+
+
+def _entry():
+    return (_lib or load_library()).entry
 
 
 def status_string(status: int) -> str:
@@ -148,17 +165,6 @@ def _act_of(dtype: torch.dtype) -> int:
 
 def _ptr(t: Optional[torch.Tensor]):
     return None if t is None else C.c_void_p(t.data_ptr())
-
-
-def _mat(t: Optional[torch.Tensor], name: str):
-    """(pointer, row stride in elements) of a 2-D tensor whose last dim is contiguous."""
-    if t is None:
-        return None, 0
-    if t.dim() != 2 or (t.shape[1] > 1 and t.stride(1) != 1):
-        raise ValueError(f"{name}: need a 2-D tensor with unit stride along the last dim")
-    if not t.is_cuda:
-        raise ValueError(f"{name}: must be a CUDA tensor")
-    return C.c_void_p(t.data_ptr()), int(t.stride(0))
 
 
 def _stream_ptr(stream) -> C.c_void_p:
@@ -247,23 +253,8 @@ def mdraft_conv_scan_prefill(layer: Layer, cache: Optional[StateCache], layer_in
                              workspace: Optional[torch.Tensor] = None, chunk_len: int = 0,
                              dev_status: Optional[torch.Tensor] = None, stream=None, flags: Optional[int] = None,
                              phase_events=None) -> None:
-    lib = load_library()
-    cl = layer.c(flags)
-    cc = cache.c() if cache is not None else None
-    px, ldx = _mat(x, "x"); pz, ldz = _mat(z, "z"); pdt, lddt = _mat(dt, "dt")
-    pB, ldb = _mat(B, "B"); pC, ldc = _mat(Cm, "C"); po, ldo = _mat(out, "out")
-    T = int(x.shape[0])
-    n_seq = 1 if cu_seqlens is None else int(cu_seqlens.numel()) - 1   # None: a single sequence of all T rows
-    if cu_seqlens is not None and cu_seqlens.dtype != torch.int32:
-        raise TypeError("cu_seqlens must be int32")
-    for t, nm in ((init_slot, "init_slot"), (final_slot, "final_slot")):
-        if t is not None and (t.dtype != torch.int32 or t.numel() != n_seq):
-            raise TypeError(f"{nm} must be int32 with one entry per sequence")
-    ws_ptr, ws_bytes = (None, 0) if workspace is None else (C.c_void_p(workspace.data_ptr()), workspace.numel() * workspace.element_size())
-    rc = lib.mdraft_conv_scan_prefill(C.byref(cl), C.byref(cc) if cc is not None else None, int(layer_index),
-                                      px, ldx, pz, ldz, pdt, lddt, pB, ldb, pC, ldc, po, ldo,
-                                      T, n_seq, int(max_seqlen), _ptr(cu_seqlens), _ptr(init_slot), _ptr(final_slot),
-                                      ws_ptr, ws_bytes, _opts(chunk_len, phase_events), _ptr(dev_status), _stream_ptr(stream))
+    rc = _host.prefill(_entry(), layer, cache, layer_index, x, z, dt, B, Cm, out, cu_seqlens, max_seqlen, init_slot, final_slot,
+                       workspace, chunk_len, dev_status, stream, flags, phase_events)
     if rc != 0:
         raise MdraftError(rc, "mdraft_conv_scan_prefill")
 
@@ -279,22 +270,8 @@ def mdraft_conv_scan_prefill_noalloc(layer: Layer, cache: Optional[StateCache], 
     """Prefill without a caller workspace: the library's own fixed scratch array is used (see the header for
     who needs this and for the sharing rules).  Raises MdraftError(MDRAFT_ERR_WORKSPACE) when the problem needs
     more than NOALLOC_SCRATCH_BYTES of scratch."""
-    lib = load_library()
-    cl = layer.c(flags)
-    cc = cache.c() if cache is not None else None
-    px, ldx = _mat(x, "x"); pz, ldz = _mat(z, "z"); pdt, lddt = _mat(dt, "dt")
-    pB, ldb = _mat(B, "B"); pC, ldc = _mat(Cm, "C"); po, ldo = _mat(out, "out")
-    T = int(x.shape[0])
-    n_seq = 1 if cu_seqlens is None else int(cu_seqlens.numel()) - 1   # None: a single sequence of all T rows
-    if cu_seqlens is not None and cu_seqlens.dtype != torch.int32:
-        raise TypeError("cu_seqlens must be int32")
-    for t, nm in ((init_slot, "init_slot"), (final_slot, "final_slot")):
-        if t is not None and (t.dtype != torch.int32 or t.numel() != n_seq):
-            raise TypeError(f"{nm} must be int32 with one entry per sequence")
-    rc = lib.mdraft_conv_scan_prefill_noalloc(C.byref(cl), C.byref(cc) if cc is not None else None, int(layer_index),
-                                              px, ldx, pz, ldz, pdt, lddt, pB, ldb, pC, ldc, po, ldo,
-                                              T, n_seq, int(max_seqlen), _ptr(cu_seqlens), _ptr(init_slot), _ptr(final_slot),
-                                              _opts(chunk_len), _ptr(dev_status), _stream_ptr(stream))
+    rc = _host.prefill_noalloc(_entry(), layer, cache, layer_index, x, z, dt, B, Cm, out, cu_seqlens, max_seqlen, init_slot, final_slot,
+                               chunk_len, dev_status, stream, flags)
     if rc != 0:
         raise MdraftError(rc, "mdraft_conv_scan_prefill_noalloc")
 
@@ -303,24 +280,8 @@ def mdraft_tree_step(layer: Layer, cache: StateCache, layer_index: int, x, z, dt
                      parent_slot: torch.Tensor, node_slot: torch.Tensor,
                      level_offsets: Optional[Sequence[int]] = None,
                      dev_status: Optional[torch.Tensor] = None, stream=None, flags: Optional[int] = None) -> None:
-    lib = load_library()
-    cl = layer.c(flags)
-    cc = cache.c()
-    px, ldx = _mat(x, "x"); pz, ldz = _mat(z, "z"); pdt, lddt = _mat(dt, "dt")
-    pB, ldb = _mat(B, "B"); pC, ldc = _mat(Cm, "C"); po, ldo = _mat(out, "out")
-    M = int(x.shape[0])
-    if parent_slot.dtype != torch.int32 or node_slot.dtype != torch.int32:
-        raise TypeError("slot index arrays must be int32")
-    if parent_slot.numel() != M or node_slot.numel() != M:
-        raise ValueError("one parent slot and one node slot per node")
-    if level_offsets is None:
-        n_levels, lo = 1, None
-    else:
-        n_levels = len(level_offsets) - 1
-        lo = (C.c_int32 * (n_levels + 1))(*[int(v) for v in level_offsets])
-    rc = lib.mdraft_tree_step(C.byref(cl), C.byref(cc), int(layer_index),
-                              px, ldx, pz, ldz, pdt, lddt, pB, ldb, pC, ldc, po, ldo,
-                              M, _ptr(parent_slot), _ptr(node_slot), n_levels, lo, _ptr(dev_status), _stream_ptr(stream))
+    rc = _host.tree_step(_entry(), layer, cache, layer_index, x, z, dt, B, Cm, out, parent_slot, node_slot, level_offsets, dev_status,
+                         stream, flags)
     if rc != 0:
         raise MdraftError(rc, "mdraft_tree_step")
 
@@ -331,35 +292,15 @@ def mdraft_tree_step_proj(layer: Layer, cache: StateCache, layer_index: int, W_x
                           nodes_per_cluster: int = 0) -> None:
     """One tree level where dt, B and C come from the block's projections of the conv output.
     W_x: (dt_rank + 2 N, D) and W_dt: (D, dt_rank), contiguous, in the layer's activation dtype."""
-    lib = load_library()
-    cl = layer.c(flags)
-    cc = cache.c()
-    px, ldx = _mat(x, "x"); pz, ldz = _mat(z, "z"); po, ldo = _mat(out, "out")
-    M = int(x.shape[0])
-    if parent_slot.dtype != torch.int32 or node_slot.dtype != torch.int32:
-        raise TypeError("slot index arrays must be int32")
-    if parent_slot.numel() != M or node_slot.numel() != M:
-        raise ValueError("one parent slot and one node slot per node")
-    if W_x.dtype != x.dtype or W_dt.dtype != x.dtype or not W_x.is_contiguous() or not W_dt.is_contiguous():
-        raise TypeError("W_x and W_dt must be contiguous and of the activation dtype")
-    R = int(W_dt.shape[1])
-    if tuple(W_dt.shape) != (layer.d_inner, R) or tuple(W_x.shape) != (R + 2 * layer.d_state, layer.d_inner):
-        raise ValueError("W_x must be (dt_rank + 2 d_state, d_inner) and W_dt (d_inner, dt_rank)")
-    pr = _SelectProj(W_x.data_ptr(), W_dt.data_ptr(), R, int(nodes_per_cluster))
-    rc = lib.mdraft_tree_step_proj(C.byref(cl), C.byref(cc), int(layer_index), C.byref(pr), px, ldx, pz, ldz, po, ldo,
-                                   M, _ptr(parent_slot), _ptr(node_slot), _ptr(dev_status), _stream_ptr(stream))
+    rc = _host.tree_step_proj(_entry(), layer, cache, layer_index, W_x, W_dt, x, z, out, parent_slot, node_slot, dev_status, stream, flags,
+                              nodes_per_cluster)
     if rc != 0:
         raise MdraftError(rc, "mdraft_tree_step_proj")
 
 
 def mdraft_state_commit(cache: StateCache, src_slot: torch.Tensor, dst_slot: torch.Tensor,
                         dev_status: Optional[torch.Tensor] = None, stream=None) -> None:
-    lib = load_library()
-    cc = cache.c()
-    if src_slot.dtype != torch.int32 or dst_slot.dtype != torch.int32 or src_slot.numel() != dst_slot.numel():
-        raise TypeError("src_slot / dst_slot must be int32 arrays of equal length")
-    rc = lib.mdraft_state_commit(C.byref(cc), cache.d_inner, cache.d_state, cache.d_conv, _act_of(cache.act),
-                                 int(src_slot.numel()), _ptr(src_slot), _ptr(dst_slot), _ptr(dev_status), _stream_ptr(stream))
+    rc = _host.commit(_entry(), cache, src_slot, dst_slot, dev_status, stream)
     if rc != 0:
         raise MdraftError(rc, "mdraft_state_commit")
 
@@ -452,22 +393,8 @@ def mdraft_ssd_prefill(layer: SsdLayer, cache: Optional[StateCache], layer_index
                        cu_seqlens: Optional[torch.Tensor], init_slot: Optional[torch.Tensor] = None,
                        final_slot: Optional[torch.Tensor] = None, workspace: Optional[torch.Tensor] = None,
                        dev_status: Optional[torch.Tensor] = None, stream=None, flags: Optional[int] = None) -> None:
-    lib = load_library()
-    cl = layer.c(flags)
-    cc = cache.c() if cache is not None else None
-    px, ldx = _mat(x, "x"); pz, ldz = _mat(z, "z"); pdt, lddt = _mat(dt, "dt")
-    pB, ldb = _mat(B, "B"); pC, ldc = _mat(Cm, "C"); po, ldo = _mat(out, "out")
-    T = int(x.shape[0])
-    n_seq = 1 if cu_seqlens is None else int(cu_seqlens.numel()) - 1
-    if cu_seqlens is not None and cu_seqlens.dtype != torch.int32:
-        raise TypeError("cu_seqlens must be int32")
-    for t, nm in ((init_slot, "init_slot"), (final_slot, "final_slot")):
-        if t is not None and (t.dtype != torch.int32 or t.numel() != n_seq):
-            raise TypeError(f"{nm} must be int32 with one entry per sequence")
-    ws_ptr, ws_bytes = (None, 0) if workspace is None else (C.c_void_p(workspace.data_ptr()), workspace.numel() * workspace.element_size())
-    rc = lib.mdraft_ssd_prefill(C.byref(cl), C.byref(cc) if cc is not None else None, int(layer_index),
-                                px, ldx, pz, ldz, pdt, lddt, pB, ldb, pC, ldc, po, ldo, T, n_seq,
-                                _ptr(cu_seqlens), _ptr(init_slot), _ptr(final_slot), ws_ptr, ws_bytes, _ptr(dev_status), _stream_ptr(stream))
+    rc = _host.ssd_prefill(_entry(), layer, cache, layer_index, x, z, dt, B, Cm, out, cu_seqlens, init_slot, final_slot, workspace, dev_status,
+                           stream, flags)
     if rc != 0:
         raise MdraftError(rc, "mdraft_ssd_prefill")
 
@@ -475,23 +402,7 @@ def mdraft_ssd_prefill(layer: SsdLayer, cache: Optional[StateCache], layer_index
 def mdraft_ssd_tree_step(layer: SsdLayer, cache: StateCache, layer_index: int, x, z, dt, B, Cm, out,
                          parent_slot: torch.Tensor, node_slot: torch.Tensor, level_offsets: Optional[Sequence[int]] = None,
                          dev_status: Optional[torch.Tensor] = None, stream=None, flags: Optional[int] = None) -> None:
-    lib = load_library()
-    cl = layer.c(flags)
-    cc = cache.c()
-    px, ldx = _mat(x, "x"); pz, ldz = _mat(z, "z"); pdt, lddt = _mat(dt, "dt")
-    pB, ldb = _mat(B, "B"); pC, ldc = _mat(Cm, "C"); po, ldo = _mat(out, "out")
-    M = int(x.shape[0])
-    if parent_slot.dtype != torch.int32 or node_slot.dtype != torch.int32:
-        raise TypeError("slot index arrays must be int32")
-    if parent_slot.numel() != M or node_slot.numel() != M:
-        raise ValueError("one parent slot and one node slot per node")
-    if level_offsets is None:
-        n_levels, lo = 1, None
-    else:
-        n_levels = len(level_offsets) - 1
-        lo = (C.c_int32 * (n_levels + 1))(*[int(v) for v in level_offsets])
-    rc = lib.mdraft_ssd_tree_step(C.byref(cl), C.byref(cc), int(layer_index),
-                                  px, ldx, pz, ldz, pdt, lddt, pB, ldb, pC, ldc, po, ldo,
-                                  M, _ptr(parent_slot), _ptr(node_slot), n_levels, lo, _ptr(dev_status), _stream_ptr(stream))
+    rc = _host.ssd_tree_step(_entry(), layer, cache, layer_index, x, z, dt, B, Cm, out, parent_slot, node_slot, level_offsets, dev_status,
+                             stream, flags)
     if rc != 0:
         raise MdraftError(rc, "mdraft_ssd_tree_step")

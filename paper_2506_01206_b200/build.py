@@ -7,7 +7,8 @@ on the GPU machine.
 
 Each ``csrc/*.cu`` is compiled to an object of its own (in parallel, and only
 when it or a header changed) and the objects are linked into the shared
-library.  ``build_library(variant="waittest")`` builds a second library,
+library.  ``csrc/host.cpp`` becomes ``_host.so``, the CPython extension that
+turns a call's tensors into the library's arguments.  ``build_library(variant="waittest")`` builds a second library,
 ``libmdraft_waittest.so``, for the failure-path tests: the same sources with a
 short limit on every on-chip wait and an overstated byte count on every
 copy barrier, so that each bounded wait runs out and the give-up paths execute.
@@ -24,6 +25,7 @@ from concurrent.futures import ThreadPoolExecutor
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libmdraft.so")
+HOST = os.path.join(HERE, "_host.so")
 OBJ_DIR = os.path.join(HERE, "_build")
 
 NVCC_FLAGS = [
@@ -58,7 +60,16 @@ def library_path(variant: str = "") -> str:
 
 
 def build_library(force: bool = False, verbose: bool = False, extra=(), variant: str = "") -> str:
+    """Builds the library (and the extension that feeds it, which every variant shares) where a source has changed."""
     lib, vflags = VARIANTS[variant]
+    host = ThreadPoolExecutor(max_workers=1).submit(build_host, force and not variant)
+    try:
+        return _build_library(lib, vflags, force, verbose, extra, variant)
+    finally:
+        host.result()
+
+
+def _build_library(lib, vflags, force, verbose, extra, variant) -> str:
     srcs, hdrs = sources(), _headers()
     if not force and not extra and not _newer(srcs + hdrs, lib):
         return lib
@@ -85,6 +96,26 @@ def build_library(force: bool = False, verbose: bool = False, extra=(), variant:
     subprocess.run([nvcc, "-shared", "-gencode", "arch=compute_100a,code=sm_100a", "-o", lib + ".tmp", *objs], check=True)
     os.replace(lib + ".tmp", lib)
     return lib
+
+
+def build_host(force: bool = False) -> str:
+    """The CPython extension that hands torch tensors to the library (``csrc/host.cpp``): host code only, one g++ run."""
+    src = os.path.join(CSRC, "host.cpp")
+    if not force and not _newer([src, *_headers()], HOST):
+        return HOST
+    import sysconfig
+
+    import torch
+    from torch.utils import cpp_extension
+    libdir = os.path.join(os.path.dirname(torch.__file__), "lib")
+    cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           *[f"-isystem{p}" for p in cpp_extension.include_paths()], f"-isystem{cuda}/include", f"-isystem{sysconfig.get_paths()['include']}",
+           src, "-o", HOST + ".tmp", f"-L{libdir}", "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
+    subprocess.run(cmd, check=True)
+    os.replace(HOST + ".tmp", HOST)
+    return HOST
 
 
 if __name__ == "__main__":
