@@ -157,6 +157,36 @@ int mdraft_conv_scan_prefill(const mdraft_layer *layer, const mdraft_cache *cach
                              void *workspace, size_t workspace_bytes, const mdraft_prefill_opts *opts,
                              int32_t *dev_status, void *stream);
 
+/* One layer's activations in a call over several layers; meanings and strides as in mdraft_conv_scan_prefill / mdraft_tree_step. */
+typedef struct {
+    const void *x, *z, *dt, *B, *C;
+    void *out;
+    int64_t ldx, ldz, lddt, ldb, ldc, ldo;
+} mdraft_io;
+
+/*
+ * The same prefill for several layers whose inputs are all there already (HOST arrays of n_layers entries each; layer i reads
+ * and writes pool layer layer_index[i]).  Paper Section 3.1: the drafter encodes a context with every layer of its stack.
+ * The results are those of one mdraft_conv_scan_prefill per layer up to the rounding of another chunk plan.  Layers that share
+ * their flags run in one launch (up to 32), which fills the GPU without cutting sequences into chunks; d_inner and act must
+ * agree over all layers (else MDRAFT_ERR_UNSUPPORTED).
+ * Hazards (caller's duty): the layers run side by side, so no layer's `out` may overlap another layer's inputs or `out`, and
+ * no pool layer may appear twice.
+ *   workspace : at least mdraft_prefill_stack_workspace_bytes(...) for layers that share their flags (the first one's)
+ * mdraft_prefill_stack_launches: kernels such a call launches (for accounting).
+ */
+size_t mdraft_prefill_stack_workspace_bytes(const mdraft_layer *layer, int32_t n_layers, int32_t total_tokens, int32_t n_seq,
+                                            int32_t max_seqlen, const mdraft_prefill_opts *opts);
+
+int32_t mdraft_prefill_stack_launches(const mdraft_layer *layer, int32_t n_layers, int32_t total_tokens, int32_t n_seq,
+                                      int32_t max_seqlen, const mdraft_prefill_opts *opts);
+
+int mdraft_conv_scan_prefill_stack(int32_t n_layers, const mdraft_layer *layers, const mdraft_cache *cache, const int32_t *layer_index,
+                                   const mdraft_io *io, int32_t total_tokens, int32_t n_seq, int32_t max_seqlen,
+                                   const int32_t *cu_seqlens, const int32_t *init_slot, const int32_t *final_slot,
+                                   void *workspace, size_t workspace_bytes, const mdraft_prefill_opts *opts,
+                                   int32_t *dev_status, void *stream);
+
 /*
  * The same prefill for callers that cannot allocate device memory.  No counterpart in the paper: this is a
  * deployment variant of mdraft_conv_scan_prefill.  Some hosts of this library must never call cudaMalloc or a
@@ -217,6 +247,16 @@ int mdraft_tree_step(const mdraft_layer *layer, const mdraft_cache *cache, int32
                      int32_t n_nodes, const int32_t *parent_slot, const int32_t *node_slot,
                      int32_t n_levels, const int32_t *level_offsets,
                      int32_t *dev_status, void *stream);
+
+/*
+ * The same tree step for several layers whose inputs are all there already: one launch per level takes every layer (up to 32
+ * with the same flags), so a round of L layers waits for n_levels dependent launches instead of L * n_levels.  HOST arrays
+ * of n_layers entries; layer i works on pool layer layer_index[i]; bit for bit the results of one mdraft_tree_step per layer.
+ * Paper Section 4.1.  Hazards: those of mdraft_tree_step, and between layers those of mdraft_conv_scan_prefill_stack.
+ */
+int mdraft_tree_step_stack(int32_t n_layers, const mdraft_layer *layers, const mdraft_cache *cache, const int32_t *layer_index,
+                           const mdraft_io *io, int32_t n_nodes, const int32_t *parent_slot, const int32_t *node_slot,
+                           int32_t n_levels, const int32_t *level_offsets, int32_t *dev_status, void *stream);
 
 /*
  * Draft-tree step with the block's own selection projections: like

@@ -10,7 +10,8 @@ from .binding import (  # noqa: F401
     MDRAFT_DEV_WAIT_EXPIRED, MDRAFT_DT_SOFTPLUS, MDRAFT_F32, MDRAFT_PRECONV,
     Layer, MdraftError, StateCache, UcbBandit, load_library, mdraft_ucb_reward,
     mdraft_classify_A, mdraft_conv_scan_prefill, mdraft_conv_scan_prefill_noalloc, mdraft_prefill_workspace_bytes,
-    NOALLOC_SCRATCH_BYTES,
+    NOALLOC_SCRATCH_BYTES, mdraft_conv_scan_prefill_stack, mdraft_prefill_stack_launches, mdraft_prefill_stack_workspace_bytes,
+    mdraft_tree_step_stack,
     SsdLayer, mdraft_ssd_prefill, mdraft_ssd_prefill_workspace_bytes, mdraft_ssd_tree_step,
     mdraft_state_commit, mdraft_tree_step, mdraft_tree_step_proj, mdraft_version, status_string,
 )

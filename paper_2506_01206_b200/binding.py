@@ -20,6 +20,7 @@ _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libmdraft.so")
 
 MDRAFT_F32, MDRAFT_BF16 = 0, 1
+MDRAFT_ERR_WORKSPACE = -4
 MDRAFT_DT_SOFTPLUS, MDRAFT_PRECONV, MDRAFT_CONV_ONLY, MDRAFT_A_POWERS = 1, 2, 4, 8
 MDRAFT_DEV_BAD_SLOT, MDRAFT_DEV_BAD_SEQLENS, MDRAFT_DEV_WAIT_EXPIRED = 1, 2, 4
 
@@ -28,6 +29,7 @@ EXPORTS = (
     "mdraft_tree_step_proj", "mdraft_state_commit", "mdraft_classify_A", "mdraft_status_string", "mdraft_version",
     "mdraft_ucb_reward", "mdraft_ucb_select", "mdraft_ucb_update",
     "mdraft_ssd_prefill_workspace_bytes", "mdraft_ssd_prefill", "mdraft_ssd_tree_step",
+    "mdraft_prefill_stack_workspace_bytes", "mdraft_prefill_stack_launches", "mdraft_conv_scan_prefill_stack", "mdraft_tree_step_stack",
 )
 
 
@@ -71,11 +73,31 @@ class _Ucb(C.Structure):
 
 
 _lib = None
-_host = None   # csrc/host.cpp
+
+
+def _load_host():
+    """The extension built from csrc/host.cpp; raises if it is missing (there is no other code path)."""
+    try:
+        from . import _host as ext
+    except ImportError as e:
+        raise ImportError(f"{_HERE}/_host.so cannot be loaded ({e}): build it with `python -m paper_2506_01206_b200.build`") from e
+    return ext
+
+
+class _NotBuilt:
+    def __getattr__(self, name):
+        return getattr(_load_host(), name)
+
+
+try:
+    _host = _load_host()
+except ImportError:   # the package has to be importable for its own build
+    _host = _NotBuilt()
 
 # entry points whose arguments csrc/host.cpp marshals, in the order of its table
 _HOST_CALLS = ("mdraft_conv_scan_prefill", "mdraft_conv_scan_prefill_noalloc", "mdraft_tree_step", "mdraft_tree_step_proj",
-               "mdraft_state_commit", "mdraft_ssd_prefill", "mdraft_ssd_tree_step")
+               "mdraft_state_commit", "mdraft_ssd_prefill", "mdraft_ssd_tree_step", "mdraft_conv_scan_prefill_stack",
+               "mdraft_tree_step_stack")
 
 
 def load_library(path: Optional[str] = None):
@@ -95,6 +117,10 @@ def load_library(path: Optional[str] = None):
     lib.mdraft_version.argtypes = []
     lib.mdraft_prefill_workspace_bytes.restype = C.c_size_t
     lib.mdraft_prefill_workspace_bytes.argtypes = [C.POINTER(_Layer), i32, i32, i32, C.POINTER(_PrefillOpts)]
+    lib.mdraft_prefill_stack_workspace_bytes.restype = C.c_size_t
+    lib.mdraft_prefill_stack_workspace_bytes.argtypes = [C.POINTER(_Layer), i32, i32, i32, i32, C.POINTER(_PrefillOpts)]
+    lib.mdraft_prefill_stack_launches.restype = i32
+    lib.mdraft_prefill_stack_launches.argtypes = [C.POINTER(_Layer), i32, i32, i32, i32, C.POINTER(_PrefillOpts)]
     lib.mdraft_conv_scan_prefill.restype = C.c_int
     lib.mdraft_conv_scan_prefill.argtypes = [C.POINTER(_Layer), C.POINTER(_Cache), i32,
                                              vp, i64, vp, i64, vp, i64, vp, i64, vp, i64, vp, i64,
@@ -131,12 +157,8 @@ def load_library(path: Optional[str] = None):
                                          vp, i64, vp, i64, vp, i64, vp, i64, vp, i64, vp, i64,
                                          i32, vp, vp, i32, C.POINTER(i32), vp, vp]
     # The calls that are issued once per layer go through the extension, which is given the addresses of this library.
-    if _host is None:
-        try:
-            from . import _host as ext
-        except ImportError as e:
-            raise ImportError(f"{_HERE}/_host.so cannot be loaded ({e}): build it with `python -m paper_2506_01206_b200.build`") from e
-        _host = ext
+    if isinstance(_host, _NotBuilt):
+        _host = _load_host()
     lib.entry = _host.table([C.cast(getattr(lib, n), C.c_void_p).value for n in _HOST_CALLS])
     if path is None:
         _lib = lib
@@ -257,6 +279,44 @@ def mdraft_conv_scan_prefill(layer: Layer, cache: Optional[StateCache], layer_in
                        workspace, chunk_len, dev_status, stream, flags, phase_events)
     if rc != 0:
         raise MdraftError(rc, "mdraft_conv_scan_prefill")
+
+
+def mdraft_prefill_stack_workspace_bytes(layer: Layer, n_layers: int, total_tokens: int, n_seq: int, max_seqlen: int) -> int:
+    cl = layer.c()
+    return int(load_library().mdraft_prefill_stack_workspace_bytes(C.byref(cl), int(n_layers), int(total_tokens), int(n_seq), int(max_seqlen), None))
+
+
+def mdraft_prefill_stack_launches(layer: Layer, n_layers: int, total_tokens: int, n_seq: int, max_seqlen: int) -> int:
+    cl = layer.c()
+    return int(load_library().mdraft_prefill_stack_launches(C.byref(cl), int(n_layers), int(total_tokens), int(n_seq), int(max_seqlen), None))
+
+
+def mdraft_conv_scan_prefill_stack(layers: Sequence[Layer], which: Sequence[int], cache: StateCache, inputs, outs,
+                                   cu_seqlens: Optional[torch.Tensor], max_seqlen: int, init_slot: Optional[torch.Tensor] = None,
+                                   final_slot: Optional[torch.Tensor] = None, workspace: Optional[torch.Tensor] = None,
+                                   dev_status: Optional[torch.Tensor] = None, stream=None) -> bool:
+    """The prefill of layers[l] for l in `which` side by side (inputs[l] = (x, z, dt, B, C)).  False, with nothing launched,
+    when they have to run one after another: a layer's output overlaps another's tensors, a layer comes twice, widths or
+    row counts differ, or the workspace is too small for all at once."""
+    rc = _host.prefill_stack(_entry(), layers, which, cache, inputs, outs, cu_seqlens, max_seqlen, init_slot, final_slot, workspace,
+                             dev_status, stream)
+    if rc is None or rc == MDRAFT_ERR_WORKSPACE:
+        return False
+    if rc != 0:
+        raise MdraftError(rc, "mdraft_conv_scan_prefill_stack")
+    return True
+
+
+def mdraft_tree_step_stack(layers: Sequence[Layer], which: Sequence[int], cache: StateCache, inputs, outs, parent_slot: torch.Tensor,
+                           node_slot: torch.Tensor, level_offsets: Optional[Sequence[int]] = None,
+                           dev_status: Optional[torch.Tensor] = None, stream=None) -> bool:
+    """The tree step of layers[l] for l in `which`, every level of all layers in one launch.  False as above."""
+    rc = _host.tree_step_stack(_entry(), layers, which, cache, inputs, outs, parent_slot, node_slot, level_offsets, dev_status, stream)
+    if rc is None:
+        return False
+    if rc != 0:
+        raise MdraftError(rc, "mdraft_tree_step_stack")
+    return True
 
 
 NOALLOC_SCRATCH_BYTES = 8 << 20

@@ -5,6 +5,8 @@
 
 #include <string.h>
 
+#include <atomic>
+
 #include "commit.cuh"
 #include "common.cuh"
 #include "prefill.cuh"
@@ -21,11 +23,14 @@ constexpr int kSmCountB200 = 148;
 // SMs of the current device; the B200's count when no device can be asked (the workspace query also runs where there
 // is none, and must then give the size the call will want on the B200 it is planned for).
 int sm_count() {
-    int dev = 0, n = 0;
+    static std::atomic<int> known{0};  // every device this library runs on is the same part
+    int dev = 0, n = known.load(std::memory_order_relaxed);
+    if (n > 0) return n;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) {
         (void)cudaGetLastError();
         return kSmCountB200;
     }
+    known.store(n, std::memory_order_relaxed);
     return n;
 }
 
@@ -86,7 +91,10 @@ struct PrefillPlan {
     int n_chunks_bound;  // upper bound on the number of chunks
     bool chunked;
     bool wide;           // 512-channel blocks (one per SM) instead of 128-channel blocks
-    size_t off_q, off_sd, off_h0, off_conv, bytes;
+    bool longest_first;  // unsplit sequences of different lengths, handed out longest first
+    bool two_per_sm;     // keep two blocks per SM (of the four that fit)
+    size_t off_q, off_sd, off_h0, off_conv, layer_bytes;
+    size_t bytes;        // what the workspace query answers: the call's layers, split
 };
 
 // Chunk length: split the token axis until every SM holds kBlocksPerSm blocks of kPrefillThreads channels (one
@@ -96,25 +104,40 @@ struct PrefillPlan {
 // uneven sequences and keeps every SM busy to the end (32 packed sequences of 1k-8k tokens: 1607 -> 1512 us).
 constexpr int kBlocksPerSm = 4, kMinChunk = 32, kOneWaveMax = 256, kManyWavesChunk = 128, kManyWavesChunkBatched = 256;
 
-PrefillPlan plan_prefill(const mdraft_layer* L, int T, int n_seq, int max_seqlen, const mdraft_prefill_opts* opts) {
+// Splitting a sequence costs a second pass over its tokens (0.75 of the output pass, for all chunks but the last) and two more
+// launches; not splitting it leaves one block per sequence, layer and 128 channels.  SM cycles a token of a block takes (128
+// channels, A = powers; a general A scales both sides alike), measured with 1, 2 and 4 resident blocks, and in wide blocks:
+constexpr double kCycOne = 228, kCycTwo = 174, kCycFour = 163, kCycWide = 144, kSplitCycles = 16000;
+
+// Estimated cycles of the unsplit form: bound by the longest sequence running alone, or by what the fullest SM is given.
+double unsplit_cycles(int64_t blocks_per_seq, int T, int n_seq, int max_seqlen, int sms) {
+    const double per_sm = (double)blocks_per_seq * T / sms, deepest = (double)((blocks_per_seq * n_seq + sms - 1) / sms) * max_seqlen;
+    double m = per_sm + 0.5 * T / n_seq;   // longest first: the last blocks to start are the short ones
+    if (m > deepest) m = deepest;
+    if (m < max_seqlen) m = max_seqlen;
+    return blocks_per_seq * n_seq <= sms ? kCycOne * max_seqlen : (kCycTwo * m > kCycOne * max_seqlen ? kCycTwo * m : kCycOne * max_seqlen);
+}
+
+PrefillPlan plan_prefill(const mdraft_layer* L, int n_layers, int T, int n_seq, int max_seqlen, const mdraft_prefill_opts* opts) {
     PrefillPlan pl;
     const int D = L->d_inner;
     const int wide_cols = kPrefillThreads * kPrefillWideBoxes;
-    const int ch_blocks = (D + kPrefillThreads - 1) / kPrefillThreads;
-    const int ch_blocks_wide = (D + wide_cols - 1) / wide_cols;
+    const int64_t ch_blocks = (int64_t)n_layers * ((D + kPrefillThreads - 1) / kPrefillThreads);
+    const int64_t ch_blocks_wide = (int64_t)n_layers * ((D + wide_cols - 1) / wide_cols);
     const int forced = opts ? opts->block_channels : 0;
+    const int sms = sm_count();
     // Wide blocks pay off when they fill the machine in one wave: every SM then runs ONE block whose 16 channel warps
     // advance together and finish together (four narrow blocks per SM finish one after another and leave the SM to
     // the last of them).  They need the channel count to (nearly) fill whole 512-channel blocks.
-    bool wide = forced == wide_cols || (forced == 0 && (int64_t)ch_blocks_wide * wide_cols * 9 <= (int64_t)D * 10);
+    bool wide = forced == wide_cols || (forced == 0 && ch_blocks_wide * wide_cols * 9 <= (int64_t)n_layers * D * 10);
     int Lc;
+    bool unsplit = false;
     if (opts && opts->chunk_len > 0) {
         Lc = opts->chunk_len < 4 ? 4 : opts->chunk_len;
     } else {
-        const int sms = sm_count();
-        int want = wide ? sms / ch_blocks_wide : sms * kBlocksPerSm / ch_blocks;
+        int64_t want = wide ? sms / ch_blocks_wide : sms * kBlocksPerSm / ch_blocks;
         if (want < 1) want = 1;
-        Lc = (T + want - 1) / want;
+        Lc = (int)((T + want - 1) / want);
         if (Lc < kMinChunk) Lc = kMinChunk;
         // A single sequence in wide blocks stays in one wave at any length: 49 x 3 equal chunks finish together
         // (32768 tokens: 344 us against 372-376 for several waves of short chunks; 65536: 675 against 724).  Packed
@@ -124,24 +147,40 @@ PrefillPlan plan_prefill(const mdraft_layer* L, int T, int n_seq, int max_seqlen
             Lc = n_seq > 1 ? kManyWavesChunkBatched : kManyWavesChunk;
             if (forced == 0) wide = false;
         }
+        const double n_chunks = n_seq + (double)T / Lc, work = (double)ch_blocks * T / sms * (wide ? kCycWide : kCycFour);
+        const double split = (work > kCycOne * Lc ? work : kCycOne * Lc) * (1.0 + 0.75 * (n_chunks - n_seq) / n_chunks) + kSplitCycles;
+        unsplit = forced == 0 && unsplit_cycles(ch_blocks, T, n_seq, max_seqlen, sms) <= split;
     }
-    pl.wide = wide;
+    pl.wide = wide && !unsplit;
     pl.chunked = Lc < max_seqlen;
-    if (!pl.chunked) {
-        pl.chunk_len = INT_MAX / 2;
-        pl.n_chunks_bound = n_seq;
-        pl.off_q = pl.off_sd = pl.off_h0 = pl.off_conv = 0;
-        pl.bytes = 0;
-        return pl;
+    pl.longest_first = pl.two_per_sm = false;
+    pl.chunk_len = INT_MAX / 2;
+    pl.n_chunks_bound = n_seq;
+    pl.off_q = pl.off_sd = pl.off_h0 = pl.off_conv = pl.layer_bytes = pl.bytes = 0;
+    if (pl.chunked) {
+        const int bound = n_seq + T / Lc;
+        const size_t Dz = (size_t)D;
+        pl.off_q = 0;
+        pl.off_sd = align_up(pl.off_q + (size_t)bound * Dz * kN * sizeof(float), 256);
+        pl.off_h0 = align_up(pl.off_sd + (size_t)bound * Dz * sizeof(float), 256);
+        pl.off_conv = align_up(pl.off_h0 + (size_t)n_seq * Dz * kN * sizeof(float), 256);
+        pl.layer_bytes = align_up(pl.off_conv + (size_t)n_seq * (kW - 1) * Dz * elem_size(L->act), 256);
+        // For one layer the query answers for the split form whichever form is taken: a workspace made for one batch then
+        // serves another of its size whose longest sequence is longer.
+        pl.bytes = pl.layer_bytes * n_layers;
+        if (!unsplit) {
+            pl.chunk_len = Lc;
+            pl.n_chunks_bound = bound;
+        }
     }
-    pl.chunk_len = Lc;
-    pl.n_chunks_bound = n_seq + T / Lc;
-    const size_t Dz = (size_t)D;
-    pl.off_q = 0;
-    pl.off_sd = align_up(pl.off_q + (size_t)pl.n_chunks_bound * Dz * kN * sizeof(float), 256);
-    pl.off_h0 = align_up(pl.off_sd + (size_t)pl.n_chunks_bound * Dz * sizeof(float), 256);
-    pl.off_conv = align_up(pl.off_h0 + (size_t)n_seq * Dz * kN * sizeof(float), 256);
-    pl.bytes = align_up(pl.off_conv + (size_t)n_seq * (kW - 1) * Dz * elem_size(L->act), 256);
+    if (unsplit) {
+        pl.chunked = false;
+        // Two blocks per SM while that holds the grid, or when lengths differ: a call that starts while the one before it
+        // drains must not stack three blocks on one SM and one on another (measured 460 against 370 us for 288 blocks), and
+        // the longest sequences set the time, which they take less of with one neighbour than with three.
+        pl.longest_first = n_seq > 1 && n_seq <= kPrefillMaxRanked;
+        pl.two_per_sm = pl.longest_first || ch_blocks * n_seq <= 2 * sms;
+    }
     return pl;
 }
 
@@ -175,6 +214,90 @@ bool encode_matrix(CUtensorMap* m, const void* base, int act, int64_t rows, int6
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Arguments of a call over several layers: the layers share a cache, so width, states, taps and type must agree.
+int check_stack(int32_t n_layers, const mdraft_layer* layers, const int32_t* layer_index, const mdraft_io* io) {
+    if (n_layers <= 0 || !layers || !layer_index || !io) return MDRAFT_ERR_INVALID_ARG;
+    for (int32_t i = 0; i < n_layers; ++i) {
+        if (int rc = check_layer(layers + i)) return rc;
+        if (layers[i].d_inner != layers->d_inner || layers[i].act != layers->act) return MDRAFT_ERR_UNSUPPORTED;
+    }
+    return MDRAFT_OK;
+}
+
+int check_io(const mdraft_io& v, const mdraft_layer& L, bool required) {
+    const bool all = required && !(L.flags & MDRAFT_CONV_ONLY);
+    int rc;
+    if ((rc = check_matrix(v.x, v.ldx, L.d_inner, L.act, required))) return rc;
+    if ((rc = check_matrix(v.out, v.ldo, L.d_inner, L.act, required))) return rc;
+    if ((rc = check_matrix(v.z, v.ldz, L.d_inner, L.act, all))) return rc;
+    if ((rc = check_matrix(v.dt, v.lddt, L.d_inner, L.act, all))) return rc;
+    if ((rc = check_matrix(v.B, v.ldb, kN, L.act, all))) return rc;
+    return check_matrix(v.C, v.ldc, kN, L.act, all);
+}
+
+// How many of the next n layers one launch takes: those with the first one's flags, at most `most`; flags beyond softplus and
+// A = powers (the split modes, whose callers work layer by layer) go one at a time.
+int32_t run_length(int32_t n, const mdraft_layer* layers, int32_t most) {
+    if ((layers->flags & ~(uint32_t)MDRAFT_A_POWERS) != (uint32_t)MDRAFT_DT_SOFTPLUS) return 1;
+    int32_t k = 1;
+    while (k < n && k < most && layers[k].flags == layers->flags) ++k;
+    return k;
+}
+
+struct PrefillCall {
+    const mdraft_cache* cache;
+    int32_t total_tokens, n_seq;
+    const int32_t *cu_seqlens, *init_slot, *final_slot;
+    char* workspace;
+    const mdraft_prefill_opts* opts;
+    int32_t* dev_status;
+    cudaStream_t stream;
+};
+
+// One launch sequence of the prefill over n_layers (at most ML) layers with the same flags.
+template <int ML>
+int run_prefill(const PrefillCall& call, const PrefillPlan& pl, int32_t n_layers, const mdraft_layer* layers, const int32_t* layer_index, const mdraft_io* io) {
+    PrefillBatch<ML> b;
+    PrefillArgs& a = b.c;
+    const int act = layers->act, D = layers->d_inner;
+    if (call.cache) {
+        a.pool = pool_dev(call.cache, act, 0);
+        a.ssm_layer_stride = call.cache->ssm_layer_stride; a.conv_layer_stride = call.cache->conv_layer_stride;
+    } else {
+        a.pool.ssm = nullptr; a.pool.conv = nullptr; a.pool.ssm_slot_stride = 0; a.pool.conv_slot_stride = 0; a.pool.n_slots = 0;
+        a.ssm_layer_stride = a.conv_layer_stride = 0;
+    }
+    a.n_layers = n_layers; a.d_inner = D;
+    a.T = call.total_tokens; a.n_seq = call.n_seq; a.chunk_len = pl.chunk_len; a.n_chunks_bound = pl.n_chunks_bound;
+    a.longest_first = pl.longest_first;
+    a.cu = call.cu_seqlens; a.init_slot = call.init_slot; a.final_slot = call.final_slot;
+    char* ws = call.workspace;
+    a.ws_q = pl.chunked ? reinterpret_cast<float*>(ws + pl.off_q) : nullptr;
+    a.ws_sd = pl.chunked ? reinterpret_cast<float*>(ws + pl.off_sd) : nullptr;
+    a.ws_h0 = pl.chunked ? reinterpret_cast<float*>(ws + pl.off_h0) : nullptr;
+    a.ws_conv = pl.chunked ? static_cast<void*>(ws + pl.off_conv) : nullptr;
+    a.ws_layer_bytes = (int64_t)pl.layer_bytes;
+    a.dev_status = call.dev_status;
+    a.pdl_inputs_ready = pl.chunked ? 1 : 0;  // the summary pass waits for the producer of the inputs on behalf of all three kernels
+    a.ev_state = call.opts ? static_cast<cudaEvent_t>(call.opts->event_after_chunk_state) : nullptr;
+    a.ev_carry = call.opts ? static_cast<cudaEvent_t>(call.opts->event_after_carry_scan) : nullptr;
+    const bool rows = call.total_tokens > 0;  // with no tokens at all (only empty sequences) nothing is ever copied: empty descriptors
+    for (int32_t i = 0; i < n_layers; ++i) {
+        PrefillLayer& p = b.l[i];
+        const mdraft_io& v = io[i];
+        p.L = layer_dev(layers + i);
+        p.layer_index = layer_index[i];
+        p.x = v.x; p.ldx = v.ldx; p.out = v.out; p.ldo = v.ldo;
+        if (!encode_matrix(&p.maps.x, rows ? v.x : nullptr, act, a.T, D, v.ldx, kPrefillThreads) ||
+            !encode_matrix(&p.maps.dt, rows ? v.dt : nullptr, act, a.T, D, v.lddt, kPrefillThreads) ||
+            !encode_matrix(&p.maps.z, rows ? v.z : nullptr, act, a.T, D, v.ldz, kPrefillThreads) ||
+            !encode_matrix(&p.maps.B, rows ? v.B : nullptr, act, a.T, kN, v.ldb, kN) ||
+            !encode_matrix(&p.maps.C, rows ? v.C : nullptr, act, a.T, kN, v.ldc, kN))
+            return MDRAFT_ERR_CUDA;
+    }
+    return launch_prefill<ML>(b, act, pl.chunked, pl.wide, pl.two_per_sm, call.stream) == cudaSuccess ? MDRAFT_OK : MDRAFT_ERR_CUDA;
+}
+
 __global__ void classify_A_kernel(const float* A, int D, int N, int32_t* res) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= D * N) return;
@@ -204,9 +327,28 @@ int mdraft_version(void) { return 100; }
 
 size_t mdraft_prefill_workspace_bytes(const mdraft_layer* layer, int32_t total_tokens, int32_t n_seq, int32_t max_seqlen,
                                       const mdraft_prefill_opts* opts) {
-    if (check_layer(layer) != MDRAFT_OK || total_tokens <= 0 || n_seq <= 0 || max_seqlen <= 0) return 0;
+    return mdraft_prefill_stack_workspace_bytes(layer, 1, total_tokens, n_seq, max_seqlen, opts);
+}
+
+size_t mdraft_prefill_stack_workspace_bytes(const mdraft_layer* layer, int32_t n_layers, int32_t total_tokens, int32_t n_seq,
+                                            int32_t max_seqlen, const mdraft_prefill_opts* opts) {
+    if (check_layer(layer) != MDRAFT_OK || n_layers <= 0 || total_tokens <= 0 || n_seq <= 0 || max_seqlen <= 0) return 0;
     // No sequence is longer than the whole batch: a looser static bound must not change the plan.
-    return plan_prefill(layer, total_tokens, n_seq, max_seqlen < total_tokens ? max_seqlen : total_tokens, opts).bytes;
+    if (n_layers > kPrefillMaxLayers) n_layers = kPrefillMaxLayers;  // launches of one call share the workspace
+    const PrefillPlan pl = plan_prefill(layer, n_layers, total_tokens, n_seq, max_seqlen < total_tokens ? max_seqlen : total_tokens, opts);
+    return n_layers == 1 || pl.chunked ? pl.bytes : 0;
+}
+
+int32_t mdraft_prefill_stack_launches(const mdraft_layer* layer, int32_t n_layers, int32_t total_tokens, int32_t n_seq,
+                                      int32_t max_seqlen, const mdraft_prefill_opts* opts) {
+    if (check_layer(layer) != MDRAFT_OK || n_layers <= 0 || total_tokens <= 0 || n_seq <= 0 || max_seqlen <= 0) return 0;
+    if (max_seqlen > total_tokens) max_seqlen = total_tokens;
+    int32_t n = 0;
+    for (int32_t l0 = 0; l0 < n_layers; l0 += kPrefillMaxLayers) {
+        const int32_t nl = n_layers - l0 < kPrefillMaxLayers ? n_layers - l0 : kPrefillMaxLayers;
+        n += !plan_prefill(layer, nl, total_tokens, n_seq, max_seqlen, opts).chunked ? 1 : (layer->flags & MDRAFT_CONV_ONLY) ? 2 : 3;
+    }
+    return n;
 }
 
 int mdraft_conv_scan_prefill(const mdraft_layer* layer, const mdraft_cache* cache, int32_t layer_index,
@@ -215,7 +357,16 @@ int mdraft_conv_scan_prefill(const mdraft_layer* layer, const mdraft_cache* cach
                              int32_t total_tokens, int32_t n_seq, int32_t max_seqlen, const int32_t* cu_seqlens,
                              const int32_t* init_slot, const int32_t* final_slot, void* workspace, size_t workspace_bytes,
                              const mdraft_prefill_opts* opts, int32_t* dev_status, void* stream) {
-    int rc = check_layer(layer);
+    const mdraft_io io = {x, z, dt, B, C, out, ldx, ldz, lddt, ldb, ldc, ldo};
+    return mdraft_conv_scan_prefill_stack(1, layer, cache, &layer_index, &io, total_tokens, n_seq, max_seqlen, cu_seqlens, init_slot,
+                                          final_slot, workspace, workspace_bytes, opts, dev_status, stream);
+}
+
+int mdraft_conv_scan_prefill_stack(int32_t n_layers, const mdraft_layer* layers, const mdraft_cache* cache, const int32_t* layer_index,
+                                   const mdraft_io* io, int32_t total_tokens, int32_t n_seq, int32_t max_seqlen,
+                                   const int32_t* cu_seqlens, const int32_t* init_slot, const int32_t* final_slot, void* workspace,
+                                   size_t workspace_bytes, const mdraft_prefill_opts* opts, int32_t* dev_status, void* stream) {
+    int rc = check_stack(n_layers, layers, layer_index, io);
     if (rc) return rc;
     if (total_tokens < 0 || n_seq < 0 || max_seqlen < 0) return MDRAFT_ERR_INVALID_ARG;
     if (opts) {
@@ -225,59 +376,42 @@ int mdraft_conv_scan_prefill(const mdraft_layer* layer, const mdraft_cache* cach
         if (opts->block_channels != 0 && opts->block_channels != kPrefillThreads && opts->block_channels != kPrefillThreads * kPrefillWideBoxes)
             return MDRAFT_ERR_INVALID_ARG;
     }
-    const bool needs_pool = init_slot || final_slot;
-    if (needs_pool || cache) {
-        rc = check_cache(cache, layer->d_inner, layer->act, layer_index);
-        if (rc) return rc;
+    const int D = layers->d_inner, act = layers->act;
+    if (init_slot || final_slot || cache) {
+        for (int32_t i = 0; i < n_layers; ++i)
+            if ((rc = check_cache(cache, D, act, layer_index[i]))) return rc;
     }
     if (n_seq == 0) return MDRAFT_OK;
     if (!cu_seqlens && n_seq != 1) return MDRAFT_ERR_INVALID_ARG;  // offsets may be omitted for a single sequence only
-    const bool conv_only = layer->flags & MDRAFT_CONV_ONLY;
-    const int D = layer->d_inner, act = layer->act;
     const bool have_rows = total_tokens > 0;
-    if ((rc = check_matrix(x, ldx, D, act, have_rows))) return rc;
-    if ((rc = check_matrix(out, ldo, D, act, have_rows))) return rc;
-    if ((rc = check_matrix(z, ldz, D, act, have_rows && !conv_only))) return rc;
-    if ((rc = check_matrix(dt, lddt, D, act, have_rows && !conv_only))) return rc;
-    if ((rc = check_matrix(B, ldb, kN, act, have_rows && !conv_only))) return rc;
-    if ((rc = check_matrix(C, ldc, kN, act, have_rows && !conv_only))) return rc;
+    for (int32_t i = 0; i < n_layers; ++i)
+        if ((rc = check_io(io[i], layers[i], have_rows))) return rc;
     // The same bound as in the workspace query: no sequence is longer than the whole batch.  A batch of empty
     // sequences therefore never takes the chunked path (and needs no workspace), whatever static bound was given.
     const int plan_tokens = total_tokens > 0 ? total_tokens : 1;
     if (max_seqlen > plan_tokens) max_seqlen = plan_tokens;
     if (max_seqlen < 1) max_seqlen = 1;
 
-    PrefillPlan pl = plan_prefill(layer, plan_tokens, n_seq, max_seqlen, opts);
-    if (pl.chunked) {
-        if (!workspace || workspace_bytes < pl.bytes) return MDRAFT_ERR_WORKSPACE;
-        if (reinterpret_cast<uintptr_t>(workspace) & 255u) return MDRAFT_ERR_MISALIGNED;
-    }
-    PrefillArgs a;
-    a.L = layer_dev(layer);
-    if (cache) a.pool = pool_dev(cache, act, layer_index);
-    else { a.pool.ssm = nullptr; a.pool.conv = nullptr; a.pool.ssm_slot_stride = 0; a.pool.conv_slot_stride = 0; a.pool.n_slots = 0; }
-    a.x = x; a.z = z; a.dt = dt; a.B = B; a.C = C; a.out = out;
-    a.ldx = ldx; a.ldz = ldz; a.lddt = lddt; a.ldb = ldb; a.ldc = ldc; a.ldo = ldo;
-    a.T = total_tokens; a.n_seq = n_seq; a.chunk_len = pl.chunk_len; a.n_chunks_bound = pl.n_chunks_bound;
-    a.cu = cu_seqlens; a.init_slot = init_slot; a.final_slot = final_slot;
-    char* ws = static_cast<char*>(workspace);
-    a.ws_q = pl.chunked ? reinterpret_cast<float*>(ws + pl.off_q) : nullptr;
-    a.ws_sd = pl.chunked ? reinterpret_cast<float*>(ws + pl.off_sd) : nullptr;
-    a.ws_h0 = pl.chunked ? reinterpret_cast<float*>(ws + pl.off_h0) : nullptr;
-    a.ws_conv = pl.chunked ? static_cast<void*>(ws + pl.off_conv) : nullptr;
-    a.dev_status = dev_status;
-    if (a.n_chunks_bound > 65535) return MDRAFT_ERR_UNSUPPORTED;
-    a.ev_state = opts ? static_cast<cudaEvent_t>(opts->event_after_chunk_state) : nullptr;
-    a.ev_carry = opts ? static_cast<cudaEvent_t>(opts->event_after_carry_scan) : nullptr;
-    PrefillMaps maps;  // with no tokens at all (only empty sequences) nothing is ever copied: empty descriptors
-    if (!encode_matrix(&maps.x, have_rows ? x : nullptr, act, total_tokens, D, ldx, kPrefillThreads) ||
-        !encode_matrix(&maps.dt, have_rows ? dt : nullptr, act, total_tokens, D, lddt, kPrefillThreads) ||
-        !encode_matrix(&maps.z, have_rows ? z : nullptr, act, total_tokens, D, ldz, kPrefillThreads) ||
-        !encode_matrix(&maps.B, have_rows ? B : nullptr, act, total_tokens, kN, ldb, kN) ||
-        !encode_matrix(&maps.C, have_rows ? C : nullptr, act, total_tokens, kN, ldc, kN))
-        return MDRAFT_ERR_CUDA;
-    cudaError_t e = launch_prefill(a, maps, act, pl.chunked, pl.wide, static_cast<cudaStream_t>(stream));
-    return e == cudaSuccess ? MDRAFT_OK : MDRAFT_ERR_CUDA;
+    const PrefillCall call = {cache, total_tokens, n_seq, cu_seqlens, init_slot, final_slot, static_cast<char*>(workspace), opts, dev_status,
+                        static_cast<cudaStream_t>(stream)};
+    for (int pass = 0; pass < 2; ++pass)  // every launch is checked before the first is made
+        for (int32_t l0 = 0; l0 < n_layers;) {
+            const int32_t nl = run_length(n_layers - l0, layers + l0, kPrefillMaxLayers);
+            const PrefillPlan pl = plan_prefill(layers + l0, nl, plan_tokens, n_seq, max_seqlen, opts);
+            if (pass == 0) {
+                if (pl.n_chunks_bound > 65535 || (int64_t)nl * n_seq > 65535) return MDRAFT_ERR_UNSUPPORTED;
+                if (pl.chunked) {
+                    if (!workspace || workspace_bytes < pl.bytes) return MDRAFT_ERR_WORKSPACE;
+                    if (reinterpret_cast<uintptr_t>(workspace) & 255u) return MDRAFT_ERR_MISALIGNED;
+                }
+            } else {
+                const int r = nl == 1 ? run_prefill<1>(call, pl, nl, layers + l0, layer_index + l0, io + l0)
+                                      : run_prefill<kPrefillMaxLayers>(call, pl, nl, layers + l0, layer_index + l0, io + l0);
+                if (r) return r;
+            }
+            l0 += nl;
+        }
+    return MDRAFT_OK;
 }
 
 int mdraft_tree_step(const mdraft_layer* layer, const mdraft_cache* cache, int32_t layer_index, const void* x, int64_t ldx,
@@ -285,9 +419,18 @@ int mdraft_tree_step(const mdraft_layer* layer, const mdraft_cache* cache, int32
                      int64_t ldc, void* out, int64_t ldo, int32_t n_nodes, const int32_t* parent_slot,
                      const int32_t* node_slot, int32_t n_levels, const int32_t* level_offsets, int32_t* dev_status,
                      void* stream) {
-    int rc = check_layer(layer);
+    const mdraft_io io = {x, z, dt, B, C, out, ldx, ldz, lddt, ldb, ldc, ldo};
+    return mdraft_tree_step_stack(1, layer, cache, &layer_index, &io, n_nodes, parent_slot, node_slot, n_levels, level_offsets, dev_status, stream);
+}
+
+int mdraft_tree_step_stack(int32_t n_layers, const mdraft_layer* layers, const mdraft_cache* cache, const int32_t* layer_index,
+                           const mdraft_io* io, int32_t n_nodes, const int32_t* parent_slot, const int32_t* node_slot,
+                           int32_t n_levels, const int32_t* level_offsets, int32_t* dev_status, void* stream) {
+    int rc = check_stack(n_layers, layers, layer_index, io);
     if (rc) return rc;
-    if ((rc = check_cache(cache, layer->d_inner, layer->act, layer_index))) return rc;
+    const int D = layers->d_inner, act = layers->act;
+    for (int32_t i = 0; i < n_layers; ++i)
+        if ((rc = check_cache(cache, D, act, layer_index[i]))) return rc;
     if (n_nodes < 0 || n_levels < 0) return MDRAFT_ERR_INVALID_ARG;
     if (n_nodes == 0) return MDRAFT_OK;
     if (!parent_slot || !node_slot) return MDRAFT_ERR_INVALID_ARG;
@@ -297,30 +440,32 @@ int mdraft_tree_step(const mdraft_layer* layer, const mdraft_cache* cache, int32
         for (int l = 0; l < n_levels; ++l)
             if (level_offsets[l + 1] < level_offsets[l]) return MDRAFT_ERR_INVALID_ARG;
     }
-    const bool conv_only = layer->flags & MDRAFT_CONV_ONLY;
-    const int D = layer->d_inner, act = layer->act;
-    if ((rc = check_matrix(x, ldx, D, act, true))) return rc;
-    if ((rc = check_matrix(out, ldo, D, act, true))) return rc;
-    if ((rc = check_matrix(z, ldz, D, act, !conv_only))) return rc;
-    if ((rc = check_matrix(dt, lddt, D, act, !conv_only))) return rc;
-    if ((rc = check_matrix(B, ldb, kN, act, !conv_only))) return rc;
-    if ((rc = check_matrix(C, ldc, kN, act, !conv_only))) return rc;
+    for (int32_t i = 0; i < n_layers; ++i)
+        if ((rc = check_io(io[i], layers[i], true))) return rc;
 
     TreeArgs a;
-    a.L = layer_dev(layer);
-    a.pool = pool_dev(cache, act, layer_index);
-    a.x = x; a.z = z; a.dt = dt; a.B = B; a.C = C; a.out = out;
-    a.ldx = ldx; a.ldz = ldz; a.lddt = lddt; a.ldb = ldb; a.ldc = ldc; a.ldo = ldo;
+    a.pool = pool_dev(cache, act, 0);
+    a.ssm_layer_stride = cache->ssm_layer_stride; a.conv_layer_stride = cache->conv_layer_stride;
     a.parent_slot = parent_slot; a.node_slot = node_slot; a.dev_status = dev_status;
     const int levels = level_offsets ? n_levels : 1;
     int launched = 0;  // an empty level launches nothing and must not count: the chaining rules go by kernels ahead
-    for (int l = 0; l < levels; ++l) {
-        a.level_in_call = launched;
-        a.lvl_begin = level_offsets ? level_offsets[l] : 0;
-        a.lvl_end = level_offsets ? level_offsets[l + 1] : n_nodes;
-        if (a.lvl_end == a.lvl_begin) continue;
-        if (launch_tree_step(a, act, static_cast<cudaStream_t>(stream)) != cudaSuccess) return MDRAFT_ERR_CUDA;
-        ++launched;
+    for (int32_t l0 = 0; l0 < n_layers;) {
+        const int32_t nl = run_length(n_layers - l0, layers + l0, kTreeMaxLayers);
+        TreeLayers<kTreeMaxLayers> tl;
+        for (int32_t i = 0; i < nl; ++i) {
+            const mdraft_io& v = io[l0 + i];
+            tl.l[i] = {layer_dev(layers + l0 + i), v.x, v.z, v.dt, v.B, v.C, v.out, v.ldx, v.ldz, v.lddt, v.ldb, v.ldc, v.ldo, layer_index[l0 + i]};
+        }
+        a.n_layers = nl;
+        for (int l = 0; l < levels; ++l) {
+            a.level_in_call = launched;
+            a.lvl_begin = level_offsets ? level_offsets[l] : 0;
+            a.lvl_end = level_offsets ? level_offsets[l + 1] : n_nodes;
+            if (a.lvl_end == a.lvl_begin) continue;
+            if (launch_tree_step(a, tl, act, static_cast<cudaStream_t>(stream)) != cudaSuccess) return MDRAFT_ERR_CUDA;
+            ++launched;
+        }
+        l0 += nl;
     }
     return MDRAFT_OK;
 }

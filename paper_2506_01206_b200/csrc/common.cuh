@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "../../include/mdraft.h"
 
 namespace mdraft {
@@ -95,6 +97,21 @@ struct PoolDev {
     int64_t conv_slot_stride;
     int n_slots;
 };
+
+// A kernel that wants more dynamic shared memory than a launch gets by default has the limit raised once per device: it is a
+// property of the loaded function, and asking for it on every call costs host time.
+template <auto kKernel>
+inline cudaError_t allow_smem(int bytes) {
+    if (bytes <= 48 * 1024) return cudaSuccess;
+    static std::atomic<uint64_t> done{0};  // bit = device
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 64 && (done.load(std::memory_order_acquire) >> dev & 1u)) return cudaSuccess;
+    const cudaError_t f = cudaFuncSetAttribute(kKernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (f == cudaSuccess && dev < 64) done.fetch_or(1ull << dev, std::memory_order_release);
+    return f;
+}
 
 __device__ __forceinline__ void flag(int32_t* dev_status, int bit) {
     if (dev_status) atomicOr(dev_status, bit);

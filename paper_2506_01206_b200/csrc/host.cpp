@@ -26,6 +26,8 @@ struct Entry {
     decltype(&mdraft_state_commit) commit;
     decltype(&mdraft_ssd_prefill) ssd_prefill;
     decltype(&mdraft_ssd_tree_step) ssd_tree_step;
+    decltype(&mdraft_conv_scan_prefill_stack) prefill_stack;
+    decltype(&mdraft_tree_step_stack) tree_step_stack;
 };
 
 struct Failed {};  // a Python exception is set
@@ -403,9 +405,92 @@ PyObject* ssd_tree_step(PyObject* const* a) {
     });
 }
 
+// The layers of a stack call, gathered; `apart` says whether they may run side by side.
+struct Stack {
+    std::vector<mdraft_layer> layers;
+    std::vector<int32_t> index;
+    std::vector<mdraft_io> io;
+    int64_t rows = 0;
+    bool apart = true;
+
+    struct Span { uintptr_t lo, hi; };
+    static Span span(const Matrix& m, int64_t cols, int64_t es) {
+        const uintptr_t p = reinterpret_cast<uintptr_t>(m.p);
+        return m.p && m.rows > 0 ? Span{p, p + (uintptr_t)(((m.rows - 1) * m.ld + cols) * es)} : Span{0, 0};
+    }
+    static bool meet(const Span& a, const Span& b) { return a.lo < b.hi && b.lo < a.hi; }
+
+    Stack(PyObject* layer_list, PyObject* which, PyObject* inputs, PyObject* outs) {
+        Ref w(PySequence_Fast(which, "layers to run"));
+        const Py_ssize_t n = PySequence_Fast_GET_SIZE(w.p);
+        std::vector<Span> in, out;
+        for (Py_ssize_t k = 0; k < n; ++k) {
+            const int64_t l = as_int(PySequence_Fast_GET_ITEM(w.p, k));
+            Ref lay(PySequence_GetItem(layer_list, l)), ins(PySequence_GetItem(inputs, l)), o(PySequence_GetItem(outs, l));
+            Ref f(PySequence_Fast(ins.p, "a layer's inputs are (x, z, dt, B, C)"));
+            if (PySequence_Fast_GET_SIZE(f.p) != 5) fail(PyExc_ValueError, "a layer's inputs are (x, z, dt, B, C)");
+            layers.push_back(layer_of(lay.p, Py_None));
+            index.push_back((int32_t)(l < 0 ? -1 : l));
+            const Matrix x(PySequence_Fast_GET_ITEM(f.p, 0), "x"), z(PySequence_Fast_GET_ITEM(f.p, 1), "z"), dt(PySequence_Fast_GET_ITEM(f.p, 2), "dt"),
+                B(PySequence_Fast_GET_ITEM(f.p, 3), "B"), C(PySequence_Fast_GET_ITEM(f.p, 4), "C"), y(o.p, "out");
+            io.push_back({x.p, z.p, dt.p, B.p, C.p, y.out(), x.ld, z.ld, dt.ld, B.ld, C.ld, y.ld});
+            const mdraft_layer& L = layers.back();
+            const int64_t es = L.act == MDRAFT_BF16 ? 2 : 4;
+            for (const Matrix* m : {&x, &z, &dt}) in.push_back(span(*m, L.d_inner, es));
+            in.push_back(span(B, L.d_state, es));
+            in.push_back(span(C, L.d_state, es));
+            out.push_back(span(y, L.d_inner, es));
+            if (k == 0) rows = x.rows;
+            apart = apart && x.rows == rows && l >= 0 && L.d_inner == layers[0].d_inner && L.act == layers[0].act;
+        }
+        // A layer that reads what another writes, or two that write the same rows or states, have to run one after another.
+        for (Py_ssize_t a = 0; a < n && apart; ++a)
+            for (Py_ssize_t b = 0; b < n && apart; ++b) {
+                if (a == b) continue;
+                apart = index[a] != index[b] && !meet(out[a], out[b]);
+                for (int i = 0; i < 5 && apart; ++i) apart = !meet(out[a], in[5 * b + i]);
+            }
+    }
+};
+
+// (table, layers, which, cache, inputs, outs, cu_seqlens, max_seqlen, init_slot, final_slot, workspace, dev_status, stream)
+// -> status, or None when the layers have to run one after another
+PyObject* prefill_stack(PyObject* const* a) {
+    const Stack k(a[1], a[2], a[4], a[5]);
+    if (!k.apart || k.layers.size() < 2) Py_RETURN_NONE;
+    const Cache c(a[3]);
+    const Sequences s(a[6], a[8], a[9]);
+    const int32_t longest = (int32_t)as_int(a[7]);
+    const Workspace ws(a[10]);
+    int32_t* st = static_cast<int32_t*>(mutable_data(a[11], "dev_status"));
+    void* stream = stream_of(a[12]);
+    const Entry& e = entry(a[0]);
+    return released([&] {
+        return e.prefill_stack((int32_t)k.layers.size(), k.layers.data(), c.get(), k.index.data(), k.io.data(), (int32_t)k.rows, (int32_t)s.n_seq,
+                               longest, s.cu, s.init, s.fin, ws.p, ws.bytes, nullptr, st, stream);
+    });
+}
+
+// (table, layers, which, cache, inputs, outs, parent_slot, node_slot, level_offsets, dev_status, stream) -> status or None, as above
+PyObject* tree_step_stack(PyObject* const* a) {
+    const Stack k(a[1], a[2], a[4], a[5]);
+    if (!k.apart || k.layers.size() < 2) Py_RETURN_NONE;
+    const Cache c(a[3]);
+    const Nodes n(a[6], a[7], k.rows);
+    const Levels lv(a[8]);
+    int32_t* st = static_cast<int32_t*>(mutable_data(a[9], "dev_status"));
+    void* stream = stream_of(a[10]);
+    const Entry& e = entry(a[0]);
+    return released([&] {
+        return e.tree_step_stack((int32_t)k.layers.size(), k.layers.data(), c.get(), k.index.data(), k.io.data(), (int32_t)k.rows, n.parent, n.node,
+                                 lv.count(), lv.get(), st, stream);
+    });
+}
+
 #define ENTRY(name) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(&guarded<name>)), METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {ENTRY(table), ENTRY(prefill), ENTRY(prefill_noalloc), ENTRY(tree_step), ENTRY(tree_step_proj),
-                         ENTRY(commit), ENTRY(ssd_prefill), ENTRY(ssd_tree_step), {nullptr, nullptr, 0, nullptr}};
+                         ENTRY(commit), ENTRY(ssd_prefill), ENTRY(ssd_tree_step), ENTRY(prefill_stack), ENTRY(tree_step_stack),
+                         {nullptr, nullptr, 0, nullptr}};
 
 PyModuleDef module_def = {PyModuleDef_HEAD_INIT, "_host", "argument marshalling for libmdraft.so", -1, methods, nullptr, nullptr, nullptr, nullptr};
 

@@ -267,6 +267,35 @@ struct ChannelScan {
     }
 };
 
+template <typename T>
+__device__ __forceinline__ T* at_bytes(T* p, int64_t off) { return reinterpret_cast<T*>(reinterpret_cast<char*>(p) + off); }  // T may be void
+
+// Unsplit sequences of different lengths: block row i takes the i-th longest (ties in sequence order), so that blocks, which
+// start in grid order, leave the short sequences for the SMs that come free first.  Called by the whole block; n_seq is
+// at most kPrefillMaxRanked.
+__device__ inline ChunkInfo ranked_sequence(const int32_t* cu, int n_seq, int T, int rank) {
+    __shared__ int s_len[kPrefillMaxRanked], s_start[kPrefillMaxRanked], s_pick;
+    for (int s = threadIdx.x; s < n_seq; s += blockDim.x) {
+        int a, len; bool bad;
+        seq_span(cu, n_seq, T, s, a, len, bad);
+        s_len[s] = len; s_start[s] = a;
+    }
+    __syncthreads();
+    for (int s = threadIdx.x; s < n_seq; s += blockDim.x) {
+        const int mine = s_len[s];
+        int r = 0;
+        for (int j = 0; j < n_seq; ++j) r += s_len[j] > mine || (s_len[j] == mine && j < s);
+        if (r == rank) s_pick = s;
+    }
+    __syncthreads();
+    ChunkInfo ci;
+    ci.seq = s_len[s_pick] > 0 ? s_pick : -1;
+    ci.k = 0; ci.nck = 1;
+    ci.s0 = ci.t0 = s_start[s_pick];
+    ci.t1 = ci.t0 + s_len[s_pick];
+    return ci;
+}
+
 // Conv window at the start of a chunk: the W-1 rows before t0, taken from the sequence itself, or (chunk 0)
 // from `src_rows` = (W-1, D) activations, or zeros.
 template <typename AT>
@@ -300,8 +329,10 @@ __device__ __forceinline__ void issue_tile(unsigned char* stage, uint64_t* bar, 
 }
 
 // ---------------------------------------------------------------------------------------------------
-template <typename AT, int SUB, bool kPow, bool kOut, bool kFast>
-__global__ void __launch_bounds__(SUB * kBoxCols + 32, SUB == 1 ? 4 : 1) chunk_kernel(const PrefillArgs p, const __grid_constant__ PrefillMaps maps) {
+template <typename AT, int SUB, bool kPow, bool kOut, bool kFast, int ML>
+__global__ void __launch_bounds__(SUB * kBoxCols + 32, SUB == 1 ? 4 : 1) chunk_kernel(const __grid_constant__ PrefillBatch<ML> batch) {
+    const PrefillArgs& c = batch.c;
+    const PrefillLayer& p = batch.l[ML == 1 ? 0 : blockIdx.z];
     constexpr int TT = TileTokens<AT>::v;
     constexpr int kCB = SUB * kBoxCols;          // channels per block, one thread each
     constexpr int kStageBytes = stage_bytes(SUB);
@@ -314,6 +345,10 @@ __global__ void __launch_bounds__(SUB * kBoxCols + 32, SUB == 1 ? 4 : 1) chunk_k
     __shared__ __align__(8) uint64_t bar_empty[kStages];  // all channel warps are done with the stage
 
     const int D = p.L.d_inner;
+    // Addresses that depend on the layer are formed where they are used: the token loop has no registers to spare.
+    auto pool_ssm = [&] { return c.pool.ssm + p.layer_index * c.ssm_layer_stride; };
+    auto pool_conv = [&] { return static_cast<AT*>(c.pool.conv) + p.layer_index * c.conv_layer_stride; };
+    auto ws_layer = [&](auto* base) { return ML == 1 ? base : at_bytes(base, blockIdx.z * c.ws_layer_bytes); };
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int d0 = blockIdx.x * kCB;
     const int cols = min(kCB, D - d0);
@@ -346,42 +381,42 @@ __global__ void __launch_bounds__(SUB * kBoxCols + 32, SUB == 1 ? 4 : 1) chunk_k
         grid_release_dependents();
     } else {
         grid_release_dependents();
-        if (!p.pdl_inputs_ready) grid_wait();  // unsplit call: no summary pass has waited for the inputs yet
+        if (!c.pdl_inputs_ready) grid_wait();  // unsplit call: no summary pass has waited for the inputs yet
     }
 
     if (kOut) {
         // Sequences without tokens have no chunk: their final state is their starting state.
-        if (cidx == 0 && p.final_slot) {
+        if (cidx == 0 && c.final_slot) {
             grid_wait();  // the state pool may be the work of the kernels before
-            for (int s = 0; s < p.n_seq; ++s) {
-                int lo = p.cu ? __ldg(p.cu + s) : 0, hi = p.cu ? __ldg(p.cu + s + 1) : p.T;
-                bool bad = (lo < 0) || (hi < lo) || (hi > p.T);
-                if (bad && blockIdx.x == 0 && tid == 0) flag(p.dev_status, MDRAFT_DEV_BAD_SEQLENS);
+            for (int s = 0; s < c.n_seq; ++s) {
+                int lo = c.cu ? __ldg(c.cu + s) : 0, hi = c.cu ? __ldg(c.cu + s + 1) : c.T;
+                bool bad = (lo < 0) || (hi < lo) || (hi > c.T);
+                if (bad && blockIdx.x == 0 && tid == 0) flag(c.dev_status, MDRAFT_DEV_BAD_SEQLENS);
                 if (bad || hi != lo) continue;
-                int fs = __ldg(p.final_slot + s), is = load_slot(p.init_slot, s);
+                int fs = __ldg(c.final_slot + s), is = load_slot(c.init_slot, s);
                 if (fs < 0 || fs == is) continue;
-                if (fs >= p.pool.n_slots || is >= p.pool.n_slots) {
-                    if (blockIdx.x == 0 && tid == 0) flag(p.dev_status, MDRAFT_DEV_BAD_SLOT);
+                if (fs >= c.pool.n_slots || is >= c.pool.n_slots) {
+                    if (blockIdx.x == 0 && tid == 0) flag(c.dev_status, MDRAFT_DEV_BAD_SLOT);
                     continue;
                 }
                 if (live) {
-                    float* dh = p.pool.ssm + (size_t)fs * p.pool.ssm_slot_stride + (size_t)d * kN;
-                    AT* dc = static_cast<AT*>(p.pool.conv) + (size_t)fs * p.pool.conv_slot_stride;
-                    const float* sh = is >= 0 ? p.pool.ssm + (size_t)is * p.pool.ssm_slot_stride + (size_t)d * kN : nullptr;
-                    const AT* sc = is >= 0 ? static_cast<const AT*>(p.pool.conv) + (size_t)is * p.pool.conv_slot_stride : nullptr;
+                    float* dh = pool_ssm() + (size_t)fs * c.pool.ssm_slot_stride + (size_t)d * kN;
+                    AT* dc = pool_conv() + (size_t)fs * c.pool.conv_slot_stride;
+                    const float* sh = is >= 0 ? pool_ssm() + (size_t)is * c.pool.ssm_slot_stride + (size_t)d * kN : nullptr;
+                    const AT* sc = is >= 0 ? pool_conv() + (size_t)is * c.pool.conv_slot_stride : nullptr;
                     for (int n = 0; n < kN; ++n) dh[n] = sh ? sh[n] : 0.0f;
                     for (int j = 0; j < kW - 1; ++j) dc[(size_t)j * D + d] = sc ? sc[(size_t)j * D + d] : Act<AT>::from_f32(0.0f);
                 }
             }
-        } else if (cidx == 0 && blockIdx.x == 0 && tid < 32 && p.cu) {
-            for (int s = tid; s < p.n_seq; s += 32) {
-                int lo = __ldg(p.cu + s), hi = __ldg(p.cu + s + 1);
-                if ((lo < 0) || (hi < lo) || (hi > p.T)) flag(p.dev_status, MDRAFT_DEV_BAD_SEQLENS);
+        } else if (cidx == 0 && blockIdx.x == 0 && blockIdx.z == 0 && tid < 32 && c.cu) {
+            for (int s = tid; s < c.n_seq; s += 32) {
+                int lo = __ldg(c.cu + s), hi = __ldg(c.cu + s + 1);
+                if ((lo < 0) || (hi < lo) || (hi > c.T)) flag(c.dev_status, MDRAFT_DEV_BAD_SEQLENS);
             }
         }
     }
 
-    const ChunkInfo ci = find_chunk(p.cu, p.n_seq, p.T, p.chunk_len, cidx);
+    const ChunkInfo ci = kOut && SUB == 1 && c.longest_first ? ranked_sequence(c.cu, c.n_seq, c.T, cidx) : find_chunk(c.cu, c.n_seq, c.T, c.chunk_len, cidx);
     if (ci.seq < 0) { if (kOut) grid_wait(); return; }
     if (!kOut) {
         // No summary is needed for an unsplit sequence or for a sequence's last chunk; in conv-only mode the only
@@ -402,12 +437,12 @@ __global__ void __launch_bounds__(SUB * kBoxCols + 32, SUB == 1 ? 4 : 1) chunk_k
     const bool want_c = kOut && !conv_only;
     const int pre = min(kStages - 1, ntiles);
     if (copy_warp && lane == 0)  // the first tiles go out before anything else is looked up
-        for (int j = 0; j < pre; ++j) issue_tile<SUB>(s_stage[j], &bar_raw[j], maps, ci.t0 + j * TT, d0, D, mask);
+        for (int j = 0; j < pre; ++j) issue_tile<SUB>(s_stage[j], &bar_raw[j], p.maps, ci.t0 + j * TT, d0, D, mask);
 
-    const int islot = load_slot(p.init_slot, ci.seq);
-    const int fslot = load_slot(p.final_slot, ci.seq);
-    if (islot >= p.pool.n_slots || fslot >= p.pool.n_slots) {  // whole sequence becomes a no-op
-        if (kOut && tid == 0 && blockIdx.x == 0 && ci.k == 0) flag(p.dev_status, MDRAFT_DEV_BAD_SLOT);
+    const int islot = load_slot(c.init_slot, ci.seq);
+    const int fslot = load_slot(c.final_slot, ci.seq);
+    if (islot >= c.pool.n_slots || fslot >= c.pool.n_slots) {  // whole sequence becomes a no-op
+        if (kOut && tid == 0 && blockIdx.x == 0 && blockIdx.z == 0 && ci.k == 0) flag(c.dev_status, MDRAFT_DEV_BAD_SLOT);
         if (copy_warp)  // the tiles already queued still land in this block's shared memory: see them in first
             for (int j = 0; j < pre; ++j) mbar_wait_bounded(&bar_raw[j], 0u);
         if (kOut) grid_wait();
@@ -438,12 +473,12 @@ __global__ void __launch_bounds__(SUB * kBoxCols + 32, SUB == 1 ? 4 : 1) chunk_k
             if (nxt < ntiles) {
                 if (nxt >= kStages) ok = mbar_wait_bounded(&bar_empty[nxt % kStages], (uint32_t)(nxt / kStages - 1) & 1u);
                 if (!ok) break;
-                if (lane == 0) issue_tile<SUB>(s_stage[nxt % kStages], &bar_raw[nxt % kStages], maps, ci.t0 + nxt * TT, d0, D, mask);
+                if (lane == 0) issue_tile<SUB>(s_stage[nxt % kStages], &bar_raw[nxt % kStages], p.maps, ci.t0 + nxt * TT, d0, D, mask);
                 queued = nxt + 1;
             }
         }
         if (!ok) {
-            if (lane == 0) flag(p.dev_status, MDRAFT_DEV_WAIT_EXPIRED);
+            if (lane == 0) flag(c.dev_status, MDRAFT_DEV_WAIT_EXPIRED);
             for (int j = landed; j < queued; ++j) mbar_wait_bounded(&bar_raw[j % kStages], (uint32_t)(j / kStages) & 1u);
         }
         if (kOut) grid_wait();
@@ -457,14 +492,14 @@ __global__ void __launch_bounds__(SUB * kBoxCols + 32, SUB == 1 ? 4 : 1) chunk_k
         if (!preconv) {
             const AT* rows = nullptr;
             if (ci.k == 0) {
-                if (kOut && split) rows = static_cast<const AT*>(p.ws_conv) + (size_t)ci.seq * (kW - 1) * D;
-                else if (islot >= 0) rows = static_cast<const AT*>(p.pool.conv) + (size_t)islot * p.pool.conv_slot_stride;
+                if (kOut && split) rows = static_cast<AT*>(ws_layer(c.ws_conv)) + (size_t)ci.seq * (kW - 1) * D;
+                else if (islot >= 0) rows = pool_conv() + (size_t)islot * c.pool.conv_slot_stride;
             }
             load_window<AT>(cs.win, x, p.ldx, d, ci.t0, ci.k, rows, D);
         }
         if (!kOut) {
             if (ci.k == 0 && !preconv) {  // stash the starting window where the output pass will look for it
-                AT* stash = static_cast<AT*>(p.ws_conv) + (size_t)ci.seq * (kW - 1) * D;
+                AT* stash = static_cast<AT*>(ws_layer(c.ws_conv)) + (size_t)ci.seq * (kW - 1) * D;
 #pragma unroll
                 for (int j = 0; j < kW - 1; ++j) stash[(size_t)j * D + d] = Act<AT>::from_f32(cs.win[j]);
             }
@@ -473,12 +508,12 @@ __global__ void __launch_bounds__(SUB * kBoxCols + 32, SUB == 1 ? 4 : 1) chunk_k
             const float4* src = nullptr;
             size_t step = 1;
             if (!split) {
-                if (islot >= 0) src = reinterpret_cast<const float4*>(p.pool.ssm + (size_t)islot * p.pool.ssm_slot_stride + (size_t)d * kN);
+                if (islot >= 0) src = reinterpret_cast<const float4*>(pool_ssm() + (size_t)islot * c.pool.ssm_slot_stride + (size_t)d * kN);
             } else if (ci.k == 0) {
-                src = reinterpret_cast<const float4*>(p.ws_h0) + ((size_t)ci.seq * (kN / 4)) * D + d;
+                src = reinterpret_cast<const float4*>(ws_layer(c.ws_h0)) + ((size_t)ci.seq * (kN / 4)) * D + d;
                 step = D;
             } else {
-                src = reinterpret_cast<const float4*>(p.ws_q) + ((size_t)(cidx - 1) * (kN / 4)) * D + d;
+                src = reinterpret_cast<const float4*>(ws_layer(c.ws_q)) + ((size_t)(cidx - 1) * (kN / 4)) * D + d;
                 step = D;
             }
             if (src) {
@@ -498,7 +533,7 @@ __global__ void __launch_bounds__(SUB * kBoxCols + 32, SUB == 1 ? 4 : 1) chunk_k
         const int rows = min(TT, ci.t1 - t);
         const uint32_t parity = (uint32_t)(j / kStages) & 1u;
         if (!mbar_wait_bounded(&bar_ready[s], parity) || !mbar_wait_bounded(&bar_raw[s], parity)) {
-            if (lane == 0) flag(p.dev_status, MDRAFT_DEV_WAIT_EXPIRED);  // the outputs of this chunk are invalid
+            if (lane == 0) flag(c.dev_status, MDRAFT_DEV_WAIT_EXPIRED);  // the outputs of this chunk are invalid
             return;
         }
         if (live) {
@@ -544,7 +579,7 @@ __global__ void __launch_bounds__(SUB * kBoxCols + 32, SUB == 1 ? 4 : 1) chunk_k
     if (!live) return;
     if (!kOut) {
         if (compute) {
-            float4* dst = reinterpret_cast<float4*>(p.ws_q) + ((size_t)cidx * (kN / 4)) * D + d;
+            float4* dst = reinterpret_cast<float4*>(ws_layer(c.ws_q)) + ((size_t)cidx * (kN / 4)) * D + d;
 #pragma unroll
             for (int q = 0; q < kN / 4; ++q) {
                 float a, b, c, e;
@@ -552,13 +587,13 @@ __global__ void __launch_bounds__(SUB * kBoxCols + 32, SUB == 1 ? 4 : 1) chunk_k
                 unpk(cs.h[2 * q + 1], c, e);
                 dst[(size_t)q * D] = make_float4(a, b, c, e);
             }
-            p.ws_sd[(size_t)cidx * D + d] = cs.sum_delta;
+            ws_layer(c.ws_sd)[(size_t)cidx * D + d] = cs.sum_delta;
         }
         return;
     }
     if (ci.k == ci.nck - 1 && fslot >= 0) {
         if (!conv_only) {
-            float4* dst = reinterpret_cast<float4*>(p.pool.ssm + (size_t)fslot * p.pool.ssm_slot_stride + (size_t)d * kN);
+            float4* dst = reinterpret_cast<float4*>(pool_ssm() + (size_t)fslot * c.pool.ssm_slot_stride + (size_t)d * kN);
 #pragma unroll
             for (int q = 0; q < kN / 4; ++q) {
                 float a, b, c, e;
@@ -568,7 +603,7 @@ __global__ void __launch_bounds__(SUB * kBoxCols + 32, SUB == 1 ? 4 : 1) chunk_k
             }
         }
         if (!preconv) {
-            AT* dc = static_cast<AT*>(p.pool.conv) + (size_t)fslot * p.pool.conv_slot_stride;
+            AT* dc = pool_conv() + (size_t)fslot * c.pool.conv_slot_stride;
 #pragma unroll
             for (int j = 0; j < kW - 1; ++j) dc[(size_t)j * D + d] = Act<AT>::from_f32(cs.win[j]);
         }
@@ -587,16 +622,19 @@ __device__ __forceinline__ float4 fold4(const float4& a, const float4& h, const 
     return make_float4(fmaf(a.x, h.x, q.x), fmaf(a.y, h.y, q.y), fmaf(a.z, h.z, q.z), fmaf(a.w, h.w, q.w));
 }
 
-__global__ void __launch_bounds__(kCarryGroups * 32) carry_kernel(const PrefillArgs p) {
+template <int ML>
+__global__ void __launch_bounds__(kCarryGroups * 32) carry_kernel(const __grid_constant__ PrefillBatch<ML> batch) {
+    const PrefillArgs& p = batch.c;
     __shared__ float4 sP[kCarryGroups][32];
     __shared__ float4 sQ[kCarryGroups][32];
-    const int D = p.L.d_inner;
+    const int D = p.d_inner;
     const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
-    const int quad = blockIdx.y, s = blockIdx.z;
+    const int quad = blockIdx.y, layer = ML == 1 ? 0 : blockIdx.z / p.n_seq, s = ML == 1 ? blockIdx.z : blockIdx.z % p.n_seq;
+    const int64_t ws_off = layer * p.ws_layer_bytes;
     const int d = blockIdx.x * 32 + lane;
     const bool live = d < D;
     const int dd = live ? d : 0;  // dead lanes shadow channel 0 and write nothing
-    float4 a2 = __ldg(reinterpret_cast<const float4*>(p.L.A + (size_t)dd * kN) + quad);
+    float4 a2 = __ldg(reinterpret_cast<const float4*>(batch.l[layer].L.A + (size_t)dd * kN) + quad);
     a2.x *= kLog2e; a2.y *= kLog2e; a2.z *= kLog2e; a2.w *= kLog2e;
     grid_release_dependents();
     // Sequence offsets, slots and the starting state are inputs of the call: the summary pass ahead of this kernel
@@ -607,14 +645,14 @@ __global__ void __launch_bounds__(kCarryGroups * 32) carry_kernel(const PrefillA
     const bool slots_ok = islot < p.pool.n_slots && fslot < p.pool.n_slots;
     float4 carry = make_float4(0.f, 0.f, 0.f, 0.f);
     if (nck > 1 && slots_ok && islot >= 0)
-        carry = *(reinterpret_cast<const float4*>(p.pool.ssm + (size_t)islot * p.pool.ssm_slot_stride + (size_t)dd * kN) + quad);
+        carry = *(reinterpret_cast<const float4*>(p.pool.ssm + batch.l[layer].layer_index * p.ssm_layer_stride + (size_t)islot * p.pool.ssm_slot_stride + (size_t)dd * kN) + quad);
     grid_wait();  // the summaries are the work of the kernel just before
     if (nck <= 1) return;
     if (!slots_ok) return;  // the output pass reports it
     const size_t per_chunk = (size_t)D * (kN / 4);  // float4s in one chunk's [N/4][D] block
     const size_t col = (size_t)quad * D + dd;        // this thread's float4 inside such a block
-    float4* wsq = reinterpret_cast<float4*>(p.ws_q);
-    if (g == 0 && live) reinterpret_cast<float4*>(p.ws_h0)[(size_t)s * per_chunk + col] = carry;
+    float4* wsq = reinterpret_cast<float4*>(at_bytes(p.ws_q, ws_off));
+    if (g == 0 && live) reinterpret_cast<float4*>(at_bytes(p.ws_h0, ws_off))[(size_t)s * per_chunk + col] = carry;
 
     const int nsum = nck - 1;  // summaries of chunks 0 .. nck-2
     for (int base = 0; base < nsum; base += kCarryGroups * kCarryPer) {
@@ -622,7 +660,7 @@ __global__ void __launch_bounds__(kCarryGroups * 32) carry_kernel(const PrefillA
         const int cnt = min(kCarryPer, nsum - c0);  // may be <= 0
         float4 q[kCarryPer], a[kCarryPer];
         const float4* qp = wsq + (size_t)(first + c0) * per_chunk + col;
-        const float* sp = p.ws_sd + (size_t)(first + c0) * D + dd;
+        const float* sp = at_bytes(p.ws_sd, ws_off) + (size_t)(first + c0) * D + dd;
 #pragma unroll
         for (int i = 0; i < kCarryPer; ++i) {
             q[i] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -658,7 +696,7 @@ __global__ void __launch_bounds__(kCarryGroups * 32) carry_kernel(const PrefillA
 
 // Launch with programmatic stream serialisation: the kernel may begin before the one ahead of it has finished.
 template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, cudaStream_t st, Args... args) {
+cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, cudaStream_t st, const Args&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(threads);
@@ -672,53 +710,49 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, int threads, size_t 
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
-// The wide block needs more dynamic shared memory than a kernel gets by default; the limit is raised once per
-// kernel and device (a property of the loaded function, not an allocation).
-template <typename K>
-cudaError_t allow_smem(K kernel, int bytes) {
-    if (bytes <= 48 * 1024) return cudaSuccess;
-    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-}
-
-template <typename AT, int SUB, bool kPow, bool kFast>
-cudaError_t launch_typed(PrefillArgs p, const PrefillMaps& maps, bool chunked, cudaStream_t st) {
-    const int D = p.L.d_inner;
+template <typename AT, int SUB, bool kPow, bool kFast, int ML>
+cudaError_t launch_typed(const PrefillBatch<ML>& b, bool chunked, bool two_per_sm, cudaStream_t st) {
+    const PrefillArgs& p = b.c;
+    const int D = p.d_inner;
     constexpr int kCB = SUB * kBoxCols, kThreads = kCB + 32, kSmem = smem_bytes(SUB);
-    dim3 grid((D + kCB - 1) / kCB, p.n_chunks_bound);
-    const bool recur = !(p.L.flags & MDRAFT_CONV_ONLY);
-    p.pdl_inputs_ready = chunked ? 1 : 0;  // the summary pass waits for the producer of the inputs on behalf of all three
+    dim3 grid((D + kCB - 1) / kCB, p.n_chunks_bound, p.n_layers);
+    const bool recur = !(b.l[0].L.flags & MDRAFT_CONV_ONLY);
     cudaError_t e = cudaSuccess;
     if (chunked) {
-        if ((e = allow_smem(chunk_kernel<AT, SUB, kPow, false, kFast>, kSmem)) != cudaSuccess) return e;
-        e = launch_pdl(chunk_kernel<AT, SUB, kPow, false, kFast>, grid, kThreads, kSmem, st, p, maps);
+        if ((e = allow_smem<chunk_kernel<AT, SUB, kPow, false, kFast, ML>>(kSmem)) != cudaSuccess) return e;
+        e = launch_pdl(chunk_kernel<AT, SUB, kPow, false, kFast, ML>, grid, kThreads, kSmem, st, b);
     }
     if (e != cudaSuccess) return e;
     if (p.ev_state) cudaEventRecord(p.ev_state, st);
     if (chunked && recur) {
-        dim3 g2((D + 31) / 32, kN / 4, p.n_seq);
-        e = launch_pdl(carry_kernel, g2, kCarryGroups * 32, 0, st, p);
+        dim3 g2((D + 31) / 32, kN / 4, p.n_seq * p.n_layers);
+        e = launch_pdl(carry_kernel<ML>, g2, kCarryGroups * 32, 0, st, b);
         if (e != cudaSuccess) return e;
     }
     if (p.ev_carry) cudaEventRecord(p.ev_carry, st);
-    if ((e = allow_smem(chunk_kernel<AT, SUB, kPow, true, kFast>, kSmem)) != cudaSuccess) return e;
-    e = launch_pdl(chunk_kernel<AT, SUB, kPow, true, kFast>, grid, kThreads, kSmem, st, p, maps);
-    if (e != cudaSuccess) return e;
-    return cudaGetLastError();
+    constexpr int kSmemTwo = 100 * 1024;  // a third block does not fit the SM's 227 KB
+    if ((e = allow_smem<chunk_kernel<AT, SUB, kPow, true, kFast, ML>>(SUB == 1 ? kSmemTwo : kSmem)) != cudaSuccess) return e;
+    return launch_pdl(chunk_kernel<AT, SUB, kPow, true, kFast, ML>, grid, kThreads, SUB == 1 && two_per_sm ? kSmemTwo : kSmem, st, b);
 }
 
-template <typename AT, int SUB>
-cudaError_t launch_act(const PrefillArgs& p, const PrefillMaps& maps, bool chunked, cudaStream_t st) {
-    const bool pow = p.L.flags & MDRAFT_A_POWERS;
-    const bool fast = (p.L.flags & ~(uint32_t)MDRAFT_A_POWERS) == (uint32_t)MDRAFT_DT_SOFTPLUS;
-    if (fast) return pow ? launch_typed<AT, SUB, true, true>(p, maps, chunked, st) : launch_typed<AT, SUB, false, true>(p, maps, chunked, st);
-    return pow ? launch_typed<AT, SUB, true, false>(p, maps, chunked, st) : launch_typed<AT, SUB, false, false>(p, maps, chunked, st);
+template <typename AT, int SUB, int ML>
+cudaError_t launch_act(const PrefillBatch<ML>& b, bool chunked, bool two_per_sm, cudaStream_t st) {
+    const uint32_t flags = b.l[0].L.flags;
+    const bool pow = flags & MDRAFT_A_POWERS;
+    if ((flags & ~(uint32_t)MDRAFT_A_POWERS) == (uint32_t)MDRAFT_DT_SOFTPLUS)
+        return pow ? launch_typed<AT, SUB, true, true>(b, chunked, two_per_sm, st) : launch_typed<AT, SUB, false, true>(b, chunked, two_per_sm, st);
+    if constexpr (ML > 1) return cudaErrorInvalidValue;  // the caller takes such layers one by one
+    else return pow ? launch_typed<AT, SUB, true, false>(b, chunked, two_per_sm, st) : launch_typed<AT, SUB, false, false>(b, chunked, two_per_sm, st);
 }
 
 }  // namespace
 
-cudaError_t launch_prefill(const PrefillArgs& p, const PrefillMaps& maps, int act, bool chunked, bool wide, cudaStream_t st) {
-    if (wide) return act == MDRAFT_F32 ? launch_act<float, kPrefillWideBoxes>(p, maps, chunked, st) : launch_act<__nv_bfloat16, kPrefillWideBoxes>(p, maps, chunked, st);
-    return act == MDRAFT_F32 ? launch_act<float, 1>(p, maps, chunked, st) : launch_act<__nv_bfloat16, 1>(p, maps, chunked, st);
+template <int ML>
+cudaError_t launch_prefill(const PrefillBatch<ML>& b, int act, bool chunked, bool wide, bool two_per_sm, cudaStream_t st) {
+    if (wide) return act == MDRAFT_F32 ? launch_act<float, kPrefillWideBoxes>(b, chunked, two_per_sm, st) : launch_act<__nv_bfloat16, kPrefillWideBoxes>(b, chunked, two_per_sm, st);
+    return act == MDRAFT_F32 ? launch_act<float, 1>(b, chunked, two_per_sm, st) : launch_act<__nv_bfloat16, 1>(b, chunked, two_per_sm, st);
 }
+template cudaError_t launch_prefill<1>(const PrefillBatch<1>&, int, bool, bool, bool, cudaStream_t);
+template cudaError_t launch_prefill<kPrefillMaxLayers>(const PrefillBatch<kPrefillMaxLayers>&, int, bool, bool, bool, cudaStream_t);
 
 }  // namespace mdraft

@@ -9,19 +9,24 @@ namespace mdraft {
 
 constexpr int kPrefillThreads = 128;  // channels per block (one thread per channel)
 
+constexpr int kPrefillMaxLayers = 32;  // layers one launch takes (their descriptors are kernel parameters: 25 of the 32 KB a launch may carry)
+constexpr int kPrefillMaxRanked = 128; // sequences a batch of unsplit sequences may have to be handed out longest first
+
+// What all layers of a call share.
 struct PrefillArgs {
-    LayerDev L;
-    PoolDev pool;
-    const void *x, *z, *dt, *B, *C;
-    void* out;
-    int64_t ldx, ldz, lddt, ldb, ldc, ldo;
+    PoolDev pool;   // of layer 0 of the cache
+    int64_t ssm_layer_stride, conv_layer_stride;
+    int n_layers, d_inner;
     int T, n_seq, chunk_len, n_chunks_bound;
+    int longest_first;  // every sequence is one chunk: block row i takes the i-th longest
     const int32_t *cu, *init_slot, *final_slot;
+    // Workspace of the call's first layer; layer l's lies ws_layer_bytes further on per layer.
     float* ws_q;    // [n_chunks_bound][N/4][D][4] zero-state result of each chunk; after the carry scan, entry c holds
                     //                             the state after chunk c = the incoming state of chunk c + 1
     float* ws_sd;   // [n_chunks_bound][D]         sum of Delta per chunk
     float* ws_h0;   // [n_seq][N/4][D][4]          starting state of each split sequence
     void* ws_conv;  // [n_seq][W-1][D]             starting conv window of each split sequence (activation type)
+    int64_t ws_layer_bytes;
     int32_t* dev_status;
     int pdl_inputs_ready;  // set by the launcher: 1 if an earlier kernel of this call has already waited for the inputs
     cudaEvent_t ev_state, ev_carry;  // optional profiling events (host side only)
@@ -35,9 +40,28 @@ struct PrefillMaps {
     CUtensorMap x, dt, z, B, C;
 };
 
+// One layer of a call.
+struct PrefillLayer {
+    LayerDev L;
+    int layer_index;  // in the cache
+    const void* x;    // for the rows before a chunk; everything else comes through the descriptors
+    void* out;
+    int64_t ldx, ldo;
+    PrefillMaps maps;
+};
+
+template <int ML>
+struct PrefillBatch {
+    PrefillArgs c;
+    PrefillLayer l[ML];
+};
+
 constexpr int kPrefillWideBoxes = 4;  // a wide block covers 4 x kPrefillThreads channels with 16 channel warps
 
-// wide: one block of 512 channels per (channel block, chunk) instead of 128 — for plans that give every SM one block.
-cudaError_t launch_prefill(const PrefillArgs& p, const PrefillMaps& maps, int act, bool chunked, bool wide, cudaStream_t st);
+// wide: one block of 512 channels per (channel block, chunk) instead of 128 - for plans that give every SM one block.
+// two_per_sm: ask for so much shared memory that an SM takes two narrow blocks, not four.
+// ML = 1, or kPrefillMaxLayers for a call over several layers (all with the same flags: softplus, A_POWERS or not).
+template <int ML>
+cudaError_t launch_prefill(const PrefillBatch<ML>& b, int act, bool chunked, bool wide, bool two_per_sm, cudaStream_t st);
 
 }  // namespace mdraft

@@ -58,8 +58,9 @@ __device__ __forceinline__ void xor_permute(float4 (&t)[4], int sw) {
     if (sw & 2) { swap4(t[0], t[2]); swap4(t[1], t[3]); }
 }
 
-template <typename AT, bool kPow>
-__global__ void __launch_bounds__(kTB) tree_step_kernel(const TreeArgs p, const int early_inputs, const int ordinary_launch) {
+template <typename AT, bool kPow, int ML>
+__global__ void __launch_bounds__(kTB) tree_step_kernel(const TreeArgs c, const __grid_constant__ TreeLayers<ML> layers, const int early_inputs,
+                                                        const int ordinary_launch) {
     __shared__ __align__(128) float4 s_h[kTB * (kN / 4)];  // state slice [channel][quad]
     __shared__ __align__(16) AT s_conv[kW - 1][kTB];
     __shared__ __align__(16) AT s_x[kTB];                 // the node's x row; receives the out row afterwards
@@ -73,17 +74,18 @@ __global__ void __launch_bounds__(kTB) tree_step_kernel(const TreeArgs p, const 
     // Launched the ordinary way nothing runs ahead of this kernel: the wait costs nothing, and passing it first lets
     // every copy be requested at once.
     if (ordinary_launch) asm volatile("griddepcontrol.wait;" ::: "memory");
+    const TreeLayer& p = layers.l[ML == 1 ? 0 : blockIdx.z];
     const int D = p.L.d_inner;
-    const int node = p.lvl_begin + blockIdx.x;
+    const int node = c.lvl_begin + blockIdx.x;
     const int tid = threadIdx.x;
     const int d0 = blockIdx.y * kTB;
     const int cols = min(kTB, D - d0);
     const int d = d0 + tid;
     const bool live = tid < cols;
-    const int pslot = __ldg(p.parent_slot + node);
-    const int nslot = __ldg(p.node_slot + node);
-    if (pslot < -1 || pslot >= p.pool.n_slots || nslot < 0 || nslot >= p.pool.n_slots) {  // the node becomes a no-op
-        if (tid == 0 && blockIdx.y == 0) flag(p.dev_status, MDRAFT_DEV_BAD_SLOT);
+    const int pslot = __ldg(c.parent_slot + node);
+    const int nslot = __ldg(c.node_slot + node);
+    if (pslot < -1 || pslot >= c.pool.n_slots || nslot < 0 || nslot >= c.pool.n_slots) {  // the node becomes a no-op
+        if (tid == 0 && blockIdx.y == 0 && blockIdx.z == 0) flag(c.dev_status, MDRAFT_DEV_BAD_SLOT);
         asm volatile("griddepcontrol.wait;" ::: "memory");
         return;
     }
@@ -91,10 +93,12 @@ __global__ void __launch_bounds__(kTB) tree_step_kernel(const TreeArgs p, const 
     const bool preconv = flags & MDRAFT_PRECONV, conv_only = flags & MDRAFT_CONV_ONLY;
     const bool have_parent = pslot >= 0;
     const uint32_t row_bytes = (uint32_t)cols * sizeof(AT), bc_bytes = (uint32_t)kN * sizeof(AT), h_bytes = (uint32_t)cols * kN * 4u;
-    float* h_parent = p.pool.ssm + (size_t)pslot * p.pool.ssm_slot_stride + (size_t)d0 * kN;
-    float* h_child = p.pool.ssm + (size_t)nslot * p.pool.ssm_slot_stride + (size_t)d0 * kN;
-    AT* conv_parent = static_cast<AT*>(p.pool.conv) + (size_t)pslot * p.pool.conv_slot_stride + d0;
-    AT* conv_child = static_cast<AT*>(p.pool.conv) + (size_t)nslot * p.pool.conv_slot_stride + d0;
+    float* pool_ssm = c.pool.ssm + p.layer_index * c.ssm_layer_stride;
+    AT* pool_conv = static_cast<AT*>(c.pool.conv) + p.layer_index * c.conv_layer_stride;
+    float* h_parent = pool_ssm + (size_t)pslot * c.pool.ssm_slot_stride + (size_t)d0 * kN;
+    float* h_child = pool_ssm + (size_t)nslot * c.pool.ssm_slot_stride + (size_t)d0 * kN;
+    AT* conv_parent = pool_conv + (size_t)pslot * c.pool.conv_slot_stride + d0;
+    AT* conv_child = pool_conv + (size_t)nslot * c.pool.conv_slot_stride + d0;
 
     // Inputs of the node (x, z, dt, B, C rows) go on one mbarrier, the parent's state and window on another: the
     // former may be requested before the kernel ahead has finished when the launch says they cannot be its work.
@@ -161,7 +165,7 @@ __global__ void __launch_bounds__(kTB) tree_step_kernel(const TreeArgs p, const 
     const bool ok = mbar_wait_bounded(&bar_in, 0u) && mbar_wait_bounded(&bar, 0u);
     if (__syncthreads_or(!ok)) {
         if (tid == 0) {
-            flag(p.dev_status, MDRAFT_DEV_WAIT_EXPIRED);
+            flag(c.dev_status, MDRAFT_DEV_WAIT_EXPIRED);
             mbar_wait_bounded(&bar_in, 0u); mbar_wait_bounded(&bar, 0u);
         }
         return;
@@ -249,8 +253,8 @@ __global__ void __launch_bounds__(kTB) tree_step_kernel(const TreeArgs p, const 
 // The first level of a call is launched the ordinary way: what runs ahead of it is usually somebody else's kernel (a
 // projection), which never releases its dependents early, and behind such a kernel a programmatic launch was measured
 // 0.8 us slower than an ordinary one.  Later levels follow a level of the same call and are launched programmatically.
-template <typename K>
-cudaError_t launch_level(K kernel, dim3 grid, cudaStream_t st, const TreeArgs& p, int early) {
+template <int ML, typename K>
+cudaError_t launch_level(K kernel, dim3 grid, cudaStream_t st, const TreeArgs& p, const TreeLayers<ML>& layers) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(kTB);
@@ -261,25 +265,26 @@ cudaError_t launch_level(K kernel, dim3 grid, cudaStream_t st, const TreeArgs& p
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = p.level_in_call > 0 ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kernel, p, early, p.level_in_call > 0 ? 0 : 1);
-}
-
-cudaError_t launch_tree_step(const TreeArgs& p, int act, cudaStream_t st) {
-    const int n = p.lvl_end - p.lvl_begin;
-    if (n <= 0) return cudaSuccess;
-    const bool pow = p.L.flags & MDRAFT_A_POWERS;
     // The first kernel of a call is an ordinary launch: it starts only after everything ahead of the call has finished.
     // A later level starts when the level before it does, so the only kernels that can still be running then are
     // levels of this call, which write states and `out` rows of other nodes only: the node's input rows cannot be
     // their work and are requested before the wait.
-    const int early = p.level_in_call >= 1 ? 1 : 0;
-    dim3 grid(n, (p.L.d_inner + kTB - 1) / kTB);
-    if (act == MDRAFT_F32) {
-        if (pow) return launch_level(tree_step_kernel<float, true>, grid, st, p, early);
-        return launch_level(tree_step_kernel<float, false>, grid, st, p, early);
-    }
-    if (pow) return launch_level(tree_step_kernel<__nv_bfloat16, true>, grid, st, p, early);
-    return launch_level(tree_step_kernel<__nv_bfloat16, false>, grid, st, p, early);
+    const int early = p.level_in_call > 0 ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, p, layers, early, 1 - early);
+}
+
+template <int ML>
+cudaError_t launch_layers(const TreeArgs& p, const TreeLayers<ML>& layers, int act, cudaStream_t st) {
+    const bool pow = layers.l[0].L.flags & MDRAFT_A_POWERS;
+    const dim3 grid(p.lvl_end - p.lvl_begin, (layers.l[0].L.d_inner + kTB - 1) / kTB, p.n_layers);
+    if (act == MDRAFT_F32) return pow ? launch_level(tree_step_kernel<float, true, ML>, grid, st, p, layers) : launch_level(tree_step_kernel<float, false, ML>, grid, st, p, layers);
+    return pow ? launch_level(tree_step_kernel<__nv_bfloat16, true, ML>, grid, st, p, layers) : launch_level(tree_step_kernel<__nv_bfloat16, false, ML>, grid, st, p, layers);
+}
+
+cudaError_t launch_tree_step(const TreeArgs& p, const TreeLayers<kTreeMaxLayers>& layers, int act, cudaStream_t st) {
+    if (p.lvl_end <= p.lvl_begin) return cudaSuccess;
+    if (p.n_layers == 1) return launch_layers(p, TreeLayers<1>{{layers.l[0]}}, act, st);
+    return launch_layers(p, layers, act, st);
 }
 
 }  // namespace mdraft

@@ -1,7 +1,9 @@
 """A stack of drafter layers driven through the C ABI: launch sequencing only.
 
 The real drafter interleaves these calls with its projections (which are outside this library); here the
-per-layer inputs are independent tensors, so one "pass" is simply every layer's call issued on one stream.
+per-layer inputs are independent tensors, so one "pass" is every layer's work side by side: one launch takes all layers
+of an encode, or of a tree level.  Where tensors overlap (a layer fed from another's output, one output buffer for all) the
+layers' calls are issued one after another on the stream instead.
 """
 
 from __future__ import annotations
@@ -22,11 +24,14 @@ class DrafterStack:
         self.cache = mb.StateCache(len(self.layers), n_slots, l0.d_inner, l0.d_state, l0.d_conv, l0.act, device)
         self.chunk_len = chunk_len
         self.ws_bytes = max(mb.mdraft_prefill_workspace_bytes(l, max_tokens, n_seq, max_seqlen, chunk_len) for l in self.layers)
-        self.workspace = torch.empty(max(self.ws_bytes, 256), dtype=torch.uint8, device=device)
+        stacked = 0 if chunk_len else mb.mdraft_prefill_stack_workspace_bytes(l0, len(self.layers), max_tokens, n_seq, max_seqlen)
+        self.workspace = torch.empty(max(self.ws_bytes, stacked, 256), dtype=torch.uint8, device=device)
         self.status = torch.zeros(1, dtype=torch.int32, device=device)
 
-    # number of kernels one prefill call launches (chunk summary + carry scan + main scan, or the main scan alone)
+    # number of kernels one layer's prefill call launches (chunk summary + carry scan + main scan, or the main scan alone)
     def prefill_launches_per_layer(self, total_tokens: int, n_seq: int, max_seqlen: int) -> int:
+        if not self.chunk_len:
+            return mb.mdraft_prefill_stack_launches(self.layers[0], 1, total_tokens, n_seq, max_seqlen)
         chunked = mb.mdraft_prefill_workspace_bytes(self.layers[0], total_tokens, n_seq, max_seqlen, self.chunk_len) > 0
         return 3 if chunked else 1
 
@@ -34,7 +39,10 @@ class DrafterStack:
                 max_seqlen: int, init_slot: Optional[torch.Tensor], final_slot: Optional[torch.Tensor], stream=None,
                 phase_events: Optional[List] = None, layer_range=None) -> None:
         """inputs[l] = (x, z, dt, B, C) of layer l.  phase_events[l] = (start, after_state, after_carry, end)."""
-        rng = range(len(self.layers)) if layer_range is None else layer_range
+        rng = range(len(self.layers)) if layer_range is None else list(layer_range)
+        if phase_events is None and not self.chunk_len and len(rng) > 1 and mb.mdraft_conv_scan_prefill_stack(
+                self.layers, rng, self.cache, inputs, outs, cu_seqlens, max_seqlen, init_slot, final_slot, self.workspace, self.status, stream):
+            return
         for l in rng:
             x, z, dt, B, C = inputs[l]
             pe = None
@@ -49,7 +57,10 @@ class DrafterStack:
 
     def tree_round(self, inputs: Sequence[Sequence[torch.Tensor]], outs: Sequence[torch.Tensor], parent_slot: torch.Tensor,
                    node_slot: torch.Tensor, level_offsets: Optional[Sequence[int]], stream=None, layer_range=None) -> None:
-        rng = range(len(self.layers)) if layer_range is None else layer_range
+        rng = range(len(self.layers)) if layer_range is None else list(layer_range)
+        if len(rng) > 1 and mb.mdraft_tree_step_stack(self.layers, rng, self.cache, inputs, outs, parent_slot, node_slot, level_offsets,
+                                                      self.status, stream):
+            return
         for l in rng:
             x, z, dt, B, C = inputs[l]
             mb.mdraft_tree_step(self.layers[l], self.cache, l, x, z, dt, B, C, outs[l], parent_slot, node_slot,
