@@ -61,6 +61,14 @@ __device__ __forceinline__ float softplus(float v) {
     return (v > 20.0f) ? v : r;
 }
 
+// softplus in base-2 units: log2(1 + 2^a) = softplus(a ln 2) log2(e), by the same two branches.
+__device__ __forceinline__ float softplus_log2(float a) {
+    const float e = ex2(a);
+    const float series = e * (kLog2e - e * (0.5f * kLog2e - e * (0.33333334f * kLog2e - e * (0.25f * kLog2e))));
+    const float r = (e < 0.03125f) ? series : lg2(1.0f + e);
+    return (a > 20.0f * kLog2e) ? a : r;
+}
+
 // ---------------------------------------------------------------- activation dtype
 template <typename T> struct Act;
 template <> struct Act<float> {

@@ -152,6 +152,13 @@ __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;
 __device__ __forceinline__ void grid_release_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // ---------------------------------------------------------------- one channel's running computation
+// The usual case (kFast: conv, softplus, recurrence, gate) works in scaled quantities, which takes the constant factors of the
+// base-2 special functions out of the token loop: step sizes are kept times log2(e) (what lg2 gives), the conv's output times
+// -log2(e) (what its SiLU's exponential takes), and so the state as h / kStateScale with kStateScale = -ln(2)^2; C is widened
+// times kStateScale, and states and summed step sizes are scaled where they enter and leave the registers.  (One layer of
+// 32 packed sequences, 141650 tokens: 1492 -> 1389 us.)
+constexpr float kStateScale = -kLn2 * kLn2;
+
 template <typename AT, bool kPow, bool kOut, bool kFast>
 struct ChannelScan {
     u64 h[kN / 2];        // state, entries (2k, 2k+1) packed
@@ -167,15 +174,17 @@ struct ChannelScan {
 #pragma unroll
         for (int q = 0; q < kN / 4; ++q) {
             float4 a = __ldg(Ap + q);
-            a2[2 * q] = pk(a.x * kLog2e, a.y * kLog2e);
-            a2[2 * q + 1] = pk(a.z * kLog2e, a.w * kLog2e);
-            if (q == 0) a20 = a.x * kLog2e;
+            constexpr float f = kFast ? 1.0f : kLog2e;
+            a2[2 * q] = pk(a.x * f, a.y * f);
+            a2[2 * q + 1] = pk(a.z * f, a.w * f);
+            if (q == 0) a20 = a.x * f;
         }
         float4 wv = __ldg(reinterpret_cast<const float4*>(L.conv_w + (size_t)d * kW));
-        w[0] = wv.x; w[1] = wv.y; w[2] = wv.z; w[3] = wv.w;
-        cb = L.conv_b ? __ldg(L.conv_b + d) : 0.0f;
-        dtb = L.dt_bias ? __ldg(L.dt_bias + d) : 0.0f;
-        dsk = L.D ? __ldg(L.D + d) : 0.0f;
+        constexpr float fu = kFast ? -kLog2e : 1.0f;
+        w[0] = wv.x * fu; w[1] = wv.y * fu; w[2] = wv.z * fu; w[3] = wv.w * fu;
+        cb = L.conv_b ? __ldg(L.conv_b + d) * fu : 0.0f;
+        dtb = L.dt_bias ? __ldg(L.dt_bias + d) * (kFast ? kLog2e : 1.0f) : 0.0f;
+        dsk = L.D ? __ldg(L.D + d) * (kFast ? -kLn2 : 1.0f) : 0.0f;
         sum_delta = 0.0f;
         flags = kFast ? (uint32_t)MDRAFT_DT_SOFTPLUS : L.flags;
 #pragma unroll
@@ -228,15 +237,31 @@ struct ChannelScan {
             acc = fmaf(w[2], win[2], acc);
             acc = fmaf(w[3], xv, acc);
             win[0] = win[1]; win[1] = win[2]; win[2] = xv;
-            e.u = silu(acc);
+            e.u = kFast ? acc * rcp(1.0f + ex2(acc)) : silu(acc);
         }
         e.delta = 0.f; e.du = 0.f; e.gate = 0.f;
         if (flags & MDRAFT_CONV_ONLY) return;
-        const float v = dtv + dtb;
-        e.delta = (flags & MDRAFT_DT_SOFTPLUS) ? softplus(v) : v;
+        if (kFast) {
+            e.delta = softplus_log2(fmaf(dtv, kLog2e, dtb));
+        } else {
+            const float v = dtv + dtb;
+            e.delta = (flags & MDRAFT_DT_SOFTPLUS) ? softplus(v) : v;
+        }
         if (!kOut) sum_delta += e.delta;
         e.du = e.delta * e.u;
         if (kOut) e.gate = silu(zv);
+    }
+    // The state as 16 floats in its own scale: what a chunk starts from, and what it leaves.
+    __device__ __forceinline__ void set_state(int q, const float4& v) {
+        constexpr float f = kFast ? 1.0f / kStateScale : 1.0f;
+        h[2 * q] = pk(v.x * f, v.y * f); h[2 * q + 1] = pk(v.z * f, v.w * f);
+    }
+    __device__ __forceinline__ float4 get_state(int q) const {
+        constexpr float f = kFast ? kStateScale : 1.0f;
+        float a, b, c, e;
+        unpk(h[2 * q], a, b);
+        unpk(h[2 * q + 1], c, e);
+        return make_float4(a * f, b * f, c * f, e * f);
     }
     // Step 2: state update and output.  Bt / Ct point at 16 fp32 values in shared memory.  Returns the output (kOut),
     // or u in conv-only mode.
@@ -245,7 +270,7 @@ struct ChannelScan {
         u64 P[kN / 2];
         decays(e.delta, P);
         const u64 DU = pk(e.du, e.du);
-        u64 y0 = pk(0.0f, 0.0f), y1 = pk(0.0f, 0.0f);
+        u64 y0, y1;
         const ulonglong2* B2 = reinterpret_cast<const ulonglong2*>(Bt);
         const ulonglong2* C2 = reinterpret_cast<const ulonglong2*>(Ct);
 #pragma unroll
@@ -255,8 +280,8 @@ struct ChannelScan {
             h[2 * q + 1] = fma2(P[2 * q + 1], h[2 * q + 1], mul2(DU, b.y));
             if (kOut) {
                 const ulonglong2 c = C2[q];
-                y0 = fma2(c.x, h[2 * q], y0);
-                y1 = fma2(c.y, h[2 * q + 1], y1);
+                y0 = q == 0 ? mul2(c.x, h[0]) : fma2(c.x, h[2 * q], y0);
+                y1 = q == 0 ? mul2(c.y, h[1]) : fma2(c.y, h[2 * q + 1], y1);
             }
         }
         if (!kOut) return 0.0f;
@@ -464,7 +489,7 @@ __global__ void __launch_bounds__(SUB * kBoxCols + 32, SUB == 1 ? 4 : 1) chunk_k
                 const AT* rc = reinterpret_cast<const AT*>(s_stage[s] + off_c(SUB));
                 for (int i = lane; i < rows * kN; i += 32) {
                     (&sBf[s][0][0])[i] = Act<AT>::to_f32(rb[i]);
-                    if (want_c) (&sCf[s][0][0])[i] = Act<AT>::to_f32(rc[i]);
+                    if (want_c) (&sCf[s][0][0])[i] = Act<AT>::to_f32(rc[i]) * (kFast ? kStateScale : 1.0f);
                 }
             }
             __syncwarp();
@@ -519,14 +544,14 @@ __global__ void __launch_bounds__(SUB * kBoxCols + 32, SUB == 1 ? 4 : 1) chunk_k
             if (src) {
 #pragma unroll
                 for (int q = 0; q < kN / 4; ++q) {
-                    const float4 v = src[(size_t)q * step];
-                    cs.h[2 * q] = pk(v.x, v.y); cs.h[2 * q + 1] = pk(v.z, v.w);
+                    cs.set_state(q, src[(size_t)q * step]);
                 }
             }
         }
     }
 
     // ---- channel warps
+    const int64_t ldo = p.ldo;
     for (int j = 0; j < ntiles; ++j) {
         const int s = j % kStages;
         const int t = ci.t0 + j * TT;
@@ -542,7 +567,7 @@ __global__ void __launch_bounds__(SUB * kBoxCols + 32, SUB == 1 ? 4 : 1) chunk_k
             const AT* sx = reinterpret_cast<const AT*>(st + off_x(SUB) + box) + col;
             const AT* sdt = reinterpret_cast<const AT*>(st + off_dt(SUB) + box) + col;
             const AT* sz = reinterpret_cast<const AT*>(st + off_z(SUB) + box) + col;
-            AT* orow = out + (size_t)t * p.ldo + d;
+            AT* orow = out + (size_t)t * ldo + d;
             typedef typename ChannelScan<AT, kPow, kOut, kFast>::Pre Pre;
             int r = 0;
             for (; r + GRP <= rows; r += GRP) {
@@ -559,7 +584,7 @@ __global__ void __launch_bounds__(SUB * kBoxCols + 32, SUB == 1 ? 4 : 1) chunk_k
                 for (int g = 0; g < GRP; ++g) o[g] = cs.post(e[g], sBf[s][r + g], sCf[s][r + g]);
                 if (kOut) {
 #pragma unroll
-                    for (int g = 0; g < GRP; ++g) orow[(size_t)(r + g) * p.ldo] = Act<AT>::from_f32(o[g]);
+                    for (int g = 0; g < GRP; ++g) orow[(size_t)(r + g) * ldo] = Act<AT>::from_f32(o[g]);
                 }
             }
             for (; r < rows; ++r) {
@@ -569,7 +594,7 @@ __global__ void __launch_bounds__(SUB * kBoxCols + 32, SUB == 1 ? 4 : 1) chunk_k
                 const float zv = want_c ? Act<AT>::to_f32(sz[r * kBoxCols]) : 0.0f;
                 cs.pre(xv, zv, dtv, e);
                 const float o = cs.post(e, sBf[s][r], sCf[s][r]);
-                if (kOut) orow[(size_t)r * p.ldo] = Act<AT>::from_f32(o);
+                if (kOut) orow[(size_t)r * ldo] = Act<AT>::from_f32(o);
             }
         }
         __syncwarp();
@@ -581,13 +606,8 @@ __global__ void __launch_bounds__(SUB * kBoxCols + 32, SUB == 1 ? 4 : 1) chunk_k
         if (compute) {
             float4* dst = reinterpret_cast<float4*>(ws_layer(c.ws_q)) + ((size_t)cidx * (kN / 4)) * D + d;
 #pragma unroll
-            for (int q = 0; q < kN / 4; ++q) {
-                float a, b, c, e;
-                unpk(cs.h[2 * q], a, b);
-                unpk(cs.h[2 * q + 1], c, e);
-                dst[(size_t)q * D] = make_float4(a, b, c, e);
-            }
-            ws_layer(c.ws_sd)[(size_t)cidx * D + d] = cs.sum_delta;
+            for (int q = 0; q < kN / 4; ++q) dst[(size_t)q * D] = cs.get_state(q);
+            ws_layer(c.ws_sd)[(size_t)cidx * D + d] = cs.sum_delta * (kFast ? kLn2 : 1.0f);
         }
         return;
     }
@@ -595,12 +615,7 @@ __global__ void __launch_bounds__(SUB * kBoxCols + 32, SUB == 1 ? 4 : 1) chunk_k
         if (!conv_only) {
             float4* dst = reinterpret_cast<float4*>(pool_ssm() + (size_t)fslot * c.pool.ssm_slot_stride + (size_t)d * kN);
 #pragma unroll
-            for (int q = 0; q < kN / 4; ++q) {
-                float a, b, c, e;
-                unpk(cs.h[2 * q], a, b);
-                unpk(cs.h[2 * q + 1], c, e);
-                dst[q] = make_float4(a, b, c, e);
-            }
+            for (int q = 0; q < kN / 4; ++q) dst[q] = cs.get_state(q);
         }
         if (!preconv) {
             AT* dc = pool_conv() + (size_t)fslot * c.pool.conv_slot_stride;
