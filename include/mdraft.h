@@ -309,6 +309,34 @@ int mdraft_tree_step_proj(const mdraft_layer *layer, const mdraft_cache *cache, 
                           int32_t *dev_status, void *stream);
 
 /*
+ * One generation of a whole drafter stack (paper Section 4.1: generation i is one batch of the nodes of level i): embedding
+ * rows of the nodes' tokens, then per layer
+ *     xz = rmsnorm(h) W_in;   y = the projection step above on (x, z) = xz;   h = h + y W_out
+ * and logits = rmsnorm(h) W_lm.  bf16 weights and activations, fp32 accumulation; h is rounded to bf16 after every layer; the
+ * norm has no weight.  All kernels of a call are chained so that each fetches its weights while the one ahead runs.
+ *   W_in[l] (d_model, 2 d_inner), W_out[l] (d_inner, d_model), W_lm (d_model, vocab), embed (vocab, d_model): row-major, dense
+ *   W_x[l], W_dt[l]     : as mdraft_select_proj       (the arrays themselves are HOST arrays of n_layers device pointers)
+ *   tokens              : n_nodes int64, device; an id outside the vocabulary raises MDRAFT_DEV_BAD_SLOT (its row is zero)
+ *   h, xz, y            : device scratch of n_nodes x d_model, x 2 d_inner, x d_inner bf16
+ *   logits              : n_nodes rows of vocab bf16, stride ldl (a multiple of 8)
+ * Layer l works on pool layer l.  No node_slot may equal another node's parent_slot or node_slot.
+ * Supported: n_nodes <= MDRAFT_BLOCK_MAX_NODES, d_model a multiple of 32 up to 1408, d_inner a multiple of 32 up to 4096, vocab
+ * a multiple of 8, dt_rank as above; anything else is MDRAFT_ERR_UNSUPPORTED.
+ */
+#define MDRAFT_BLOCK_MAX_NODES 64
+typedef struct {
+    int32_t n_layers, d_model, dt_rank, vocab;
+    const mdraft_layer *layers;   /* HOST, n_layers */
+    const void *const *W_in, *const *W_x, *const *W_dt, *const *W_out;
+    const void *embed, *W_lm;
+    float eps;                    /* of the norms */
+} mdraft_block_stack;
+
+int mdraft_block_generation(const mdraft_block_stack *stack, const mdraft_cache *cache, const int64_t *tokens, int32_t n_nodes,
+                            const int32_t *parent_slot, const int32_t *node_slot, void *h, void *xz, void *y,
+                            void *logits, int64_t ldl, int32_t *dev_status, void *stream);
+
+/*
  * ---------------------------------------------------------------------------------------------------------
  * Mamba-2 (SSD) drafter layer.  The paper names Mamba-2 as the model whose advances "directly benefit" the approach
  * (Section 1, the paragraph before Related Work) and defines nothing about it; what is computed here is the cited

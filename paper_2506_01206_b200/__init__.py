@@ -11,7 +11,7 @@ from .binding import (  # noqa: F401
     Layer, MdraftError, StateCache, UcbBandit, load_library, mdraft_ucb_reward,
     mdraft_classify_A, mdraft_conv_scan_prefill, mdraft_conv_scan_prefill_noalloc, mdraft_prefill_workspace_bytes,
     NOALLOC_SCRATCH_BYTES, mdraft_conv_scan_prefill_stack, mdraft_prefill_stack_launches, mdraft_prefill_stack_workspace_bytes,
-    mdraft_tree_step_stack,
+    mdraft_tree_step_stack, mdraft_block_generation,
     SsdLayer, mdraft_ssd_prefill, mdraft_ssd_prefill_workspace_bytes, mdraft_ssd_tree_step,
     mdraft_state_commit, mdraft_tree_step, mdraft_tree_step_proj, mdraft_version, status_string,
 )

@@ -30,6 +30,7 @@ EXPORTS = (
     "mdraft_ucb_reward", "mdraft_ucb_select", "mdraft_ucb_update",
     "mdraft_ssd_prefill_workspace_bytes", "mdraft_ssd_prefill", "mdraft_ssd_tree_step",
     "mdraft_prefill_stack_workspace_bytes", "mdraft_prefill_stack_launches", "mdraft_conv_scan_prefill_stack", "mdraft_tree_step_stack",
+    "mdraft_block_generation",
 )
 
 
@@ -97,7 +98,7 @@ except ImportError:   # the package has to be importable for its own build
 # entry points whose arguments csrc/host.cpp marshals, in the order of its table
 _HOST_CALLS = ("mdraft_conv_scan_prefill", "mdraft_conv_scan_prefill_noalloc", "mdraft_tree_step", "mdraft_tree_step_proj",
                "mdraft_state_commit", "mdraft_ssd_prefill", "mdraft_ssd_tree_step", "mdraft_conv_scan_prefill_stack",
-               "mdraft_tree_step_stack")
+               "mdraft_tree_step_stack", "mdraft_block_generation")
 
 
 def load_library(path: Optional[str] = None):
@@ -317,6 +318,16 @@ def mdraft_tree_step_stack(layers: Sequence[Layer], which: Sequence[int], cache:
     if rc != 0:
         raise MdraftError(rc, "mdraft_tree_step_stack")
     return True
+
+
+def mdraft_block_generation(layers: Sequence[Layer], weights, cache: StateCache, tokens: torch.Tensor, parent_slot: torch.Tensor,
+                            node_slot: torch.Tensor, h: torch.Tensor, xz: torch.Tensor, y: torch.Tensor, logits: torch.Tensor,
+                            dev_status: Optional[torch.Tensor] = None, stream=None, flags: Optional[int] = None, eps: float = 1e-5) -> None:
+    """One generation of a block stack.  weights = (W_in list, W_x list, W_dt list, W_out list, embed, W_lm), bf16; h, xz, y are
+    contiguous scratch tensors with at least one row per node."""
+    rc = _host.block_generation(_entry(), layers, weights, cache, tokens, parent_slot, node_slot, h, xz, y, logits, dev_status, stream, flags, eps)
+    if rc != 0:
+        raise MdraftError(rc, "mdraft_block_generation")
 
 
 NOALLOC_SCRATCH_BYTES = 8 << 20

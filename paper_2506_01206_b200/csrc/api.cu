@@ -7,6 +7,7 @@
 
 #include <atomic>
 
+#include "block.cuh"
 #include "commit.cuh"
 #include "common.cuh"
 #include "prefill.cuh"
@@ -497,9 +498,60 @@ int mdraft_tree_step_proj(const mdraft_layer* layer, const mdraft_cache* cache, 
     a.x = x; a.z = z; a.out = out;
     a.ldx = ldx; a.ldz = ldz; a.ldo = ldo;
     a.W_x = proj->W_x; a.W_dt = proj->W_dt; a.dt_rank = proj->dt_rank; a.nodes_per_cluster = proj->nodes_per_cluster;
-    a.parent_slot = parent_slot; a.node_slot = node_slot; a.n_nodes = n_nodes; a.dev_status = dev_status;
+    a.parent_slot = parent_slot; a.node_slot = node_slot; a.n_nodes = n_nodes; a.chained = 0; a.dev_status = dev_status;
     if (launch_tree_proj(a, act, static_cast<cudaStream_t>(stream)) != cudaSuccess) return MDRAFT_ERR_CUDA;
     return MDRAFT_OK;
+}
+
+int mdraft_block_generation(const mdraft_block_stack* stack, const mdraft_cache* cache, const int64_t* tokens, int32_t n_nodes,
+                            const int32_t* parent_slot, const int32_t* node_slot, void* h, void* xz, void* y, void* logits, int64_t ldl,
+                            int32_t* dev_status, void* stream) {
+    if (!stack || stack->n_layers <= 0 || !stack->layers || !stack->W_in || !stack->W_x || !stack->W_dt || !stack->W_out || !stack->embed || !stack->W_lm)
+        return MDRAFT_ERR_INVALID_ARG;
+    if (n_nodes < 0) return MDRAFT_ERR_INVALID_ARG;
+    const int D = stack->layers->d_inner, M = stack->d_model, R = stack->dt_rank;
+    int rc;
+    for (int32_t l = 0; l < stack->n_layers; ++l) {
+        const mdraft_layer* L = stack->layers + l;
+        if ((rc = check_layer(L))) return rc;
+        if (L->d_inner != D || L->act != MDRAFT_BF16) return MDRAFT_ERR_UNSUPPORTED;
+        if (L->flags & (MDRAFT_PRECONV | MDRAFT_CONV_ONLY)) return MDRAFT_ERR_INVALID_ARG;
+        if ((rc = check_cache(cache, D, MDRAFT_BF16, l))) return rc;
+        for (const void* w : {stack->W_in[l], stack->W_x[l], stack->W_dt[l], stack->W_out[l]}) {
+            if (!w) return MDRAFT_ERR_INVALID_ARG;
+            if (!aligned16(w)) return MDRAFT_ERR_MISALIGNED;
+        }
+    }
+    if (M < 32 || M > kBlockMaxModel || M % 32 || D % 32 || D > kBlockMaxInner || stack->vocab < 8 || stack->vocab % 8 || R < 8 || R > kProjMaxRank ||
+        R % 8 || tree_proj_block_channels(D) == 0 || n_nodes > kBlockMaxNodes)
+        return MDRAFT_ERR_UNSUPPORTED;
+    if (n_nodes == 0) return MDRAFT_OK;
+    if (!tokens || !parent_slot || !node_slot || !h || !xz || !y || !logits || ldl < stack->vocab) return MDRAFT_ERR_INVALID_ARG;
+    for (const void* q : {(const void*)h, (const void*)xz, (const void*)y, (const void*)logits, stack->embed, stack->W_lm})
+        if (!aligned16(q)) return MDRAFT_ERR_MISALIGNED;
+    if (ldl % 8) return MDRAFT_ERR_MISALIGNED;
+    typedef __nv_bfloat16 bf;
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    bf *hb = static_cast<bf*>(h), *xzb = static_cast<bf*>(xz), *yb = static_cast<bf*>(y);
+    // The first kernel is an ordinary launch: everything ahead of the call is complete before a kernel of the call reads
+    // a parent's state, which no other kernel of the call writes.  Each later kernel may start while the one ahead runs.
+    cudaError_t e = launch_embed(tokens, static_cast<const bf*>(stack->embed), hb, n_nodes, M, stack->vocab, dev_status, st);
+    for (int32_t l = 0; l < stack->n_layers && e == cudaSuccess; ++l) {
+        e = launch_small_linear({hb, static_cast<const bf*>(stack->W_in[l]), nullptr, xzb, M, 2 * (int64_t)D, 2 * (int64_t)D, n_nodes, 2 * D, M, stack->eps}, st);
+        if (e != cudaSuccess) break;
+        TreeProjArgs a;
+        a.L = layer_dev(stack->layers + l);
+        a.pool = pool_dev(cache, MDRAFT_BF16, l);
+        a.x = xzb; a.z = xzb + D; a.out = yb;
+        a.ldx = a.ldz = 2 * (int64_t)D; a.ldo = D;
+        a.W_x = stack->W_x[l]; a.W_dt = stack->W_dt[l]; a.dt_rank = R; a.nodes_per_cluster = 0;
+        a.parent_slot = parent_slot; a.node_slot = node_slot; a.n_nodes = n_nodes; a.chained = 1; a.dev_status = dev_status;
+        if ((e = launch_tree_proj(a, MDRAFT_BF16, st)) != cudaSuccess) break;
+        e = launch_small_linear({yb, static_cast<const bf*>(stack->W_out[l]), hb, hb, D, M, M, n_nodes, M, D, -1.0f}, st);
+    }
+    if (e == cudaSuccess)
+        e = launch_small_linear({hb, static_cast<const bf*>(stack->W_lm), nullptr, static_cast<bf*>(logits), M, stack->vocab, ldl, n_nodes, stack->vocab, M, stack->eps}, st);
+    return e == cudaSuccess ? MDRAFT_OK : MDRAFT_ERR_CUDA;
 }
 
 int mdraft_state_commit(const mdraft_cache* cache, int32_t d_inner, int32_t d_state, int32_t d_conv, int32_t act,

@@ -1,0 +1,27 @@
+// Launch interface of the drafter block's matrix products (internal to the library).
+#pragma once
+
+#include "common.cuh"
+
+namespace mdraft {
+
+constexpr int kBlockMaxNodes = 64;    // rows of a generation these kernels take
+constexpr int kBlockMaxModel = 1408;  // a block's columns of W fit its shared memory: d_model for in_proj and the LM head,
+constexpr int kBlockMaxInner = 4096;  // d_inner for out_proj
+
+// out[m][n] = sum_k a[m][k] W[k][n], all bf16, fp32 accumulation; rows of a optionally normalised, out optionally added to.
+// k a multiple of 32, n of 8, m at most kBlockMaxNodes.
+struct SmallLinear {
+    const __nv_bfloat16 *a, *W;
+    const __nv_bfloat16* add;  // same shape and stride as out, or NULL
+    __nv_bfloat16* out;
+    int64_t lda, ldw, ldo;
+    int m, n, k;
+    float eps;                 // >= 0: the sum is scaled by 1 / sqrt(mean_k a[m][k]^2 + eps); < 0: not
+};
+
+cudaError_t launch_small_linear(const SmallLinear& p, cudaStream_t st);
+
+cudaError_t launch_embed(const int64_t* tokens, const __nv_bfloat16* embed, __nv_bfloat16* h, int m, int d, int vocab, int32_t* dev_status, cudaStream_t st);
+
+}  // namespace mdraft

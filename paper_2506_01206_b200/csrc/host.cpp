@@ -28,6 +28,7 @@ struct Entry {
     decltype(&mdraft_ssd_tree_step) ssd_tree_step;
     decltype(&mdraft_conv_scan_prefill_stack) prefill_stack;
     decltype(&mdraft_tree_step_stack) tree_step_stack;
+    decltype(&mdraft_block_generation) block_generation;
 };
 
 struct Failed {};  // a Python exception is set
@@ -487,9 +488,68 @@ PyObject* tree_step_stack(PyObject* const* a) {
     });
 }
 
+// A list of dense bf16 matrices of one shape, as addresses.
+std::vector<const void*> dense(PyObject* list, const char* name, int64_t rows, int64_t cols) {
+    Ref f(PySequence_Fast(list, name));
+    std::vector<const void*> v;
+    for (Py_ssize_t i = 0; i < PySequence_Fast_GET_SIZE(f.p); ++i) {
+        const at::Tensor& t = tensor(PySequence_Fast_GET_ITEM(f.p, i), name);
+        if (t.scalar_type() != at::kBFloat16 || t.dim() != 2 || t.size(0) != rows || t.size(1) != cols || !t.is_contiguous() || !t.is_cuda())
+            fail(PyExc_ValueError, std::string(name) + ": need contiguous bf16 CUDA matrices of " + std::to_string(rows) + " x " + std::to_string(cols));
+        v.push_back(t.const_data_ptr());
+    }
+    return v;
+}
+void* scratch(PyObject* o, const char* name, int64_t rows, int64_t cols) {
+    const at::Tensor& t = tensor(o, name);
+    if (t.scalar_type() != at::kBFloat16 || t.dim() != 2 || t.size(0) < rows || t.size(1) != cols || !t.is_contiguous())
+        fail(PyExc_ValueError, std::string(name) + ": need a contiguous bf16 matrix with " + std::to_string(cols) + " columns and a row per node");
+    return t.data_ptr();
+}
+
+// (table, layers, (W_in, W_x, W_dt, W_out, embed, W_lm), cache, tokens, parent_slot, node_slot, h, xz, y, logits, dev_status,
+//  stream, flags, eps)
+PyObject* block_generation(PyObject* const* a) {
+    Ref ls(PySequence_Fast(a[1], "layers")), w(PySequence_Fast(a[2], "weights"));
+    if (PySequence_Fast_GET_SIZE(w.p) != 6) fail(PyExc_ValueError, "weights are (W_in, W_x, W_dt, W_out, embed, W_lm)");
+    std::vector<mdraft_layer> layers;
+    for (Py_ssize_t i = 0; i < PySequence_Fast_GET_SIZE(ls.p); ++i) layers.push_back(layer_of(PySequence_Fast_GET_ITEM(ls.p, i), a[13]));
+    if (layers.empty()) fail(PyExc_ValueError, "no layers");
+    const at::Tensor &embed = tensor(PySequence_Fast_GET_ITEM(w.p, 4), "embed"), &lm = tensor(PySequence_Fast_GET_ITEM(w.p, 5), "W_lm");
+    Ref dts(PySequence_Fast(PySequence_Fast_GET_ITEM(w.p, 2), "W_dt"));
+    if (PySequence_Fast_GET_SIZE(dts.p) < 1) fail(PyExc_ValueError, "no W_dt");
+    const at::Tensor& wdt = tensor(PySequence_Fast_GET_ITEM(dts.p, 0), "W_dt");
+    if (embed.dim() != 2 || lm.dim() != 2 || wdt.dim() != 2 || embed.scalar_type() != at::kBFloat16 || lm.scalar_type() != at::kBFloat16 ||
+        !embed.is_contiguous() || !lm.is_contiguous() || embed.size(0) != lm.size(1) || embed.size(1) != lm.size(0))
+        fail(PyExc_ValueError, "embed (vocab, d_model) and W_lm (d_model, vocab) must be contiguous bf16 matrices");
+    const int64_t D = layers[0].d_inner, M = embed.size(1), V = embed.size(0), R = wdt.size(1);
+    const auto W_in = dense(PySequence_Fast_GET_ITEM(w.p, 0), "W_in", M, 2 * D), W_x = dense(PySequence_Fast_GET_ITEM(w.p, 1), "W_x", R + 2 * layers[0].d_state, D),
+               W_dt = dense(dts.p, "W_dt", D, R), W_out = dense(PySequence_Fast_GET_ITEM(w.p, 3), "W_out", D, M);
+    const size_t n = layers.size();
+    if (W_in.size() != n || W_x.size() != n || W_dt.size() != n || W_out.size() != n) fail(PyExc_ValueError, "one matrix of each kind per layer");
+    const mdraft_block_stack stack = {(int32_t)n, (int32_t)M, (int32_t)R, (int32_t)V, layers.data(), W_in.data(), W_x.data(), W_dt.data(), W_out.data(),
+                                      embed.const_data_ptr(), lm.const_data_ptr(), (float)PyFloat_AsDouble(a[14])};
+    if (PyErr_Occurred()) throw Failed();
+    const Cache c(a[3]);
+    const at::Tensor& tok = tensor(a[4], "tokens");
+    if (tok.scalar_type() != at::kLong || !tok.is_contiguous()) fail(PyExc_TypeError, "tokens must be contiguous int64");
+    const int64_t m = tok.numel();
+    const Nodes nodes(a[5], a[6], m);
+    void *h = scratch(a[7], "h", m, M), *xz = scratch(a[8], "xz", m, 2 * D), *y = scratch(a[9], "y", m, D);
+    const Matrix logits(a[10], "logits");
+    if (logits.rows != m || tensor(a[10], "logits").scalar_type() != at::kBFloat16) fail(PyExc_ValueError, "logits: one bf16 row per node");
+    int32_t* st = static_cast<int32_t*>(mutable_data(a[11], "dev_status"));
+    void* stream = stream_of(a[12]);
+    const Entry& e = entry(a[0]);
+    return released([&] {
+        return e.block_generation(&stack, c.get(), static_cast<const int64_t*>(tok.const_data_ptr()), (int32_t)m, nodes.parent, nodes.node, h, xz, y,
+                                  logits.out(), logits.ld, st, stream);
+    });
+}
+
 #define ENTRY(name) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(&guarded<name>)), METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {ENTRY(table), ENTRY(prefill), ENTRY(prefill_noalloc), ENTRY(tree_step), ENTRY(tree_step_proj),
-                         ENTRY(commit), ENTRY(ssd_prefill), ENTRY(ssd_tree_step), ENTRY(prefill_stack), ENTRY(tree_step_stack),
+                         ENTRY(commit), ENTRY(ssd_prefill), ENTRY(ssd_tree_step), ENTRY(prefill_stack), ENTRY(tree_step_stack), ENTRY(block_generation),
                          {nullptr, nullptr, 0, nullptr}};
 
 PyModuleDef module_def = {PyModuleDef_HEAD_INIT, "_host", "argument marshalling for libmdraft.so", -1, methods, nullptr, nullptr, nullptr, nullptr};

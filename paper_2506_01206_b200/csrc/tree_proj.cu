@@ -15,6 +15,10 @@
 // state, window and output leave by bulk stores.  All waits on the mbarriers are bounded.  The cluster barrier is
 // executed unconditionally by every thread of every block of the cluster (a block that gave up on its copies still
 // takes part), so no block can wait for one that left.
+//
+// Behind a kernel of this library that produces x and z (an in_proj of csrc/block.cu) the step is launched with programmatic stream
+// serialisation: slots, constants, the rows of W_x and W_dt and the parent's state and window are requested before the
+// wait for that kernel, x and z after it.
 #include "common.cuh"
 #include "tree_proj.cuh"
 
@@ -151,6 +155,7 @@ __global__ void __launch_bounds__(CB) tree_proj_kernel(const TreeProjArgs p) {
     float* const s_s = reinterpret_cast<float*>(s_dyn + S::kS);
     uint64_t* const bars = reinterpret_cast<uint64_t*>(s_dyn + S::kBars);  // [i][0]: x + window, [i][1]: z + state
 
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // no effect unless the next kernel asks for it
     const int D = p.L.d_inner, R = p.dt_rank, rows = R + 2 * kN;
     const int node0 = blockIdx.x * NT;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -176,6 +181,8 @@ __global__ void __launch_bounds__(CB) tree_proj_kernel(const TreeProjArgs p) {
         }
     }
 
+    auto issue_x = [&](int i) { bulk_load(s_x + i * CB, static_cast<const AT*>(p.x) + (size_t)(node0 + i) * p.ldx + d0, row_bytes, &bars[2 * i]); };
+    auto issue_z = [&](int i) { bulk_load(s_z + i * CB, static_cast<const AT*>(p.z) + (size_t)(node0 + i) * p.ldz + d0, row_bytes, &bars[2 * i + 1]); };
     if (tid == 0) {
 #pragma unroll
         for (int i = 0; i < 2 * NT; ++i) mbar_init(&bars[i], 1);
@@ -186,7 +193,7 @@ __global__ void __launch_bounds__(CB) tree_proj_kernel(const TreeProjArgs p) {
             const bool have_parent = pslot[i] >= 0;
             const AT* conv_parent = static_cast<const AT*>(p.pool.conv) + (size_t)pslot[i] * p.pool.conv_slot_stride + d0;
             mbar_expect_tx(&bars[2 * i], row_bytes + (have_parent ? (kW - 1) * row_bytes : 0u));
-            bulk_load(s_x + i * CB, static_cast<const AT*>(p.x) + (size_t)(node0 + i) * p.ldx + d0, row_bytes, &bars[2 * i]);
+            if (!p.chained) issue_x(i);
             if (have_parent)
                 for (int j = 0; j < kW - 1; ++j) bulk_load(s_conv + (i * (kW - 1) + j) * CB, conv_parent + (size_t)j * D, row_bytes, &bars[2 * i]);
         }
@@ -197,7 +204,7 @@ __global__ void __launch_bounds__(CB) tree_proj_kernel(const TreeProjArgs p) {
             mbar_expect_tx(&bars[2 * i + 1], row_bytes + (have_parent ? h_bytes : 0u));
             if (have_parent)
                 bulk_load(s_h + i * CB * (kN / 4), p.pool.ssm + (size_t)pslot[i] * p.pool.ssm_slot_stride + (size_t)d0 * kN, h_bytes, &bars[2 * i + 1]);
-            bulk_load(s_z + i * CB, static_cast<const AT*>(p.z) + (size_t)(node0 + i) * p.ldz + d0, row_bytes, &bars[2 * i + 1]);
+            if (!p.chained) issue_z(i);
         }
     }
 
@@ -245,6 +252,17 @@ __global__ void __launch_bounds__(CB) tree_proj_kernel(const TreeProjArgs p) {
     for (int j = 0; j < kPreDt; ++j)
         dpre[j].load(wr + (8 * j < R ? 8 * j : 0));
 
+    if (p.chained) {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        if (tid == 0) {
+#pragma unroll
+            for (int i = 0; i < NT; ++i)
+                if (valid[i]) issue_x(i);
+#pragma unroll
+            for (int i = 0; i < NT; ++i)
+                if (valid[i]) issue_z(i);
+        }
+    }
     __syncthreads();  // the mbarriers are initialised for everyone
     bool waited = true;
 #pragma unroll
@@ -499,20 +517,19 @@ cudaError_t launch_nt(const TreeProjArgs& p, int n_blocks, cudaStream_t st) {
     cfg.blockDim = dim3(CB, 1, 1);
     cfg.dynamicSmemBytes = kSmem;
     cfg.stream = st;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = 1;
     at[0].val.clusterDim.y = (unsigned)n_blocks;  // the blocks of one group of nodes
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.numAttrs = p.chained ? 2 : 1;
     const bool pow = p.L.flags & MDRAFT_A_POWERS;
-    auto kernel = pow ? tree_proj_kernel<AT, CB, NT, true> : tree_proj_kernel<AT, CB, NT, false>;
-    if (kSmem > 48 * 1024) {  // a property of the loaded function, not an allocation
-        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
-        if (e != cudaSuccess) return e;
-    }
-    return cudaLaunchKernelEx(&cfg, kernel, p);
+    const cudaError_t e = pow ? allow_smem<tree_proj_kernel<AT, CB, NT, true>>(kSmem) : allow_smem<tree_proj_kernel<AT, CB, NT, false>>(kSmem);
+    if (e != cudaSuccess) return e;
+    return cudaLaunchKernelEx(&cfg, pow ? tree_proj_kernel<AT, CB, NT, true> : tree_proj_kernel<AT, CB, NT, false>, p);
 }
 
 template <typename AT>

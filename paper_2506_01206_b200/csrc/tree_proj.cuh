@@ -20,6 +20,7 @@ struct TreeProjArgs {
     int nodes_per_cluster;  // 0: chosen from the level's width; else 1, 2 or 4
     const int32_t *parent_slot, *node_slot;
     int n_nodes;
+    int chained;       // 1: launched behind a kernel that releases it early; only x and z are that kernel's work
     int32_t* dev_status;
 };
 

@@ -3,13 +3,15 @@
 In a Mamba block the step size, B and C are projections of the conv output, so the fused conv+scan call cannot be
 fed by a real model.  The library offers two ways: the split mode, `MDRAFT_CONV_ONLY` (conv window + SiLU), the
 caller's projections, then `MDRAFT_PRECONV` (recurrence + gate); or `mdraft_tree_step_proj`, which takes the two
-projection matrices and does conv step, projections, recurrence and gate in one launch (`fused=True` here).  This
-module is the caller, for drafting only: embedding,
+projection matrices and does conv step, projections, recurrence and gate in one launch (`fused=True` here).  With
+bf16 weights and levels of at most BLOCK_MAX_NODES nodes a generation is one call, `mdraft_block_generation`, whose kernels
+take the norms and the other projections in as well (in either mode: what the modes round to bf16 in between differs,
+and the call rounds least).  This module is the caller, for drafting only: embedding,
 24 x [RMSNorm, in_proj, conv step, x_proj, dt_proj, S6 step, out_proj, residual], final norm, LM head, and
 tree-structured drafting by batch generation (paper Section 4.1): generation i is one batch of all nodes of level
 i, each node forks its parent's conv / SSM state by slot index, and the children of a node are its N_i most
-probable next tokens.  The projections are plain torch matmuls on random weights (they are outside the library,
-and there are no trained weights here): what this measures is the drafting LATENCY of the whole stack per round,
+probable next tokens.  Otherwise the projections are plain torch matmuls.  Weights are random
+(there are no trained weights here): what this measures is the drafting LATENCY of the whole stack per round,
 the quantity of the paper's Table 4, not acceptance.
 
 Slots: 0 = the sequence's committed state; node i of the current round = slot 1 + i.
@@ -27,6 +29,9 @@ from . import binding as mb
 # Above this many nodes in a level the one-launch projection step loses to the split mode (its per-node re-reads of
 # the two projection matrices cost more than the split mode's matrix products); the stack switches path there.
 PROJ_STEP_MAX_NODES = 256
+
+# Above this many nodes in a level the torch matmuls amortise the weights better than the block kernels' 32-row tiles.
+BLOCK_MAX_NODES = 64
 
 
 class ToyDrafter:
@@ -46,7 +51,10 @@ class ToyDrafter:
         self.W_out = [rnd(d_inner, d_model, scale=d_inner ** -0.5 / (2 * n_layers) ** 0.5) for _ in range(n_layers)]
         self.W_lm = rnd(d_model, vocab, scale=d_model ** -0.5)
         self.fused = fused
-        if fused:   # the library takes both matrices as (out features, in features), rows contiguous
+        # what mdraft_block_generation takes (include/mdraft.h)
+        self.block_kernels = (act == torch.bfloat16 and d_model % 32 == 0 and d_model <= 1408 and d_inner % 32 == 0 and d_inner <= 4096
+                              and vocab % 8 == 0 and dt_rank % 8 == 0 and 8 <= dt_rank <= 256)
+        if fused or self.block_kernels:   # the library takes both matrices as (out features, in features), rows contiguous
             self.W_x_rows = [w.T.contiguous() for w in self.W_x]
             self.W_dt_rows = [w.T.contiguous() for w in self.W_dt]
         A = -torch.arange(1, N + 1, dtype=torch.float32, device=device).repeat(d_inner, 1).contiguous()
@@ -65,6 +73,10 @@ class ToyDrafter:
         self.u = torch.zeros((max_nodes, d_inner), dtype=act, device=device)
         self.y = torch.zeros((max_nodes, d_inner), dtype=act, device=device)
         self.logits = torch.zeros((max_nodes, vocab), dtype=act, device=device)
+        if self.block_kernels:
+            rows = min(max_nodes, BLOCK_MAX_NODES)
+            self._h = torch.empty((rows, d_model), dtype=act, device=device)
+            self._xz = torch.empty((rows, 2 * d_inner), dtype=act, device=device)
         self._graphs = {}
         self._round_graphs = {}
         self.root_token = torch.zeros(1, dtype=torch.int64, device=device)   # read by the round, so that a captured round can be replayed with another root
@@ -76,6 +88,11 @@ class ToyDrafter:
     def _generation(self, lo: int, hi: int) -> None:
         """One batch-generation step for nodes [lo, hi): tokens / parent_slot / node_slot rows lo..hi-1 are read,
         logits rows lo..hi-1 are written; conv and SSM states of the nodes' slots are written."""
+        if self.block_kernels and hi - lo <= BLOCK_MAX_NODES:
+            mb.mdraft_block_generation(self.layers, (self.W_in, self.W_x_rows, self.W_dt_rows, self.W_out, self.embed, self.W_lm), self.cache,
+                                       self.tokens[lo:hi], self.parent_slot[lo:hi], self.node_slot[lo:hi], self._h, self._xz, self.y,
+                                       self.logits[lo:hi], self.status, flags=mb.MDRAFT_DT_SOFTPLUS | mb.MDRAFT_A_POWERS)
+            return
         N, R = 16, self.dt_rank
         h = self.embed[self.tokens[lo:hi]]
         ps, ns = self.parent_slot[lo:hi], self.node_slot[lo:hi]
