@@ -320,7 +320,7 @@ int mdraft_tree_step_proj(const mdraft_layer *layer, const mdraft_cache *cache, 
  *   h, xz, y            : device scratch of n_nodes x d_model, x 2 d_inner, x d_inner bf16
  *   logits              : n_nodes rows of vocab bf16, stride ldl (a multiple of 8)
  * Layer l works on pool layer l.  No node_slot may equal another node's parent_slot or node_slot.
- * Supported: n_nodes <= MDRAFT_BLOCK_MAX_NODES, d_model a multiple of 32 up to 1408, d_inner a multiple of 32 up to 4096, vocab
+ * Supported: n_nodes <= MDRAFT_BLOCK_MAX_NODES, d_model a multiple of 32 up to 1408, d_inner a multiple of 32 up to 2048, vocab
  * a multiple of 8, dt_rank as above; anything else is MDRAFT_ERR_UNSUPPORTED.
  */
 #define MDRAFT_BLOCK_MAX_NODES 64

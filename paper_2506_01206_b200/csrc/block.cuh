@@ -7,7 +7,7 @@ namespace mdraft {
 
 constexpr int kBlockMaxNodes = 64;    // rows of a generation these kernels take
 constexpr int kBlockMaxModel = 1408;  // a block's columns of W fit its shared memory: d_model for in_proj and the LM head,
-constexpr int kBlockMaxInner = 4096;  // d_inner for out_proj
+constexpr int kBlockMaxInner = 2048;  // d_inner for out_proj, beside 32 rows of its activations
 
 // out[m][n] = sum_k a[m][k] W[k][n], all bf16, fp32 accumulation; rows of a optionally normalised, out optionally added to.
 // k a multiple of 32, n of 8, m at most kBlockMaxNodes.
@@ -15,8 +15,9 @@ struct SmallLinear {
     const __nv_bfloat16 *a, *W;
     const __nv_bfloat16* add;  // same shape and stride as out, or NULL
     __nv_bfloat16* out;
-    int64_t lda, ldw, ldo;
+    int64_t ldw, ldo;          // rows of a are dense (k values)
     int m, n, k;
+    int32_t* dev_status;
     float eps;                 // >= 0: the sum is scaled by 1 / sqrt(mean_k a[m][k]^2 + eps); < 0: not
 };
 

@@ -52,7 +52,7 @@ class ToyDrafter:
         self.W_lm = rnd(d_model, vocab, scale=d_model ** -0.5)
         self.fused = fused
         # what mdraft_block_generation takes (include/mdraft.h)
-        self.block_kernels = (act == torch.bfloat16 and d_model % 32 == 0 and d_model <= 1408 and d_inner % 32 == 0 and d_inner <= 4096
+        self.block_kernels = (act == torch.bfloat16 and d_model % 32 == 0 and d_model <= 1408 and d_inner % 32 == 0 and d_inner <= 2048
                               and vocab % 8 == 0 and dt_rank % 8 == 0 and 8 <= dt_rank <= 256)
         if fused or self.block_kernels:   # the library takes both matrices as (out features, in features), rows contiguous
             self.W_x_rows = [w.T.contiguous() for w in self.W_x]
