@@ -398,7 +398,7 @@ int mdraft_ssd_prefill(const mdraft_ssd_layer *layer, const mdraft_cache *cache,
 /*
  * Draft-tree step of an SSD layer: one token for each node of a level, node i from slot parent_slot[i] into slot
  * node_slot[i] (paper Section 4.1, as mdraft_tree_step).  x, z, out: (M, D); dt: (M, H); B, C: (M, 128).  Levels,
- * hazards and device-side faults as in mdraft_tree_step; every level is an ordinary launch.  All arithmetic is
+ * hazards (early input rows included) and device-side faults as in mdraft_tree_step.  All arithmetic is
  * fp32 (no tensor cores: one token per node is a memory-bound update of a (D, 128) state).
  */
 int mdraft_ssd_tree_step(const mdraft_ssd_layer *layer, const mdraft_cache *cache, int32_t layer_index,

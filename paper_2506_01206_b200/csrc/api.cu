@@ -757,10 +757,13 @@ int mdraft_ssd_tree_step(const mdraft_ssd_layer* layer, const mdraft_cache* cach
     a.ldx = ldx; a.ldz = ldz; a.lddt = lddt; a.ldb = ldb; a.ldc = ldc; a.ldo = ldo;
     a.parent_slot = parent_slot; a.node_slot = node_slot; a.dev_status = dev_status;
     const int levels = level_offsets ? n_levels : 1;
+    a.level_in_call = 0;
     for (int l = 0; l < levels; ++l) {
         a.lvl_begin = level_offsets ? level_offsets[l] : 0;
         a.lvl_end = level_offsets ? level_offsets[l + 1] : n_nodes;
+        if (a.lvl_end == a.lvl_begin) continue;
         if (launch_ssd_step(a, static_cast<cudaStream_t>(stream)) != cudaSuccess) return MDRAFT_ERR_CUDA;
+        ++a.level_in_call;
     }
     return MDRAFT_OK;
 }

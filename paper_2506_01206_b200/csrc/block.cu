@@ -75,22 +75,29 @@ __device__ __forceinline__ int place_of(int k) { return ((k & 6) << 2) + ((k >> 
 __host__ __device__ constexpr int w_pitch(int nt) { return nt * 2 + 16; }
 __host__ __device__ constexpr int part_pitch(int nt) { return nt + 4; }
 
-// One block of 32 of the contraction: acc += W^T a for the block's columns and the first `tiles` groups of 8 nodes.
+// Fragments of W^T for one block of 32 of the contraction and kColTiles x 16 columns: both steps of 16.
+template <int kColTiles> struct WFrag { uint32_t v[kColTiles][2][4]; };
 template <int kColTiles>
-__device__ __forceinline__ void multiply_block(float (&acc)[kColTiles][kNodeTiles][4], const uint4 (&a)[kNodeTiles], int tiles, uint32_t w_rows, int pitch, int lane) {
+__device__ __forceinline__ void load_w(WFrag<kColTiles>& w, uint32_t w_rows, int pitch, int lane) {
 #pragma unroll
     for (int j = 0; j < kColTiles; ++j) {
         // lanes 0-7, 8-15, .. give the rows of the four 8 x 8 blocks of a fragment: columns 0-7 / 8-15 of the first 8 places,
         // then of the next 8; places 16.. are the second step
         const uint32_t at = w_rows + (uint32_t)(((lane & 7) + ((lane >> 4) << 3)) * pitch + j * 32 + ((lane >> 3) & 1) * 16);
-        uint32_t w0[4], w1[4];
-        ldmatrix_x4_trans(w0, at);
-        ldmatrix_x4_trans(w1, at + 16 * pitch);
+        ldmatrix_x4_trans(w.v[j][0], at);
+        ldmatrix_x4_trans(w.v[j][1], at + 16 * pitch);
+    }
+}
+// acc += W^T a for the first `tiles` groups of 8 nodes.
+template <int kColTiles>
+__device__ __forceinline__ void multiply(float (&acc)[kColTiles][kNodeTiles][4], const WFrag<kColTiles>& w, const uint4 (&a)[kNodeTiles], int tiles) {
 #pragma unroll
-        for (int i = 0; i < kNodeTiles; ++i) {
-            if (i < tiles) {
-                mma16816(acc[j][i], w0[0], w0[1], w0[2], w0[3], a[i].x, a[i].y);
-                mma16816(acc[j][i], w1[0], w1[1], w1[2], w1[3], a[i].z, a[i].w);
+    for (int i = 0; i < kNodeTiles; ++i) {
+        if (i < tiles) {
+#pragma unroll
+            for (int j = 0; j < kColTiles; ++j) {
+                mma16816(acc[j][i], w.v[j][0][0], w.v[j][0][1], w.v[j][0][2], w.v[j][0][3], a[i].x, a[i].y);
+                mma16816(acc[j][i], w.v[j][1][0], w.v[j][1][1], w.v[j][1][2], w.v[j][1][3], a[i].z, a[i].w);
             }
         }
     }
@@ -117,9 +124,9 @@ __device__ __forceinline__ void put_part(float* part, const float (&acc)[kColTil
 #pragma unroll
                 for (int e = 0; e < 4; ++e) part[(i * 8 + 2 * t + (e & 1)) * kPitch + j * 16 + (e >> 1) * 8 + g] = acc[j][i][e];
 }
-// The warps' shares added up in order, normalised, added to, rounded and stored.
+// The warps' shares added up in order, normalised, added to (add0: what the thread's first pair is added to), rounded, stored.
 template <int NT, int NW, bool NORM>
-__device__ __forceinline__ void finish(const SmallLinear& p, const float* part, const float (*s_sq)[kRows], int rows, int m0, int n0) {
+__device__ __forceinline__ void finish(const SmallLinear& p, const float* part, const float (*s_sq)[kRows], int rows, int m0, int n0, const __nv_bfloat162& add0) {
     constexpr int kPitch = part_pitch(NT);
     for (int idx = threadIdx.x; idx < rows * NT / 2; idx += NW * 32) {
         const int r = idx / (NT / 2), c = (idx - r * (NT / 2)) * 2, col = n0 + c;
@@ -137,7 +144,7 @@ __device__ __forceinline__ void finish(const SmallLinear& p, const float* part, 
         }
         const size_t at = (size_t)(m0 + r) * p.ldo + col;
         if (p.add) {
-            const __nv_bfloat162 b = *reinterpret_cast<const __nv_bfloat162*>(p.add + at);
+            const __nv_bfloat162 b = idx == threadIdx.x ? add0 : *reinterpret_cast<const __nv_bfloat162*>(p.add + at);
             x += __bfloat162float(b.x); y += __bfloat162float(b.y);
         }
         *reinterpret_cast<__nv_bfloat162*>(p.out + at) = __floats2bfloat162_rn(x, y);
@@ -149,8 +156,9 @@ __host__ __device__ inline int rows_offset(int k, int nt, int nw) {   // W or th
     return ((w > part ? w : part) + 127) / 128 * 128;
 }
 
-template <int NT, int NW, bool NORM>
-__global__ void __launch_bounds__(NW * 32) small_linear_kernel(const SmallLinear p) {
+// PRE: blocks of the contraction whose fragments of W a warp takes into registers before the wait.
+template <int NT, int NW, int PRE, bool NORM>
+__global__ void __launch_bounds__(NW * 32, PRE > 0 ? 1 : 2) small_linear_kernel(const SmallLinear p) {
     constexpr int kCols = NT / 16, kPitch = w_pitch(NT);
     extern __shared__ __align__(128) unsigned char s_w[];   // W as [k][NT], later the warps' partial results [NW][kRows][NT]; then the activations
     __shared__ float s_sq[NW][kRows];
@@ -176,27 +184,48 @@ __global__ void __launch_bounds__(NW * 32) small_linear_kernel(const SmallLinear
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
     unsigned char* const s_a = s_w + rows_offset(p.k, NT, NW);
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
+    WFrag<kCols> w[PRE > 0 ? PRE : 1];
+#pragma unroll
+    for (int q = 0; q < PRE; ++q)
+        if (warp + q * NW < kblocks) load_w<kCols>(w[q], smem_u32(s_w) + (uint32_t)((warp + q * NW) * 32 * kPitch), kPitch, lane);
     grid_wait();   // the activations are the work of the kernel ahead
     if (threadIdx.x == 0) {
         mbar_expect_tx(&bar, (uint32_t)(rows * p.k * 2));
         bulk_load(s_a, p.a + (size_t)m0 * p.k, (uint32_t)(rows * p.k * 2), &bar);
     }
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    // What the thread's first result is added to is on its way meanwhile.
+    __nv_bfloat162 add0 = __floats2bfloat162_rn(0.0f, 0.0f);
+    {
+        const int r = threadIdx.x / (NT / 2), c = n0 + (threadIdx.x % (NT / 2)) * 2;
+        if (p.add && r < rows && c < p.n) add0 = *reinterpret_cast<const __nv_bfloat162*>(p.add + (size_t)(m0 + r) * p.ldo + c);
+    }
     const bool ok = mbar_wait_bounded(&bar, 0u);
-    __syncwarp();
 
     float acc[kCols][kNodeTiles][4] = {};
     float sq[kNodeTiles] = {};
-    for (int kb = warp; kb < kblocks; kb += NW) {
-        uint4 a[kNodeTiles];
+    auto load_a = [&](uint4 (&a)[kNodeTiles], int kb) {
 #pragma unroll
         for (int i = 0; i < kNodeTiles; ++i) {
             a[i] = make_uint4(0u, 0u, 0u, 0u);
             if (i * 8 + g < rows) a[i] = *reinterpret_cast<const uint4*>(s_a + (i * 8 + g) * p.k * 2 + kb * 64 + t * 16);
             if (NORM) sq[i] = squares(a[i], sq[i]);
         }
-        multiply_block<kCols>(acc, a, tiles, smem_u32(s_w) + (uint32_t)(kb * 32 * kPitch), kPitch, lane);
+    };
+#pragma unroll
+    for (int q = 0; q < PRE; ++q)
+        if (warp + q * NW < kblocks) {
+            uint4 a[kNodeTiles];
+            load_a(a, warp + q * NW);
+            multiply<kCols>(acc, w[q], a, tiles);
+        }
+#pragma unroll 1
+    for (int kb = warp + PRE * NW; kb < kblocks; kb += NW) {
+        uint4 a[kNodeTiles];
+        load_a(a, kb);
+        load_w<kCols>(w[0], smem_u32(s_w) + (uint32_t)(kb * 32 * kPitch), kPitch, lane);
+        multiply<kCols>(acc, w[0], a, tiles);
     }
     if (NORM) put_squares(s_sq[warp], sq, g, t);
     const bool all_ok = !__syncthreads_or(!ok);   // and nobody reads W any more
@@ -204,7 +233,7 @@ __global__ void __launch_bounds__(NW * 32) small_linear_kernel(const SmallLinear
     put_part<kCols>(part + warp * kRows * part_pitch(NT), acc, tiles, g, t);
     __syncthreads();
     if (all_ok) {
-        finish<NT, NW, NORM>(p, part, s_sq, rows, m0, n0);
+        finish<NT, NW, NORM>(p, part, s_sq, rows, m0, n0, add0);
     } else if (threadIdx.x == 0) {
         flag(p.dev_status, MDRAFT_DEV_WAIT_EXPIRED);
         mbar_wait_bounded(&bar, 0u);   // the copy targets this block's shared memory: one more bounded chance
@@ -269,7 +298,11 @@ __global__ void __launch_bounds__(kWideWarps * 32, 1) wide_linear_kernel(const S
 #pragma unroll
         for (int q = 0; q < kWideBlocks; ++q) {
             const int kb = warp + q * NW;
-            if (kb < kblocks) multiply_block<kCols>(acc, a[q], node_tiles, smem_u32(s_w) + (uint32_t)(stage * stage_bytes + kb * 32 * kPitch), kPitch, lane);
+            if (kb < kblocks) {
+                WFrag<kCols> w;
+                load_w<kCols>(w, smem_u32(s_w) + (uint32_t)(stage * stage_bytes + kb * 32 * kPitch), kPitch, lane);
+                multiply<kCols>(acc, w, a[q], node_tiles);
+            }
         }
         __syncwarp();
         const int ahead = stage + kWideStages - 1;   // the stage of the tile before this one, which this warp is done with
@@ -278,7 +311,7 @@ __global__ void __launch_bounds__(kWideWarps * 32, 1) wide_linear_kernel(const S
         __syncthreads();   // the partial results of the tile before have been read
         put_part<kCols>(part + warp * kRows * part_pitch(NT), acc, node_tiles, g, t);
         __syncthreads();
-        finish<NT, NW, NORM>(p, part, s_sq, rows, m0, tile * NT);
+        finish<NT, NW, NORM>(p, part, s_sq, rows, m0, tile * NT, __nv_bfloat162());
     }
 }
 
@@ -312,10 +345,10 @@ cudaError_t launch_chained(dim3 grid, int threads, int smem, const SmallLinear& 
     return cudaLaunchKernelEx(&cfg, kKernel, p);
 }
 
-template <int NT, int NW, bool NORM>
+template <int NT, int NW, int PRE, bool NORM>
 cudaError_t launch_tile(const SmallLinear& p, cudaStream_t st) {
     const int rows = p.m < kRows ? p.m : kRows;
-    return launch_chained<small_linear_kernel<NT, NW, NORM>>(dim3((p.n + NT - 1) / NT, (p.m + kRows - 1) / kRows), NW * 32,
+    return launch_chained<small_linear_kernel<NT, NW, PRE, NORM>>(dim3((p.n + NT - 1) / NT, (p.m + kRows - 1) / kRows), NW * 32,
                                                              rows_offset(p.k, NT, NW) + rows * p.k * 2, p, st);
 }
 
@@ -333,9 +366,16 @@ cudaError_t launch_small_linear(const SmallLinear& p, cudaStream_t st) {
                         : launch_chained<wide_linear_kernel<false>>(grid, kWideWarps * 32, smem, p, st);
     }
     // The narrow tile for a narrow n, whose blocks are few, and for a contraction too long for the wide one's shared memory.
+    // Fragments of W in registers ahead of the wait while one row tile leaves room for the kernels of the chain beside each
+    // other (18 nodes: 329 -> 304 us a generation); with two, the registers they take cost more (64 nodes: 486 -> 534 us).
     const int rows = p.m < kRows ? p.m : kRows;
-    if (p.n <= 16 * 148 || rows_offset(p.k, 32, 12) + rows * p.k * 2 > kMaxSmem) return norm ? launch_tile<16, 12, true>(p, st) : launch_tile<16, 12, false>(p, st);
-    return norm ? launch_tile<32, 12, true>(p, st) : launch_tile<32, 12, false>(p, st);
+    const bool narrow = p.n <= 16 * 148 || rows_offset(p.k, 32, 12) + rows * p.k * 2 > kMaxSmem;
+    if (p.m <= kRows) {
+        if (narrow) return norm ? launch_tile<16, 12, 4, true>(p, st) : launch_tile<16, 12, 4, false>(p, st);
+        return norm ? launch_tile<32, 12, 2, true>(p, st) : launch_tile<32, 12, 2, false>(p, st);
+    }
+    if (narrow) return norm ? launch_tile<16, 12, 0, true>(p, st) : launch_tile<16, 12, 0, false>(p, st);
+    return norm ? launch_tile<32, 12, 0, true>(p, st) : launch_tile<32, 12, 0, false>(p, st);
 }
 
 cudaError_t launch_embed(const int64_t* tokens, const __nv_bfloat16* embed, __nv_bfloat16* h, int m, int d, int vocab, int32_t* dev_status, cudaStream_t st) {

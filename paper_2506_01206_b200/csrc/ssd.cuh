@@ -55,6 +55,7 @@ struct SsdStepArgs {
     __nv_bfloat16* out;
     int64_t ldx, ldz, lddt, ldb, ldc, ldo;
     const int32_t *parent_slot, *node_slot;
+    int level_in_call;   // kernels this call has launched before this level
     int lvl_begin, lvl_end;
     int32_t* dev_status;
 };
