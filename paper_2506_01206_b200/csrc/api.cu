@@ -91,9 +91,9 @@ struct PrefillPlan {
     int chunk_len;       // tokens per chunk (INT_MAX/2 when every sequence is one chunk)
     int n_chunks_bound;  // upper bound on the number of chunks
     bool chunked;
-    bool wide;           // 512-channel blocks (one per SM) instead of 128-channel blocks
+    int boxes;           // 128-channel boxes per block: 1, 2 (unsplit sequences only) or 4 (one block per SM)
     bool longest_first;  // unsplit sequences of different lengths, handed out longest first
-    bool two_per_sm;     // keep two blocks per SM (of the four that fit)
+    bool alone;          // unsplit sequences: one block per SM
     size_t off_q, off_sd, off_h0, off_conv, layer_bytes;
     size_t bytes;        // what the workspace query answers: the call's layers, split
 };
@@ -103,20 +103,23 @@ struct PrefillPlan {
 // When one wave would need chunks longer than kOneWaveMax tokens and the chunks would be uneven (packed batches) or the
 // blocks narrow, several waves of short chunks do better: blocks are then handed out as SMs free up, which evens out
 // uneven sequences and keeps every SM busy to the end (32 packed sequences of 1k-8k tokens: 1607 -> 1512 us).
-constexpr int kBlocksPerSm = 4, kMinChunk = 32, kOneWaveMax = 256, kManyWavesChunk = 128, kManyWavesChunkBatched = 256;
+constexpr int kBlocksPerSm = 3, kMinChunk = 32, kOneWaveMax = 256, kManyWavesChunk = 128, kManyWavesChunkBatched = 256;
 
 // Splitting a sequence costs a second pass over its tokens (0.75 of the output pass, for all chunks but the last) and two more
-// launches; not splitting it leaves one block per sequence, layer and 128 channels.  SM cycles a token of a block takes (128
-// channels, A = powers; a general A scales both sides alike), measured with 1, 2 and 4 resident blocks, and in wide blocks:
-constexpr double kCycOne = 228, kCycTwo = 174, kCycFour = 163, kCycWide = 144, kSplitCycles = 16000;
+// launches; not splitting it leaves one block per sequence, layer and 128 or 256 channels.  SM cycles a token of a block takes
+// (A = powers; a general A scales all alike), measured: a block of 128 channels alone on its SM, one of 256 channels alone,
+// three of 128 side by side (per block), and a wide one per 128 channels.  Blocks that share an SM are not served evenly (of two,
+// one ran 548k cycles and the other 708k over the same 2048 tokens) and the last one finishes alone at the rate of one warp per
+// scheduler; the warps of one block advance together.  Hence 256 channels in one block rather than two blocks of 128.
+constexpr double kCycOne = 217, kCycPair = 268, kCycMany = 163 * 1.25, kCycWide = 144, kSplitCycles = 16000, kBlockCycles = 10000;
 
-// Estimated cycles of the unsplit form: bound by the longest sequence running alone, or by what the fullest SM is given.
-double unsplit_cycles(int64_t blocks_per_seq, int T, int n_seq, int max_seqlen, int sms) {
-    const double per_sm = (double)blocks_per_seq * T / sms, deepest = (double)((blocks_per_seq * n_seq + sms - 1) / sms) * max_seqlen;
-    double m = per_sm + 0.5 * T / n_seq;   // longest first: the last blocks to start are the short ones
-    if (m > deepest) m = deepest;
+// Estimated cycles of the unsplit form with one block per SM: the longest sequence, or what the fullest SM is given.
+double unsplit_cycles(int64_t blocks_per_seq, double cycles, int T, int n_seq, int max_seqlen, int sms) {
+    const int64_t rounds = (blocks_per_seq * n_seq + sms - 1) / sms;
+    double m = (double)blocks_per_seq * T / sms + 0.5 * T / n_seq;   // longest first: the last blocks to start are the short ones
+    if (m > (double)rounds * max_seqlen) m = (double)rounds * max_seqlen;
     if (m < max_seqlen) m = max_seqlen;
-    return blocks_per_seq * n_seq <= sms ? kCycOne * max_seqlen : (kCycTwo * m > kCycOne * max_seqlen ? kCycTwo * m : kCycOne * max_seqlen);
+    return cycles * m + kBlockCycles * rounds;
 }
 
 PrefillPlan plan_prefill(const mdraft_layer* L, int n_layers, int T, int n_seq, int max_seqlen, const mdraft_prefill_opts* opts) {
@@ -125,6 +128,7 @@ PrefillPlan plan_prefill(const mdraft_layer* L, int n_layers, int T, int n_seq, 
     const int wide_cols = kPrefillThreads * kPrefillWideBoxes;
     const int64_t ch_blocks = (int64_t)n_layers * ((D + kPrefillThreads - 1) / kPrefillThreads);
     const int64_t ch_blocks_wide = (int64_t)n_layers * ((D + wide_cols - 1) / wide_cols);
+    const int64_t ch_blocks_pair = (int64_t)n_layers * ((D + 2 * kPrefillThreads - 1) / (2 * kPrefillThreads));
     const int forced = opts ? opts->block_channels : 0;
     const int sms = sm_count();
     // Wide blocks pay off when they fill the machine in one wave: every SM then runs ONE block whose 16 channel warps
@@ -132,7 +136,8 @@ PrefillPlan plan_prefill(const mdraft_layer* L, int n_layers, int T, int n_seq, 
     // the last of them).  They need the channel count to (nearly) fill whole 512-channel blocks.
     bool wide = forced == wide_cols || (forced == 0 && ch_blocks_wide * wide_cols * 9 <= (int64_t)n_layers * D * 10);
     int Lc;
-    bool unsplit = false;
+    bool unsplit = false, alone = false;
+    int unsplit_boxes = 1;
     if (opts && opts->chunk_len > 0) {
         Lc = opts->chunk_len < 4 ? 4 : opts->chunk_len;
     } else {
@@ -148,13 +153,22 @@ PrefillPlan plan_prefill(const mdraft_layer* L, int n_layers, int T, int n_seq, 
             Lc = n_seq > 1 ? kManyWavesChunkBatched : kManyWavesChunk;
             if (forced == 0) wide = false;
         }
-        const double n_chunks = n_seq + (double)T / Lc, work = (double)ch_blocks * T / sms * (wide ? kCycWide : kCycFour);
+        const double n_chunks = n_seq + (double)T / Lc, work = (double)ch_blocks * T / sms * (wide ? kCycWide : kCycMany);
         const double split = (work > kCycOne * Lc ? work : kCycOne * Lc) * (1.0 + 0.75 * (n_chunks - n_seq) / n_chunks) + kSplitCycles;
-        unsplit = forced == 0 && unsplit_cycles(ch_blocks, T, n_seq, max_seqlen, sms) <= split;
+        // The unsplit forms: 128 channels alone, 256 channels alone, and three blocks of 128 channels to an SM for many short sequences.
+        const double one = unsplit_cycles(ch_blocks, kCycOne, T, n_seq, max_seqlen, sms), pair = unsplit_cycles(ch_blocks_pair, kCycPair, T, n_seq, max_seqlen, sms);
+        double many = kCycMany * ch_blocks * T / sms;
+        if (many < kCycOne * max_seqlen) many = kCycOne * max_seqlen;
+        many += kBlockCycles;
+        unsplit = forced == 0 && (one <= split || pair <= split || many <= split);
+        if (unsplit) {
+            unsplit_boxes = pair < one && pair < many ? 2 : 1;
+            alone = unsplit_boxes == 2 || one <= many;
+        }
     }
-    pl.wide = wide && !unsplit;
+    pl.boxes = unsplit ? unsplit_boxes : wide ? kPrefillWideBoxes : 1;
     pl.chunked = Lc < max_seqlen;
-    pl.longest_first = pl.two_per_sm = false;
+    pl.longest_first = pl.alone = false;
     pl.chunk_len = INT_MAX / 2;
     pl.n_chunks_bound = n_seq;
     pl.off_q = pl.off_sd = pl.off_h0 = pl.off_conv = pl.layer_bytes = pl.bytes = 0;
@@ -176,11 +190,8 @@ PrefillPlan plan_prefill(const mdraft_layer* L, int n_layers, int T, int n_seq, 
     }
     if (unsplit) {
         pl.chunked = false;
-        // Two blocks per SM while that holds the grid, or when lengths differ: a call that starts while the one before it
-        // drains must not stack three blocks on one SM and one on another (measured 460 against 370 us for 288 blocks), and
-        // the longest sequences set the time, which they take less of with one neighbour than with three.
         pl.longest_first = n_seq > 1 && n_seq <= kPrefillMaxRanked;
-        pl.two_per_sm = pl.longest_first || ch_blocks * n_seq <= 2 * sms;
+        pl.alone = alone;
     }
     return pl;
 }
@@ -296,7 +307,7 @@ int run_prefill(const PrefillCall& call, const PrefillPlan& pl, int32_t n_layers
             !encode_matrix(&p.maps.C, rows ? v.C : nullptr, act, a.T, kN, v.ldc, kN))
             return MDRAFT_ERR_CUDA;
     }
-    return launch_prefill<ML>(b, act, pl.chunked, pl.wide, pl.two_per_sm, call.stream) == cudaSuccess ? MDRAFT_OK : MDRAFT_ERR_CUDA;
+    return launch_prefill<ML>(b, act, pl.chunked, pl.boxes, pl.alone, call.stream) == cudaSuccess ? MDRAFT_OK : MDRAFT_ERR_CUDA;
 }
 
 __global__ void classify_A_kernel(const float* A, int D, int N, int32_t* res) {

@@ -158,7 +158,7 @@ __host__ __device__ inline int rows_offset(int k, int nt, int nw) {   // W or th
 
 // PRE: blocks of the contraction whose fragments of W a warp takes into registers before the wait.
 template <int NT, int NW, int PRE, bool NORM>
-__global__ void __launch_bounds__(NW * 32, PRE > 0 ? 1 : 2) small_linear_kernel(const SmallLinear p) {
+__global__ void __launch_bounds__(NW * 32, PRE > 0 ? 0 : 2) small_linear_kernel(const SmallLinear p) {
     constexpr int kCols = NT / 16, kPitch = w_pitch(NT);
     extern __shared__ __align__(128) unsigned char s_w[];   // W as [k][NT], later the warps' partial results [NW][kRows][NT]; then the activations
     __shared__ float s_sq[NW][kRows];

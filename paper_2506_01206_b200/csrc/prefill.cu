@@ -192,9 +192,8 @@ struct ChannelScan {
     }
 
     // The 16 decays exp(A[d][n] * delta) as 8 packed pairs.
-    __device__ __forceinline__ void decays(float delta, u64 (&P)[kN / 2]) const {
+    __device__ __forceinline__ void decays(float delta, float r1, u64 (&P)[kN / 2]) const {
         if (kPow) {
-            const float r1 = ex2(delta * a20);
             const float r2 = r1 * r1;
             P[0] = pk(r1, r2);
             P[1] = mul2(P[0], pk(r2, r2));
@@ -226,7 +225,7 @@ struct ChannelScan {
 
     // A token is processed in two steps, so that the first, which has no dependence between tokens, can be run for a
     // group of tokens at once (their special-function latencies overlap) before the second walks the state forward.
-    struct Pre { float u, delta, du, gate; };  // conv+SiLU output, step size, their product, SiLU(z)
+    struct Pre { float u, delta, du, gate, r1; };  // conv+SiLU output, step size, their product, SiLU(z)
     // Step 1: everything that does not touch the state.
     __device__ __forceinline__ void pre(float xv, float zv, float dtv, Pre& e) {
         if (flags & MDRAFT_PRECONV) {
@@ -249,6 +248,7 @@ struct ChannelScan {
         }
         if (!kOut) sum_delta += e.delta;
         e.du = e.delta * e.u;
+        if (kPow) e.r1 = ex2(e.delta * a20);
         if (kOut) e.gate = silu(zv);
     }
     // The state as 16 floats in its own scale: what a chunk starts from, and what it leaves.
@@ -268,7 +268,7 @@ struct ChannelScan {
     __device__ __forceinline__ float post(const Pre& e, const float* Bt, const float* Ct) {
         if (flags & MDRAFT_CONV_ONLY) return e.u;
         u64 P[kN / 2];
-        decays(e.delta, P);
+        decays(e.delta, e.r1, P);
         const u64 DU = pk(e.du, e.du);
         u64 y0, y1;
         const ulonglong2* B2 = reinterpret_cast<const ulonglong2*>(Bt);
@@ -355,7 +355,7 @@ __device__ __forceinline__ void issue_tile(unsigned char* stage, uint64_t* bar, 
 
 // ---------------------------------------------------------------------------------------------------
 template <typename AT, int SUB, bool kPow, bool kOut, bool kFast, int ML>
-__global__ void __launch_bounds__(SUB * kBoxCols + 32, SUB == 1 ? 4 : 1) chunk_kernel(const __grid_constant__ PrefillBatch<ML> batch) {
+__global__ void __launch_bounds__(SUB * kBoxCols + 32, SUB == 1 ? 3 : 1) chunk_kernel(const __grid_constant__ PrefillBatch<ML> batch) {
     const PrefillArgs& c = batch.c;
     const PrefillLayer& p = batch.l[ML == 1 ? 0 : blockIdx.z];
     constexpr int TT = TileTokens<AT>::v;
@@ -441,7 +441,7 @@ __global__ void __launch_bounds__(SUB * kBoxCols + 32, SUB == 1 ? 4 : 1) chunk_k
         }
     }
 
-    const ChunkInfo ci = kOut && SUB == 1 && c.longest_first ? ranked_sequence(c.cu, c.n_seq, c.T, cidx) : find_chunk(c.cu, c.n_seq, c.T, c.chunk_len, cidx);
+    const ChunkInfo ci = kOut && SUB <= 2 && c.longest_first ? ranked_sequence(c.cu, c.n_seq, c.T, cidx) : find_chunk(c.cu, c.n_seq, c.T, c.chunk_len, cidx);
     if (ci.seq < 0) { if (kOut) grid_wait(); return; }
     if (!kOut) {
         // No summary is needed for an unsplit sequence or for a sequence's last chunk; in conv-only mode the only
@@ -569,32 +569,37 @@ __global__ void __launch_bounds__(SUB * kBoxCols + 32, SUB == 1 ? 4 : 1) chunk_k
             const AT* sz = reinterpret_cast<const AT*>(st + off_z(SUB) + box) + col;
             AT* orow = out + (size_t)t * ldo + d;
             typedef typename ChannelScan<AT, kPow, kOut, kFast>::Pre Pre;
-            int r = 0;
-            for (; r + GRP <= rows; r += GRP) {
+            const float *pB = sBf[s][0], *pC = sCf[s][0];
+#pragma unroll 1
+            for (int left = rows; left > 0; left -= GRP) {
                 Pre e[GRP];
                 float o[GRP];
+                if (left >= GRP) {
 #pragma unroll
                 for (int g = 0; g < GRP; ++g) {
-                    const float xv = Act<AT>::to_f32(sx[(r + g) * kBoxCols]);
-                    const float dtv = conv_only ? 0.0f : Act<AT>::to_f32(sdt[(r + g) * kBoxCols]);
-                    const float zv = want_c ? Act<AT>::to_f32(sz[(r + g) * kBoxCols]) : 0.0f;
+                    const float xv = Act<AT>::to_f32(sx[g * kBoxCols]);
+                    const float dtv = conv_only ? 0.0f : Act<AT>::to_f32(sdt[g * kBoxCols]);
+                    const float zv = want_c ? Act<AT>::to_f32(sz[g * kBoxCols]) : 0.0f;
                     cs.pre(xv, zv, dtv, e[g]);
                 }
 #pragma unroll
-                for (int g = 0; g < GRP; ++g) o[g] = cs.post(e[g], sBf[s][r + g], sCf[s][r + g]);
+                for (int g = 0; g < GRP; ++g) o[g] = cs.post(e[g], pB + g * kN, pC + g * kN);
                 if (kOut) {
 #pragma unroll
-                    for (int g = 0; g < GRP; ++g) orow[(size_t)(r + g) * ldo] = Act<AT>::from_f32(o[g]);
+                    for (int g = 0; g < GRP; ++g) { *orow = Act<AT>::from_f32(o[g]); orow += ldo; }
                 }
-            }
-            for (; r < rows; ++r) {
-                Pre e;
-                const float xv = Act<AT>::to_f32(sx[r * kBoxCols]);
-                const float dtv = conv_only ? 0.0f : Act<AT>::to_f32(sdt[r * kBoxCols]);
-                const float zv = want_c ? Act<AT>::to_f32(sz[r * kBoxCols]) : 0.0f;
-                cs.pre(xv, zv, dtv, e);
-                const float o = cs.post(e, sBf[s][r], sCf[s][r]);
-                if (kOut) orow[(size_t)r * ldo] = Act<AT>::from_f32(o);
+                sx += GRP * kBoxCols; sdt += GRP * kBoxCols; sz += GRP * kBoxCols; pB += GRP * kN; pC += GRP * kN;
+                } else {
+#pragma unroll 1
+                for (int g = 0; g < left; ++g) {
+                    const float xv = Act<AT>::to_f32(sx[g * kBoxCols]);
+                    const float dtv = conv_only ? 0.0f : Act<AT>::to_f32(sdt[g * kBoxCols]);
+                    const float zv = want_c ? Act<AT>::to_f32(sz[g * kBoxCols]) : 0.0f;
+                    cs.pre(xv, zv, dtv, e[0]);
+                    o[0] = cs.post(e[0], pB + g * kN, pC + g * kN);
+                    if (kOut) { *orow = Act<AT>::from_f32(o[0]); orow += ldo; }
+                }
+                }
             }
         }
         __syncwarp();
@@ -726,13 +731,14 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, int threads, size_t 
 }
 
 template <typename AT, int SUB, bool kPow, bool kFast, int ML>
-cudaError_t launch_typed(const PrefillBatch<ML>& b, bool chunked, bool two_per_sm, cudaStream_t st) {
+cudaError_t launch_typed(const PrefillBatch<ML>& b, bool chunked, bool alone, cudaStream_t st) {
     const PrefillArgs& p = b.c;
     const int D = p.d_inner;
     constexpr int kCB = SUB * kBoxCols, kThreads = kCB + 32, kSmem = smem_bytes(SUB);
     dim3 grid((D + kCB - 1) / kCB, p.n_chunks_bound, p.n_layers);
     const bool recur = !(b.l[0].L.flags & MDRAFT_CONV_ONLY);
     cudaError_t e = cudaSuccess;
+    if constexpr (SUB != 2)  // blocks of 256 channels take unsplit sequences only
     if (chunked) {
         if ((e = allow_smem<chunk_kernel<AT, SUB, kPow, false, kFast, ML>>(kSmem)) != cudaSuccess) return e;
         e = launch_pdl(chunk_kernel<AT, SUB, kPow, false, kFast, ML>, grid, kThreads, kSmem, st, b);
@@ -745,29 +751,33 @@ cudaError_t launch_typed(const PrefillBatch<ML>& b, bool chunked, bool two_per_s
         if (e != cudaSuccess) return e;
     }
     if (p.ev_carry) cudaEventRecord(p.ev_carry, st);
-    constexpr int kSmemTwo = 100 * 1024;  // a third block does not fit the SM's 227 KB
-    if ((e = allow_smem<chunk_kernel<AT, SUB, kPow, true, kFast, ML>>(SUB == 1 ? kSmemTwo : kSmem)) != cudaSuccess) return e;
-    return launch_pdl(chunk_kernel<AT, SUB, kPow, true, kFast, ML>, grid, kThreads, SUB == 1 && two_per_sm ? kSmemTwo : kSmem, st, b);
+    // Alone on its SM: ask for more than half of the SM's shared memory.
+    constexpr int kSmemAlone = 116 * 1024;
+    if ((e = allow_smem<chunk_kernel<AT, SUB, kPow, true, kFast, ML>>(SUB < 4 ? kSmemAlone : kSmem)) != cudaSuccess) return e;
+    return launch_pdl(chunk_kernel<AT, SUB, kPow, true, kFast, ML>, grid, kThreads, SUB < 4 && alone ? kSmemAlone : kSmem, st, b);
 }
 
 template <typename AT, int SUB, int ML>
-cudaError_t launch_act(const PrefillBatch<ML>& b, bool chunked, bool two_per_sm, cudaStream_t st) {
+cudaError_t launch_act(const PrefillBatch<ML>& b, bool chunked, bool alone, cudaStream_t st) {
     const uint32_t flags = b.l[0].L.flags;
     const bool pow = flags & MDRAFT_A_POWERS;
     if ((flags & ~(uint32_t)MDRAFT_A_POWERS) == (uint32_t)MDRAFT_DT_SOFTPLUS)
-        return pow ? launch_typed<AT, SUB, true, true>(b, chunked, two_per_sm, st) : launch_typed<AT, SUB, false, true>(b, chunked, two_per_sm, st);
+        return pow ? launch_typed<AT, SUB, true, true>(b, chunked, alone, st) : launch_typed<AT, SUB, false, true>(b, chunked, alone, st);
     if constexpr (ML > 1) return cudaErrorInvalidValue;  // the caller takes such layers one by one
-    else return pow ? launch_typed<AT, SUB, true, false>(b, chunked, two_per_sm, st) : launch_typed<AT, SUB, false, false>(b, chunked, two_per_sm, st);
+    else return pow ? launch_typed<AT, SUB, true, false>(b, chunked, alone, st) : launch_typed<AT, SUB, false, false>(b, chunked, alone, st);
 }
 
 }  // namespace
 
 template <int ML>
-cudaError_t launch_prefill(const PrefillBatch<ML>& b, int act, bool chunked, bool wide, bool two_per_sm, cudaStream_t st) {
-    if (wide) return act == MDRAFT_F32 ? launch_act<float, kPrefillWideBoxes>(b, chunked, two_per_sm, st) : launch_act<__nv_bfloat16, kPrefillWideBoxes>(b, chunked, two_per_sm, st);
-    return act == MDRAFT_F32 ? launch_act<float, 1>(b, chunked, two_per_sm, st) : launch_act<__nv_bfloat16, 1>(b, chunked, two_per_sm, st);
+cudaError_t launch_prefill(const PrefillBatch<ML>& b, int act, bool chunked, int boxes, bool alone, cudaStream_t st) {
+    switch (boxes) {
+        case 1: return act == MDRAFT_F32 ? launch_act<float, 1>(b, chunked, alone, st) : launch_act<__nv_bfloat16, 1>(b, chunked, alone, st);
+        case 2: return act == MDRAFT_F32 ? launch_act<float, 2>(b, chunked, alone, st) : launch_act<__nv_bfloat16, 2>(b, chunked, alone, st);
+        default: return act == MDRAFT_F32 ? launch_act<float, kPrefillWideBoxes>(b, chunked, alone, st) : launch_act<__nv_bfloat16, kPrefillWideBoxes>(b, chunked, alone, st);
+    }
 }
-template cudaError_t launch_prefill<1>(const PrefillBatch<1>&, int, bool, bool, bool, cudaStream_t);
-template cudaError_t launch_prefill<kPrefillMaxLayers>(const PrefillBatch<kPrefillMaxLayers>&, int, bool, bool, bool, cudaStream_t);
+template cudaError_t launch_prefill<1>(const PrefillBatch<1>&, int, bool, int, bool, cudaStream_t);
+template cudaError_t launch_prefill<kPrefillMaxLayers>(const PrefillBatch<kPrefillMaxLayers>&, int, bool, int, bool, cudaStream_t);
 
 }  // namespace mdraft

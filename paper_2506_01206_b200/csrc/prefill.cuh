@@ -58,10 +58,9 @@ struct PrefillBatch {
 
 constexpr int kPrefillWideBoxes = 4;  // a wide block covers 4 x kPrefillThreads channels with 16 channel warps
 
-// wide: one block of 512 channels per (channel block, chunk) instead of 128 - for plans that give every SM one block.
-// two_per_sm: ask for so much shared memory that an SM takes two narrow blocks, not four.
+// boxes: 128-channel boxes per block (1, 2 or kPrefillWideBoxes; 2 for unsplit sequences only).  alone: one block per SM.
 // ML = 1, or kPrefillMaxLayers for a call over several layers (all with the same flags: softplus, A_POWERS or not).
 template <int ML>
-cudaError_t launch_prefill(const PrefillBatch<ML>& b, int act, bool chunked, bool wide, bool two_per_sm, cudaStream_t st);
+cudaError_t launch_prefill(const PrefillBatch<ML>& b, int act, bool chunked, int boxes, bool alone, cudaStream_t st);
 
 }  // namespace mdraft
