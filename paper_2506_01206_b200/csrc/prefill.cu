@@ -23,6 +23,8 @@
 // when it is done, so the channel warps never wait for one another.  Every wait on an mbarrier is bounded: if
 // it runs out, the warp raises MDRAFT_DEV_WAIT_EXPIRED and stops; the copy warp first gives the copies it still
 // has in flight a bounded chance to land (they target this block's shared memory).
+#include <type_traits>
+
 #include "common.cuh"
 #include "chunk_map.cuh"
 #include "prefill.cuh"
@@ -46,7 +48,10 @@ __host__ __device__ constexpr int off_b(int sub) { return 3 * sub * kTileBytes; 
 __host__ __device__ constexpr int off_c(int sub) { return 3 * sub * kTileBytes + kBCBytes; }
 __host__ __device__ constexpr int smem_bytes(int sub) { return kStages * (stage_bytes(sub) + 2 * kBCBytes * 2); }  // + fp32 B, C
 constexpr int kFmaPairs = 1;            // pairs of decays per token computed on the FMA pipe when A is general (measured: 0 -> 43.8, 1 -> 42.5, 2 -> 43.0, 3 -> 45.6 us per 2048x1536 call)
-constexpr int GRP = 4;                  // tokens whose state-independent part is computed together (measured: 2 % faster than one by one)
+// Tokens whose state-independent part is computed together, so that their special-function latencies overlap: 8 for A = powers
+// (4 instead: 642 against 610 us for 148 wide blocks of 2048 tokens, 250 against 226 us for blocks of 128 channels), 4 for a
+// general A, whose 16 exponentials a token keep the unit busy (8: 870 against 828 us).
+__host__ __device__ constexpr int group_tokens(bool pow) { return pow ? 8 : 4; }
 
 template <typename AT> struct TileTokens { static constexpr int v = kPrefillTileRowBytes / (int)sizeof(AT); };  // 16 (bf16) or 8 (fp32)
 
@@ -273,12 +278,20 @@ struct ChannelScan {
         u64 y0, y1;
         const ulonglong2* B2 = reinterpret_cast<const ulonglong2*>(Bt);
         const ulonglong2* C2 = reinterpret_cast<const ulonglong2*>(Ct);
+        // h = DU * b + (P * h): with DU in all eight multiply-adds the register file delivers four operands to each instead of six
+        // (it delivers two 32-bit operands a cycle to a scheduler: an fma.rn.f32x2 with three distinct pairs takes 3.1 cycles, one
+        // with a repeated pair 2.2).
+#pragma unroll
+        for (int k = 0; k < kN / 2; ++k) P[k] = mul2(P[k], h[k]);
 #pragma unroll
         for (int q = 0; q < kN / 4; ++q) {
             const ulonglong2 b = B2[q];
-            h[2 * q] = fma2(P[2 * q], h[2 * q], mul2(DU, b.x));
-            h[2 * q + 1] = fma2(P[2 * q + 1], h[2 * q + 1], mul2(DU, b.y));
-            if (kOut) {
+            h[2 * q] = fma2(DU, b.x, P[2 * q]);
+            h[2 * q + 1] = fma2(DU, b.y, P[2 * q + 1]);
+        }
+        if (kOut) {
+#pragma unroll
+            for (int q = 0; q < kN / 4; ++q) {
                 const ulonglong2 c = C2[q];
                 y0 = q == 0 ? mul2(c.x, h[0]) : fma2(c.x, h[2 * q], y0);
                 y1 = q == 0 ? mul2(c.y, h[1]) : fma2(c.y, h[2 * q + 1], y1);
@@ -358,7 +371,7 @@ template <typename AT, int SUB, bool kPow, bool kOut, bool kFast, int ML>
 __global__ void __launch_bounds__(SUB * kBoxCols + 32, SUB == 1 ? 3 : 1) chunk_kernel(const __grid_constant__ PrefillBatch<ML> batch) {
     const PrefillArgs& c = batch.c;
     const PrefillLayer& p = batch.l[ML == 1 ? 0 : blockIdx.z];
-    constexpr int TT = TileTokens<AT>::v;
+    constexpr int TT = TileTokens<AT>::v, GRP = group_tokens(kPow);
     constexpr int kCB = SUB * kBoxCols;          // channels per block, one thread each
     constexpr int kStageBytes = stage_bytes(SUB);
     extern __shared__ __align__(128) unsigned char s_dyn[];
@@ -570,37 +583,31 @@ __global__ void __launch_bounds__(SUB * kBoxCols + 32, SUB == 1 ? 3 : 1) chunk_k
             AT* orow = out + (size_t)t * ldo + d;
             typedef typename ChannelScan<AT, kPow, kOut, kFast>::Pre Pre;
             const float *pB = sBf[s][0], *pC = sCf[s][0];
-#pragma unroll 1
-            for (int left = rows; left > 0; left -= GRP) {
-                Pre e[GRP];
-                float o[GRP];
-                if (left >= GRP) {
+            auto run_group = [&](auto size) {
+                constexpr int G = decltype(size)::value;
+                Pre e[G];
+                float o[G];
 #pragma unroll
-                for (int g = 0; g < GRP; ++g) {
+                for (int g = 0; g < G; ++g) {
                     const float xv = Act<AT>::to_f32(sx[g * kBoxCols]);
                     const float dtv = conv_only ? 0.0f : Act<AT>::to_f32(sdt[g * kBoxCols]);
                     const float zv = want_c ? Act<AT>::to_f32(sz[g * kBoxCols]) : 0.0f;
                     cs.pre(xv, zv, dtv, e[g]);
                 }
 #pragma unroll
-                for (int g = 0; g < GRP; ++g) o[g] = cs.post(e[g], pB + g * kN, pC + g * kN);
+                for (int g = 0; g < G; ++g) o[g] = cs.post(e[g], pB + g * kN, pC + g * kN);
                 if (kOut) {
 #pragma unroll
-                    for (int g = 0; g < GRP; ++g) { *orow = Act<AT>::from_f32(o[g]); orow += ldo; }
+                    for (int g = 0; g < G; ++g) { *orow = Act<AT>::from_f32(o[g]); orow += ldo; }
                 }
-                sx += GRP * kBoxCols; sdt += GRP * kBoxCols; sz += GRP * kBoxCols; pB += GRP * kN; pC += GRP * kN;
-                } else {
+                sx += G * kBoxCols; sdt += G * kBoxCols; sz += G * kBoxCols; pB += G * kN; pC += G * kN;
+            };
+            int left = rows;
 #pragma unroll 1
-                for (int g = 0; g < left; ++g) {
-                    const float xv = Act<AT>::to_f32(sx[g * kBoxCols]);
-                    const float dtv = conv_only ? 0.0f : Act<AT>::to_f32(sdt[g * kBoxCols]);
-                    const float zv = want_c ? Act<AT>::to_f32(sz[g * kBoxCols]) : 0.0f;
-                    cs.pre(xv, zv, dtv, e[0]);
-                    o[0] = cs.post(e[0], pB + g * kN, pC + g * kN);
-                    if (kOut) { *orow = Act<AT>::from_f32(o[0]); orow += ldo; }
-                }
-                }
-            }
+            for (; left >= GRP; left -= GRP) run_group(std::integral_constant<int, GRP>());
+            if (GRP > 4 && left >= 4) { run_group(std::integral_constant<int, 4>()); left -= 4; }
+#pragma unroll 1
+            for (; left > 0; --left) run_group(std::integral_constant<int, 1>());
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(&bar_empty[s]);
