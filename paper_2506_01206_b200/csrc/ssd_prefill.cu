@@ -17,9 +17,10 @@
 //      log-decays of the chunk's rows; the sequence's last chunk also leaves the conv window.
 //   2. ssd_state_passing: per (channel, 4 states) the chunk states of a sequence are chained in token order; every
 //      chunk's incoming state is left in the operand layout the next kernel wants, the final state goes to its slot.
-//   3. ssd_chunk_scan: per (head, chunk) G = C B^T (issued before the kernel's wait: inputs only), the causal decay mask applied to G on its way from tensor memory to
-//      shared memory, Y = (G o L) Xd and C H_in^T on the tensor cores, then skip term, gate and store.  It touches no
-//      x, dt or conv weight: its shared memory is three operand tiles, so that two blocks share an SM.
+//   3. ssd_chunk_scan: per (head, chunk) G = C B^T (issued before the kernel's wait: inputs only), the causal decay mask applied
+//      to G on its way out of tensor memory and back into it as the operand of Y = (G o L) Xd; C H_in^T on the tensor cores;
+//      then skip term, gate and store.  It touches no x, dt or conv weight: with the masked G in tensor memory its shared
+//      memory is two operand tiles, and three blocks share an SM (all blocks of a 2048-token layer in one wave).
 //
 // Operands live in shared memory in the tensor core's canonical un-swizzled layout: 16-byte units of 8 bf16 values,
 // 8 units = one 8 x 8 "core matrix" of 128 contiguous bytes; one descriptor field gives the byte step between core
@@ -97,6 +98,16 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// 16 columns of the warp's 32 lanes, written.
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
+        ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]),
+          "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+        : "memory");
+}
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
 // Shared-memory operand descriptor, un-swizzled canonical layout.  `lead` / `stride` are the two byte steps between core
 // matrices: for a K-major operand lead = along the contraction index, stride = along rows; for an MN-major operand
 // lead = along the contraction index (groups of 8), stride = along the row index (groups of 8).
@@ -127,6 +138,14 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64
         "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, {%5, %5, %5, %5}, p;\n\t}"
         ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate ? 1u : 0u), "r"(0u)
+        : "memory");
+}
+// The same with A out of tensor memory: lane = row, two consecutive bf16 values of the contraction per column.
+__device__ __forceinline__ void mma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc, bool accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, {%5, %5, %5, %5}, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate ? 1u : 0u), "r"(0u)
         : "memory");
 }
 // All tensor-core work issued so far by this thread arrives on the mbarrier when it has completed.
@@ -423,23 +442,27 @@ __global__ void __launch_bounds__(kPassThreads) ssd_state_passing_kernel(const S
 }
 
 // ---------------------------------------------------------------- kernel 3: outputs of a chunk
-// Shared memory is three operand tiles that are re-used as the phases go by:
-//   region A: C rows (operand of G and of C H_in^T)  ->  Xd (fetched from the workspace once those products are done)
-//   region B: B rows (operand of G)                   ->  masked G (operand of Y)
-//   region H: incoming state, value + remainder        ->  the z box (fetched once C H_in^T is done)
-//   regions A + B                                       ->  y rows on their way from accumulator lanes to channel-contiguous stores
+// Bound by latency: a block walks phases that wait for one another, so what counts is that every block of the call is resident
+// at once.  Shared memory is two operand tiles and tensor memory 128 columns, both re-used as the phases go by:
+//   region A: C rows (operand of G and of C H_in^T)          ->  Xd (fetched once those products are done)
+//   region B: B rows (operand of G)  ->  incoming state, value + remainder (fetched once G is done)  ->  the z box
+//   regions A + B                                            ->  y rows on their way from accumulator lanes to channel-contiguous stores
+//   columns 0-127: G  ->  columns 0-63: masked G as bf16 pairs (operand of Y); columns 64-127: C H_in^T, then Y
+// A form with the masked G in shared memory took three tiles and 256 columns: two blocks per SM, and 88 of 384 blocks in a
+// wave of their own.
 struct ScanSmem {
     unsigned char regA[N / 8 * Q * 16];   // C rows [2][Q][64] bf16, 128-byte swizzle (K-major operand)  ->  Xd [(P/8)][Q + 1 unit][8] (MN-major operand, from kernel 1)
-    unsigned char regB[N / 8 * Q * 16];   // B rows [2][Q][64] bf16, 128-byte swizzle (K-major operand)  ->  masked G [Q/8][Q][8] (K-major over the source token)
-    unsigned char regH[2 * N * P * 2];    // incoming state [2][N/8][P][8] bf16 (value, remainder; K-major operands)  ->  z box [Q][P] bf16
+    unsigned char regB[N / 8 * Q * 16];   // B rows, likewise  ->  incoming state [2][N/8][P][8] bf16 (value, remainder; K-major operands)  ->  (second half) z box [Q][P] bf16
     float csl[Q];                         // running log2-decay of the chunk's rows (from kernel 1)
-    uint64_t bar_cb, bar_in, bar_late, bar_g, bar_x, bar_y;
+    uint64_t bar_cb, bar_dec, bar_in, bar_late, bar_g, bar_x, bar_y;
     uint32_t tmem_base;
 };
-static_assert(sizeof(float) * Q * (P + 1) <= 2 * (N / 8 * Q * 16), "the y staging rows must fit the two operand tiles they lie over");
-static_assert((P / 8) * kXdColBytes <= N / 8 * Q * 16 && Q * P * 2 <= 2 * N * P * 2, "re-used regions too small");
+constexpr int kZOffset = 2 * N * P * 2 - Q * P * 2;   // of the z box in region B, behind the y rows' last bytes
+static_assert(sizeof(float) * Q * (P + 1) <= N / 8 * Q * 16 + kZOffset, "the y staging rows must end before the z box");
+static_assert((P / 8) * kXdColBytes <= N / 8 * Q * 16 && 2 * N * P * 2 <= N / 8 * Q * 16, "re-used regions too small");
+static_assert(3 * (sizeof(ScanSmem) + 1024 + 1024) <= 227 * 1024, "three blocks per SM");
 
-__global__ void __launch_bounds__(kThreads, 2) ssd_chunk_scan_kernel(const SsdPrefillArgs p, const __grid_constant__ SsdMaps maps) {
+__global__ void __launch_bounds__(kThreads, 3) ssd_chunk_scan_kernel(const SsdPrefillArgs p, const __grid_constant__ SsdMaps maps) {
     extern __shared__ __align__(1024) unsigned char s_raw[];
     ScanSmem& sm = *reinterpret_cast<ScanSmem*>(s_raw + ((1024u - (smem_u32(s_raw) & 1023u)) & 1023u));   // swizzled tiles start on 1024-byte boundaries
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -453,15 +476,15 @@ __global__ void __launch_bounds__(kThreads, 2) ssd_chunk_scan_kernel(const SsdPr
     if (islot >= p.pool.n_slots || fslot >= p.pool.n_slots) { grid_wait(); return; }
     const int rows = ci.t1 - ci.t0;
     const size_t ch_head = (size_t)cidx * H + head;
-    __nv_bfloat16 (*Mt)[Q][8] = reinterpret_cast<__nv_bfloat16 (*)[Q][8]>(sm.regB);
-    unsigned char* xd = sm.regA;
     constexpr uint32_t kXdBytes = (P / 8) * kXdColBytes;
-    __nv_bfloat16* hin = reinterpret_cast<__nv_bfloat16*>(sm.regH);
-    __nv_bfloat16* zs = reinterpret_cast<__nv_bfloat16*>(sm.regH);
-    float (*ystage)[P + 1] = reinterpret_cast<float (*)[P + 1]>(sm.regA);   // runs on into regB
+    unsigned char* const xd = sm.regA;
+    __nv_bfloat16* const hin = reinterpret_cast<__nv_bfloat16*>(sm.regB);
+    __nv_bfloat16* const zs = reinterpret_cast<__nv_bfloat16*>(sm.regB + kZOffset);
+    float (*const ystage)[P + 1] = reinterpret_cast<float (*)[P + 1]>(sm.regA);   // runs on into regB
 
     if (tid == 0) {
-        mbar_init(&sm.bar_cb, 1); mbar_init(&sm.bar_in, 1); mbar_init(&sm.bar_late, 1); mbar_init(&sm.bar_g, 1); mbar_init(&sm.bar_x, 1); mbar_init(&sm.bar_y, 1);
+        mbar_init(&sm.bar_cb, 1); mbar_init(&sm.bar_dec, 1); mbar_init(&sm.bar_in, 1); mbar_init(&sm.bar_late, 1);
+        mbar_init(&sm.bar_g, 1); mbar_init(&sm.bar_x, 1); mbar_init(&sm.bar_y, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         mbar_expect_tx(&sm.bar_cb, 2 * Q * N * 2);
         // two boxes of 64 states x 128 tokens per matrix
@@ -470,17 +493,16 @@ __global__ void __launch_bounds__(kThreads, 2) ssd_chunk_scan_kernel(const SsdPr
         tma_box(sm.regB, &maps.Bs, 0, ci.t0, &sm.bar_cb);
         tma_box(sm.regB + Q * 128, &maps.Bs, 64, ci.t0, &sm.bar_cb);
     }
-    if (warp == 0) { tmem_alloc(&sm.tmem_base, 256); tc_fence_before(); }
+    if (warp == 0) { tmem_alloc(&sm.tmem_base, 128); tc_fence_before(); }
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = sm.tmem_base;
-    const uint32_t tG = tmem, tYi = tmem + 128, tYx = tmem + 192;   // accumulator columns: G, Y inside the chunk, C H_in^T
+    const uint32_t tG = tmem, tM = tmem, tY = tmem + 64;
     // Operand descriptors are built once; an instruction's descriptor is a base plus the step along the contraction index
     // (the start-address field counts 16-byte units and cannot carry out of its 14 bits: shared memory ends below 256 KB).
     // C and B rows: swizzled tiles; contraction step k (16 states) starts 32 bytes further on inside a half of 64 states,
-    // the second half lies one 16 KB box further on.  The masked G that replaces the B rows is un-swizzled.
+    // the second half lies one 16 KB box further on.
     const uint64_t dC = operand_desc_sw128(smem_u32(sm.regA)), dB = operand_desc_sw128(smem_u32(sm.regB));
-    const uint64_t dM = operand_desc(smem_u32(sm.regB), kColBytes, 128);
     const uint64_t dH = operand_desc(smem_u32(hin), kHinColBytes, 128), dX = operand_desc(smem_u32(xd), 128, kXdColBytes);
     auto kstep = [](int k) { return (uint64_t)(((k >> 2) * (Q * 128) + (k & 3) * 32) >> 4); };
 
@@ -494,96 +516,102 @@ __global__ void __launch_bounds__(kThreads, 2) ssd_chunk_scan_kernel(const SsdPr
             mma_bf16(tG, dC + kstep(k), dB + kstep(k), idG, k > 0);
         mma_commit(&sm.bar_g);
     }
+    const bool g_ok = cb_ok && mbar_wait_bounded(&sm.bar_g, 0u);
     grid_wait();   // the incoming states and the running decays are the work of the kernels just before
-    if (tid == 0) {
-        mbar_expect_tx(&sm.bar_in, 2 * N * P * 2 + Q * 4);
+    if (g_ok && tid == 0) {   // G is complete: its B rows make room for the incoming state
+        mbar_expect_tx(&sm.bar_dec, Q * 4);
+        bulk_load(sm.csl, p.ws_csl + ch_head * Q, Q * 4, &sm.bar_dec);
+        mbar_expect_tx(&sm.bar_in, 2 * N * P * 2);
         bulk_load(hin, p.ws_hin + ch_head * 2 * N * P, 2 * N * P * 2, &sm.bar_in);
-        bulk_load(sm.csl, p.ws_csl + ch_head * Q, Q * 4, &sm.bar_in);
     }
-    // skip term inputs of the warp's rows (u of this lane's channel pair, from kernel 1): requested now, used at the very end
-    const int d = head * P + 2 * lane;
-    uint32_t uraw[kRowsPerWarp];
-#pragma unroll
-    for (int i = 0; i < kRowsPerWarp; ++i) {
-        const int r = warp * kRowsPerWarp + i;
-        uraw[i] = r < rows ? *reinterpret_cast<const uint32_t*>(p.ws_u + (size_t)(ci.t0 + r) * p.L.d_inner + d) : 0u;
-    }
-
-    const bool ok = cb_ok && mbar_wait_bounded(&sm.bar_in, 0u);
-    if (ok && tid == 0) {
+    const bool dec_ok = g_ok && mbar_wait_bounded(&sm.bar_dec, 0u);
+    const int rb = warp & 3, row = rb * 32 + lane, half = warp >> 2;
+    const uint32_t lanes = (uint32_t)(rb * 32) << 16;
+    uint32_t packed[2][16];
+    if (dec_ok) {
         tc_fence_after();
-        constexpr uint32_t idX = instr_desc(P, false, false);
-#pragma unroll
-        for (int k = 0; k < 2 * (N / 16); ++k) {   // Yx[t][p] = sum_n C[t][n] h_in[p][n], value then remainder
-            const int kk = k % (N / 16), part = k / (N / 16);
-            mma_bf16(tYx, dC + kstep(kk), dH + (uint64_t)((part * (N * P * 2) + kk * 2 * kHinColBytes) >> 4), idX, k > 0);
-        }
-        mma_commit(&sm.bar_x);
-    }
-    // The mask needs G and the decays only: it is written while C H_in^T runs.
-    const bool g_ok = ok && mbar_wait_bounded(&sm.bar_g, 0u);
-    if (g_ok) {
-        tc_fence_after();
-        // row t of G, masked: M[t][s] = G[t][s] exp(cs_t - cs_s) for s <= t, else 0; written over the B boxes (G is complete).
-        // Warps w and w + 4 own rows 32 (w % 4) ..: the first takes column blocks 0 and 3, the second 1 and 2 (five
-        // non-zero blocks of 32 x 32 on each side of the split).
-        const int rb = warp & 3, row = rb * 32 + lane;
+        // Row t of G, masked: M[t][s] = G[t][s] exp(cs_t - cs_s) for s <= t, else 0.  Warps w and w + 4 own rows 32 (w % 4) ..:
+        // the first takes column blocks 0 and 3, the second 1 and 2 (five non-zero blocks of 32 x 32 on each side of the split).
         const float my = sm.csl[row];
-#pragma unroll 1
+#pragma unroll
         for (int q = 0; q < 2; ++q) {
-            const int cb = warp < 4 ? (q == 0 ? 0 : 3) : (q == 0 ? 1 : 2);
-            uint32_t packed[16];
+            const int cb = half == 0 ? (q == 0 ? 0 : 3) : (q == 0 ? 1 : 2);
             if (cb <= rb) {   // column blocks right of the warp's rows are all zero
                 float g[32];
-                tmem_ld32(tG + ((uint32_t)(rb * 32) << 16) + cb * 32, g);
+                tmem_ld32(tG + lanes + cb * 32, g);
 #pragma unroll
                 for (int j = 0; j < 32; j += 2) {
                     const int s0 = cb * 32 + j;
                     const float m0 = s0 <= row ? g[j] * ex2(my - sm.csl[s0]) : 0.0f;
                     const float m1 = s0 + 1 <= row ? g[j + 1] * ex2(my - sm.csl[s0 + 1]) : 0.0f;
-                    packed[j >> 1] = pack_bf(m0, m1);
+                    packed[q][j >> 1] = pack_bf(m0, m1);
                 }
             } else {
 #pragma unroll
-                for (int j = 0; j < 16; ++j) packed[j] = 0u;
+                for (int j = 0; j < 16; ++j) packed[q][j] = 0u;
             }
-#pragma unroll
-            for (int u4 = 0; u4 < 4; ++u4)
-                *reinterpret_cast<uint4*>(&Mt[cb * 4 + u4][row][0]) = make_uint4(packed[4 * u4], packed[4 * u4 + 1], packed[4 * u4 + 2], packed[4 * u4 + 3]);
         }
     }
-    // Warp 4 has only zeros to write above.  Once C H_in^T is complete, the tiles it read take Xd and the z box.
-    if (warp == 4 && g_ok && mbar_wait_bounded(&sm.bar_x, 0u) && lane == 0) {
-        mbar_expect_tx(&sm.bar_late, kXdBytes + Q * P * 2);
-        bulk_load(xd, p.ws_xd + ch_head * (kXdBytes / 2), kXdBytes, &sm.bar_late);
-        tma_box(zs, &maps.z, head * P, ci.t0, &sm.bar_late);
-    }
-    const bool late_ok = g_ok && mbar_wait_bounded(&sm.bar_late, 0u);
-    fence_async_smem();
+    const bool in_ok = dec_ok && mbar_wait_bounded(&sm.bar_in, 0u);
     tc_fence_before();
-    const bool all_ok = !__syncthreads_or(!late_ok);
+    const bool mask_ok = !__syncthreads_or(!in_ok);   // every warp has its part of G in registers: the columns are free
+    if (mask_ok) {
+        tc_fence_after();
+        if (tid == 0) {
+            constexpr uint32_t idX = instr_desc(P, false, false);
+#pragma unroll
+            for (int k = 0; k < 2 * (N / 16); ++k) {   // C H_in^T: sum_n C[t][n] h_in[p][n], value then remainder
+                const int kk = k % (N / 16), part = k / (N / 16);
+                mma_bf16(tY, dC + kstep(kk), dH + (uint64_t)((part * (N * P * 2) + kk * 2 * kHinColBytes) >> 4), idX, k > 0);
+            }
+            mma_commit(&sm.bar_x);
+        }
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < 2; ++q) tmem_st16(tM + lanes + (half == 0 ? (q == 0 ? 0 : 3) : (q == 0 ? 1 : 2)) * 16, packed[q]);
+        tmem_wait_st();
+    }
+    const bool x_ok = mask_ok && mbar_wait_bounded(&sm.bar_x, 0u);
+    float y[32];
+    if (x_ok) {
+        if (tid == 0) {   // the tiles that C H_in^T read take Xd and the z box
+            mbar_expect_tx(&sm.bar_late, kXdBytes + Q * P * 2);
+            bulk_load(xd, p.ws_xd + ch_head * (kXdBytes / 2), kXdBytes, &sm.bar_late);
+            tma_box(zs, &maps.z, head * P, ci.t0, &sm.bar_late);
+        }
+        __syncwarp();
+        tc_fence_after();
+        const float scale = ex2(sm.csl[row]);   // decay from the chunk's start through this row
+        tmem_ld32(tY + lanes + half * 32, y);
+#pragma unroll
+        for (int j = 0; j < 32; ++j) y[j] *= scale;
+    }
+    const bool late_ok = x_ok && mbar_wait_bounded(&sm.bar_late, 0u);
+    tc_fence_before();
+    const bool all_ok = !__syncthreads_or(!late_ok);   // C H_in^T has been read by all: its columns take Y
     if (all_ok && tid == 0) {
         tc_fence_after();
         constexpr uint32_t idY = instr_desc(P, false, true);
 #pragma unroll
-        for (int k = 0; k < Q / 16; ++k)   // Yi[t][p] = sum_s M[t][s] Xd[s][p]; the masked G lies where the B rows were
-            mma_bf16(tYi, dM + (uint64_t)(k * 2 * kColBytes >> 4), dX + (uint64_t)(k * 256 >> 4), idY, k > 0);
+        for (int k = 0; k < Q / 16; ++k)   // Y[t][p] = sum_s M[t][s] Xd[s][p]
+            mma_bf16_ts(tY, tM + k * 8, dX + (uint64_t)(k * 256 >> 4), idY, k > 0);
         mma_commit(&sm.bar_y);
     }
     bool y_ok = all_ok && mbar_wait_bounded(&sm.bar_y, 0u);
     if (y_ok) {
         tc_fence_after();
-        const int rb = warp & 3, row = rb * 32 + lane, half = warp >> 2;
-        const float scale = ex2(sm.csl[row]);   // decay from the chunk's start through this row
-        float yi[32], yx[32];
-        tmem_ld32(tYi + ((uint32_t)(rb * 32) << 16) + half * 32, yi);
-        tmem_ld32(tYx + ((uint32_t)(rb * 32) << 16) + half * 32, yx);
-        __syncwarp();
-#pragma unroll
-        for (int j = 0; j < 32; ++j) yi[j] = fmaf(scale, yx[j], yi[j]);
         // the staging rows lie over the operand tiles of the product that has just completed
+        float yi[32];
+        tmem_ld32(tY + lanes + half * 32, yi);
 #pragma unroll
-        for (int j = 0; j < 32; ++j) ystage[row][half * 32 + j] = yi[j];
+        for (int j = 0; j < 32; ++j) ystage[row][half * 32 + j] = y[j] + yi[j];
+    }
+    const int d = head * P + 2 * lane;
+    uint32_t uraw[kRowsPerWarp];   // skip term inputs of the warp's rows (u of this lane's channel pair, from kernel 1)
+#pragma unroll
+    for (int i = 0; i < kRowsPerWarp; ++i) {
+        const int r = warp * kRowsPerWarp + i;
+        uraw[i] = r < rows ? *reinterpret_cast<const uint32_t*>(p.ws_u + (size_t)(ci.t0 + r) * p.L.d_inner + d) : 0u;
     }
     y_ok = !__syncthreads_or(!y_ok);
     if (y_ok) {
@@ -603,18 +631,19 @@ __global__ void __launch_bounds__(kThreads, 2) ssd_chunk_scan_kernel(const SsdPr
     } else if (tid == 0) {
         flag(p.dev_status, MDRAFT_DEV_WAIT_EXPIRED);
         if (!cb_ok) mbar_wait_bounded(&sm.bar_cb, 0u);   // copies target this block's shared memory: one more bounded chance
-        if (!ok) mbar_wait_bounded(&sm.bar_in, 0u);
-        if (g_ok && !late_ok) mbar_wait_bounded(&sm.bar_late, 0u);
+        if (g_ok && !dec_ok) mbar_wait_bounded(&sm.bar_dec, 0u);
+        if (g_ok && !in_ok) mbar_wait_bounded(&sm.bar_in, 0u);
+        if (x_ok && !late_ok) mbar_wait_bounded(&sm.bar_late, 0u);
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == 0) tmem_free(tmem, 256);
+    if (warp == 0) tmem_free(tmem, 128);
 }
 
 template <typename K>
 cudaError_t allow_smem(K kernel, size_t bytes) {
-    // two blocks of ~100 KB per SM: ask for the largest shared-memory carve-out up front, so that the second block of
-    // an SM does not wait for the split to be changed
+    // three blocks of 67 KB per SM: ask for the largest shared-memory carve-out up front, so that the next block of an SM
+    // does not wait for the split to be changed
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
     if (e != cudaSuccess) return e;
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
