@@ -575,32 +575,32 @@ __global__ void __launch_bounds__(SUB * kBoxCols + 32, SUB == 1 ? 3 : 1) chunk_k
             return;
         }
         if (live) {
-            const unsigned char* st = s_stage[s];
-            const int box = (tid / kBoxCols) * kTileBytes, col = tid % kBoxCols;  // this thread's box of 128 channels and its column in it
-            const AT* sx = reinterpret_cast<const AT*>(st + off_x(SUB) + box) + col;
-            const AT* sdt = reinterpret_cast<const AT*>(st + off_dt(SUB) + box) + col;
-            const AT* sz = reinterpret_cast<const AT*>(st + off_z(SUB) + box) + col;
-            AT* orow = out + (size_t)t * ldo + d;
+            // One pointer for the thread's x, dt and z values and one for B and C: the others lie at constant distances.
+            const unsigned char* q = s_stage[s] + (tid / kBoxCols) * kTileBytes + (tid % kBoxCols) * sizeof(AT);
+            const float* pB = sBf[s][0];
+            constexpr int kToC = kStages * TT * kN;
+            AT* orow = out + (size_t)t * p.ldo + d;
             typedef typename ChannelScan<AT, kPow, kOut, kFast>::Pre Pre;
-            const float *pB = sBf[s][0], *pC = sCf[s][0];
+            auto value = [&](int off, int g) { return Act<AT>::to_f32(*reinterpret_cast<const AT*>(q + off + g * (kBoxCols * (int)sizeof(AT)))); };
             auto run_group = [&](auto size) {
                 constexpr int G = decltype(size)::value;
                 Pre e[G];
                 float o[G];
 #pragma unroll
                 for (int g = 0; g < G; ++g) {
-                    const float xv = Act<AT>::to_f32(sx[g * kBoxCols]);
-                    const float dtv = conv_only ? 0.0f : Act<AT>::to_f32(sdt[g * kBoxCols]);
-                    const float zv = want_c ? Act<AT>::to_f32(sz[g * kBoxCols]) : 0.0f;
+                    const float xv = value(off_x(SUB), g);
+                    const float dtv = conv_only ? 0.0f : value(off_dt(SUB), g);
+                    const float zv = want_c ? value(off_z(SUB), g) : 0.0f;
                     cs.pre(xv, zv, dtv, e[g]);
                 }
 #pragma unroll
-                for (int g = 0; g < G; ++g) o[g] = cs.post(e[g], pB + g * kN, pC + g * kN);
+                for (int g = 0; g < G; ++g) o[g] = cs.post(e[g], pB + g * kN, pB + kToC + g * kN);
                 if (kOut) {
 #pragma unroll
                     for (int g = 0; g < G; ++g) { *orow = Act<AT>::from_f32(o[g]); orow += ldo; }
                 }
-                sx += G * kBoxCols; sdt += G * kBoxCols; sz += G * kBoxCols; pB += G * kN; pC += G * kN;
+                q += G * kBoxCols * sizeof(AT);
+                pB += G * kN;
             };
             int left = rows;
 #pragma unroll 1
