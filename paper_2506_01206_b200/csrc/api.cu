@@ -98,12 +98,17 @@ struct PrefillPlan {
     size_t bytes;        // what the workspace query answers: the call's layers, split
 };
 
-// Chunk length: split the token axis until every SM holds kBlocksPerSm blocks of kPrefillThreads channels (one
-// resident wave, no tail), but never into chunks shorter than kMinChunk tokens (per-chunk set-up would dominate).
+// Chunk length: split the token axis until every SM holds kBlocksPerSm blocks of kPrefillThreads channels, or one wide block
+// (one resident wave, no tail).  Narrow blocks have more registers a thread, hide one another's set-up and can be 16 tokens
+// short; wide ones take fewer cycles a token.  Measured (one layer, narrow against wide): 1536 channels x 256 tokens 15.0
+// against 26.0 us, 512 x 4096 27.5 against 31.0, 1536 x 2048 34.4 against 32.7 with A = powers and 41.7 against 42.5 with a
+// general A, 1536 x 32768 357 against 338 and 507 against 491: narrow while one wave of them takes chunks of at most
+// kNarrowChunk (kNarrowChunkGeneral) tokens.  Shorter chunks than a 128th of the sequence cost the carry scan more than they give.
 // When one wave would need chunks longer than kOneWaveMax tokens and the chunks would be uneven (packed batches) or the
 // blocks narrow, several waves of short chunks do better: blocks are then handed out as SMs free up, which evens out
 // uneven sequences and keeps every SM busy to the end (32 packed sequences of 1k-8k tokens: 1607 -> 1512 us).
-constexpr int kBlocksPerSm = 3, kMinChunk = 32, kOneWaveMax = 256, kManyWavesChunk = 128, kManyWavesChunkBatched = 256;
+constexpr int kBlocksPerSm = 3, kMinChunk = 16, kMinChunkWide = 32, kNarrowChunk = 48, kNarrowChunkGeneral = 72;
+constexpr int kOneWaveMax = 256, kManyWavesChunk = 128, kManyWavesChunkBatched = 256;
 
 // Splitting a sequence costs a second pass over its tokens (0.75 of the output pass, for all chunks but the last) and two more
 // launches; not splitting it leaves one block per sequence, layer and 128 or 256 channels.  SM cycles a token of a block takes
@@ -111,7 +116,7 @@ constexpr int kBlocksPerSm = 3, kMinChunk = 32, kOneWaveMax = 256, kManyWavesChu
 // three of 128 side by side (per block), and a wide one per 128 channels.  Blocks that share an SM are not served evenly (of two,
 // one ran 548k cycles and the other 708k over the same 2048 tokens) and the last one finishes alone at the rate of one warp per
 // scheduler; the warps of one block advance together.  Hence 256 channels in one block rather than two blocks of 128.
-constexpr double kCycOne = 217, kCycPair = 268, kCycMany = 163 * 1.25, kCycWide = 144, kSplitCycles = 16000, kBlockCycles = 10000;
+constexpr double kCycOne = 200, kCycPair = 268, kCycMany = 163 * 1.25, kCycWide = 144, kSplitCycles = 16000, kBlockCycles = 6500;
 
 // Estimated cycles of the unsplit form with one block per SM: the longest sequence, or what the fullest SM is given.
 double unsplit_cycles(int64_t blocks_per_seq, double cycles, int T, int n_seq, int max_seqlen, int sms) {
@@ -132,7 +137,7 @@ PrefillPlan plan_prefill(const mdraft_layer* L, int n_layers, int T, int n_seq, 
     const int forced = opts ? opts->block_channels : 0;
     const int sms = sm_count();
     // Wide blocks pay off when they fill the machine in one wave: every SM then runs ONE block whose 16 channel warps
-    // advance together and finish together (four narrow blocks per SM finish one after another and leave the SM to
+    // advance together and finish together (narrow blocks side by side finish one after another and leave the SM to
     // the last of them).  They need the channel count to (nearly) fill whole 512-channel blocks.
     bool wide = forced == wide_cols || (forced == 0 && ch_blocks_wide * wide_cols * 9 <= (int64_t)n_layers * D * 10);
     int Lc;
@@ -141,14 +146,31 @@ PrefillPlan plan_prefill(const mdraft_layer* L, int n_layers, int T, int n_seq, 
     if (opts && opts->chunk_len > 0) {
         Lc = opts->chunk_len < 4 ? 4 : opts->chunk_len;
     } else {
-        int64_t want = wide ? sms / ch_blocks_wide : sms * kBlocksPerSm / ch_blocks;
-        if (want < 1) want = 1;
-        Lc = (int)((T + want - 1) / want);
-        if (Lc < kMinChunk) Lc = kMinChunk;
+        // Every sequence may leave one chunk unfilled: of a wave's narrow blocks, n_seq - 1 chunks' worth are set aside for that.
+        const int64_t want_narrow = sms * kBlocksPerSm / ch_blocks - (n_seq - 1);
+        int64_t narrow = want_narrow > 0 ? (T + want_narrow - 1) / want_narrow : INT_MAX / 2;
+        int shortest = max_seqlen / 128;
+        shortest = shortest < kMinChunk ? kMinChunk : shortest > kMinChunkWide ? kMinChunkWide : shortest;
+        if (narrow < shortest) narrow = shortest;
+        if (forced == 0 && narrow <= ((L->flags & MDRAFT_A_POWERS) ? kNarrowChunk : kNarrowChunkGeneral)) wide = false;
+        if (wide) {
+            int64_t want = sms / ch_blocks_wide;
+            if (want < 1) want = 1;
+            Lc = (int)((T + want - 1) / want);
+            if (Lc < kMinChunkWide) Lc = kMinChunkWide;
+        } else {
+            Lc = (int)narrow;
+            // Tokens past the last group of four go one by one: round up, unless it is a single one.  And where whole tiles would
+            // leave only a few tokens over a full wave of one sequence, those make a short last chunk instead of one more
+            // step for every chunk (1777 tokens x 1536 channels: 48-token chunks 35.8 us, 49-token chunks 38.4).
+            const int tile = kPrefillTileRowBytes / (int)elem_size(L->act), down = Lc / tile * tile;
+            if (n_seq == 1 && down >= kMinChunk && T - want_narrow * down <= 4) Lc = down;
+            else if (Lc % 4 >= 2) Lc += 4 - Lc % 4;
+        }
         // A single sequence in wide blocks stays in one wave at any length: 49 x 3 equal chunks finish together
         // (32768 tokens: 344 us against 372-376 for several waves of short chunks; 65536: 675 against 724).  Packed
         // batches, whose sequences differ in length, and widths that do not fill wide blocks take several waves of
-        // short chunks in narrow blocks, four to an SM, so that a new block's set-up hides behind the others.
+        // short chunks in narrow blocks, several to an SM, so that a new block's set-up hides behind the others.
         if (Lc > kOneWaveMax && !(wide && n_seq == 1)) {
             Lc = n_seq > 1 ? kManyWavesChunkBatched : kManyWavesChunk;
             if (forced == 0) wide = false;

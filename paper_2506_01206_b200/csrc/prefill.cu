@@ -422,19 +422,21 @@ __global__ void __launch_bounds__(SUB * kBoxCols + 32, SUB == 1 ? 3 : 1) chunk_k
         if (!c.pdl_inputs_ready) grid_wait();  // unsplit call: no summary pass has waited for the inputs yet
     }
 
-    if (kOut) {
-        // Sequences without tokens have no chunk: their final state is their starting state.
-        if (cidx == 0 && c.final_slot) {
-            grid_wait();  // the state pool may be the work of the kernels before
-            for (int s = 0; s < c.n_seq; ++s) {
-                int lo = c.cu ? __ldg(c.cu + s) : 0, hi = c.cu ? __ldg(c.cu + s + 1) : c.T;
-                bool bad = (lo < 0) || (hi < lo) || (hi > c.T);
-                if (bad && blockIdx.x == 0 && tid == 0) flag(c.dev_status, MDRAFT_DEV_BAD_SEQLENS);
-                if (bad || hi != lo) continue;
-                int fs = __ldg(c.final_slot + s), is = load_slot(c.init_slot, s);
+    if (kOut && cidx == 0 && (c.final_slot || c.cu)) {
+        // Sequences without tokens have no chunk: their final state is their starting state.  All sequences are looked at
+        // side by side, and before the wait: only a batch that has such a sequence waits here for the kernels ahead.
+        for (int sb = 0; sb < c.n_seq; sb += 32) {
+            int a, len; bool bad;
+            seq_span(c.cu, c.n_seq, c.T, sb + lane, a, len, bad);
+            if (bad && warp == 0 && blockIdx.x == 0 && blockIdx.z == 0) flag(c.dev_status, MDRAFT_DEV_BAD_SEQLENS);
+            unsigned empty = __ballot_sync(0xffffffffu, c.final_slot && sb + lane < c.n_seq && !bad && len == 0);
+            if (empty) grid_wait();  // the state pool may be the work of the kernels before
+            for (; empty; empty &= empty - 1) {
+                const int s = sb + __ffs(empty) - 1;
+                const int fs = __ldg(c.final_slot + s), is = load_slot(c.init_slot, s);
                 if (fs < 0 || fs == is) continue;
                 if (fs >= c.pool.n_slots || is >= c.pool.n_slots) {
-                    if (blockIdx.x == 0 && tid == 0) flag(c.dev_status, MDRAFT_DEV_BAD_SLOT);
+                    if (blockIdx.x == 0 && blockIdx.z == 0 && tid == 0) flag(c.dev_status, MDRAFT_DEV_BAD_SLOT);
                     continue;
                 }
                 if (live) {
@@ -445,11 +447,6 @@ __global__ void __launch_bounds__(SUB * kBoxCols + 32, SUB == 1 ? 3 : 1) chunk_k
                     for (int n = 0; n < kN; ++n) dh[n] = sh ? sh[n] : 0.0f;
                     for (int j = 0; j < kW - 1; ++j) dc[(size_t)j * D + d] = sc ? sc[(size_t)j * D + d] : Act<AT>::from_f32(0.0f);
                 }
-            }
-        } else if (cidx == 0 && blockIdx.x == 0 && blockIdx.z == 0 && tid < 32 && c.cu) {
-            for (int s = tid; s < c.n_seq; s += 32) {
-                int lo = __ldg(c.cu + s), hi = __ldg(c.cu + s + 1);
-                if ((lo < 0) || (hi < lo) || (hi > c.T)) flag(c.dev_status, MDRAFT_DEV_BAD_SEQLENS);
             }
         }
     }
