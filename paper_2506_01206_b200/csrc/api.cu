@@ -146,8 +146,8 @@ PrefillPlan plan_prefill(const mdraft_layer* L, int n_layers, int T, int n_seq, 
     if (opts && opts->chunk_len > 0) {
         Lc = opts->chunk_len < 4 ? 4 : opts->chunk_len;
     } else {
-        // Every sequence may leave one chunk unfilled: of a wave's narrow blocks, n_seq - 1 chunks' worth are set aside for that.
-        const int64_t want_narrow = sms * kBlocksPerSm / ch_blocks - (n_seq - 1);
+        // Every sequence leaves its last chunk half unfilled, on average.
+        const int64_t want_narrow = sms * kBlocksPerSm / ch_blocks - (n_seq - 1) / 2;
         int64_t narrow = want_narrow > 0 ? (T + want_narrow - 1) / want_narrow : INT_MAX / 2;
         int shortest = max_seqlen / 128;
         shortest = shortest < kMinChunk ? kMinChunk : shortest > kMinChunkWide ? kMinChunkWide : shortest;
@@ -160,12 +160,10 @@ PrefillPlan plan_prefill(const mdraft_layer* L, int n_layers, int T, int n_seq, 
             if (Lc < kMinChunkWide) Lc = kMinChunkWide;
         } else {
             Lc = (int)narrow;
-            // Tokens past the last group of four go one by one: round up, unless it is a single one.  And where whole tiles would
-            // leave only a few tokens over a full wave of one sequence, those make a short last chunk instead of one more
-            // step for every chunk (1777 tokens x 1536 channels: 48-token chunks 35.8 us, 49-token chunks 38.4).
+            // Where whole tiles would leave only a few tokens over a full wave of one sequence, those make a short last chunk
+            // instead of one more step for every chunk (1777 tokens x 1536 channels: 48-token chunks 35.8 us, 49-token chunks 38.4).
             const int tile = kPrefillTileRowBytes / (int)elem_size(L->act), down = Lc / tile * tile;
             if (n_seq == 1 && down >= kMinChunk && T - want_narrow * down <= 4) Lc = down;
-            else if (Lc % 4 >= 2) Lc += 4 - Lc % 4;
         }
         // A single sequence in wide blocks stays in one wave at any length: 49 x 3 equal chunks finish together
         // (32768 tokens: 344 us against 372-376 for several waves of short chunks; 65536: 675 against 724).  Packed
