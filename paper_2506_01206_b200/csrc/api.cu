@@ -104,19 +104,22 @@ struct PrefillPlan {
 // against 26.0 us, 512 x 4096 27.5 against 31.0, 1536 x 2048 34.4 against 32.7 with A = powers and 41.7 against 42.5 with a
 // general A, 1536 x 32768 357 against 338 and 507 against 491: narrow while one wave of them takes chunks of at most
 // kNarrowChunk (kNarrowChunkGeneral) tokens.  Shorter chunks than a 128th of the sequence cost the carry scan more than they give.
-// When one wave would need chunks longer than kOneWaveMax tokens and the chunks would be uneven (packed batches) or the
-// blocks narrow, several waves of short chunks do better: blocks are then handed out as SMs free up, which evens out
-// uneven sequences and keeps every SM busy to the end (32 packed sequences of 1k-8k tokens: 1607 -> 1512 us).
+// When one wave of narrow blocks would need longer chunks, a single sequence takes one wave of wide blocks, or, where its width
+// does not fill them, several waves of kManyWavesChunk tokens once one wave would need more than kOneWaveMax.  Packed batches,
+// whose chunks are uneven, take about three waves of narrow blocks, kManyWavesMin to kManyWavesChunk tokens a chunk: blocks are
+// handed out as SMs free up, which evens them out (8 x 2000 tokens x 512 channels: wide 83.7 us, 48-64 tokens 73.5, 128 79.8; 26
+// sequences of 4k-12k tokens x 152 channels: 64 tokens 331, 128 321, 256 334).
 constexpr int kBlocksPerSm = 3, kMinChunk = 16, kMinChunkWide = 32, kNarrowChunk = 48, kNarrowChunkGeneral = 72;
-constexpr int kOneWaveMax = 256, kManyWavesChunk = 128, kManyWavesChunkBatched = 256;
+constexpr int kOneWaveMax = 256, kManyWavesChunk = 128, kManyWavesMin = 48;
 
 // Splitting a sequence costs a second pass over its tokens (0.75 of the output pass, for all chunks but the last) and two more
 // launches; not splitting it leaves one block per sequence, layer and 128 or 256 channels.  SM cycles a token of a block takes
 // (A = powers; a general A scales all alike), measured: a block of 128 channels alone on its SM, one of 256 channels alone,
-// three of 128 side by side (per block), and a wide one per 128 channels.  Blocks that share an SM are not served evenly (of two,
+// three of 128 side by side (per block; in many waves of short chunks, and in one wave of unsplit sequences), and a wide one per
+// 128 channels.  Blocks that share an SM are not served evenly (of two,
 // one ran 548k cycles and the other 708k over the same 2048 tokens) and the last one finishes alone at the rate of one warp per
 // scheduler; the warps of one block advance together.  Hence 256 channels in one block rather than two blocks of 128.
-constexpr double kCycOne = 200, kCycPair = 268, kCycMany = 163 * 1.25, kCycWide = 144, kSplitCycles = 16000, kBlockCycles = 6500;
+constexpr double kCycOne = 200, kCycPair = 268, kCycMany = 170, kCycCrowd = 204, kCycWide = 144, kSplitCycles = 16000, kBlockCycles = 6500;
 
 // Estimated cycles of the unsplit form with one block per SM: the longest sequence, or what the fullest SM is given.
 double unsplit_cycles(int64_t blocks_per_seq, double cycles, int T, int n_seq, int max_seqlen, int sms) {
@@ -127,7 +130,18 @@ double unsplit_cycles(int64_t blocks_per_seq, double cycles, int T, int n_seq, i
     return cycles * m + kBlockCycles * rounds;
 }
 
-PrefillPlan plan_prefill(const mdraft_layer* L, int n_layers, int T, int n_seq, int max_seqlen, const mdraft_prefill_opts* opts) {
+// Workspace of one layer with this many chunks; with `pl`, where its parts lie.
+size_t workspace_of(const mdraft_layer* L, int n_seq, int chunks, PrefillPlan* pl = nullptr) {
+    const size_t Dz = (size_t)L->d_inner;
+    const size_t sd = align_up((size_t)chunks * Dz * kN * sizeof(float), 256);
+    const size_t h0 = align_up(sd + (size_t)chunks * Dz * sizeof(float), 256);
+    const size_t conv = align_up(h0 + (size_t)n_seq * Dz * kN * sizeof(float), 256);
+    if (pl) { pl->off_q = 0; pl->off_sd = sd; pl->off_h0 = h0; pl->off_conv = conv; }
+    return align_up(conv + (size_t)n_seq * (kW - 1) * Dz * elem_size(L->act), 256);
+}
+
+// coarse: the fewest chunks that still give every SM a block or two, for a call whose workspace was sized for another batch.
+PrefillPlan plan_prefill(const mdraft_layer* L, int n_layers, int T, int n_seq, int max_seqlen, const mdraft_prefill_opts* opts, bool coarse = false) {
     PrefillPlan pl;
     const int D = L->d_inner;
     const int wide_cols = kPrefillThreads * kPrefillWideBoxes;
@@ -147,12 +161,14 @@ PrefillPlan plan_prefill(const mdraft_layer* L, int n_layers, int T, int n_seq, 
         Lc = opts->chunk_len < 4 ? 4 : opts->chunk_len;
     } else {
         // Every sequence leaves its last chunk half unfilled, on average.
-        const int64_t want_narrow = sms * kBlocksPerSm / ch_blocks - (n_seq - 1) / 2;
+        int64_t want_narrow = sms * kBlocksPerSm / ch_blocks - (n_seq - 1) / 2;
+        if (coarse) want_narrow = sms * 4 / ch_blocks;
         int64_t narrow = want_narrow > 0 ? (T + want_narrow - 1) / want_narrow : INT_MAX / 2;
         int shortest = max_seqlen / 128;
         shortest = shortest < kMinChunk ? kMinChunk : shortest > kMinChunkWide ? kMinChunkWide : shortest;
         if (narrow < shortest) narrow = shortest;
-        if (forced == 0 && narrow <= ((L->flags & MDRAFT_A_POWERS) ? kNarrowChunk : kNarrowChunkGeneral)) wide = false;
+        if (coarse && narrow < kMinChunkWide) narrow = kMinChunkWide;
+        if (forced == 0 && !coarse && narrow <= ((L->flags & MDRAFT_A_POWERS) ? kNarrowChunk : kNarrowChunkGeneral)) wide = false;
         if (wide) {
             int64_t want = sms / ch_blocks_wide;
             if (want < 1) want = 1;
@@ -165,19 +181,33 @@ PrefillPlan plan_prefill(const mdraft_layer* L, int n_layers, int T, int n_seq, 
             const int tile = kPrefillTileRowBytes / (int)elem_size(L->act), down = Lc / tile * tile;
             if (n_seq == 1 && down >= kMinChunk && T - want_narrow * down <= 4) Lc = down;
         }
+        // More chunks are not taken at the price of a workspace that the fixed scratch array does not hold, where fewer would fit it.
+        auto too_big = [&](int chunk, int instead) {
+            const size_t most = MDRAFT_NOALLOC_SCRATCH_BYTES;
+            return workspace_of(L, n_seq, n_seq + T / chunk) > most && workspace_of(L, n_seq, n_seq + T / instead) <= most;
+        };
         // A single sequence in wide blocks stays in one wave at any length: 49 x 3 equal chunks finish together
-        // (32768 tokens: 344 us against 372-376 for several waves of short chunks; 65536: 675 against 724).  Packed
-        // batches, whose sequences differ in length, and widths that do not fill wide blocks take several waves of
-        // short chunks in narrow blocks, several to an SM, so that a new block's set-up hides behind the others.
-        if (Lc > kOneWaveMax && !(wide && n_seq == 1)) {
-            Lc = n_seq > 1 ? kManyWavesChunkBatched : kManyWavesChunk;
+        // (32768 tokens: 344 us against 372-376 for several waves of short chunks; 65536: 675 against 724).
+        if (n_seq == 1) {
+            if (Lc > kOneWaveMax && !wide && !too_big(kManyWavesChunk, Lc)) Lc = kManyWavesChunk;
+        } else if (forced == 0 && !coarse && narrow > ((L->flags & MDRAFT_A_POWERS) ? kNarrowChunk : kNarrowChunkGeneral)) {
+            int64_t waves = narrow / 3;
+            waves = waves < kManyWavesMin ? kManyWavesMin : waves > kManyWavesChunk ? kManyWavesChunk : waves;
+            const bool one_wave = wide && Lc <= kOneWaveMax;
+            const int fewer = one_wave ? Lc : kOneWaveMax;
+            const bool keep = too_big((int)waves, fewer);
+            Lc = keep ? fewer : (int)waves;
+            wide = keep && one_wave;
+        } else if (Lc > kOneWaveMax) {
+            Lc = kOneWaveMax;
             if (forced == 0) wide = false;
         }
+        if (n_seq + (int64_t)T / Lc > 65535 && Lc < kOneWaveMax) Lc = kOneWaveMax;  // a launch's grid
         const double n_chunks = n_seq + (double)T / Lc, work = (double)ch_blocks * T / sms * (wide ? kCycWide : kCycMany);
         const double split = (work > kCycOne * Lc ? work : kCycOne * Lc) * (1.0 + 0.75 * (n_chunks - n_seq) / n_chunks) + kSplitCycles;
         // The unsplit forms: 128 channels alone, 256 channels alone, and three blocks of 128 channels to an SM for many short sequences.
         const double one = unsplit_cycles(ch_blocks, kCycOne, T, n_seq, max_seqlen, sms), pair = unsplit_cycles(ch_blocks_pair, kCycPair, T, n_seq, max_seqlen, sms);
-        double many = kCycMany * ch_blocks * T / sms;
+        double many = kCycCrowd * ch_blocks * T / sms;
         if (many < kCycOne * max_seqlen) many = kCycOne * max_seqlen;
         many += kBlockCycles;
         unsplit = forced == 0 && (one <= split || pair <= split || many <= split);
@@ -194,12 +224,7 @@ PrefillPlan plan_prefill(const mdraft_layer* L, int n_layers, int T, int n_seq, 
     pl.off_q = pl.off_sd = pl.off_h0 = pl.off_conv = pl.layer_bytes = pl.bytes = 0;
     if (pl.chunked) {
         const int bound = n_seq + T / Lc;
-        const size_t Dz = (size_t)D;
-        pl.off_q = 0;
-        pl.off_sd = align_up(pl.off_q + (size_t)bound * Dz * kN * sizeof(float), 256);
-        pl.off_h0 = align_up(pl.off_sd + (size_t)bound * Dz * sizeof(float), 256);
-        pl.off_conv = align_up(pl.off_h0 + (size_t)n_seq * Dz * kN * sizeof(float), 256);
-        pl.layer_bytes = align_up(pl.off_conv + (size_t)n_seq * (kW - 1) * Dz * elem_size(L->act), 256);
+        pl.layer_bytes = workspace_of(L, n_seq, bound, &pl);
         // For one layer the query answers for the split form whichever form is taken: a workspace made for one batch then
         // serves another of its size whose longest sequence is longer.
         pl.bytes = pl.layer_bytes * n_layers;
@@ -428,8 +453,9 @@ int mdraft_conv_scan_prefill_stack(int32_t n_layers, const mdraft_layer* layers,
                         static_cast<cudaStream_t>(stream)};
     for (int pass = 0; pass < 2; ++pass)  // every launch is checked before the first is made
         for (int32_t l0 = 0; l0 < n_layers;) {
-            const int32_t nl = run_length(n_layers - l0, layers + l0, kPrefillMaxLayers);
-            const PrefillPlan pl = plan_prefill(layers + l0, nl, plan_tokens, n_seq, max_seqlen, opts);
+            const int32_t nl = run_length(n_layers - l0, layers + l0, n_seq > 65535 / kPrefillMaxLayers ? 1 : kPrefillMaxLayers);
+            PrefillPlan pl = plan_prefill(layers + l0, nl, plan_tokens, n_seq, max_seqlen, opts);
+            if (pl.chunked && workspace_bytes < pl.bytes) pl = plan_prefill(layers + l0, nl, plan_tokens, n_seq, max_seqlen, opts, true);
             if (pass == 0) {
                 if (pl.n_chunks_bound > 65535 || (int64_t)nl * n_seq > 65535) return MDRAFT_ERR_UNSUPPORTED;
                 if (pl.chunked) {

@@ -40,8 +40,10 @@ extern "C" int mdraft_conv_scan_prefill_noalloc(const mdraft_layer* layer, const
                                                 int32_t* dev_status, void* stream) {
     // Size check first, on the host: an oversized problem is refused before CUDA is touched at all.
     size_t need = 0;
-    if (layer && total_tokens > 0 && n_seq > 0)
-        need = mdraft_prefill_workspace_bytes(layer, total_tokens, n_seq, max_seqlen > 0 ? max_seqlen : 1, opts);
+    // (The query answers for the split form; a call of one launch is unsplit and uses no scratch.)
+    const int32_t longest = max_seqlen > 0 ? max_seqlen : 1;
+    if (layer && total_tokens > 0 && n_seq > 0 && mdraft_prefill_stack_launches(layer, 1, total_tokens, n_seq, longest, opts) != 1)
+        need = mdraft_prefill_workspace_bytes(layer, total_tokens, n_seq, longest, opts);
     if (need > (size_t)MDRAFT_NOALLOC_SCRATCH_BYTES) return MDRAFT_ERR_WORKSPACE;
     void* scratch = nullptr;
     if (need > 0) {
