@@ -354,9 +354,8 @@ def run_ours(args):
     split = kernel_split(stack, 3)
     split_general = kernel_split(stack_general, 2)
 
-    # ---- the output-pass kernel alone, in the launch configuration of the call above, replayed from a graph: the same
-    # 2048 rows given as 49 independent sequences of 42 tokens are not split, so the call launches ONLY the output pass,
-    # with the grid, block, shared memory and tokens per block that the chunked call gives it (49 chunks of 42 tokens).
+    # ---- the output-pass kernel alone, replayed from a graph: the same 2048 rows given as 49 independent sequences of 42
+    # tokens are not split, so the call launches ONLY the output pass (one launch for all 24 layers).
     n_ck = -(-T // 42)
     cu_alone = i32(np.minimum(np.arange(n_ck + 1) * 42, T), dev)
     alone_stack = DrafterStack(stack.layers, n_ck, T, n_ck, 42, 0, dev)
@@ -489,7 +488,7 @@ def run_ours(args):
                 "algorithmic_bytes_per_layer": bytes_l, "hbm_frac": bytes_l / (ms * 1e-3) / 1e9 / load_peaks()[0],
                 "fp32_issue_frac_82_ops": ALU_LANE_OPS_PER_UNIT * units / (ms * 1e-3) / (SM_COUNT * FP32_LANES_PER_SM * SM_MAX_MHZ * 1e6),
                 "fp32_issue_frac_70_ops": 70 * units / (ms * 1e-3) / (SM_COUNT * FP32_LANES_PER_SM * SM_MAX_MHZ * 1e6),
-                "buffers": n_buf, "launches_per_layer": 3}
+                "buffers": n_buf, "launches": md.mdraft_prefill_stack_launches(lays[0], n_buf, T_l, S_l, max(lens))}
 
     peak_hbm = load_peaks()[0]
     prefill_shapes = None
@@ -629,8 +628,8 @@ def run_ours(args):
     node_updates = NL * M
     value = replicas.whole_job_throughput(units_step, ms_step, world)
     peak, peak_src = load_peaks()
-    pre_launches = stack.prefill_launches_per_layer(T, 1, T)
-    launches = NL * pre_launches + NL * (len(levels) - 1) + 1
+    # one launch takes all layers (up to 32) of the encode, or of a tree level
+    launches = md.mdraft_prefill_stack_launches(stack.layers[0], NL, T, 1, T) + -(-NL // 32) * (len(levels) - 1) + 1
     alu_peak = SM_COUNT * FP32_LANES_PER_SM * SM_MAX_MHZ * 1e6  # fp32 lane-ops/s at the maximum SM clock
 
     # dominant kernel: the output pass of the prefill (chunk_kernel<bf16, kOut>).  Algorithmic bytes of one layer's
@@ -649,14 +648,14 @@ def run_ours(args):
         "traffic": ncu_traffic("prefill_output_pass")[0], "traffic_kernel": ncu_traffic("prefill_output_pass")[1],
         "peak_source": "148 SMs x 128 fp32 lanes x %.0f MHz (clocks.max.sm)" % SM_MAX_MHZ,
         "algorithmic_lane_ops_per_launch": lane_ops, "algorithmic_bytes_per_launch": pb, "launch_us": output_pass_us,
-        "timed": "CUDA-graph replay of 24 launches of this kernel alone (the 2048 rows as 49 unsplit sequences of 42 tokens: same grid, block and tokens per block as in the chunked call), time / 24",
+        "timed": "CUDA-graph replay of one launch of this kernel over 24 layers (the 2048 rows as 49 unsplit sequences of 42 tokens), time / 24",
         "launch_us_between_events": split[2],
         "hbm": {"achieved": pb / scan_s / 1e9, "peak": peak, "unit": "GB/s", "frac": pb / scan_s / 1e9 / peak, "peak_source": peak_src,
                 "frac_of_nominal_8000": pb / scan_s / 1e9 / 8000.0},
         "whole_prefill_call": {"us": call_s * 1e6, "achieved": pb / call_s / 1e9, "frac": pb / call_s / 1e9 / peak,
                                "alu_frac": lane_ops / call_s / alu_peak,
                                "summary_pass_us": split[0], "carry_scan_us": split[1], "output_pass_us": split[2],
-                               "timed": "call: CUDA-graph replay of the 24 calls; per-kernel: CUDA events recorded by the library between the kernels of a call, launched eagerly with the host queued ahead (no overlap between the kernels, event gaps included)"},
+                               "timed": "call: CUDA-graph replay of the call over 24 layers, time / 24; per-kernel: CUDA events recorded by the library between the kernels of a call, launched eagerly with the host queued ahead (no overlap between the kernels, event gaps included)"},
     }
     tb = w.tree_bytes_per_layer()
     bt_round_bytes = sum(bt.level_bytes(a, b) for a, b in zip(bt.levels[:-1], bt.levels[1:]))
@@ -666,7 +665,7 @@ def run_ours(args):
         "achieved": NL * bt_wide_bytes / (ms_bt_widest * 1e-3) / 1e9, "peak": peak, "unit": "GB/s",
         "frac": NL * bt_wide_bytes / (ms_bt_widest * 1e-3) / 1e9 / peak, "traffic": ncu_traffic("tree_step_widest_level")[0], "traffic_kernel": ncu_traffic("tree_step_widest_level")[1],
         "algorithmic_bytes_per_launch": bt_wide_bytes, "launch_us": 1e3 * ms_bt_widest / NL,
-        "timed": "CUDA-graph replay of 24 launches (one per layer, distinct 110 MB pools), time / 24",
+        "timed": "CUDA-graph replay of the level, one launch over 24 layers (distinct 110 MB pools), time / 24",
         "whole_round": {"ms": ms_bt_round, "levels": [b - a for a, b in zip(bt.levels[:-1], bt.levels[1:])],
                         "node_updates_per_s": world * NL * bt.M / (ms_bt_round * 1e-3),
                         "hbm_frac": NL * bt_round_bytes / (ms_bt_round * 1e-3) / 1e9 / peak},
