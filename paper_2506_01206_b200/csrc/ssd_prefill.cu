@@ -517,6 +517,19 @@ __global__ void __launch_bounds__(kThreads, 3) ssd_chunk_scan_kernel(const SsdPr
         mma_commit(&sm.bar_g);
     }
     const bool g_ok = cb_ok && mbar_wait_bounded(&sm.bar_g, 0u);
+    // Row t of G, masked: M[t][s] = G[t][s] exp(cs_t - cs_s) for s <= t, else 0.  Warps w and w + 4 own rows 32 (w % 4) ..:
+    // the first takes column blocks 0 and 3, the second 1 and 2 (five non-zero blocks of 32 x 32 on each side of the split).
+    // Blocks 2 and 3 are taken into registers ahead of the wait: their columns are free for C H_in^T then.
+    const int rb = warp & 3, row = rb * 32 + lane, half = warp >> 2;
+    const int cb0 = half, cb1 = 3 - half;
+    const uint32_t lanes = (uint32_t)(rb * 32) << 16;
+    float g1[32];
+    if (g_ok) {
+        tc_fence_after();
+        if (cb1 <= rb) tmem_ld32(tG + lanes + cb1 * 32, g1);
+        tc_fence_before();
+    }
+    __syncthreads();
     grid_wait();   // the incoming states and the running decays are the work of the kernels just before
     if (g_ok && tid == 0) {   // G is complete: its B rows make room for the incoming state
         mbar_expect_tx(&sm.bar_dec, Q * 4);
@@ -524,40 +537,13 @@ __global__ void __launch_bounds__(kThreads, 3) ssd_chunk_scan_kernel(const SsdPr
         mbar_expect_tx(&sm.bar_in, 2 * N * P * 2);
         bulk_load(hin, p.ws_hin + ch_head * 2 * N * P, 2 * N * P * 2, &sm.bar_in);
     }
-    const bool dec_ok = g_ok && mbar_wait_bounded(&sm.bar_dec, 0u);
-    const int rb = warp & 3, row = rb * 32 + lane, half = warp >> 2;
-    const uint32_t lanes = (uint32_t)(rb * 32) << 16;
-    uint32_t packed[2][16];
-    if (dec_ok) {
-        tc_fence_after();
-        // Row t of G, masked: M[t][s] = G[t][s] exp(cs_t - cs_s) for s <= t, else 0.  Warps w and w + 4 own rows 32 (w % 4) ..:
-        // the first takes column blocks 0 and 3, the second 1 and 2 (five non-zero blocks of 32 x 32 on each side of the split).
-        const float my = sm.csl[row];
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const int cb = half == 0 ? (q == 0 ? 0 : 3) : (q == 0 ? 1 : 2);
-            if (cb <= rb) {   // column blocks right of the warp's rows are all zero
-                float g[32];
-                tmem_ld32(tG + lanes + cb * 32, g);
-#pragma unroll
-                for (int j = 0; j < 32; j += 2) {
-                    const int s0 = cb * 32 + j;
-                    const float m0 = s0 <= row ? g[j] * ex2(my - sm.csl[s0]) : 0.0f;
-                    const float m1 = s0 + 1 <= row ? g[j + 1] * ex2(my - sm.csl[s0 + 1]) : 0.0f;
-                    packed[q][j >> 1] = pack_bf(m0, m1);
-                }
-            } else {
-#pragma unroll
-                for (int j = 0; j < 16; ++j) packed[q][j] = 0u;
-            }
-        }
-    }
-    const bool in_ok = dec_ok && mbar_wait_bounded(&sm.bar_in, 0u);
-    tc_fence_before();
-    const bool mask_ok = !__syncthreads_or(!in_ok);   // every warp has its part of G in registers: the columns are free
-    if (mask_ok) {
-        tc_fence_after();
-        if (tid == 0) {
+    // Warp 4 has only zeros to mask: it issues C H_in^T, which runs while the others form the mask, and refills the tiles
+    // that this product read with Xd and the z box.
+    bool in_ok = true;
+    if (warp == 4) {
+        in_ok = g_ok && mbar_wait_bounded(&sm.bar_in, 0u);
+        if (in_ok && lane == 0) {
+            tc_fence_after();
             constexpr uint32_t idX = instr_desc(P, false, false);
 #pragma unroll
             for (int k = 0; k < 2 * (N / 16); ++k) {   // C H_in^T: sum_n C[t][n] h_in[p][n], value then remainder
@@ -567,19 +553,47 @@ __global__ void __launch_bounds__(kThreads, 3) ssd_chunk_scan_kernel(const SsdPr
             mma_commit(&sm.bar_x);
         }
         __syncwarp();
-#pragma unroll
-        for (int q = 0; q < 2; ++q) tmem_st16(tM + lanes + (half == 0 ? (q == 0 ? 0 : 3) : (q == 0 ? 1 : 2)) * 16, packed[q]);
-        tmem_wait_st();
-    }
-    const bool x_ok = mask_ok && mbar_wait_bounded(&sm.bar_x, 0u);
-    float y[32];
-    if (x_ok) {
-        if (tid == 0) {   // the tiles that C H_in^T read take Xd and the z box
+        in_ok = in_ok && mbar_wait_bounded(&sm.bar_x, 0u);
+        if (in_ok && lane == 0) {
             mbar_expect_tx(&sm.bar_late, kXdBytes + Q * P * 2);
             bulk_load(xd, p.ws_xd + ch_head * (kXdBytes / 2), kXdBytes, &sm.bar_late);
             tma_box(zs, &maps.z, head * P, ci.t0, &sm.bar_late);
         }
         __syncwarp();
+    }
+    const bool dec_ok = g_ok && mbar_wait_bounded(&sm.bar_dec, 0u);
+    uint32_t packed[2][16];
+    auto mask_block = [&](int cb, const float (&g)[32], uint32_t (&m)[16]) {
+        const float my = sm.csl[row];
+#pragma unroll
+        for (int j = 0; j < 32; j += 2) {
+            const int s0 = cb * 32 + j;
+            const float m0 = s0 <= row ? g[j] * ex2(my - sm.csl[s0]) : 0.0f;
+            const float m1 = s0 + 1 <= row ? g[j + 1] * ex2(my - sm.csl[s0 + 1]) : 0.0f;
+            m[j >> 1] = pack_bf(m0, m1);
+        }
+    };
+#pragma unroll
+    for (int j = 0; j < 16; ++j) { packed[0][j] = 0u; packed[1][j] = 0u; }   // column blocks right of the warp's rows stay zero
+    if (dec_ok) {
+        if (cb1 <= rb) mask_block(cb1, g1, packed[1]);
+        if (cb0 <= rb) {
+            float g0[32];
+            tmem_ld32(tG + lanes + cb0 * 32, g0);
+            mask_block(cb0, g0, packed[0]);
+        }
+    }
+    tc_fence_before();
+    const bool mask_ok = !__syncthreads_or(!dec_ok || !in_ok);   // every warp has its part of G in registers: the columns are free
+    if (mask_ok) {
+        tc_fence_after();
+        tmem_st16(tM + lanes + cb0 * 16, packed[0]);
+        tmem_st16(tM + lanes + cb1 * 16, packed[1]);
+        tmem_wait_st();
+    }
+    const bool x_ok = mask_ok && mbar_wait_bounded(&sm.bar_x, 0u);   // complete: warp 4 has seen it
+    float y[32];
+    if (x_ok) {
         tc_fence_after();
         const float scale = ex2(sm.csl[row]);   // decay from the chunk's start through this row
         tmem_ld32(tY + lanes + half * 32, y);
@@ -632,7 +646,11 @@ __global__ void __launch_bounds__(kThreads, 3) ssd_chunk_scan_kernel(const SsdPr
         flag(p.dev_status, MDRAFT_DEV_WAIT_EXPIRED);
         if (!cb_ok) mbar_wait_bounded(&sm.bar_cb, 0u);   // copies target this block's shared memory: one more bounded chance
         if (g_ok && !dec_ok) mbar_wait_bounded(&sm.bar_dec, 0u);
-        if (g_ok && !in_ok) mbar_wait_bounded(&sm.bar_in, 0u);
+        if (g_ok && !mask_ok) {   // ... and for the product that reads them, and the copies that follow it, which warp 4 may have begun
+            mbar_wait_bounded(&sm.bar_in, 0u);
+            mbar_wait_bounded(&sm.bar_x, 0u);
+            mbar_wait_bounded(&sm.bar_late, 0u);
+        }
         if (x_ok && !late_ok) mbar_wait_bounded(&sm.bar_late, 0u);
     }
     tc_fence_before();
