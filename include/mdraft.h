@@ -22,7 +22,7 @@
  *     y_t     = sum_n C[t][n] * h_t[n] + D[d] * u_t
  *     out[t][d] = y_t * SiLU(z[t][d])                        (rounded to the activation type)
  *
- * The in/x/dt/out projections of the block are outside the library.
+ * The in/x/dt/out projections of the block are outside these formulas; mdraft_tree_step_proj and mdraft_block_generation include them.
  *
  * State.  Per sequence (or tree node) and layer: the SSM state h (D x N, fp32,
  * n contiguous) and the conv window = the last W-1 RAW inputs x (W-1 rows of D,

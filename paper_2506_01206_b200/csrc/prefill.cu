@@ -55,37 +55,6 @@ __host__ __device__ constexpr int group_tokens(bool pow) { return pow ? 8 : 4; }
 
 template <typename AT> struct TileTokens { static constexpr int v = kPrefillTileRowBytes / (int)sizeof(AT); };  // 16 (bf16) or 8 (fp32)
 
-typedef unsigned long long u64;
-
-// ---------------------------------------------------------------- packed fp32 pairs
-__device__ __forceinline__ u64 pk(float lo, float hi) {
-    u64 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void unpk(u64 v, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
-__device__ __forceinline__ float hi_of(u64 v) {
-    float lo, hi;
-    unpk(v, lo, hi);
-    return hi;
-}
-__device__ __forceinline__ u64 fma2(u64 a, u64 b, u64 c) {
-    u64 d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ u64 mul2(u64 a, u64 b) {
-    u64 d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-
-__device__ __forceinline__ u64 add2(u64 a, u64 b) {
-    u64 d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-
 // 2^x for a pair of arguments x <= 0 on the FMA pipe instead of the special-function unit (which a general A keeps
 // busy with 16 exponentials per token, channel and pass).  x = j + f with j = round(x) taken from the mantissa of
 // x + 1.5*2^23 and f in [-0.5, 0.5]; 2^f = 1 + f g(f) with g of degree 4 interpolated at Chebyshev nodes (relative error
