@@ -70,12 +70,6 @@ __device__ __forceinline__ float peer_block_float(const float* local, uint32_t r
     return v;
 }
 
-__device__ __forceinline__ void swap4(float4& a, float4& b) { const float4 t = a; a = b; b = t; }
-__device__ __forceinline__ void xor_permute(float4 (&t)[4], int sw) {
-    if (sw & 1) { swap4(t[0], t[1]); swap4(t[2], t[3]); }
-    if (sw & 2) { swap4(t[0], t[2]); swap4(t[1], t[3]); }
-}
-
 // Four consecutive weights as floats.
 __device__ __forceinline__ float4 load_w4(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
 __device__ __forceinline__ float4 load_w4(const __nv_bfloat16* p) {
@@ -209,19 +203,24 @@ __global__ void __launch_bounds__(CB) tree_proj_kernel(const TreeProjArgs p) {
     }
 
     // Layer constants travel by ordinary loads while the copies are in flight.
-    float a2[kPow ? 1 : kN];
+    // Position i of a channel's state quads is quad i ^ sw (no bank conflicts between neighbouring threads); decays, B and C are
+    // made and read in that order.
+    const int sw = (tid >> 1) & 3;
+    u64 a2[kPow ? 1 : kN / 2];
+    float a20 = 0.f;
     float4 wv = make_float4(0.f, 0.f, 0.f, 0.f);
     float cb = 0.f, dtb = 0.f, dsk = 0.f;
     if (live) {
         wv = __ldg(reinterpret_cast<const float4*>(p.L.conv_w + (size_t)d * kW));
         cb = p.L.conv_b ? __ldg(p.L.conv_b + d) : 0.f;
         if constexpr (kPow) {
-            a2[0] = __ldg(p.L.A + (size_t)d * kN) * kLog2e;
+            a20 = __ldg(p.L.A + (size_t)d * kN) * kLog2e;
         } else {
 #pragma unroll
-            for (int q = 0; q < kN / 4; ++q) {
-                const float4 a = __ldg(reinterpret_cast<const float4*>(p.L.A + (size_t)d * kN) + q);
-                a2[4 * q] = a.x * kLog2e; a2[4 * q + 1] = a.y * kLog2e; a2[4 * q + 2] = a.z * kLog2e; a2[4 * q + 3] = a.w * kLog2e;
+            for (int k = 0; k < kN / 4; ++k) {
+                const float4 a = __ldg(reinterpret_cast<const float4*>(p.L.A + (size_t)d * kN) + (k ^ sw));
+                a2[2 * k] = pk(a.x * kLog2e, a.y * kLog2e);
+                a2[2 * k + 1] = pk(a.z * kLog2e, a.w * kLog2e);
             }
         }
         dtb = p.L.dt_bias ? __ldg(p.L.dt_bias + d) : 0.f;
@@ -434,52 +433,57 @@ __global__ void __launch_bounds__(CB) tree_proj_kernel(const TreeProjArgs p) {
 #pragma unroll
     for (int i = 0; i < NT; ++i) {
         if (!(live && !bad && valid[i])) continue;
-        // ---- one step of the recurrence.  The quads of a channel are visited in an order that differs between
-        // neighbouring threads, which keeps the 128-bit shared-memory accesses free of bank conflicts.
-        float4* hs = s_h + (i * CB + tid) * (kN / 4);
+        // ---- one step of the recurrence, two states at a time
+        ulonglong2* const hs = reinterpret_cast<ulonglong2*>(s_h + (i * CB + tid) * (kN / 4));
         const float* ss = s_s + i * kMaxRows;
-        const int sw = (tid >> 1) & 3;
-        float4 hq[kN / 4];
+        ulonglong2 h[kN / 4];
 #pragma unroll
-        for (int k = 0; k < kN / 4; ++k) hq[k] = pslot[i] >= 0 ? hs[k ^ sw] : make_float4(0.f, 0.f, 0.f, 0.f);
-        xor_permute(hq, sw);
+        for (int k = 0; k < kN / 4; ++k) {
+            h[k] = make_ulonglong2(0ull, 0ull);
+            if (pslot[i] >= 0) h[k] = hs[k ^ sw];
+        }
         const float zv = Act<AT>::to_f32(s_z[i * CB + tid]);
         const float v = dtv[i] + dtb;
         const float delta = (flags & MDRAFT_DT_SOFTPLUS) ? softplus(v) : v;
         const float du = delta * u[i];
-        float P[kN];
-        if constexpr (kPow) {
-            const float r1 = ex2(delta * a2[0]);
-            const float r2 = r1 * r1, r4 = r2 * r2, r8 = r4 * r4;
-            P[0] = r1; P[1] = r2; P[2] = r2 * r1; P[3] = r4;
-            P[4] = r4 * r1; P[5] = r4 * r2; P[6] = r4 * P[2]; P[7] = r8;
+        u64 P[kN / 2];
+        if constexpr (kPow) {   // quad q: r^(4q) (r, r^2, r^3, r^4), with r^(4 (k ^ sw)) made of the two bits of k ^ sw
+            const float r1 = ex2(delta * a20), r2 = r1 * r1;
+            const u64 p01 = pk(r1, r2), p23 = mul2(p01, pk(r2, r2));
+            const float r4 = hi_of(p23), r8 = r4 * r4;
+            const float l0 = sw & 1 ? r4 : 1.0f, l1 = sw & 1 ? 1.0f : r4, u0 = sw & 2 ? r8 : 1.0f, u1 = sw & 2 ? 1.0f : r8;
+            const float Rq[kN / 4] = {l0 * u0, l1 * u0, l0 * u1, l1 * u1};
 #pragma unroll
-            for (int n = 0; n < 8; ++n) P[8 + n] = r8 * P[n];
+            for (int k = 0; k < kN / 4; ++k) {
+                const u64 R2 = pk(Rq[k], Rq[k]);
+                P[2 * k] = mul2(p01, R2);
+                P[2 * k + 1] = mul2(p23, R2);
+            }
         } else {
+            const u64 dd = pk(delta, delta);
 #pragma unroll
-            for (int n = 0; n < kN; ++n) P[n] = ex2(delta * a2[n]);
+            for (int k = 0; k < kN / 2; ++k) {
+                float lo, hi;
+                unpk(mul2(dd, a2[k]), lo, hi);
+                P[k] = pk(ex2(lo), ex2(hi));
+            }
         }
-        float h[kN], Bv[kN], Cv[kN];
+        const u64 DU = pk(du, du);
+        u64 y0 = 0ull, y1 = 0ull;
 #pragma unroll
-        for (int q = 0; q < kN / 4; ++q) {
-            h[4 * q] = hq[q].x; h[4 * q + 1] = hq[q].y; h[4 * q + 2] = hq[q].z; h[4 * q + 3] = hq[q].w;
-            const float4 b = *reinterpret_cast<const float4*>(&ss[R + 4 * q]);
-            const float4 c = *reinterpret_cast<const float4*>(&ss[R + kN + 4 * q]);
-            Bv[4 * q] = b.x; Bv[4 * q + 1] = b.y; Bv[4 * q + 2] = b.z; Bv[4 * q + 3] = b.w;
-            Cv[4 * q] = c.x; Cv[4 * q + 1] = c.y; Cv[4 * q + 2] = c.z; Cv[4 * q + 3] = c.w;
-        }
-        float y0 = 0.f, y1 = 0.f;
-#pragma unroll
-        for (int n = 0; n < kN; ++n) {
-            h[n] = fmaf(P[n], h[n], du * Bv[n]);
-            if (n & 1) y1 = fmaf(Cv[n], h[n], y1); else y0 = fmaf(Cv[n], h[n], y0);
+        for (int k = 0; k < kN / 4; ++k) {
+            const ulonglong2 b = reinterpret_cast<const ulonglong2*>(ss + R)[k ^ sw], c = reinterpret_cast<const ulonglong2*>(ss + R + kN)[k ^ sw];
+            h[k].x = fma2(DU, b.x, mul2(P[2 * k], h[k].x));
+            h[k].y = fma2(DU, b.y, mul2(P[2 * k + 1], h[k].y));
+            y0 = fma2(c.x, h[k].x, y0);
+            y1 = fma2(c.y, h[k].y, y1);
         }
 #pragma unroll
-        for (int q = 0; q < kN / 4; ++q) hq[q] = make_float4(h[4 * q], h[4 * q + 1], h[4 * q + 2], h[4 * q + 3]);
-        xor_permute(hq, sw);
-#pragma unroll
-        for (int k = 0; k < kN / 4; ++k) hs[k ^ sw] = hq[k];
-        s_x[i * CB + tid] = Act<AT>::from_f32(fmaf(dsk, u[i], y0 + y1) * silu(zv));
+        for (int k = 0; k < kN / 4; ++k) hs[k ^ sw] = h[k];
+        float ya, yb, yc, yd;
+        unpk(y0, ya, yb);
+        unpk(y1, yc, yd);
+        s_x[i * CB + tid] = Act<AT>::from_f32(fmaf(dsk, u[i], (ya + yb) + (yc + yd)) * silu(zv));
     }
     // Shared-memory writes above must be visible to the copy engine before it reads them.
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
