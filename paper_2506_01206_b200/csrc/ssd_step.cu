@@ -10,7 +10,8 @@
 // is still running, fetch everything that no level of the call writes (slots, constants, the node's input rows) and form
 // decay and input term's factors that need no state, and only then wait; the parent's state and window, just written and
 // mostly still in L2, are all that follows.  As ordinary launches the six levels of a 150-node round of one 130M layer spent
-// more than half their 63 us ramping up and draining.  The first level of a call is an ordinary launch (what runs
+// more than half their 63 us ramping up and draining.  On wide levels issue slots count beside HBM: two states per instruction
+// brought the round from 45.1 to 40.9 us (five or six blocks per SM by fewer registers: 48.7 and 53.0, spills).  The first level of a call is an ordinary launch (what runs
 // ahead of it is usually not this library's).
 #include "common.cuh"
 #include "ssd.cuh"
@@ -23,7 +24,7 @@ constexpr int kStepThreads = 256, kStepChannels = 32;
 
 __device__ __forceinline__ float bfv(const __nv_bfloat16* p) { return __bfloat162float(*p); }
 
-__global__ void __launch_bounds__(kStepThreads) ssd_step_kernel(const SsdStepArgs p) {
+__global__ void __launch_bounds__(kStepThreads, 4) ssd_step_kernel(const SsdStepArgs p) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the next level may begin its own look-ups
     const int D = p.L.d_inner;
     const int node = p.lvl_begin + blockIdx.x;
@@ -41,8 +42,8 @@ __global__ void __launch_bounds__(kStepThreads) ssd_step_kernel(const SsdStepArg
     const bool have_parent = pslot >= 0;
     const __nv_bfloat16* conv_parent = static_cast<const __nv_bfloat16*>(p.pool.conv) + (size_t)pslot * p.pool.conv_slot_stride + d;
     __nv_bfloat16* conv_child = static_cast<__nv_bfloat16*>(p.pool.conv) + (size_t)nslot * p.pool.conv_slot_stride + d;
-    const float4* hp = reinterpret_cast<const float4*>(p.pool.ssm + (size_t)pslot * p.pool.ssm_slot_stride + (size_t)d * kSsdN) + j;
-    float4* hc = reinterpret_cast<float4*>(p.pool.ssm + (size_t)nslot * p.pool.ssm_slot_stride + (size_t)d * kSsdN) + j;
+    const ulonglong2* hp = reinterpret_cast<const ulonglong2*>(p.pool.ssm + (size_t)pslot * p.pool.ssm_slot_stride + (size_t)d * kSsdN) + j;
+    ulonglong2* hc = reinterpret_cast<ulonglong2*>(p.pool.ssm + (size_t)nslot * p.pool.ssm_slot_stride + (size_t)d * kSsdN) + j;
 
     // Inputs and constants: no level of the call writes them.
     const float xv = bfv(p.x + (size_t)node * p.ldx + d), zv = bfv(p.z + (size_t)node * p.ldz + d);
@@ -59,9 +60,12 @@ __global__ void __launch_bounds__(kStepThreads) ssd_step_kernel(const SsdStepArg
     const float decay = ex2(delta * __ldg(p.L.A + head) * kLog2e);
 
     asm volatile("griddepcontrol.wait;" ::: "memory");   // the parent's state may be the work of the level ahead
-    float4 h[4];
+    ulonglong2 h[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) h[i] = have_parent ? hp[8 * i] : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int i = 0; i < 4; ++i) {
+        h[i] = make_ulonglong2(0ull, 0ull);
+        if (have_parent) h[i] = hp[8 * i];
+    }
     float w0 = 0.f, w1 = 0.f, w2 = 0.f;
     if (have_parent) { w0 = bfv(conv_parent); w1 = bfv(conv_parent + D); w2 = bfv(conv_parent + 2 * (size_t)D); }
     float acc = fmaf(wv.x, w0, cb);
@@ -71,18 +75,21 @@ __global__ void __launch_bounds__(kStepThreads) ssd_step_kernel(const SsdStepArg
     const float u = silu(acc);
     const float du = delta * u;
 
-    float y = 0.f;
+    auto wide = [](uint32_t v) { return pk(__uint_as_float(v << 16), __uint_as_float(v & 0xffff0000u)); };
+    const u64 DU = pk(du, du), K = pk(decay, decay);
+    u64 y0 = 0ull, y1 = 0ull;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const float b0 = __uint_as_float(braw[i].x << 16), b1 = __uint_as_float(braw[i].x & 0xffff0000u);
-        const float b2 = __uint_as_float(braw[i].y << 16), b3 = __uint_as_float(braw[i].y & 0xffff0000u);
-        const float c0 = __uint_as_float(craw[i].x << 16), c1 = __uint_as_float(craw[i].x & 0xffff0000u);
-        const float c2 = __uint_as_float(craw[i].y << 16), c3 = __uint_as_float(craw[i].y & 0xffff0000u);
-        h[i].x = fmaf(decay, h[i].x, du * b0); h[i].y = fmaf(decay, h[i].y, du * b1);
-        h[i].z = fmaf(decay, h[i].z, du * b2); h[i].w = fmaf(decay, h[i].w, du * b3);
-        y = fmaf(c0, h[i].x, y); y = fmaf(c1, h[i].y, y); y = fmaf(c2, h[i].z, y); y = fmaf(c3, h[i].w, y);
+    for (int i = 0; i < 4; ++i) {   // two states at a time
+        h[i].x = fma2(DU, wide(braw[i].x), mul2(K, h[i].x));
+        h[i].y = fma2(DU, wide(braw[i].y), mul2(K, h[i].y));
         hc[8 * i] = h[i];
+        y0 = fma2(wide(craw[i].x), h[i].x, y0);
+        y1 = fma2(wide(craw[i].y), h[i].y, y1);
     }
+    float ya, yb, yc, yd;
+    unpk(y0, ya, yb);
+    unpk(y1, yc, yd);
+    float y = (ya + yb) + (yc + yd);
     y += __shfl_xor_sync(0xffffffffu, y, 1);
     y += __shfl_xor_sync(0xffffffffu, y, 2);
     y += __shfl_xor_sync(0xffffffffu, y, 4);
