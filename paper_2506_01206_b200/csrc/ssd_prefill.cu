@@ -185,15 +185,15 @@ struct RowScalars {
     float warp_sum[4];
 };
 
-__device__ __forceinline__ void row_scalars(RowScalars& rs, const SsdPrefillArgs& p, int head, int t0, int rows) {
+__device__ __forceinline__ void row_scalars(RowScalars& rs, const SsdPrefillArgs& p, int head, int t0, int rows, float a_head, float dtb) {
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const bool owner = t < Q;   // threads Q.. only take part in the barriers
     float delta = 0.0f;
     if (owner && t < rows) {
-        const float v = __bfloat162float(p.dt[(size_t)(t0 + t) * p.lddt + head]) + (p.L.dt_bias ? __ldg(p.L.dt_bias + head) : 0.0f);
+        const float v = __bfloat162float(p.dt[(size_t)(t0 + t) * p.lddt + head]) + dtb;
         delta = (p.L.flags & MDRAFT_DT_SOFTPLUS) ? softplus(v) : v;
     }
-    float la = delta * __ldg(p.L.A + head);
+    float la = delta * a_head;
     // inclusive scan over the 128 rows: inside the warp by shuffles, across the four warps through shared memory
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -235,14 +235,25 @@ __device__ __forceinline__ void load_rows(const __nv_bfloat16* xs_ext, uint32_t 
     for (int i = 0; i < kRowsPerWarp + 3; ++i) xr[i] = col[(r0 + i) * (P / 2)];
 }
 
+// Taps and bias of this lane's channel pair.
+struct Taps {
+    float4 wa, wb;
+    float ba, bb;
+    __device__ __forceinline__ Taps(const SsdLayerDev& L, int head) {
+        const int d = head * P + 2 * (threadIdx.x & 31);
+        wa = __ldg(reinterpret_cast<const float4*>(L.conv_w + (size_t)d * kW));
+        wb = __ldg(reinterpret_cast<const float4*>(L.conv_w + (size_t)(d + 1) * kW));
+        ba = L.conv_b ? __ldg(L.conv_b + d) : 0.0f;
+        bb = L.conv_b ? __ldg(L.conv_b + d + 1) : 0.0f;
+    }
+};
+
 // conv + SiLU of those rows; calls f(row, index in the warp, u_lo, u_hi).
 template <typename F>
-__device__ __forceinline__ void conv_rows(const uint32_t (&xr)[kRowsPerWarp + 3], const SsdLayerDev& L, int head, F&& f) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int d = head * P + 2 * lane;
-    const float4 wa = __ldg(reinterpret_cast<const float4*>(L.conv_w + (size_t)d * kW));
-    const float4 wb = __ldg(reinterpret_cast<const float4*>(L.conv_w + (size_t)(d + 1) * kW));
-    const float ba = L.conv_b ? __ldg(L.conv_b + d) : 0.0f, bb = L.conv_b ? __ldg(L.conv_b + d + 1) : 0.0f;
+__device__ __forceinline__ void conv_rows(const uint32_t (&xr)[kRowsPerWarp + 3], const Taps& k, F&& f) {
+    const int warp = threadIdx.x >> 5;
+    const float4 wa = k.wa, wb = k.wb;
+    const float ba = k.ba, bb = k.bb;
     const int r0 = warp * kRowsPerWarp;
 #pragma unroll
     for (int i = 0; i < kRowsPerWarp; ++i) {
@@ -274,8 +285,10 @@ __global__ void __launch_bounds__(kThreads, 3) ssd_chunk_state_kernel(const SsdP
     StateSmem& sm = *reinterpret_cast<StateSmem*>(s_raw + ((1024u - (smem_u32(s_raw) & 1023u)) & 1023u));   // the swizzled tile starts on a 1024-byte boundary
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int head = blockIdx.x, cidx = blockIdx.y, H = p.L.n_heads;
+    const Taps taps(p.L, head);   // layer constants: no kernel of this library writes them
+    const float a_head = __ldg(p.L.A + head), dtb = p.L.dt_bias ? __ldg(p.L.dt_bias + head) : 0.0f;
     // The inputs may be the work of the kernel ahead of this call, and the workspace is still being read by the call
-    // before this one: nothing is touched before that kernel is complete.  Only then may the next kernels start, which
+    // before this one: nothing else is touched before that kernel is complete.  Only then may the next kernels start, which
     // lets them read the call's inputs without a wait of their own.
     grid_wait();
     grid_release_dependents();
@@ -298,7 +311,7 @@ __global__ void __launch_bounds__(kThreads, 3) ssd_chunk_state_kernel(const SsdP
     }
     if (warp == 0) { tmem_alloc(&sm.tmem_base, 64); tc_fence_before(); }
     load_halo(xs_ext, p, ci, head, islot);
-    row_scalars(sm.rs, p, head, ci.t0, rows);   // two block-wide barriers inside: barrier init and tmem_base are visible after it
+    row_scalars(sm.rs, p, head, ci.t0, rows, a_head, dtb);   // two block-wide barriers inside: barrier init and tmem_base are visible after it
     tc_fence_after();
     const uint32_t tmem = sm.tmem_base;
 
@@ -316,7 +329,7 @@ __global__ void __launch_bounds__(kThreads, 3) ssd_chunk_state_kernel(const SsdP
     if (ok) {
         const float cs_end_l = sm.rs.csl[Q - 1];
         unsigned char* xd_g = reinterpret_cast<unsigned char*>(p.ws_xd) + ((size_t)cidx * H + head) * ((P / 8) * kXdColBytes);
-        conv_rows(xr, p.L, head, [&](int r, int, float ua, float ub) {
+        conv_rows(xr, taps, [&](int r, int, float ua, float ub) {
             const float wgt = r < rows ? sm.rs.delta[r] * ex2(cs_end_l - sm.rs.csl[r]) : 0.0f;
             const float va = r < rows ? wgt * ua : 0.0f, vb = r < rows ? wgt * ub : 0.0f;
             const uint32_t hi = pack_bf(va, vb);
@@ -627,10 +640,10 @@ __global__ void __launch_bounds__(kThreads, 3) ssd_chunk_scan_kernel(const SsdPr
         const int r = warp * kRowsPerWarp + i;
         uraw[i] = r < rows ? *reinterpret_cast<const uint32_t*>(p.ws_u + (size_t)(ci.t0 + r) * p.L.d_inner + d) : 0u;
     }
+    const float da = p.L.D ? __ldg(p.L.D + d) : 0.0f, db = p.L.D ? __ldg(p.L.D + d + 1) : 0.0f;
     y_ok = !__syncthreads_or(!y_ok);
     if (y_ok) {
         // skip term, gate, store: the warp's rows, this lane's channel pair (128 contiguous bytes per row and warp)
-        const float da = p.L.D ? __ldg(p.L.D + d) : 0.0f, db = p.L.D ? __ldg(p.L.D + d + 1) : 0.0f;
         const uint32_t* zc = reinterpret_cast<const uint32_t*>(zs) + lane;
 #pragma unroll
         for (int i = 0; i < kRowsPerWarp; ++i) {
