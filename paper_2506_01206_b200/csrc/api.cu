@@ -106,20 +106,22 @@ struct PrefillPlan {
 // kNarrowChunk (kNarrowChunkGeneral) tokens.  Shorter chunks than a 128th of the sequence cost the carry scan more than they give.
 // When one wave of narrow blocks would need longer chunks, a single sequence takes one wave of wide blocks, or, where its width
 // does not fill them, several waves of kManyWavesChunk tokens once one wave would need more than kOneWaveMax.  Packed batches,
-// whose chunks are uneven, take about three waves of narrow blocks, kManyWavesMin to kManyWavesChunk tokens a chunk: blocks are
+// whose chunks are uneven, take one to three waves of narrow blocks, kManyWavesMin to kManyWavesChunk tokens a chunk: blocks are
 // handed out as SMs free up, which evens them out (8 x 2000 tokens x 512 channels: wide 83.7 us, 48-64 tokens 73.5, 128 79.8; 26
 // sequences of 4k-12k tokens x 152 channels: 64 tokens 331, 128 321, 256 334).
 constexpr int kBlocksPerSm = 3, kMinChunk = 16, kMinChunkWide = 32, kNarrowChunk = 48, kNarrowChunkGeneral = 72;
-constexpr int kOneWaveMax = 256, kManyWavesChunk = 128, kManyWavesMin = 48;
+constexpr int kOneWaveMax = 256, kManyWavesChunk = 128, kManyWavesMin = 48, kOneWaveNarrow = 110;
 
 // Splitting a sequence costs a second pass over its tokens (0.75 of the output pass, for all chunks but the last) and two more
 // launches; not splitting it leaves one block per sequence, layer and 128 or 256 channels.  SM cycles a token of a block takes
-// (A = powers; a general A scales all alike), measured: a block of 128 channels alone on its SM, one of 256 channels alone,
+// (A = powers), measured: a block of 128 channels alone on its SM, one of 256 channels alone,
 // three of 128 side by side (per block; in many waves of short chunks, and in one wave of unsplit sequences), and a wide one per
 // 128 channels.  Blocks that share an SM are not served evenly (of two,
 // one ran 548k cycles and the other 708k over the same 2048 tokens) and the last one finishes alone at the rate of one warp per
 // scheduler; the warps of one block advance together.  Hence 256 channels in one block rather than two blocks of 128.
-constexpr double kCycOne = 200, kCycPair = 268, kCycMany = 170, kCycCrowd = 204, kCycWide = 144, kSplitCycles = 16000, kBlockCycles = 6500;
+constexpr double kCycOne = 205, kCycPair = 315, kCycMany = 170, kCycCrowd = 204, kCycWide = 146, kSplitCycles = 20500, kOffsetCycles = 5000, kBlockCycles = 6500;
+constexpr double kGeneralOne = 1.38, kGeneralMany = 1.26;   // a general A takes so much more: few warps per scheduler, many
+constexpr double kFloatOne = 1.1;                            // fp32 activations, few warps per scheduler
 
 // Estimated cycles of the unsplit form with one block per SM: the longest sequence, or what the fullest SM is given.
 double unsplit_cycles(int64_t blocks_per_seq, double cycles, int T, int n_seq, int max_seqlen, int sms) {
@@ -191,24 +193,32 @@ PrefillPlan plan_prefill(const mdraft_layer* L, int n_layers, int T, int n_seq, 
         if (n_seq == 1) {
             if (Lc > kOneWaveMax && !wide && !too_big(kManyWavesChunk, Lc)) Lc = kManyWavesChunk;
         } else if (forced == 0 && !coarse && narrow > ((L->flags & MDRAFT_A_POWERS) ? kNarrowChunk : kNarrowChunkGeneral)) {
-            int64_t waves = narrow / 3;
+            // One wave while its chunks are short and the sequences' unfilled last chunks few (5 x 3172 tokens x 256 channels: 73-token
+            // chunks 53.9 us, 48 59.6), then two, then three.
+            int64_t waves = narrow <= kOneWaveNarrow && n_seq * narrow * 20 <= T ? narrow : narrow / (narrow <= 2 * kOneWaveNarrow ? 2 : 3);
             waves = waves < kManyWavesMin ? kManyWavesMin : waves > kManyWavesChunk ? kManyWavesChunk : waves;
-            const bool one_wave = wide && Lc <= kOneWaveMax;
-            const int fewer = one_wave ? Lc : kOneWaveMax;
+            // ... with as few more tokens a chunk as make the workspace fit, up to one wave of them.
+            const int64_t wave4 = sms * 4 / ch_blocks;
+            const int64_t one_wave = wave4 > 0 ? (T + wave4 - 1) / wave4 : kOneWaveMax;
+            const int fewer = wide && Lc <= kOneWaveMax ? Lc : one_wave < waves ? (int)waves : one_wave < kOneWaveMax ? (int)one_wave : kOneWaveMax;
             const bool keep = too_big((int)waves, fewer);
-            Lc = keep ? fewer : (int)waves;
-            wide = keep && one_wave;
+            Lc = (int)waves;
+            if (keep)
+                while (Lc < fewer && too_big(Lc, fewer)) Lc = Lc + 8 < fewer ? Lc + 8 : fewer;
+            wide = false;
         } else if (Lc > kOneWaveMax) {
             Lc = kOneWaveMax;
             if (forced == 0) wide = false;
         }
         if (n_seq + (int64_t)T / Lc > 65535 && Lc < kOneWaveMax) Lc = kOneWaveMax;  // a launch's grid
-        const double n_chunks = n_seq + (double)T / Lc, work = (double)ch_blocks * T / sms * (wide ? kCycWide : kCycMany);
-        const double split = (work > kCycOne * Lc ? work : kCycOne * Lc) * (1.0 + 0.75 * (n_chunks - n_seq) / n_chunks) + kSplitCycles;
+        const bool general = !(L->flags & MDRAFT_A_POWERS);
+        const double g1 = (general ? kGeneralOne : 1.0) * (L->act == MDRAFT_F32 ? kFloatOne : 1.0), gm = general ? kGeneralMany : 1.0;
+        const double n_chunks = n_seq + (double)T / Lc, work = (double)ch_blocks * T / sms * (wide ? kCycWide * g1 : kCycMany * gm);
+        const double split = (work > g1 * kCycOne * Lc ? work : g1 * kCycOne * Lc) * (1.0 + 0.75 * (n_chunks - n_seq) / n_chunks) + kSplitCycles + (n_seq > 1 ? kOffsetCycles : 0.0);
         // The unsplit forms: 128 channels alone, 256 channels alone, and three blocks of 128 channels to an SM for many short sequences.
-        const double one = unsplit_cycles(ch_blocks, kCycOne, T, n_seq, max_seqlen, sms), pair = unsplit_cycles(ch_blocks_pair, kCycPair, T, n_seq, max_seqlen, sms);
-        double many = kCycCrowd * ch_blocks * T / sms;
-        if (many < kCycOne * max_seqlen) many = kCycOne * max_seqlen;
+        const double one = unsplit_cycles(ch_blocks, g1 * kCycOne, T, n_seq, max_seqlen, sms), pair = unsplit_cycles(ch_blocks_pair, g1 * kCycPair, T, n_seq, max_seqlen, sms);
+        double many = gm * kCycCrowd * ((double)ch_blocks * T / sms + 0.7 * max_seqlen);   // uneven neighbours on an SM
+        if (many < g1 * kCycOne * max_seqlen) many = g1 * kCycOne * max_seqlen;
         many += kBlockCycles;
         unsplit = forced == 0 && (one <= split || pair <= split || many <= split);
         if (unsplit) {
@@ -235,7 +245,9 @@ PrefillPlan plan_prefill(const mdraft_layer* L, int n_layers, int T, int n_seq, 
     }
     if (unsplit) {
         pl.chunked = false;
-        pl.longest_first = n_seq > 1 && n_seq <= kPrefillMaxRanked;
+        // Where every block starts at once the order is worth nothing.
+        const bool at_once = (pl.boxes == 2 ? ch_blocks_pair : ch_blocks) * n_seq <= sms;
+        pl.longest_first = !at_once && n_seq > 1 && n_seq <= kPrefillMaxRanked;
         pl.alone = alone;
     }
     return pl;

@@ -83,7 +83,7 @@ def test_a_workspace_for_fewer_chunks_still_serves():
     lay, dev = upload_layer(prob.params, "bf16"), [to_device(a, torch.bfloat16) for a in (prob.x, prob.z, prob.dt, prob.B, prob.C)]
     need = md.mdraft_prefill_workspace_bytes(lay, 40000, 2, 30000)
     res = []
-    for n in (need, need // 2):
+    for n in (need, need * 3 // 4):
         cache, out = md.StateCache(1, 2, Dn), torch.empty((40000, Dn), dtype=torch.bfloat16, device="cuda")
         md.mdraft_conv_scan_prefill(lay, cache, 0, *dev, out, i32(prob.cu), 30000, None, i32([0, 1]), torch.empty(n, dtype=torch.uint8, device="cuda"))
         torch.cuda.synchronize()
