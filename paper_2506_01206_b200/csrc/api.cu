@@ -186,7 +186,8 @@ PrefillPlan plan_prefill(const mdraft_layer* L, int n_layers, int T, int n_seq, 
         // More chunks are not taken at the price of a workspace that the fixed scratch array does not hold, where fewer would fit it.
         auto too_big = [&](int chunk, int instead) {
             const size_t most = MDRAFT_NOALLOC_SCRATCH_BYTES;
-            return workspace_of(L, n_seq, n_seq + T / chunk) > most && workspace_of(L, n_seq, n_seq + T / instead) <= most;
+            auto need = [&](int len) { return len < max_seqlen ? workspace_of(L, n_seq, n_seq + T / len) : (size_t)0; };
+            return need(chunk) > most && need(instead) <= most;
         };
         // A single sequence in wide blocks stays in one wave at any length: 49 x 3 equal chunks finish together
         // (32768 tokens: 344 us against 372-376 for several waves of short chunks; 65536: 675 against 724).
