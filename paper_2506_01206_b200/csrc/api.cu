@@ -181,7 +181,7 @@ PrefillPlan plan_prefill(const mdraft_layer* L, int n_layers, int T, int n_seq, 
             // Where whole tiles would leave only a few tokens over a full wave of one sequence, those make a short last chunk
             // instead of one more step for every chunk (1777 tokens x 1536 channels: 48-token chunks 35.8 us, 49-token chunks 38.4).
             const int tile = kPrefillTileRowBytes / (int)elem_size(L->act), down = Lc / tile * tile;
-            if (n_seq == 1 && down >= kMinChunk && T - want_narrow * down <= 4) Lc = down;
+            if (n_seq == 1 && !coarse && down >= kMinChunk && T - want_narrow * down <= 4) Lc = down;
         }
         // More chunks are not taken at the price of a workspace that the fixed scratch array does not hold, where fewer would fit it.
         auto too_big = [&](int chunk, int instead) {
@@ -201,7 +201,7 @@ PrefillPlan plan_prefill(const mdraft_layer* L, int n_layers, int T, int n_seq, 
             // ... with as few more tokens a chunk as make the workspace fit, up to one wave of them.
             const int64_t wave4 = sms * 4 / ch_blocks;
             const int64_t one_wave = wave4 > 0 ? (T + wave4 - 1) / wave4 : kOneWaveMax;
-            const int fewer = wide && Lc <= kOneWaveMax ? Lc : one_wave < waves ? (int)waves : one_wave < kOneWaveMax ? (int)one_wave : kOneWaveMax;
+            const int fewer = wide ? (Lc <= kOneWaveMax ? Lc : kOneWaveMax) : one_wave < waves ? (int)waves : one_wave < kOneWaveMax ? (int)one_wave : kOneWaveMax;
             const bool keep = too_big((int)waves, fewer);
             Lc = (int)waves;
             if (keep)
