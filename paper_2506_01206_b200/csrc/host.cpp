@@ -248,9 +248,11 @@ PyObject* released(F&& call) {
     return PyLong_FromLong(rc);
 }
 
-// Every function below: C++ exceptions become Python exceptions.
-template <PyObject* (*body)(PyObject* const*)>
-PyObject* guarded(PyObject*, PyObject* const* a, Py_ssize_t) {
+// Every function below takes exactly kArgs arguments, which it reads without asking for their number again; C++ exceptions
+// become Python exceptions.
+template <PyObject* (*body)(PyObject* const*), int kArgs>
+PyObject* guarded(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    if (n != kArgs) return PyErr_Format(PyExc_TypeError, "expected %d arguments, got %zd", kArgs, n);
     try {
         return body(a);
     } catch (const Failed&) {
@@ -547,10 +549,10 @@ PyObject* block_generation(PyObject* const* a) {
     });
 }
 
-#define ENTRY(name) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(&guarded<name>)), METH_FASTCALL, nullptr}
-PyMethodDef methods[] = {ENTRY(table), ENTRY(prefill), ENTRY(prefill_noalloc), ENTRY(tree_step), ENTRY(tree_step_proj),
-                         ENTRY(commit), ENTRY(ssd_prefill), ENTRY(ssd_tree_step), ENTRY(prefill_stack), ENTRY(tree_step_stack), ENTRY(block_generation),
-                         {nullptr, nullptr, 0, nullptr}};
+#define ENTRY(name, args) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(&guarded<name, args>)), METH_FASTCALL, nullptr}
+PyMethodDef methods[] = {ENTRY(table, 1), ENTRY(prefill, 20), ENTRY(prefill_noalloc, 18), ENTRY(tree_step, 16), ENTRY(tree_step_proj, 15),
+                         ENTRY(commit, 6), ENTRY(ssd_prefill, 17), ENTRY(ssd_tree_step, 16), ENTRY(prefill_stack, 13),
+                         ENTRY(tree_step_stack, 11), ENTRY(block_generation, 15), {nullptr, nullptr, 0, nullptr}};
 
 PyModuleDef module_def = {PyModuleDef_HEAD_INIT, "_host", "argument marshalling for libmdraft.so", -1, methods, nullptr, nullptr, nullptr, nullptr};
 

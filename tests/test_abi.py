@@ -227,3 +227,14 @@ def test_ssd_host_side_checks(lib):
     # the commit call moves 128-state slots too, and nothing between the two sizes
     commit = lambda ds: lib.mdraft_state_commit(C.byref(cache), 128, ds, 4, 1, 0, None, None, None, None)
     assert commit(128) == 0 and commit(64) == UNSUPPORTED
+
+
+@pytest.mark.parametrize("name,count", [("table", 1), ("prefill", 20), ("prefill_noalloc", 18), ("tree_step", 16), ("tree_step_proj", 15), ("commit", 6),
+                                        ("ssd_prefill", 17), ("ssd_tree_step", 16), ("prefill_stack", 13), ("tree_step_stack", 11), ("block_generation", 15)])
+def test_the_extension_checks_how_many_arguments_it_is_given(lib, name, count):
+    """The extension's functions index an argument array: a call with another number of arguments must not reach that."""
+    from paper_2506_01206_b200 import binding
+    f = getattr(binding._host, name)
+    for n in (0, count - 1, count + 1):
+        with pytest.raises(TypeError, match=f"expected {count} arguments, got {n}"):
+            f(*[None] * n)
