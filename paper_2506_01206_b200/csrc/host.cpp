@@ -166,7 +166,8 @@ struct Cache {
     const mdraft_cache* get() const { return present ? &c : nullptr; }
 };
 
-// chunk_len: tokens per chunk, or a pair (tokens, channels per block); events: None or two events to record.
+// chunk_len: tokens per chunk (0 or None: the library's plan), or a pair (tokens, channels per block); events: None or two events
+// to record.
 struct Opts {
     mdraft_prefill_opts o = {};
     bool present = false;
@@ -176,7 +177,7 @@ struct Opts {
             if (PySequence_Fast_GET_SIZE(f.p) != 2) fail(PyExc_ValueError, "chunk_len: an int or a pair (chunk_len, block_channels)");
             o.chunk_len = (int32_t)as_int(PySequence_Fast_GET_ITEM(f.p, 0));
             o.block_channels = (int32_t)as_int(PySequence_Fast_GET_ITEM(f.p, 1));
-        } else {
+        } else if (chunk != Py_None) {
             o.chunk_len = (int32_t)as_int(chunk);
         }
         present = o.chunk_len || o.block_channels || events != Py_None;

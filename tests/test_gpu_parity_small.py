@@ -100,6 +100,13 @@ def test_prefill_matches_oracle(act, Dn, lens, chunk_len, general_A, conv_bias, 
     assert np.array_equal(g_conv, o_conv), "conv window must be an exact copy of the last raw inputs"
 
 
+def test_no_chunk_length_may_be_given_as_none():
+    cfg = parity.small_config(64, "f32", 1)
+    prob = parity.make_problem(cfg, [256])
+    for got, want in zip(run_gpu_prefill(prob, md.MDRAFT_DT_SOFTPLUS, None), run_gpu_prefill(prob, md.MDRAFT_DT_SOFTPLUS, 0)):
+        assert np.array_equal(got, want)
+
+
 @pytest.mark.parametrize("act", ["f32", "bf16"])
 def test_prefill_in_place_slots_and_strided_views(act):
     cfg = parity.small_config(264, act, 3)
