@@ -124,6 +124,46 @@ def test_prefill_with_zero_step_size_leaves_the_state_bit_identical(act, powers,
     assert_close(g_out, o_out, TOL[act], "out = (C.h0 + D u) * SiLU(z)")
 
 
+@pytest.mark.parametrize("act", ["f32", "bf16"])
+@pytest.mark.parametrize("powers", [False, True])
+@pytest.mark.parametrize("chunk_len", [16, 4096])
+def test_prefill_whose_softplus_underflows_leaves_the_state_bit_identical(act, powers, chunk_len):
+    """The same with the step size from softplus: log(1 + exp(-200)) is 0 in fp32."""
+    g = np.random.default_rng(18)
+    lens = [90, 41]
+    cfg = parity.small_config(136, act, len(lens), cid=93)
+    prob = parity.make_problem(cfg, lens, conv_bias=True, general_A=not powers)
+    shape_A(prob.params, "", powers, g)
+    prob.dt = gen.round_to_act(g.normal(size=prob.dt.shape).astype(np.float32), act)
+    prob.params.dt_bias[:] = -200.0
+    flags = flags_for(False, powers)
+    h0 = g.normal(size=(len(lens), 136, 16)).astype(np.float32)
+    c0 = gen.round_to_act(g.normal(size=(len(lens), 3, 136)).astype(np.float32), act)
+    g_out, _, g_h = run_gpu_prefill(prob, flags, chunk_len, c0, h0)
+    assert np.array_equal(g_h.astype(np.float32).view(np.uint32), h0.view(np.uint32)), "a zero step size must freeze the state exactly"
+    o_out, _, _ = run_oracle_prefill(prob, flags, c0, h0)
+    assert_close(g_out, o_out, TOL[act], "out = (C.h0 + D u) * SiLU(z)")
+
+
+@pytest.mark.parametrize("act", ["f32", "bf16"])
+@pytest.mark.parametrize("powers", [False, True])
+def test_prefill_in_pieces_is_the_whole_bit_for_bit(act, powers):
+    """A state that goes through a slot between two unsplit calls is the state that stays in registers."""
+    cfg = parity.small_config(136, act, 1, cid=93)
+    prob = parity.make_problem(cfg, [160], conv_bias=True, general_A=not powers)
+    flags = flags_for(False, powers)
+    whole = run_gpu_prefill(prob, flags, 4096)
+    outs, conv, h = [], None, None
+    for lo, hi in ((0, 48), (48, 160)):
+        piece = parity.make_problem(cfg, [hi - lo], conv_bias=True, general_A=not powers)
+        piece.params = prob.params
+        for name in ("x", "z", "dt", "B", "C"):
+            setattr(piece, name, getattr(prob, name)[lo:hi])
+        o, conv, h = run_gpu_prefill(piece, flags, 4096, conv, h)
+        outs.append(o)
+    assert np.array_equal(np.concatenate(outs), whole[0]) and np.array_equal(conv, whole[1]) and np.array_equal(h, whole[2])
+
+
 def _tree_rig(regime, act, powers, g, Dn=200):
     cfg = parity.small_config(Dn, act, cid=93)
     rig = TreeRig(cfg, gen.paper_tree((3, 2, 2, 1, 1)), conv_bias=True, general_A=not powers)
