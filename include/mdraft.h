@@ -65,7 +65,7 @@ typedef enum {
     MDRAFT_ERR_INVALID_ARG = -1,  /* NULL where data is required, negative size, bad index   */
     MDRAFT_ERR_UNSUPPORTED = -2,  /* shape or dtype outside the supported set                */
     MDRAFT_ERR_MISALIGNED  = -3,  /* pointer or stride not a multiple of 16 bytes            */
-    MDRAFT_ERR_WORKSPACE   = -4,  /* workspace NULL or smaller than the query says           */
+    MDRAFT_ERR_WORKSPACE   = -4,  /* workspace NULL, or smaller than the call can do with    */
     MDRAFT_ERR_CUDA        = -5   /* a CUDA runtime call or launch failed                    */
 } mdraft_status;
 
@@ -141,8 +141,13 @@ typedef struct {
  *   final_slot : n_seq int32 or NULL; slot that receives the state after the last token, -1 / NULL = discard.
  *                init_slot[s] == final_slot[s] is allowed (encode a context in pieces).
  *   max_seqlen : an upper bound on the longest sequence (HOST value, used to size the launch)
- *   workspace  : device scratch of at least mdraft_prefill_workspace_bytes(...) bytes, 256-byte aligned;
- *                contents need not be initialised and are garbage afterwards
+ *   workspace  : device scratch, 256-byte aligned; contents need not be initialised and are garbage afterwards.
+ *                mdraft_prefill_workspace_bytes(...) says how much the call would like.  With less it cuts the sequences
+ *                into fewer, longer chunks (slower, and another rounding), as long as those give every SM four blocks
+ *                of 128 channels (one of 512 where the width fills those) or are, for several sequences, at most 256
+ *                tokens; less is MDRAFT_ERR_WORKSPACE.  Sequences that the library leaves whole need none, although
+ *                the query for a single layer answers as if they were cut.  A chunk length given in `opts` is kept:
+ *                it needs all that the query says
  *   dev_status : device int32 or NULL (see mdraft_dev_status bits); never cleared by the library
  */
 size_t mdraft_prefill_workspace_bytes(const mdraft_layer *layer, int32_t total_tokens, int32_t n_seq,
@@ -197,8 +202,8 @@ int mdraft_conv_scan_prefill_stack(int32_t n_layers, const mdraft_layer *layers,
  * until the process exits).  Inputs, outputs and the state pool are still the caller's.
  *
  * Arguments and results are those of mdraft_conv_scan_prefill without `workspace` / `workspace_bytes`; the output
- * is the same, bit for bit, as that call given a workspace of its own.
- *   - A problem whose workspace (mdraft_prefill_workspace_bytes) exceeds MDRAFT_NOALLOC_SCRATCH_BYTES returns
+ * is the same, bit for bit, as that call given a workspace of MDRAFT_NOALLOC_SCRATCH_BYTES bytes of its own.
+ *   - A problem that such a workspace does not serve (see `workspace` above: not even with the longest chunks) returns
  *     MDRAFT_ERR_WORKSPACE before anything is launched: shorten the call (encode the context in pieces through
  *     init_slot / final_slot) or use the entry point above with your own buffer.
  *   - The first call on each device looks up the array's device address (the device must be current); make that

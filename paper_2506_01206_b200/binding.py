@@ -339,8 +339,8 @@ def mdraft_conv_scan_prefill_noalloc(layer: Layer, cache: Optional[StateCache], 
                                      chunk_len: int = 0, dev_status: Optional[torch.Tensor] = None, stream=None,
                                      flags: Optional[int] = None) -> None:
     """Prefill without a caller workspace: the library's own fixed scratch array is used (see the header for
-    who needs this and for the sharing rules).  Raises MdraftError(MDRAFT_ERR_WORKSPACE) when the problem needs
-    more than NOALLOC_SCRATCH_BYTES of scratch."""
+    who needs this and for the sharing rules).  Raises MdraftError(MDRAFT_ERR_WORKSPACE) when a workspace of
+    NOALLOC_SCRATCH_BYTES would not serve the ordinary call."""
     rc = _host.prefill_noalloc(_entry(), layer, cache, layer_index, x, z, dt, B, Cm, out, cu_seqlens, max_seqlen, init_slot, final_slot,
                                chunk_len, dev_status, stream, flags)
     if rc != 0:

@@ -142,8 +142,11 @@ size_t workspace_of(const mdraft_layer* L, int n_seq, int chunks, PrefillPlan* p
     return align_up(conv + (size_t)n_seq * (kW - 1) * Dz * elem_size(L->act), 256);
 }
 
-// coarse: the fewest chunks that still give every SM a block or two, for a call whose workspace was sized for another batch.
-PrefillPlan plan_prefill(const mdraft_layer* L, int n_layers, int T, int n_seq, int max_seqlen, const mdraft_prefill_opts* opts, bool coarse = false) {
+constexpr size_t kAnyWorkspace = SIZE_MAX;  // "whatever the plan asks for"
+
+// workspace: bytes that the call has.  A call that has fewer than the plan would like gets fewer chunks; one that has fewer than
+// the longest chunks need gets a plan with bytes > workspace, which the caller refuses.
+PrefillPlan plan_prefill(const mdraft_layer* L, int n_layers, int T, int n_seq, int max_seqlen, const mdraft_prefill_opts* opts, size_t workspace) {
     PrefillPlan pl;
     const int D = L->d_inner;
     const int wide_cols = kPrefillThreads * kPrefillWideBoxes;
@@ -164,13 +167,17 @@ PrefillPlan plan_prefill(const mdraft_layer* L, int n_layers, int T, int n_seq, 
     } else {
         // Every sequence leaves its last chunk half unfilled, on average.
         int64_t want_narrow = sms * kBlocksPerSm / ch_blocks - (n_seq - 1) / 2;
-        if (coarse) want_narrow = sms * 4 / ch_blocks;
         int64_t narrow = want_narrow > 0 ? (T + want_narrow - 1) / want_narrow : INT_MAX / 2;
         int shortest = max_seqlen / 128;
         shortest = shortest < kMinChunk ? kMinChunk : shortest > kMinChunkWide ? kMinChunkWide : shortest;
         if (narrow < shortest) narrow = shortest;
-        if (coarse && narrow < kMinChunkWide) narrow = kMinChunkWide;
-        if (forced == 0 && !coarse && narrow <= ((L->flags & MDRAFT_A_POWERS) ? kNarrowChunk : kNarrowChunkGeneral)) wide = false;
+        // The longest chunks that a call is given: one wide block or four narrow ones to an SM, at least kMinChunkWide tokens and, for
+        // several sequences, at most kOneWaveMax.
+        const int64_t most = wide ? sms / ch_blocks_wide : sms * 4 / ch_blocks;
+        int64_t longest = (T + (most < 1 ? 1 : most) - 1) / (most < 1 ? 1 : most);
+        const bool longest_wide = wide && (n_seq == 1 || longest <= kOneWaveMax);
+        longest = longest < kMinChunkWide ? kMinChunkWide : longest > kOneWaveMax && n_seq > 1 ? kOneWaveMax : longest;
+        if (forced == 0 && narrow <= ((L->flags & MDRAFT_A_POWERS) ? kNarrowChunk : kNarrowChunkGeneral)) wide = false;
         if (wide) {
             int64_t want = sms / ch_blocks_wide;
             if (want < 1) want = 1;
@@ -181,7 +188,7 @@ PrefillPlan plan_prefill(const mdraft_layer* L, int n_layers, int T, int n_seq, 
             // Where whole tiles would leave only a few tokens over a full wave of one sequence, those make a short last chunk
             // instead of one more step for every chunk (1777 tokens x 1536 channels: 48-token chunks 35.8 us, 49-token chunks 38.4).
             const int tile = kPrefillTileRowBytes / (int)elem_size(L->act), down = Lc / tile * tile;
-            if (n_seq == 1 && !coarse && down >= kMinChunk && T - want_narrow * down <= 4) Lc = down;
+            if (n_seq == 1 && down >= kMinChunk && T - want_narrow * down <= 4) Lc = down;
         }
         // More chunks are not taken at the price of a workspace that the fixed scratch array does not hold, where fewer would fit it.
         auto too_big = [&](int chunk, int instead) {
@@ -193,7 +200,7 @@ PrefillPlan plan_prefill(const mdraft_layer* L, int n_layers, int T, int n_seq, 
         // (32768 tokens: 344 us against 372-376 for several waves of short chunks; 65536: 675 against 724).
         if (n_seq == 1) {
             if (Lc > kOneWaveMax && !wide && !too_big(kManyWavesChunk, Lc)) Lc = kManyWavesChunk;
-        } else if (forced == 0 && !coarse && narrow > ((L->flags & MDRAFT_A_POWERS) ? kNarrowChunk : kNarrowChunkGeneral)) {
+        } else if (forced == 0 && narrow > ((L->flags & MDRAFT_A_POWERS) ? kNarrowChunk : kNarrowChunkGeneral)) {
             // One wave while its chunks are short and the sequences' unfilled last chunks few (5 x 3172 tokens x 256 channels: 73-token
             // chunks 53.9 us, 48 59.6), then two, then three.
             int64_t waves = narrow <= kOneWaveNarrow && n_seq * narrow * 20 <= T ? narrow : narrow / (narrow <= 2 * kOneWaveNarrow ? 2 : 3);
@@ -214,14 +221,27 @@ PrefillPlan plan_prefill(const mdraft_layer* L, int n_layers, int T, int n_seq, 
         if (n_seq + (int64_t)T / Lc > 65535 && Lc < kOneWaveMax) Lc = kOneWaveMax;  // a launch's grid
         const bool general = !(L->flags & MDRAFT_A_POWERS);
         const double g1 = (general ? kGeneralOne : 1.0) * (L->act == MDRAFT_F32 ? kFloatOne : 1.0), gm = general ? kGeneralMany : 1.0;
-        const double n_chunks = n_seq + (double)T / Lc, work = (double)ch_blocks * T / sms * (wide ? kCycWide * g1 : kCycMany * gm);
-        const double split = (work > g1 * kCycOne * Lc ? work : g1 * kCycOne * Lc) * (1.0 + 0.75 * (n_chunks - n_seq) / n_chunks) + kSplitCycles + (n_seq > 1 ? kOffsetCycles : 0.0);
         // The unsplit forms: 128 channels alone, 256 channels alone, and three blocks of 128 channels to an SM for many short sequences.
         const double one = unsplit_cycles(ch_blocks, g1 * kCycOne, T, n_seq, max_seqlen, sms), pair = unsplit_cycles(ch_blocks_pair, g1 * kCycPair, T, n_seq, max_seqlen, sms);
         double many = gm * kCycCrowd * ((double)ch_blocks * T / sms + 0.7 * max_seqlen);   // uneven neighbours on an SM
         if (many < g1 * kCycOne * max_seqlen) many = g1 * kCycOne * max_seqlen;
         many += kBlockCycles;
-        unsplit = forced == 0 && (one <= split || pair <= split || many <= split);
+        auto better_whole = [&](int64_t chunk, bool wide_blocks) {
+            const double n_chunks = n_seq + (double)T / chunk, work = (double)ch_blocks * T / sms * (wide_blocks ? kCycWide * g1 : kCycMany * gm);
+            const double split = (work > g1 * kCycOne * chunk ? work : g1 * kCycOne * chunk) * (1.0 + 0.75 * (n_chunks - n_seq) / n_chunks) + kSplitCycles + (n_seq > 1 ? kOffsetCycles : 0.0);
+            return forced == 0 && (one <= split || pair <= split || many <= split);
+        };
+        unsplit = better_whole(Lc, wide);
+        auto need = [&](int64_t len) { return len < max_seqlen ? n_layers * workspace_of(L, n_seq, (int)(n_seq + T / len)) : (size_t)0; };
+        if (!unsplit && need(Lc) > workspace) {
+            if (Lc < longest) {  // the shortest chunks that fit, in whole groups of tokens
+                int64_t lo = Lc, hi = longest;  // need(lo) > workspace; need() falls with the length
+                while (hi - lo > 1) (need((lo + hi) / 2) > workspace ? lo : hi) = (lo + hi) / 2;
+                hi = (hi + 7) / 8 * 8;
+                Lc = (int)(hi < longest ? hi : longest);
+            }
+            unsplit = need(Lc) > workspace ? better_whole(longest, longest_wide) : better_whole(Lc, wide);
+        }
         if (unsplit) {
             unsplit_boxes = pair < one && pair < many ? 2 : 1;
             alone = unsplit_boxes == 2 || one <= many;
@@ -379,6 +399,14 @@ __global__ void classify_A_kernel(const float* A, int D, int N, int32_t* res) {
 
 }  // namespace
 
+size_t mdraft::prefill_scratch_bytes(const mdraft_layer* layer, int32_t total_tokens, int32_t n_seq, int32_t max_seqlen, const mdraft_prefill_opts* opts,
+                                     size_t available) {
+    if (check_layer(layer) != MDRAFT_OK || total_tokens <= 0 || n_seq <= 0) return 0;
+    if (max_seqlen < 1) max_seqlen = 1;
+    const PrefillPlan pl = plan_prefill(layer, 1, total_tokens, n_seq, max_seqlen < total_tokens ? max_seqlen : total_tokens, opts, available);
+    return pl.chunked ? pl.bytes : 0;
+}
+
 extern "C" {
 
 const char* mdraft_status_string(int status) {
@@ -405,7 +433,7 @@ size_t mdraft_prefill_stack_workspace_bytes(const mdraft_layer* layer, int32_t n
     if (check_layer(layer) != MDRAFT_OK || n_layers <= 0 || total_tokens <= 0 || n_seq <= 0 || max_seqlen <= 0) return 0;
     // No sequence is longer than the whole batch: a looser static bound must not change the plan.
     if (n_layers > kPrefillMaxLayers) n_layers = kPrefillMaxLayers;  // launches of one call share the workspace
-    const PrefillPlan pl = plan_prefill(layer, n_layers, total_tokens, n_seq, max_seqlen < total_tokens ? max_seqlen : total_tokens, opts);
+    const PrefillPlan pl = plan_prefill(layer, n_layers, total_tokens, n_seq, max_seqlen < total_tokens ? max_seqlen : total_tokens, opts, kAnyWorkspace);
     return n_layers == 1 || pl.chunked ? pl.bytes : 0;
 }
 
@@ -416,7 +444,7 @@ int32_t mdraft_prefill_stack_launches(const mdraft_layer* layer, int32_t n_layer
     int32_t n = 0;
     for (int32_t l0 = 0; l0 < n_layers; l0 += kPrefillMaxLayers) {
         const int32_t nl = n_layers - l0 < kPrefillMaxLayers ? n_layers - l0 : kPrefillMaxLayers;
-        n += !plan_prefill(layer, nl, total_tokens, n_seq, max_seqlen, opts).chunked ? 1 : (layer->flags & MDRAFT_CONV_ONLY) ? 2 : 3;
+        n += !plan_prefill(layer, nl, total_tokens, n_seq, max_seqlen, opts, kAnyWorkspace).chunked ? 1 : (layer->flags & MDRAFT_CONV_ONLY) ? 2 : 3;
     }
     return n;
 }
@@ -467,8 +495,7 @@ int mdraft_conv_scan_prefill_stack(int32_t n_layers, const mdraft_layer* layers,
     for (int pass = 0; pass < 2; ++pass)  // every launch is checked before the first is made
         for (int32_t l0 = 0; l0 < n_layers;) {
             const int32_t nl = run_length(n_layers - l0, layers + l0, n_seq > 65535 / kPrefillMaxLayers ? 1 : kPrefillMaxLayers);
-            PrefillPlan pl = plan_prefill(layers + l0, nl, plan_tokens, n_seq, max_seqlen, opts);
-            if (pl.chunked && workspace_bytes < pl.bytes) pl = plan_prefill(layers + l0, nl, plan_tokens, n_seq, max_seqlen, opts, true);
+            const PrefillPlan pl = plan_prefill(layers + l0, nl, plan_tokens, n_seq, max_seqlen, opts, workspace ? workspace_bytes : 0);
             if (pass == 0) {
                 if (pl.n_chunks_bound > 65535 || (int64_t)nl * n_seq > 65535) return MDRAFT_ERR_UNSUPPORTED;
                 if (pl.chunked) {

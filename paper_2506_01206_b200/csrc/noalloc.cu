@@ -2,7 +2,7 @@
 // array inside the library image instead of a caller-supplied workspace.
 #include <mutex>
 
-#include "common.cuh"
+#include "prefill.cuh"
 
 namespace {
 
@@ -39,11 +39,7 @@ extern "C" int mdraft_conv_scan_prefill_noalloc(const mdraft_layer* layer, const
                                                 const int32_t* final_slot, const mdraft_prefill_opts* opts,
                                                 int32_t* dev_status, void* stream) {
     // Size check first, on the host: an oversized problem is refused before CUDA is touched at all.
-    size_t need = 0;
-    // (The query answers for the split form; a call of one launch is unsplit and uses no scratch.)
-    const int32_t longest = max_seqlen > 0 ? max_seqlen : 1;
-    if (layer && total_tokens > 0 && n_seq > 0 && mdraft_prefill_stack_launches(layer, 1, total_tokens, n_seq, longest, opts) != 1)
-        need = mdraft_prefill_workspace_bytes(layer, total_tokens, n_seq, longest, opts);
+    const size_t need = mdraft::prefill_scratch_bytes(layer, total_tokens, n_seq, max_seqlen, opts, MDRAFT_NOALLOC_SCRATCH_BYTES);
     if (need > (size_t)MDRAFT_NOALLOC_SCRATCH_BYTES) return MDRAFT_ERR_WORKSPACE;
     void* scratch = nullptr;
     if (need > 0) {
@@ -51,5 +47,5 @@ extern "C" int mdraft_conv_scan_prefill_noalloc(const mdraft_layer* layer, const
         if (rc != MDRAFT_OK) return rc;
     }
     return mdraft_conv_scan_prefill(layer, cache, layer_index, x, ldx, z, ldz, dt, lddt, B, ldb, C, ldc, out, ldo, total_tokens,
-                                    n_seq, max_seqlen, cu_seqlens, init_slot, final_slot, scratch, need, opts, dev_status, stream);
+                                    n_seq, max_seqlen, cu_seqlens, init_slot, final_slot, scratch, scratch ? MDRAFT_NOALLOC_SCRATCH_BYTES : 0, opts, dev_status, stream);
 }

@@ -63,4 +63,9 @@ constexpr int kPrefillWideBoxes = 4;  // a wide block covers 4 x kPrefillThreads
 template <int ML>
 cudaError_t launch_prefill(const PrefillBatch<ML>& b, int act, bool chunked, int boxes, bool alone, cudaStream_t st);
 
+// Of a workspace of `available` bytes, how many a call for one layer uses: 0 if it needs none, more than `available` if it would be
+// refused.  Arguments that the call itself would turn away give 0.
+size_t prefill_scratch_bytes(const mdraft_layer* layer, int32_t total_tokens, int32_t n_seq, int32_t max_seqlen, const mdraft_prefill_opts* opts,
+                             size_t available);
+
 }  // namespace mdraft

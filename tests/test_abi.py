@@ -174,6 +174,50 @@ def test_prefill_plan_seen_through_the_workspace_query(lib):
     assert q(0, 1, 8) == 0 and q(8, 0, 8) == 0     # nonsense sizes give 0, not garbage
 
 
+def _takes(lib, binding, layer, T, S, longest, workspace_bytes):
+    """Whether the prefill is content with that much workspace.  Nothing can be launched: the workspace is misaligned, which is
+    looked at next."""
+    D = layer.d_inner
+    rc = _prefill(lib, binding, layer, None, ldx=D, ldz=D, lddt=D, ldo=D, T=T, n_seq=S, max_seqlen=longest, ws=0x900010, ws_bytes=workspace_bytes)
+    assert rc in (-3, -4)
+    return rc != -4
+
+
+def _noalloc_takes(lib, layer, T, S, longest):
+    """The same of the fixed scratch array (x is missing, which is looked at after the size)."""
+    D = layer.d_inner
+    rc = lib.mdraft_conv_scan_prefill_noalloc(C.byref(layer), None, 0, None, D, 0x200000, D, 0x300000, D, 0x400000, 16, 0x500000, 16, 0x600000, D,
+                                              T, S, longest, 0x700000, None, None, None, None, None)
+    assert rc != 0
+    return rc != -4
+
+
+@pytest.mark.parametrize("S,T,longest,D,act", [(33, 425, 130, 1520, 1), (32, 304, 119, 1528, 1), (48, 625, 129, 1016, 1), (73, 798, 111, 608, 0)])
+def test_a_workspace_that_only_fewer_chunks_fit_is_taken(lib, S, T, longest, D, act):
+    """Batches whose preferred chunks want more than the fixed scratch array holds, where fewer chunks do not."""
+    from paper_2506_01206_b200 import binding
+    layer = _layer(binding, d_inner=D, act=act)
+    want = lib.mdraft_prefill_workspace_bytes(C.byref(layer), T, S, longest, None)
+    assert want > 8 << 20 and _noalloc_takes(lib, layer, T, S, longest)
+    assert _takes(lib, binding, layer, T, S, longest, want) and _takes(lib, binding, layer, T, S, longest, 8 << 20)
+    # one chunk a sequence and one more for every 32 tokens is what the longest chunks need; without any workspace there is no call
+    fewest = (S + T // 32 + 1) * D * 17 * 4 + S * D * (16 * 4 + 3 * 4) + 1024
+    assert _takes(lib, binding, layer, T, S, longest, fewest) and not _takes(lib, binding, layer, T, S, longest, 256)
+
+
+def test_a_workspace_too_small_for_the_longest_chunks_is_refused(lib):
+    from paper_2506_01206_b200 import binding
+    layer = _layer(binding, d_inner=1536, act=1)
+    assert not _noalloc_takes(lib, layer, 32000, 4, 8000)
+    for T, S, longest in ((2048, 1, 2048), (32000, 4, 8000), (16000, 8, 2000)):
+        want = lib.mdraft_prefill_workspace_bytes(C.byref(layer), T, S, longest, None)
+        lo, hi = 0, want
+        while hi - lo > 256:
+            mid = (lo + hi) // 2
+            lo, hi = (lo, mid) if _takes(lib, binding, layer, T, S, longest, mid) else (mid, hi)
+        assert want // 8 < hi <= want, "some chunks are needed, and never more than the query says"
+
+
 def test_ssd_host_side_checks(lib):
     """The SSD entry points turn unsupported shapes and bad arguments away before any launch."""
     from paper_2506_01206_b200 import binding
