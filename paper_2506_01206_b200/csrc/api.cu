@@ -171,12 +171,13 @@ PrefillPlan plan_prefill(const mdraft_layer* L, int n_layers, int T, int n_seq, 
         int shortest = max_seqlen / 128;
         shortest = shortest < kMinChunk ? kMinChunk : shortest > kMinChunkWide ? kMinChunkWide : shortest;
         if (narrow < shortest) narrow = shortest;
-        // The longest chunks that a call is given: one wide block or four narrow ones to an SM, at least kMinChunkWide tokens and, for
-        // several sequences, at most kOneWaveMax.
+        // The longest chunks that a call is given: one wide block or four narrow ones (three for a single sequence) to an SM, at least
+        // kMinChunkWide tokens and, for several sequences, at most kOneWaveMax.
         const int64_t most = wide ? sms / ch_blocks_wide : sms * 4 / ch_blocks;
         int64_t longest = (T + (most < 1 ? 1 : most) - 1) / (most < 1 ? 1 : most);
         const bool longest_wide = wide && (n_seq == 1 || longest <= kOneWaveMax);
         longest = longest < kMinChunkWide ? kMinChunkWide : longest > kOneWaveMax && n_seq > 1 ? kOneWaveMax : longest;
+        if (n_seq == 1 && !wide && longest < narrow) longest = narrow;
         if (forced == 0 && narrow <= ((L->flags & MDRAFT_A_POWERS) ? kNarrowChunk : kNarrowChunkGeneral)) wide = false;
         if (wide) {
             int64_t want = sms / ch_blocks_wide;
@@ -190,29 +191,16 @@ PrefillPlan plan_prefill(const mdraft_layer* L, int n_layers, int T, int n_seq, 
             const int tile = kPrefillTileRowBytes / (int)elem_size(L->act), down = Lc / tile * tile;
             if (n_seq == 1 && down >= kMinChunk && T - want_narrow * down <= 4) Lc = down;
         }
-        // More chunks are not taken at the price of a workspace that the fixed scratch array does not hold, where fewer would fit it.
-        auto too_big = [&](int chunk, int instead) {
-            const size_t most = MDRAFT_NOALLOC_SCRATCH_BYTES;
-            auto need = [&](int len) { return len < max_seqlen ? workspace_of(L, n_seq, n_seq + T / len) : (size_t)0; };
-            return need(chunk) > most && need(instead) <= most;
-        };
         // A single sequence in wide blocks stays in one wave at any length: 49 x 3 equal chunks finish together
         // (32768 tokens: 344 us against 372-376 for several waves of short chunks; 65536: 675 against 724).
         if (n_seq == 1) {
-            if (Lc > kOneWaveMax && !wide && !too_big(kManyWavesChunk, Lc)) Lc = kManyWavesChunk;
+            if (Lc > kOneWaveMax && !wide) Lc = kManyWavesChunk;
         } else if (forced == 0 && narrow > ((L->flags & MDRAFT_A_POWERS) ? kNarrowChunk : kNarrowChunkGeneral)) {
             // One wave while its chunks are short and the sequences' unfilled last chunks few (5 x 3172 tokens x 256 channels: 73-token
             // chunks 53.9 us, 48 59.6), then two, then three.
             int64_t waves = narrow <= kOneWaveNarrow && n_seq * narrow * 20 <= T ? narrow : narrow / (narrow <= 2 * kOneWaveNarrow ? 2 : 3);
             waves = waves < kManyWavesMin ? kManyWavesMin : waves > kManyWavesChunk ? kManyWavesChunk : waves;
-            // ... with as few more tokens a chunk as make the workspace fit, up to one wave of them.
-            const int64_t wave4 = sms * 4 / ch_blocks;
-            const int64_t one_wave = wave4 > 0 ? (T + wave4 - 1) / wave4 : kOneWaveMax;
-            const int fewer = wide ? (Lc <= kOneWaveMax ? Lc : kOneWaveMax) : one_wave < waves ? (int)waves : one_wave < kOneWaveMax ? (int)one_wave : kOneWaveMax;
-            const bool keep = too_big((int)waves, fewer);
             Lc = (int)waves;
-            if (keep)
-                while (Lc < fewer && too_big(Lc, fewer)) Lc = Lc + 8 < fewer ? Lc + 8 : fewer;
             wide = false;
         } else if (Lc > kOneWaveMax) {
             Lc = kOneWaveMax;

@@ -192,6 +192,24 @@ def _noalloc_takes(lib, layer, T, S, longest):
     return rc != -4
 
 
+def _chunks(lib, layer, T, S, longest):
+    """The bound on the number of chunks, read back from the workspace query (include/mdraft.h: states, summed step sizes, starting states, windows)."""
+    up = lambda v: (v + 255) // 256 * 256
+    D, es = layer.d_inner, 2 if layer.act else 4
+    want = lib.mdraft_prefill_workspace_bytes(C.byref(layer), T, S, longest, None)
+    for n in range(S, S + T + 1):
+        if up(up(up(up(n * D * 64) + n * D * 4) + S * D * 64) + S * 3 * D * es) == want:
+            return n
+    raise AssertionError(f"no chunk count gives {want} bytes")
+
+
+@pytest.mark.parametrize("S,T,longest,D,chunk_len", [(8, 16000, 2000, 1536, 128), (4, 8000, 2000, 1536, 74)])
+def test_ordinary_calls_are_not_planned_around_the_fixed_scratch_array(lib, S, T, longest, D, chunk_len):
+    """Three waves of chunks where they are long (at most 128 tokens), two where not, whatever the fixed array would hold."""
+    from paper_2506_01206_b200 import binding
+    assert _chunks(lib, _layer(binding, d_inner=D, act=1, flags=1 | 8), T, S, longest) == S + T // chunk_len
+
+
 @pytest.mark.parametrize("S,T,longest,D,act", [(33, 425, 130, 1520, 1), (32, 304, 119, 1528, 1), (48, 625, 129, 1016, 1), (73, 798, 111, 608, 0)])
 def test_a_workspace_that_only_fewer_chunks_fit_is_taken(lib, S, T, longest, D, act):
     """Batches whose preferred chunks want more than the fixed scratch array holds, where fewer chunks do not."""
