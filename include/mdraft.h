@@ -177,7 +177,8 @@ typedef struct {
  * agree over all layers (else MDRAFT_ERR_UNSUPPORTED).
  * Hazards (caller's duty): the layers run side by side, so no layer's `out` may overlap another layer's inputs or `out`, and
  * no pool layer may appear twice.
- *   workspace : at least mdraft_prefill_stack_workspace_bytes(...) for layers that share their flags (the first one's)
+ *   workspace : as above; mdraft_prefill_stack_workspace_bytes answers for layers that share the flags of `layer`.  The
+ *               launches of a call share it, so layers with different flags need the largest answer over their groups
  * mdraft_prefill_stack_launches: kernels such a call launches (for accounting).
  */
 size_t mdraft_prefill_stack_workspace_bytes(const mdraft_layer *layer, int32_t n_layers, int32_t total_tokens, int32_t n_seq,

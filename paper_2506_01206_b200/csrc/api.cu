@@ -315,11 +315,23 @@ int check_io(const mdraft_io& v, const mdraft_layer& L, bool required) {
 
 // How many of the next n layers one launch takes: those with the first one's flags, at most `most`; flags beyond softplus and
 // A = powers (the split modes, whose callers work layer by layer) go one at a time.
+bool one_at_a_time(const mdraft_layer* layer) { return (layer->flags & ~(uint32_t)MDRAFT_A_POWERS) != (uint32_t)MDRAFT_DT_SOFTPLUS; }
 int32_t run_length(int32_t n, const mdraft_layer* layers, int32_t most) {
-    if ((layers->flags & ~(uint32_t)MDRAFT_A_POWERS) != (uint32_t)MDRAFT_DT_SOFTPLUS) return 1;
+    if (one_at_a_time(layers)) return 1;
     int32_t k = 1;
     while (k < n && k < most && layers[k].flags == layers->flags) ++k;
     return k;
+}
+
+// Layers that one launch of the prefill may take: its grid's last dimension also counts sequences (in the carry scan).
+int32_t prefill_most_layers(int32_t n_seq) { return n_seq > 65535 / kPrefillMaxLayers ? 1 : kPrefillMaxLayers; }
+
+// The launches of a prefill of n_layers layers with this one's flags: f(layers of a launch, how many such launches).
+template <typename F>
+void for_each_prefill_run(const mdraft_layer* layer, int32_t n_layers, int32_t n_seq, F&& f) {
+    const int32_t most = one_at_a_time(layer) ? 1 : prefill_most_layers(n_seq);
+    if (n_layers >= most) f(most, n_layers / most);
+    if (n_layers % most) f(n_layers % most, 1);
 }
 
 struct PrefillCall {
@@ -420,9 +432,13 @@ size_t mdraft_prefill_stack_workspace_bytes(const mdraft_layer* layer, int32_t n
                                             int32_t max_seqlen, const mdraft_prefill_opts* opts) {
     if (check_layer(layer) != MDRAFT_OK || n_layers <= 0 || total_tokens <= 0 || n_seq <= 0 || max_seqlen <= 0) return 0;
     // No sequence is longer than the whole batch: a looser static bound must not change the plan.
-    if (n_layers > kPrefillMaxLayers) n_layers = kPrefillMaxLayers;  // launches of one call share the workspace
-    const PrefillPlan pl = plan_prefill(layer, n_layers, total_tokens, n_seq, max_seqlen < total_tokens ? max_seqlen : total_tokens, opts, kAnyWorkspace);
-    return n_layers == 1 || pl.chunked ? pl.bytes : 0;
+    if (max_seqlen > total_tokens) max_seqlen = total_tokens;
+    size_t bytes = 0;  // the launches of one call share the workspace
+    for_each_prefill_run(layer, n_layers, n_seq, [&](int32_t nl, int32_t) {
+        const PrefillPlan pl = plan_prefill(layer, nl, total_tokens, n_seq, max_seqlen, opts, kAnyWorkspace);
+        if ((n_layers == 1 || pl.chunked) && pl.bytes > bytes) bytes = pl.bytes;
+    });
+    return bytes;
 }
 
 int32_t mdraft_prefill_stack_launches(const mdraft_layer* layer, int32_t n_layers, int32_t total_tokens, int32_t n_seq,
@@ -430,10 +446,9 @@ int32_t mdraft_prefill_stack_launches(const mdraft_layer* layer, int32_t n_layer
     if (check_layer(layer) != MDRAFT_OK || n_layers <= 0 || total_tokens <= 0 || n_seq <= 0 || max_seqlen <= 0) return 0;
     if (max_seqlen > total_tokens) max_seqlen = total_tokens;
     int32_t n = 0;
-    for (int32_t l0 = 0; l0 < n_layers; l0 += kPrefillMaxLayers) {
-        const int32_t nl = n_layers - l0 < kPrefillMaxLayers ? n_layers - l0 : kPrefillMaxLayers;
-        n += !plan_prefill(layer, nl, total_tokens, n_seq, max_seqlen, opts, kAnyWorkspace).chunked ? 1 : (layer->flags & MDRAFT_CONV_ONLY) ? 2 : 3;
-    }
+    for_each_prefill_run(layer, n_layers, n_seq, [&](int32_t nl, int32_t times) {
+        n += times * (!plan_prefill(layer, nl, total_tokens, n_seq, max_seqlen, opts, kAnyWorkspace).chunked ? 1 : (layer->flags & MDRAFT_CONV_ONLY) ? 2 : 3);
+    });
     return n;
 }
 
@@ -482,7 +497,7 @@ int mdraft_conv_scan_prefill_stack(int32_t n_layers, const mdraft_layer* layers,
                         static_cast<cudaStream_t>(stream)};
     for (int pass = 0; pass < 2; ++pass)  // every launch is checked before the first is made
         for (int32_t l0 = 0; l0 < n_layers;) {
-            const int32_t nl = run_length(n_layers - l0, layers + l0, n_seq > 65535 / kPrefillMaxLayers ? 1 : kPrefillMaxLayers);
+            const int32_t nl = run_length(n_layers - l0, layers + l0, prefill_most_layers(n_seq));
             const PrefillPlan pl = plan_prefill(layers + l0, nl, plan_tokens, n_seq, max_seqlen, opts, workspace ? workspace_bytes : 0);
             if (pass == 0) {
                 if (pl.n_chunks_bound > 65535 || (int64_t)nl * n_seq > 65535) return MDRAFT_ERR_UNSUPPORTED;

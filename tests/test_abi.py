@@ -236,6 +236,30 @@ def test_a_workspace_too_small_for_the_longest_chunks_is_refused(lib):
         assert want // 8 < hi <= want, "some chunks are needed, and never more than the query says"
 
 
+@pytest.mark.parametrize("n_layers,flags,T,S,D,act", [
+    (33, 1, 2048, 1, 1536, 1),          # a launch of 32 unsplit layers and one of a single layer that is cut into chunks
+    (40, 1 | 8, 4000, 1, 512, 0), (24, 1 | 2, 2048, 1, 1536, 1), (24, 4, 2048, 1, 1536, 1), (3, 1, 50000, 2100, 64, 1)])
+def test_the_workspace_query_covers_every_launch_of_a_call(lib, n_layers, flags, T, S, D, act):
+    from paper_2506_01206_b200 import binding
+
+    class Io(C.Structure):
+        _fields_ = [(n, C.c_void_p) for n in ("x", "z", "dt", "B", "C", "out")] + [(n, C.c_int64) for n in ("ldx", "ldz", "lddt", "ldb", "ldc", "ldo")]
+
+    one = _layer(binding, d_inner=D, act=act, flags=flags)
+    layers, index = (binding._Layer * n_layers)(*[one] * n_layers), (C.c_int32 * n_layers)(*range(n_layers))
+    io = (Io * n_layers)(*[Io(0x100000, 0x200000, 0x300000, 0x400000, 0x500000, 0x600000, D, D, D, 16, 16, D)] * n_layers)
+    longest = T if S == 1 else 20000
+    want = lib.mdraft_prefill_stack_workspace_bytes(C.byref(one), n_layers, T, S, longest, None)
+    assert want > 0
+    rc = lib.mdraft_conv_scan_prefill_stack(C.c_int32(n_layers), layers, None, index, io, C.c_int32(T), C.c_int32(S), C.c_int32(longest), C.c_void_p(0x700000),
+                                            None, None, C.c_void_p(0x900010), C.c_size_t(want), None, None, None)
+    assert rc == -3, "the workspace is large enough; only its alignment is wrong"
+    per_layer = lib.mdraft_prefill_stack_launches(C.byref(one), 1, T, S, longest, None)
+    alone = flags & 6 or S > 2047       # the split modes, and more sequences than a launch's grid takes times 32 layers
+    got = lib.mdraft_prefill_stack_launches(C.byref(one), n_layers, T, S, longest, None)
+    assert got == n_layers * per_layer if alone else got < n_layers * per_layer
+
+
 def test_ssd_host_side_checks(lib):
     """The SSD entry points turn unsupported shapes and bad arguments away before any launch."""
     from paper_2506_01206_b200 import binding
