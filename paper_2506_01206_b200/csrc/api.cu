@@ -103,7 +103,11 @@ struct PrefillPlan {
 // short; wide ones take fewer cycles a token.  Measured (one layer, narrow against wide): 1536 channels x 256 tokens 15.0
 // against 26.0 us, 512 x 4096 27.5 against 31.0, 1536 x 2048 34.4 against 32.7 with A = powers and 41.7 against 42.5 with a
 // general A, 1536 x 32768 357 against 338 and 507 against 491: narrow while one wave of them takes chunks of at most
-// kNarrowChunk (kNarrowChunkGeneral) tokens.  Shorter chunks than a 128th of the sequence cost the carry scan more than they give.
+// kNarrowChunk (kNarrowChunkGeneral) tokens.
+// Where one sequence is one or two channel blocks wide, chunks of less than a 128th of it (to the nearest 8 tokens) cost the carry scan
+// more than they give the passes (3000 tokens x 64 / 128 / 192 channels: 16-token chunks 16.8 / 18.3 / 20.4 us, 24-token 15.7 / 16.8 /
+// 18.8; 4000 x 64 / 256: 16-token 20.1 / 25.4, 32-token 16.7 / 24.9); with more channel blocks, or with two and a general A, whose passes
+// cost more, they pay (3300 x 256, general A: 16-token chunks 23.3, 24 25.5, 32 28.3; 3000 x 384: 21 23.1, 32 23.5).
 // When one wave of narrow blocks would need longer chunks, a single sequence takes one wave of wide blocks, or, where its width
 // does not fill them, several waves of kManyWavesChunk tokens once one wave would need more than kOneWaveMax.  Packed batches,
 // whose chunks are uneven, take one to three waves of narrow blocks, kManyWavesMin to kManyWavesChunk tokens a chunk: blocks are
@@ -167,18 +171,19 @@ PrefillPlan plan_prefill(const mdraft_layer* L, int n_layers, int T, int n_seq, 
     } else {
         // Every sequence leaves its last chunk half unfilled, on average.
         int64_t want_narrow = sms * kBlocksPerSm / ch_blocks - (n_seq - 1) / 2;
-        int64_t narrow = want_narrow > 0 ? (T + want_narrow - 1) / want_narrow : INT_MAX / 2;
+        const int64_t even = want_narrow > 0 ? (T + want_narrow - 1) / want_narrow : INT_MAX / 2;
         int shortest = max_seqlen / 128;
+        if (n_seq == 1) shortest = ch_blocks == 1 || (ch_blocks == 2 && (L->flags & MDRAFT_A_POWERS)) ? (shortest + 4) / 8 * 8 : kMinChunk;
         shortest = shortest < kMinChunk ? kMinChunk : shortest > kMinChunkWide ? kMinChunkWide : shortest;
-        if (narrow < shortest) narrow = shortest;
+        const int64_t narrow = even < shortest ? shortest : even;
         // The longest chunks that a call is given: one wide block or four narrow ones (three for a single sequence) to an SM, at least
         // kMinChunkWide tokens and, for several sequences, at most kOneWaveMax.
         const int64_t most = wide ? sms / ch_blocks_wide : sms * 4 / ch_blocks;
         int64_t longest = (T + (most < 1 ? 1 : most) - 1) / (most < 1 ? 1 : most);
         const bool longest_wide = wide && (n_seq == 1 || longest <= kOneWaveMax);
         longest = longest < kMinChunkWide ? kMinChunkWide : longest > kOneWaveMax && n_seq > 1 ? kOneWaveMax : longest;
-        if (n_seq == 1 && !wide && longest < narrow) longest = narrow;
         if (forced == 0 && narrow <= ((L->flags & MDRAFT_A_POWERS) ? kNarrowChunk : kNarrowChunkGeneral)) wide = false;
+        if (n_seq == 1 && !wide && longest < narrow) longest = narrow;
         if (wide) {
             int64_t want = sms / ch_blocks_wide;
             if (want < 1) want = 1;
@@ -186,10 +191,13 @@ PrefillPlan plan_prefill(const mdraft_layer* L, int n_layers, int T, int n_seq, 
             if (Lc < kMinChunkWide) Lc = kMinChunkWide;
         } else {
             Lc = (int)narrow;
-            // Where whole tiles would leave only a few tokens over a full wave of one sequence, those make a short last chunk
-            // instead of one more step for every chunk (1777 tokens x 1536 channels: 48-token chunks 35.8 us, 49-token chunks 38.4).
-            const int tile = kPrefillTileRowBytes / (int)elem_size(L->act), down = Lc / tile * tile;
-            if (n_seq == 1 && down >= kMinChunk && T - want_narrow * down <= 4) Lc = down;
+            // One sequence: where whole tiles would leave a few tokens over a full wave, those make a short last chunk instead of one more
+            // step for every chunk.  It starts when the wave's first blocks are done and is hidden while it is shorter than they finish
+            // apart: up to a third of a chunk and 16 tokens (1536 channels, general A, 48-token chunks against 49: 1777 tokens 37.8
+            // and 39.2 us, 1790 38.5 and 39.1; against 50: 1821 42.6 and 39.9.  16 against 17: 596 17.3 and 17.0, 601 17.7 and 17.0).
+            const int tile = kPrefillTileRowBytes / (int)elem_size(L->act), down = (int)narrow / tile * tile;
+            const int64_t over = T - want_narrow * down;
+            if (n_seq == 1 && narrow == even && down >= kMinChunk && over <= 16 && over * 3 <= down) Lc = down;
         }
         // A single sequence in wide blocks stays in one wave at any length: 49 x 3 equal chunks finish together
         // (32768 tokens: 344 us against 372-376 for several waves of short chunks; 65536: 675 against 724).

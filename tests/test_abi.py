@@ -210,6 +210,20 @@ def test_ordinary_calls_are_not_planned_around_the_fixed_scratch_array(lib, S, T
     assert _chunks(lib, _layer(binding, d_inner=D, act=1, flags=1 | 8), T, S, longest) == S + T // chunk_len
 
 
+def test_one_sequence_takes_whole_tiles_wherever_few_tokens_are_over(lib):
+    """No special length: the chunk count follows the length without a step between 1780 and 1781, and a width whose SMs the shortest
+    chunks do not fill keeps to a 128th of the sequence."""
+    from paper_2506_01206_b200 import binding
+    general = _layer(binding, d_inner=1536, act=1)
+    assert {_chunks(lib, general, T, 1, T) for T in range(1777, 1793)} == {1 + 1777 // 48}
+    for T, chunk_len in ((1776, 48), (1793, 49), (1813, 49), (1850, 50)):
+        assert _chunks(lib, general, T, 1, T) == 1 + T // chunk_len
+    for T, least in ((3000, 24), (4000, 32)):
+        for D, flags in ((64, 1), (128, 1), (64, 9), (128, 9), (192, 9), (256, 9)):
+            n = _chunks(lib, _layer(binding, d_inner=D, act=1, flags=flags), T, 1, T)
+            assert n <= 1 + T // least, (T, D, flags, n)
+
+
 @pytest.mark.parametrize("S,T,longest,D,act", [(33, 425, 130, 1520, 1), (32, 304, 119, 1528, 1), (48, 625, 129, 1016, 1), (73, 798, 111, 608, 0)])
 def test_a_workspace_that_only_fewer_chunks_fit_is_taken(lib, S, T, longest, D, act):
     """Batches whose preferred chunks want more than the fixed scratch array holds, where fewer chunks do not."""
