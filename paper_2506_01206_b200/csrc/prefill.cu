@@ -127,11 +127,11 @@ __device__ __forceinline__ void grid_release_dependents() { asm volatile("gridde
 
 // ---------------------------------------------------------------- one channel's running computation
 // The usual case (kFast: conv, softplus, recurrence, gate) works in scaled quantities, which takes the constant factors of the
-// base-2 special functions out of the token loop: step sizes are kept times log2(e) (what lg2 gives), the conv's output times
-// -log2(e) (what its SiLU's exponential takes), and B is widened times kInputScale = -ln(2)^2, which takes both factors out of
-// the product again: the state itself is never scaled, so that it enters and leaves the registers bit for bit.  (One layer of
-// 32 packed sequences, 141650 tokens: 1492 -> 1389 us.)
-constexpr float kInputScale = -kLn2 * kLn2;
+// base-2 special functions out of the token loop: step sizes are kept times log2(e) (what lg2 gives) and the conv's sum times
+// -log2(e) (what its SiLU's exponential takes).  The SiLU's denominator is formed times kSiluScale = -log2(e)^2, by the multiply-add that
+// would be the addition of 1, so that u comes out times ln(2) and its product with the step size in units of its own: the state is
+// never scaled, it enters and leaves the registers bit for bit.  (One layer of 32 packed sequences, 141650 tokens: 1492 -> 1389 us.)
+constexpr float kSiluScale = -kLog2e * kLog2e;
 
 template <typename AT, bool kPow, bool kOut, bool kFast>
 struct ChannelScan {
@@ -158,7 +158,7 @@ struct ChannelScan {
         w[0] = wv.x * fu; w[1] = wv.y * fu; w[2] = wv.z * fu; w[3] = wv.w * fu;
         cb = L.conv_b ? __ldg(L.conv_b + d) * fu : 0.0f;
         dtb = L.dt_bias ? __ldg(L.dt_bias + d) * (kFast ? kLog2e : 1.0f) : 0.0f;
-        dsk = L.D ? __ldg(L.D + d) * (kFast ? -kLn2 : 1.0f) : 0.0f;
+        dsk = L.D ? __ldg(L.D + d) * (kFast ? kLog2e : 1.0f) : 0.0f;
         sum_delta = 0.0f;
         flags = kFast ? (uint32_t)MDRAFT_DT_SOFTPLUS : L.flags;
 #pragma unroll
@@ -210,7 +210,7 @@ struct ChannelScan {
             acc = fmaf(w[2], win[2], acc);
             acc = fmaf(w[3], xv, acc);
             win[0] = win[1]; win[1] = win[2]; win[2] = xv;
-            e.u = kFast ? acc * rcp(1.0f + ex2(acc)) : silu(acc);
+            e.u = kFast ? acc * rcp(fmaf(ex2(acc), kSiluScale, kSiluScale)) : silu(acc);
         }
         e.delta = 0.f; e.du = 0.f; e.gate = 0.f;
         if (flags & MDRAFT_CONV_ONLY) return;
@@ -465,7 +465,7 @@ __global__ void __launch_bounds__(SUB * kBoxCols + 32, SUB == 1 ? 3 : 1) chunk_k
                 const AT* rb = reinterpret_cast<const AT*>(s_stage[s] + off_b(SUB));
                 const AT* rc = reinterpret_cast<const AT*>(s_stage[s] + off_c(SUB));
                 for (int i = lane; i < rows * kN; i += 32) {
-                    (&sBf[s][0][0])[i] = Act<AT>::to_f32(rb[i]) * (kFast ? kInputScale : 1.0f);
+                    (&sBf[s][0][0])[i] = Act<AT>::to_f32(rb[i]);
                     if (want_c) (&sCf[s][0][0])[i] = Act<AT>::to_f32(rc[i]);
                 }
             }
