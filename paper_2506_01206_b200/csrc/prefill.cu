@@ -128,10 +128,12 @@ __device__ __forceinline__ void grid_release_dependents() { asm volatile("gridde
 // ---------------------------------------------------------------- one channel's running computation
 // The usual case (kFast: conv, softplus, recurrence, gate) works in scaled quantities, which takes the constant factors of the
 // base-2 special functions out of the token loop: step sizes are kept times log2(e) (what lg2 gives) and the conv's sum times
-// -log2(e) (what its SiLU's exponential takes).  The SiLU's denominator is formed times kSiluScale = -log2(e)^2, by the multiply-add that
-// would be the addition of 1, so that u comes out times ln(2) and its product with the step size in units of its own: the state is
-// never scaled, it enters and leaves the registers bit for bit.  (One layer of 32 packed sequences, 141650 tokens: 1492 -> 1389 us.)
-constexpr float kSiluScale = -kLog2e * kLog2e;
+// -log2(e) (what its SiLU's exponential takes).  Both factors leave the product of step size, u and B again at no cost, so that the
+// state is never scaled and enters and leaves the registers bit for bit: with A = powers the SiLU's denominator is formed times
+// kSiluScale, by the multiply-add that would be the addition of 1, and u comes out times ln(2); a general A has no register to spare
+// for that constant (one sequence of 20821 x 264, fp32: 99.4 against 109 us), there B is widened times kInputScale.
+// (One layer of 32 packed sequences, 141650 tokens: 1492 -> 1389 us.)
+constexpr float kSiluScale = -kLog2e * kLog2e, kInputScale = -kLn2 * kLn2;
 
 template <typename AT, bool kPow, bool kOut, bool kFast>
 struct ChannelScan {
@@ -158,7 +160,7 @@ struct ChannelScan {
         w[0] = wv.x * fu; w[1] = wv.y * fu; w[2] = wv.z * fu; w[3] = wv.w * fu;
         cb = L.conv_b ? __ldg(L.conv_b + d) * fu : 0.0f;
         dtb = L.dt_bias ? __ldg(L.dt_bias + d) * (kFast ? kLog2e : 1.0f) : 0.0f;
-        dsk = L.D ? __ldg(L.D + d) * (kFast ? kLog2e : 1.0f) : 0.0f;
+        dsk = L.D ? __ldg(L.D + d) * (kFast ? (kPow ? kLog2e : -kLn2) : 1.0f) : 0.0f;
         sum_delta = 0.0f;
         flags = kFast ? (uint32_t)MDRAFT_DT_SOFTPLUS : L.flags;
 #pragma unroll
@@ -210,7 +212,7 @@ struct ChannelScan {
             acc = fmaf(w[2], win[2], acc);
             acc = fmaf(w[3], xv, acc);
             win[0] = win[1]; win[1] = win[2]; win[2] = xv;
-            e.u = kFast ? acc * rcp(fmaf(ex2(acc), kSiluScale, kSiluScale)) : silu(acc);
+            e.u = !kFast ? silu(acc) : kPow ? acc * rcp(fmaf(ex2(acc), kSiluScale, kSiluScale)) : acc * rcp(1.0f + ex2(acc));
         }
         e.delta = 0.f; e.du = 0.f; e.gate = 0.f;
         if (flags & MDRAFT_CONV_ONLY) return;
@@ -465,7 +467,7 @@ __global__ void __launch_bounds__(SUB * kBoxCols + 32, SUB == 1 ? 3 : 1) chunk_k
                 const AT* rb = reinterpret_cast<const AT*>(s_stage[s] + off_b(SUB));
                 const AT* rc = reinterpret_cast<const AT*>(s_stage[s] + off_c(SUB));
                 for (int i = lane; i < rows * kN; i += 32) {
-                    (&sBf[s][0][0])[i] = Act<AT>::to_f32(rb[i]);
+                    (&sBf[s][0][0])[i] = Act<AT>::to_f32(rb[i]) * (kFast && !kPow ? kInputScale : 1.0f);
                     if (want_c) (&sCf[s][0][0])[i] = Act<AT>::to_f32(rc[i]);
                 }
             }
