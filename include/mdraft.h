@@ -143,7 +143,7 @@ typedef struct {
  *   max_seqlen : an upper bound on the longest sequence (HOST value, used to size the launch)
  *   workspace  : device scratch, 256-byte aligned; contents need not be initialised and are garbage afterwards.
  *                mdraft_prefill_workspace_bytes(...) says how much the call would like.  With less it cuts the sequences
- *                into fewer, longer chunks (slower, and another rounding), as long as those give every SM four blocks
+ *                into fewer, longer chunks (slower, and another rounding), as long as those give every SM three or four blocks
  *                of 128 channels (one of 512 where the width fills those) or are, for several sequences, at most 256
  *                tokens; less is MDRAFT_ERR_WORKSPACE.  Sequences that the library leaves whole need none, although
  *                the query for a single layer answers as if they were cut.  A chunk length given in `opts` is kept:

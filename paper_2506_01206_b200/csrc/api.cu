@@ -70,6 +70,9 @@ int check_matrix(const void* p, int64_t ld, int cols, int act, bool required) {
     return MDRAFT_OK;
 }
 
+// Flags beyond softplus and A = powers: the split modes and raw step sizes, which have kernels of their own that take one layer.
+bool one_at_a_time(const mdraft_layer* layer) { return (layer->flags & ~(uint32_t)MDRAFT_A_POWERS) != (uint32_t)MDRAFT_DT_SOFTPLUS; }
+
 LayerDev layer_dev(const mdraft_layer* L) {
     LayerDev d;
     d.A = L->A; d.D = L->D; d.conv_w = L->conv_w; d.conv_b = L->conv_b; d.dt_bias = L->dt_bias;
@@ -90,15 +93,13 @@ PoolDev pool_dev(const mdraft_cache* c, int act, int layer_index) {
 struct PrefillPlan {
     int chunk_len;       // tokens per chunk (INT_MAX/2 when every sequence is one chunk)
     int n_chunks_bound;  // upper bound on the number of chunks
-    bool chunked;
-    int boxes;           // 128-channel boxes per block: 1, 2 (unsplit sequences only) or 4 (one block per SM)
+    PrefillForm form;
     bool longest_first;  // unsplit sequences of different lengths, handed out longest first
-    bool alone;          // unsplit sequences: one block per SM
     size_t off_q, off_sd, off_h0, off_conv, layer_bytes;
     size_t bytes;        // what the workspace query answers: the call's layers, split
 };
 
-// Chunk length: split the token axis until every SM holds kBlocksPerSm blocks of kPrefillThreads channels, or one wide block
+// Chunk length: split the token axis until every SM holds three blocks of kPrefillThreads channels, or one wide block
 // (one resident wave, no tail).  Narrow blocks have more registers a thread, hide one another's set-up and can be 16 tokens
 // short; wide ones take fewer cycles a token.  Measured (one layer, narrow against wide): 1536 channels x 256 tokens 15.0
 // against 26.0 us, 512 x 4096 27.5 against 31.0, 1536 x 2048 34.4 against 32.7 with A = powers and 41.7 against 42.5 with a
@@ -106,15 +107,20 @@ struct PrefillPlan {
 // kNarrowChunk (kNarrowChunkGeneral) tokens.
 // Where one sequence is one or two channel blocks wide, chunks of less than a 128th of it (to the nearest 8 tokens) cost the carry scan
 // more than they give the passes (3000 tokens x 64 / 128 / 192 channels: 16-token chunks 16.8 / 18.3 / 20.4 us, 24-token 15.7 / 16.8 /
-// 18.8; 4000 x 64 / 256: 16-token 20.1 / 25.4, 32-token 16.7 / 24.9); with more channel blocks, or with two and a general A, whose passes
+// 18.8; 4000 x 64 / 256: 16-token 20.1 / 25.4, 32-token 16.7 / 24.9), up to kOneBlockChunk tokens for one channel block, whose chunks then
+// have an SM each (5000 x 128: 32-token 23.1, 40-token 20.4; 6976 x 112, general A: 31.7, 56-token 28.1; 8000 x 64: 23.9, 64-token
+// 24.9, two blocks of 32 tokens an SM again), and up to kMinChunkWide for two; with more channel blocks, or with two and a general A, whose passes
 // cost more, they pay (3300 x 256, general A: 16-token chunks 23.3, 24 25.5, 32 28.3; 3000 x 384: 21 23.1, 32 23.5).
 // When one wave of narrow blocks would need longer chunks, a single sequence takes one wave of wide blocks, or, where its width
 // does not fill them, several waves of kManyWavesChunk tokens once one wave would need more than kOneWaveMax.  Packed batches,
 // whose chunks are uneven, take one to three waves of narrow blocks, kManyWavesMin to kManyWavesChunk tokens a chunk: blocks are
 // handed out as SMs free up, which evens them out (8 x 2000 tokens x 512 channels: wide 83.7 us, 48-64 tokens 73.5, 128 79.8; 26
 // sequences of 4k-12k tokens x 152 channels: 64 tokens 331, 128 321, 256 334).
-constexpr int kBlocksPerSm = 3, kMinChunk = 16, kMinChunkWide = 32, kNarrowChunk = 48, kNarrowChunkGeneral = 72;
-constexpr int kOneWaveMax = 256, kManyWavesChunk = 128, kManyWavesMin = 48, kOneWaveNarrow = 110;
+// Three narrow blocks to an SM have 128 registers a thread, four have 96.  Four are up to 17 % faster where the width leaves a warp of each
+// block idle and the batch is packed (32 sequences, 91k tokens x 72 channels 94.7 -> 85.1 us; 20, 37k x 88, general A 59.3 -> 48.8;
+// 32, 17k x 288 72.2 -> 65.6), slower elsewhere (full blocks, general A: 2-5 %; one sequence of 13608 x 96 38.7 -> 41.6).
+constexpr int kMinChunk = 16, kMinChunkWide = 32, kNarrowChunk = 48, kNarrowChunkGeneral = 72;
+constexpr int kOneWaveMax = 256, kManyWavesChunk = 128, kManyWavesMin = 48, kOneWaveNarrow = 110, kOneBlockChunk = 56;
 
 // Splitting a sequence costs a second pass over its tokens (0.75 of the output pass, for all chunks but the last) and two more
 // launches; not splitting it leaves one block per sequence, layer and 128 or 256 channels.  SM cycles a token of a block takes
@@ -164,26 +170,37 @@ PrefillPlan plan_prefill(const mdraft_layer* L, int n_layers, int T, int n_seq, 
     // the last of them).  They need the channel count to (nearly) fill whole 512-channel blocks.
     bool wide = forced == wide_cols || (forced == 0 && ch_blocks_wide * wide_cols * 9 <= (int64_t)n_layers * D * 10);
     int Lc;
-    bool unsplit = false, alone = false;
+    bool unsplit = false, alone = false, four = false;
     int unsplit_boxes = 1;
+    const bool general = !(L->flags & MDRAFT_A_POWERS);
     if (opts && opts->chunk_len > 0) {
         Lc = opts->chunk_len < 4 ? 4 : opts->chunk_len;
     } else {
-        // Every sequence leaves its last chunk half unfilled, on average.
-        int64_t want_narrow = sms * kBlocksPerSm / ch_blocks - (n_seq - 1) / 2;
-        const int64_t even = want_narrow > 0 ? (T + want_narrow - 1) / want_narrow : INT_MAX / 2;
+        // Four narrow blocks to an SM instead of three: for packed batches whose blocks have a warp of four to spare (the width fills at
+        // most three quarters of them) and whose wave of four takes whole tiles; with several channel blocks for A = powers only.
+        four = n_layers == 1 && n_seq > 1 && !one_at_a_time(L) && (D + 31) / 32 <= 3 * ch_blocks && (!general || ch_blocks == 1) &&
+               T >= kMinChunk * (sms * 4 / ch_blocks - (n_seq - 1) / 2);
+        const int per_sm = four ? 4 : 3;
+        // Chunks of a wave of so many blocks to an SM; every sequence leaves its last chunk half unfilled, on average.
+        auto wave_chunks = [&](int blocks) { return sms * blocks / ch_blocks - (n_seq - 1) / 2; };
+        auto wave_length = [&](int blocks) { return wave_chunks(blocks) > 0 ? (T + wave_chunks(blocks) - 1) / wave_chunks(blocks) : (int64_t)(INT_MAX / 2); };
+        const int64_t want_narrow = wave_chunks(per_sm), even = wave_length(per_sm);
         int shortest = max_seqlen / 128;
-        if (n_seq == 1) shortest = ch_blocks == 1 || (ch_blocks == 2 && (L->flags & MDRAFT_A_POWERS)) ? (shortest + 4) / 8 * 8 : kMinChunk;
-        shortest = shortest < kMinChunk ? kMinChunk : shortest > kMinChunkWide ? kMinChunkWide : shortest;
+        if (n_seq == 1) shortest = ch_blocks == 1 || (ch_blocks == 2 && !general) ? (shortest + (shortest > 40 ? 7 : 4)) / 8 * 8 : kMinChunk;
+        const int most_shortest = n_seq == 1 && ch_blocks == 1 && shortest <= kOneBlockChunk ? kOneBlockChunk : kMinChunkWide;
+        shortest = shortest < kMinChunk ? kMinChunk : shortest > most_shortest ? most_shortest : shortest;
         const int64_t narrow = even < shortest ? shortest : even;
-        // The longest chunks that a call is given: one wide block or four narrow ones (three for a single sequence) to an SM, at least
-        // kMinChunkWide tokens and, for several sequences, at most kOneWaveMax.
-        const int64_t most = wide ? sms / ch_blocks_wide : sms * 4 / ch_blocks;
-        int64_t longest = (T + (most < 1 ? 1 : most) - 1) / (most < 1 ? 1 : most);
-        const bool longest_wide = wide && (n_seq == 1 || longest <= kOneWaveMax);
-        longest = longest < kMinChunkWide ? kMinChunkWide : longest > kOneWaveMax && n_seq > 1 ? kOneWaveMax : longest;
-        if (forced == 0 && narrow <= ((L->flags & MDRAFT_A_POWERS) ? kNarrowChunk : kNarrowChunkGeneral)) wide = false;
-        if (n_seq == 1 && !wide && longest < narrow) longest = narrow;
+        const bool short_chunks = narrow * per_sm <= (general ? kNarrowChunkGeneral : kNarrowChunk) * 3;
+        // The longest chunks that a call is given when its workspace does not hold the preferred ones: one wide block or four narrow ones to
+        // an SM, at least kMinChunkWide tokens and, for several sequences, at most kOneWaveMax (`coarse`); three narrow ones where that
+        // is what a wave of short chunks may be.  Where not even those fit, leaving the sequences whole is weighed against `coarse` chunks.
+        const int64_t most = wide ? sms / ch_blocks_wide : sms * 4 / ch_blocks, uncapped = (T + (most < 1 ? 1 : most) - 1) / (most < 1 ? 1 : most);
+        const bool coarse_wide = wide && (n_seq == 1 || uncapped <= kOneWaveMax);
+        const int64_t coarse = uncapped < kMinChunkWide ? kMinChunkWide : uncapped > kOneWaveMax && n_seq > 1 ? kOneWaveMax : uncapped;
+        if (forced == 0 && short_chunks) wide = false;
+        int64_t longest = !wide && (n_seq == 1 || four) ? wave_length(3) : coarse;
+        if (n_seq > 1 && longest > kOneWaveMax) longest = kOneWaveMax;
+        if (longest < coarse) longest = coarse;
         if (wide) {
             int64_t want = sms / ch_blocks_wide;
             if (want < 1) want = 1;
@@ -203,10 +220,11 @@ PrefillPlan plan_prefill(const mdraft_layer* L, int n_layers, int T, int n_seq, 
         // (32768 tokens: 344 us against 372-376 for several waves of short chunks; 65536: 675 against 724).
         if (n_seq == 1) {
             if (Lc > kOneWaveMax && !wide) Lc = kManyWavesChunk;
-        } else if (forced == 0 && narrow > ((L->flags & MDRAFT_A_POWERS) ? kNarrowChunk : kNarrowChunkGeneral)) {
+        } else if (forced == 0 && !short_chunks) {
             // One wave while its chunks are short and the sequences' unfilled last chunks few (5 x 3172 tokens x 256 channels: 73-token
             // chunks 53.9 us, 48 59.6), then two, then three.
-            int64_t waves = narrow <= kOneWaveNarrow && n_seq * narrow * 20 <= T ? narrow : narrow / (narrow <= 2 * kOneWaveNarrow ? 2 : 3);
+            const int64_t one_wave = narrow * per_sm / 3;   // tokens a chunk of a wave of three blocks to an SM
+            int64_t waves = one_wave <= kOneWaveNarrow && n_seq * narrow * 20 <= T ? narrow : narrow / (one_wave <= 2 * kOneWaveNarrow ? 2 : 3);
             waves = waves < kManyWavesMin ? kManyWavesMin : waves > kManyWavesChunk ? kManyWavesChunk : waves;
             Lc = (int)waves;
             wide = false;
@@ -215,7 +233,6 @@ PrefillPlan plan_prefill(const mdraft_layer* L, int n_layers, int T, int n_seq, 
             if (forced == 0) wide = false;
         }
         if (n_seq + (int64_t)T / Lc > 65535 && Lc < kOneWaveMax) Lc = kOneWaveMax;  // a launch's grid
-        const bool general = !(L->flags & MDRAFT_A_POWERS);
         const double g1 = (general ? kGeneralOne : 1.0) * (L->act == MDRAFT_F32 ? kFloatOne : 1.0), gm = general ? kGeneralMany : 1.0;
         // The unsplit forms: 128 channels alone, 256 channels alone, and three blocks of 128 channels to an SM for many short sequences.
         const double one = unsplit_cycles(ch_blocks, g1 * kCycOne, T, n_seq, max_seqlen, sms), pair = unsplit_cycles(ch_blocks_pair, g1 * kCycPair, T, n_seq, max_seqlen, sms);
@@ -236,20 +253,21 @@ PrefillPlan plan_prefill(const mdraft_layer* L, int n_layers, int T, int n_seq, 
                 hi = (hi + 7) / 8 * 8;
                 Lc = (int)(hi < longest ? hi : longest);
             }
-            unsplit = need(Lc) > workspace ? better_whole(longest, longest_wide) : better_whole(Lc, wide);
+            unsplit = need(Lc) > workspace ? better_whole(coarse, coarse_wide) : better_whole(Lc, wide);
         }
         if (unsplit) {
             unsplit_boxes = pair < one && pair < many ? 2 : 1;
             alone = unsplit_boxes == 2 || one <= many;
         }
     }
-    pl.boxes = unsplit ? unsplit_boxes : wide ? kPrefillWideBoxes : 1;
-    pl.chunked = Lc < max_seqlen;
-    pl.longest_first = pl.alone = false;
+    pl.form.boxes = unsplit ? unsplit_boxes : wide ? kPrefillWideBoxes : 1;
+    pl.form.chunked = Lc < max_seqlen;
+    pl.longest_first = pl.form.alone = false;
+    pl.form.four = four && !unsplit && !wide;
     pl.chunk_len = INT_MAX / 2;
     pl.n_chunks_bound = n_seq;
     pl.off_q = pl.off_sd = pl.off_h0 = pl.off_conv = pl.layer_bytes = pl.bytes = 0;
-    if (pl.chunked) {
+    if (pl.form.chunked) {
         const int bound = n_seq + T / Lc;
         pl.layer_bytes = workspace_of(L, n_seq, bound, &pl);
         // For one layer the query answers for the split form whichever form is taken: a workspace made for one batch then
@@ -261,11 +279,11 @@ PrefillPlan plan_prefill(const mdraft_layer* L, int n_layers, int T, int n_seq, 
         }
     }
     if (unsplit) {
-        pl.chunked = false;
+        pl.form.chunked = false;
         // Where every block starts at once the order is worth nothing.
-        const bool at_once = (pl.boxes == 2 ? ch_blocks_pair : ch_blocks) * n_seq <= sms;
+        const bool at_once = (pl.form.boxes == 2 ? ch_blocks_pair : ch_blocks) * n_seq <= sms;
         pl.longest_first = !at_once && n_seq > 1 && n_seq <= kPrefillMaxRanked;
-        pl.alone = alone;
+        pl.form.alone = alone;
     }
     return pl;
 }
@@ -321,9 +339,7 @@ int check_io(const mdraft_io& v, const mdraft_layer& L, bool required) {
     return check_matrix(v.C, v.ldc, kN, L.act, all);
 }
 
-// How many of the next n layers one launch takes: those with the first one's flags, at most `most`; flags beyond softplus and
-// A = powers (the split modes, whose callers work layer by layer) go one at a time.
-bool one_at_a_time(const mdraft_layer* layer) { return (layer->flags & ~(uint32_t)MDRAFT_A_POWERS) != (uint32_t)MDRAFT_DT_SOFTPLUS; }
+// How many of the next n layers one launch takes: those with the first one's flags, at most `most`.
 int32_t run_length(int32_t n, const mdraft_layer* layers, int32_t most) {
     if (one_at_a_time(layers)) return 1;
     int32_t k = 1;
@@ -370,13 +386,13 @@ int run_prefill(const PrefillCall& call, const PrefillPlan& pl, int32_t n_layers
     a.longest_first = pl.longest_first;
     a.cu = call.cu_seqlens; a.init_slot = call.init_slot; a.final_slot = call.final_slot;
     char* ws = call.workspace;
-    a.ws_q = pl.chunked ? reinterpret_cast<float*>(ws + pl.off_q) : nullptr;
-    a.ws_sd = pl.chunked ? reinterpret_cast<float*>(ws + pl.off_sd) : nullptr;
-    a.ws_h0 = pl.chunked ? reinterpret_cast<float*>(ws + pl.off_h0) : nullptr;
-    a.ws_conv = pl.chunked ? static_cast<void*>(ws + pl.off_conv) : nullptr;
+    a.ws_q = pl.form.chunked ? reinterpret_cast<float*>(ws + pl.off_q) : nullptr;
+    a.ws_sd = pl.form.chunked ? reinterpret_cast<float*>(ws + pl.off_sd) : nullptr;
+    a.ws_h0 = pl.form.chunked ? reinterpret_cast<float*>(ws + pl.off_h0) : nullptr;
+    a.ws_conv = pl.form.chunked ? static_cast<void*>(ws + pl.off_conv) : nullptr;
     a.ws_layer_bytes = (int64_t)pl.layer_bytes;
     a.dev_status = call.dev_status;
-    a.pdl_inputs_ready = pl.chunked ? 1 : 0;  // the summary pass waits for the producer of the inputs on behalf of all three kernels
+    a.pdl_inputs_ready = pl.form.chunked ? 1 : 0;  // the summary pass waits for the producer of the inputs on behalf of all three kernels
     a.ev_state = call.opts ? static_cast<cudaEvent_t>(call.opts->event_after_chunk_state) : nullptr;
     a.ev_carry = call.opts ? static_cast<cudaEvent_t>(call.opts->event_after_carry_scan) : nullptr;
     const bool rows = call.total_tokens > 0;  // with no tokens at all (only empty sequences) nothing is ever copied: empty descriptors
@@ -393,7 +409,7 @@ int run_prefill(const PrefillCall& call, const PrefillPlan& pl, int32_t n_layers
             !encode_matrix(&p.maps.C, rows ? v.C : nullptr, act, a.T, kN, v.ldc, kN))
             return MDRAFT_ERR_CUDA;
     }
-    return launch_prefill<ML>(b, act, pl.chunked, pl.boxes, pl.alone, call.stream) == cudaSuccess ? MDRAFT_OK : MDRAFT_ERR_CUDA;
+    return launch_prefill<ML>(b, act, pl.form, call.stream) == cudaSuccess ? MDRAFT_OK : MDRAFT_ERR_CUDA;
 }
 
 __global__ void classify_A_kernel(const float* A, int D, int N, int32_t* res) {
@@ -412,7 +428,7 @@ size_t mdraft::prefill_scratch_bytes(const mdraft_layer* layer, int32_t total_to
     if (check_layer(layer) != MDRAFT_OK || total_tokens <= 0 || n_seq <= 0) return 0;
     if (max_seqlen < 1) max_seqlen = 1;
     const PrefillPlan pl = plan_prefill(layer, 1, total_tokens, n_seq, max_seqlen < total_tokens ? max_seqlen : total_tokens, opts, available);
-    return pl.chunked ? pl.bytes : 0;
+    return pl.form.chunked ? pl.bytes : 0;
 }
 
 extern "C" {
@@ -444,7 +460,7 @@ size_t mdraft_prefill_stack_workspace_bytes(const mdraft_layer* layer, int32_t n
     size_t bytes = 0;  // the launches of one call share the workspace
     for_each_prefill_run(layer, n_layers, n_seq, [&](int32_t nl, int32_t) {
         const PrefillPlan pl = plan_prefill(layer, nl, total_tokens, n_seq, max_seqlen, opts, kAnyWorkspace);
-        if ((n_layers == 1 || pl.chunked) && pl.bytes > bytes) bytes = pl.bytes;
+        if ((n_layers == 1 || pl.form.chunked) && pl.bytes > bytes) bytes = pl.bytes;
     });
     return bytes;
 }
@@ -455,7 +471,7 @@ int32_t mdraft_prefill_stack_launches(const mdraft_layer* layer, int32_t n_layer
     if (max_seqlen > total_tokens) max_seqlen = total_tokens;
     int32_t n = 0;
     for_each_prefill_run(layer, n_layers, n_seq, [&](int32_t nl, int32_t times) {
-        n += times * (!plan_prefill(layer, nl, total_tokens, n_seq, max_seqlen, opts, kAnyWorkspace).chunked ? 1 : (layer->flags & MDRAFT_CONV_ONLY) ? 2 : 3);
+        n += times * (!plan_prefill(layer, nl, total_tokens, n_seq, max_seqlen, opts, kAnyWorkspace).form.chunked ? 1 : (layer->flags & MDRAFT_CONV_ONLY) ? 2 : 3);
     });
     return n;
 }
@@ -509,7 +525,7 @@ int mdraft_conv_scan_prefill_stack(int32_t n_layers, const mdraft_layer* layers,
             const PrefillPlan pl = plan_prefill(layers + l0, nl, plan_tokens, n_seq, max_seqlen, opts, workspace ? workspace_bytes : 0);
             if (pass == 0) {
                 if (pl.n_chunks_bound > 65535 || (int64_t)nl * n_seq > 65535) return MDRAFT_ERR_UNSUPPORTED;
-                if (pl.chunked) {
+                if (pl.form.chunked) {
                     if (!workspace || workspace_bytes < pl.bytes) return MDRAFT_ERR_WORKSPACE;
                     if (reinterpret_cast<uintptr_t>(workspace) & 255u) return MDRAFT_ERR_MISALIGNED;
                 }

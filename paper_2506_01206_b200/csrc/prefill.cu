@@ -336,8 +336,9 @@ __device__ __forceinline__ void issue_tile(unsigned char* stage, uint64_t* bar, 
 }
 
 // ---------------------------------------------------------------------------------------------------
-template <typename AT, int SUB, bool kPow, bool kOut, bool kFast, int ML>
-__global__ void __launch_bounds__(SUB * kBoxCols + 32, SUB == 1 ? 3 : 1) chunk_kernel(const __grid_constant__ PrefillBatch<ML> batch) {
+// PER_SM: blocks that share an SM.  Blocks of 128 channels come in two forms, for three (128 registers a thread) and for four (96).
+template <typename AT, int SUB, bool kPow, bool kOut, bool kFast, int ML, int PER_SM>
+__global__ void __launch_bounds__(SUB * kBoxCols + 32, PER_SM) chunk_kernel(const __grid_constant__ PrefillBatch<ML> batch) {
     const PrefillArgs& c = batch.c;
     const PrefillLayer& p = batch.l[ML == 1 ? 0 : blockIdx.z];
     constexpr int TT = TileTokens<AT>::v, GRP = group_tokens(kPow);
@@ -703,7 +704,7 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, int threads, size_t 
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
-template <typename AT, int SUB, bool kPow, bool kFast, int ML>
+template <typename AT, int SUB, bool kPow, bool kFast, int ML, int PER_SM = SUB == 1 ? 3 : 1>
 cudaError_t launch_typed(const PrefillBatch<ML>& b, bool chunked, bool alone, cudaStream_t st) {
     const PrefillArgs& p = b.c;
     const int D = p.d_inner;
@@ -713,8 +714,8 @@ cudaError_t launch_typed(const PrefillBatch<ML>& b, bool chunked, bool alone, cu
     cudaError_t e = cudaSuccess;
     if constexpr (SUB != 2)  // blocks of 256 channels take unsplit sequences only
     if (chunked) {
-        if ((e = allow_smem<chunk_kernel<AT, SUB, kPow, false, kFast, ML>>(kSmem)) != cudaSuccess) return e;
-        e = launch_pdl(chunk_kernel<AT, SUB, kPow, false, kFast, ML>, grid, kThreads, kSmem, st, b);
+        if ((e = allow_smem<chunk_kernel<AT, SUB, kPow, false, kFast, ML, PER_SM>>(kSmem)) != cudaSuccess) return e;
+        e = launch_pdl(chunk_kernel<AT, SUB, kPow, false, kFast, ML, PER_SM>, grid, kThreads, kSmem, st, b);
     }
     if (e != cudaSuccess) return e;
     if (p.ev_state) cudaEventRecord(p.ev_state, st);
@@ -726,14 +727,16 @@ cudaError_t launch_typed(const PrefillBatch<ML>& b, bool chunked, bool alone, cu
     if (p.ev_carry) cudaEventRecord(p.ev_carry, st);
     // Alone on its SM: ask for more than half of the SM's shared memory.
     constexpr int kSmemAlone = 116 * 1024;
-    if ((e = allow_smem<chunk_kernel<AT, SUB, kPow, true, kFast, ML>>(SUB < 4 ? kSmemAlone : kSmem)) != cudaSuccess) return e;
-    return launch_pdl(chunk_kernel<AT, SUB, kPow, true, kFast, ML>, grid, kThreads, SUB < 4 && alone ? kSmemAlone : kSmem, st, b);
+    if ((e = allow_smem<chunk_kernel<AT, SUB, kPow, true, kFast, ML, PER_SM>>(SUB < 4 ? kSmemAlone : kSmem)) != cudaSuccess) return e;
+    return launch_pdl(chunk_kernel<AT, SUB, kPow, true, kFast, ML, PER_SM>, grid, kThreads, SUB < 4 && alone ? kSmemAlone : kSmem, st, b);
 }
 
 template <typename AT, int SUB, int ML>
-cudaError_t launch_act(const PrefillBatch<ML>& b, bool chunked, bool alone, cudaStream_t st) {
+cudaError_t launch_act(const PrefillBatch<ML>& b, const PrefillForm& form, cudaStream_t st) {
     const uint32_t flags = b.l[0].L.flags;
-    const bool pow = flags & MDRAFT_A_POWERS;
+    const bool pow = flags & MDRAFT_A_POWERS, chunked = form.chunked, alone = form.alone;
+    if constexpr (SUB == 1 && ML == 1)
+        if (form.four) return pow ? launch_typed<AT, SUB, true, true, ML, 4>(b, chunked, alone, st) : launch_typed<AT, SUB, false, true, ML, 4>(b, chunked, alone, st);
     if ((flags & ~(uint32_t)MDRAFT_A_POWERS) == (uint32_t)MDRAFT_DT_SOFTPLUS)
         return pow ? launch_typed<AT, SUB, true, true>(b, chunked, alone, st) : launch_typed<AT, SUB, false, true>(b, chunked, alone, st);
     if constexpr (ML > 1) return cudaErrorInvalidValue;  // the caller takes such layers one by one
@@ -743,14 +746,14 @@ cudaError_t launch_act(const PrefillBatch<ML>& b, bool chunked, bool alone, cuda
 }  // namespace
 
 template <int ML>
-cudaError_t launch_prefill(const PrefillBatch<ML>& b, int act, bool chunked, int boxes, bool alone, cudaStream_t st) {
-    switch (boxes) {
-        case 1: return act == MDRAFT_F32 ? launch_act<float, 1>(b, chunked, alone, st) : launch_act<__nv_bfloat16, 1>(b, chunked, alone, st);
-        case 2: return act == MDRAFT_F32 ? launch_act<float, 2>(b, chunked, alone, st) : launch_act<__nv_bfloat16, 2>(b, chunked, alone, st);
-        default: return act == MDRAFT_F32 ? launch_act<float, kPrefillWideBoxes>(b, chunked, alone, st) : launch_act<__nv_bfloat16, kPrefillWideBoxes>(b, chunked, alone, st);
+cudaError_t launch_prefill(const PrefillBatch<ML>& b, int act, const PrefillForm& form, cudaStream_t st) {
+    switch (form.boxes) {
+        case 1: return act == MDRAFT_F32 ? launch_act<float, 1>(b, form, st) : launch_act<__nv_bfloat16, 1>(b, form, st);
+        case 2: return act == MDRAFT_F32 ? launch_act<float, 2>(b, form, st) : launch_act<__nv_bfloat16, 2>(b, form, st);
+        default: return act == MDRAFT_F32 ? launch_act<float, kPrefillWideBoxes>(b, form, st) : launch_act<__nv_bfloat16, kPrefillWideBoxes>(b, form, st);
     }
 }
-template cudaError_t launch_prefill<1>(const PrefillBatch<1>&, int, bool, int, bool, cudaStream_t);
-template cudaError_t launch_prefill<kPrefillMaxLayers>(const PrefillBatch<kPrefillMaxLayers>&, int, bool, int, bool, cudaStream_t);
+template cudaError_t launch_prefill<1>(const PrefillBatch<1>&, int, const PrefillForm&, cudaStream_t);
+template cudaError_t launch_prefill<kPrefillMaxLayers>(const PrefillBatch<kPrefillMaxLayers>&, int, const PrefillForm&, cudaStream_t);
 
 }  // namespace mdraft

@@ -58,10 +58,17 @@ struct PrefillBatch {
 
 constexpr int kPrefillWideBoxes = 4;  // a wide block covers 4 x kPrefillThreads channels with 16 channel warps
 
-// boxes: 128-channel boxes per block (1, 2 or kPrefillWideBoxes; 2 for unsplit sequences only).  alone: one block per SM.
+// How a call is launched.
+struct PrefillForm {
+    bool chunked;  // sequences are cut into chunks: three kernels instead of one
+    int boxes;     // 128-channel boxes per block: 1, 2 (unsplit sequences only) or kPrefillWideBoxes (one block per SM)
+    bool alone;    // unsplit sequences: one block per SM
+    bool four;     // blocks of 128 channels: four to an SM instead of three (one layer, softplus step sizes only)
+};
+
 // ML = 1, or kPrefillMaxLayers for a call over several layers (all with the same flags: softplus, A_POWERS or not).
 template <int ML>
-cudaError_t launch_prefill(const PrefillBatch<ML>& b, int act, bool chunked, int boxes, bool alone, cudaStream_t st);
+cudaError_t launch_prefill(const PrefillBatch<ML>& b, int act, const PrefillForm& form, cudaStream_t st);
 
 // Of a workspace of `available` bytes, how many a call for one layer uses: 0 if it needs none, more than `available` if it would be
 // refused.  Arguments that the call itself would turn away give 0.

@@ -100,6 +100,23 @@ def test_prefill_matches_oracle(act, Dn, lens, chunk_len, general_A, conv_bias, 
     assert np.array_equal(g_conv, o_conv), "conv window must be an exact copy of the last raw inputs"
 
 
+@pytest.mark.parametrize("act,Dn,lens,general_A", [
+    ("f32", 64, [3000, 0, 4500, 1, 2111], True),     # a wave of four blocks to an SM just above 16 tokens a chunk
+    ("bf16", 96, [700] * 16, True), ("bf16", 72, [5000, 17, 12000, 40], False), ("f32", 88, [333] * 40, False),
+    ("bf16", 264, [900, 31, 2800], False),           # three channel blocks, the last one of a single warp
+    ("f32", 64, [5000], True), ("bf16", 128, [3000], False), ("bf16", 256, [3300], True)])   # one sequence: floors under the chunk length
+def test_prefill_default_plan_of_narrow_problems_matches_oracle(act, Dn, lens, general_A):
+    cfg = parity.small_config(Dn, act, len(lens))
+    prob = parity.make_problem(cfg, lens, conv_bias=True, general_A=general_A)
+    ci, hi = random_state(cfg, len(lens), 6)
+    flags = md.MDRAFT_DT_SOFTPLUS | (0 if general_A else md.MDRAFT_A_POWERS)
+    g_out, g_conv, g_h = run_gpu_prefill(prob, flags, 0, ci, hi)
+    o_out, o_conv, o_h = run_oracle_prefill(prob, flags, ci, hi)
+    assert_close(g_out, o_out, TOL[act], "out")
+    assert_close(g_h, o_h, TOL_STATE, "final SSM state")
+    assert np.array_equal(g_conv, o_conv)
+
+
 def test_no_chunk_length_may_be_given_as_none():
     cfg = parity.small_config(64, "f32", 1)
     prob = parity.make_problem(cfg, [256])
