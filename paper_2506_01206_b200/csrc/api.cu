@@ -17,13 +17,10 @@
 
 using namespace mdraft;
 
-namespace {
-
-constexpr int kSmCountB200 = 148;
-
 // SMs of the current device; the B200's count when no device can be asked (the workspace query also runs where there
 // is none, and must then give the size the call will want on the B200 it is planned for).
-int sm_count() {
+int mdraft::sm_count() {
+    constexpr int kSmCountB200 = 148;
     static std::atomic<int> known{0};  // every device this library runs on is the same part
     int dev = 0, n = known.load(std::memory_order_relaxed);
     if (n > 0) return n;
@@ -34,6 +31,8 @@ int sm_count() {
     known.store(n, std::memory_order_relaxed);
     return n;
 }
+
+namespace {
 
 inline size_t elem_size(int act) { return act == MDRAFT_BF16 ? 2 : 4; }
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }

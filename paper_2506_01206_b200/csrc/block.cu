@@ -240,12 +240,11 @@ __global__ void __launch_bounds__(NW * 32, PRE > 0 ? 0 : 2) small_linear_kernel(
     }
 }
 
-// The same product for a wide n (the LM head: 77 MB of weights for the 130M shape), bound by HBM: one block per SM takes every
+// The same product, normalised, for a wide n (the LM head: 77 MB of weights for the 130M shape), bound by HBM: one block per SM takes every
 // gridDim.x-th tile of 32 columns and keeps the next two tiles' weights in flight (cp.async ring of three) while it multiplies
 // one.  A warp's share of the contraction stays the same from tile to tile, so its activations stay in registers.
 constexpr int kWideNT = 32, kWideWarps = 8, kWideStages = 3, kWideBlocks = 4;   // kWideBlocks: blocks of 32 of the contraction a warp may hold
 
-template <bool NORM>
 __global__ void __launch_bounds__(kWideWarps * 32, 1) wide_linear_kernel(const SmallLinear p) {
     constexpr int NW = kWideWarps, NT = kWideNT, kCols = NT / 16, kPitch = w_pitch(NT);
     extern __shared__ __align__(128) unsigned char s_w[];   // [kWideStages][k][NT], then the warps' partial results [NW][kRows][NT]
@@ -283,13 +282,11 @@ __global__ void __launch_bounds__(kWideWarps * 32, 1) wide_linear_kernel(const S
             a[q][i] = make_uint4(0u, 0u, 0u, 0u);
             if (kb < kblocks && row < rows) a[q][i] = *reinterpret_cast<const uint4*>(p.a + (size_t)(m0 + row) * p.k + kb * 32 + t * 8);
         }
-    if (NORM) {
 #pragma unroll
-        for (int q = 0; q < kWideBlocks; ++q)
+    for (int q = 0; q < kWideBlocks; ++q)
 #pragma unroll
-            for (int i = 0; i < kNodeTiles; ++i) sq[i] = squares(a[q][i], sq[i]);
-        put_squares(s_sq[warp], sq, g, t);
-    }
+        for (int i = 0; i < kNodeTiles; ++i) sq[i] = squares(a[q][i], sq[i]);
+    put_squares(s_sq[warp], sq, g, t);
     int stage = 0;
     for (int tile = blockIdx.x; tile < tiles; tile += step) {
         asm volatile("cp.async.wait_group %0;" ::"n"(kWideStages - 2) : "memory");
@@ -311,7 +308,7 @@ __global__ void __launch_bounds__(kWideWarps * 32, 1) wide_linear_kernel(const S
         __syncthreads();   // the partial results of the tile before have been read
         put_part<kCols>(part + warp * kRows * part_pitch(NT), acc, node_tiles, g, t);
         __syncthreads();
-        finish<NT, NW, NORM>(p, part, s_sq, rows, m0, tile * NT, __nv_bfloat162());
+        finish<NT, NW, true>(p, part, s_sq, rows, m0, tile * NT, __nv_bfloat162());
     }
 }
 
@@ -355,27 +352,22 @@ cudaError_t launch_tile(const SmallLinear& p, cudaStream_t st) {
 }  // namespace
 
 cudaError_t launch_small_linear(const SmallLinear& p, cudaStream_t st) {
-    const bool norm = p.eps >= 0.0f;
-    // Beyond one wave of 32-column tiles the persistent form, where the contraction fits its registers (it does not add).
-    if (p.n > 32 * 148 && !p.add && p.k <= kWideWarps * kWideBlocks * 32) {
-        const int tiles = (p.n + kWideNT - 1) / kWideNT, mt = (p.m + kRows - 1) / kRows, per_row = 148 / mt;
-        const dim3 grid(tiles < per_row ? tiles : per_row, mt);
-        const int smem = kWideStages * p.k * w_pitch(kWideNT) + kWideWarps * kRows * part_pitch(kWideNT) * 4;
-        if (smem <= kMaxSmem)
-            return norm ? launch_chained<wide_linear_kernel<true>>(grid, kWideWarps * 32, smem, p, st)
-                        : launch_chained<wide_linear_kernel<false>>(grid, kWideWarps * 32, smem, p, st);
-    }
-    // The narrow tile for a narrow n, whose blocks are few, and for a contraction too long for the wide one's shared memory.
+    const int sms = sm_count();
+    const bool one_tile = p.m <= kRows;
+    // out_proj (the only product that is added to something and not normalised) has at most kBlockMaxModel columns: few blocks even
+    // of the narrow tile.
     // Fragments of W in registers ahead of the wait while one row tile leaves room for the kernels of the chain beside each
     // other (18 nodes: 329 -> 304 us a generation); with two, the registers they take cost more (64 nodes: 486 -> 534 us).
-    const int rows = p.m < kRows ? p.m : kRows;
-    const bool narrow = p.n <= 16 * 148 || rows_offset(p.k, 32, 12) + rows * p.k * 2 > kMaxSmem;
-    if (p.m <= kRows) {
-        if (narrow) return norm ? launch_tile<16, 12, 4, true>(p, st) : launch_tile<16, 12, 4, false>(p, st);
-        return norm ? launch_tile<32, 12, 2, true>(p, st) : launch_tile<32, 12, 2, false>(p, st);
+    if (p.eps < 0.0f) return one_tile ? launch_tile<16, 12, 4, false>(p, st) : launch_tile<16, 12, 0, false>(p, st);
+    // Beyond one wave of 32-column tiles the persistent form, where the contraction fits its registers and shared memory.
+    const int smem = kWideStages * p.k * w_pitch(kWideNT) + kWideWarps * kRows * part_pitch(kWideNT) * 4;
+    if (p.n > 32 * sms && p.k <= kWideWarps * kWideBlocks * 32 && smem <= kMaxSmem) {
+        const int tiles = (p.n + kWideNT - 1) / kWideNT, mt = (p.m + kRows - 1) / kRows, per_row = sms / mt;
+        return launch_chained<wide_linear_kernel>(dim3(tiles < per_row ? tiles : per_row, mt), kWideWarps * 32, smem, p, st);
     }
-    if (narrow) return norm ? launch_tile<16, 12, 0, true>(p, st) : launch_tile<16, 12, 0, false>(p, st);
-    return norm ? launch_tile<32, 12, 0, true>(p, st) : launch_tile<32, 12, 0, false>(p, st);
+    // The narrow tile for a narrow n, whose blocks are few.
+    if (p.n <= 16 * sms) return one_tile ? launch_tile<16, 12, 4, true>(p, st) : launch_tile<16, 12, 0, true>(p, st);
+    return one_tile ? launch_tile<32, 12, 2, true>(p, st) : launch_tile<32, 12, 0, true>(p, st);
 }
 
 cudaError_t launch_embed(const int64_t* tokens, const __nv_bfloat16* embed, __nv_bfloat16* h, int m, int d, int vocab, int32_t* dev_status, cudaStream_t st) {

@@ -9,11 +9,11 @@ constexpr int kBlockMaxNodes = 64;    // rows of a generation these kernels take
 constexpr int kBlockMaxModel = 1408;  // a block's columns of W fit its shared memory: d_model for in_proj and the LM head,
 constexpr int kBlockMaxInner = 2048;  // d_inner for out_proj, beside 32 rows of its activations
 
-// out[m][n] = sum_k a[m][k] W[k][n], all bf16, fp32 accumulation; rows of a optionally normalised, out optionally added to.
+// out[m][n] = sum_k a[m][k] W[k][n], all bf16, fp32 accumulation; either with the rows of a normalised, or added to something.
 // k a multiple of 32, n of 8, m at most kBlockMaxNodes.
 struct SmallLinear {
     const __nv_bfloat16 *a, *W;
-    const __nv_bfloat16* add;  // same shape and stride as out, or NULL
+    const __nv_bfloat16* add;  // same shape and stride as out; NULL for a normalised product
     __nv_bfloat16* out;
     int64_t ldw, ldo;          // rows of a are dense (k values)
     int m, n, k;

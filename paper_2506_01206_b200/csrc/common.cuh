@@ -137,6 +137,9 @@ struct PoolDev {
     int n_slots;
 };
 
+// SMs of the current device (api.cu).
+int sm_count();
+
 // A kernel that wants more dynamic shared memory than a launch gets by default has the limit raised once per device: it is a
 // property of the loaded function, and asking for it on every call costs host time.
 template <auto kKernel>

@@ -543,7 +543,7 @@ cudaError_t launch_act(const TreeProjArgs& p, cudaStream_t st) {
     // Nodes per cluster: one while the level is narrow (latency is what counts and every node gets its own SMs);
     // two or four once the level is wide enough that re-reading the two matrices per node is what costs.
     int nt = p.nodes_per_cluster;
-    if (nt <= 0) nt = p.n_nodes * n_blocks <= 2 * 148 ? 1 : (p.n_nodes * n_blocks <= 4 * 148 ? 2 : 4);
+    if (nt <= 0) nt = p.n_nodes * n_blocks <= 2 * sm_count() ? 1 : (p.n_nodes * n_blocks <= 4 * sm_count() ? 2 : 4);
     if (cb == 512) nt = 1;  // the widest block has no registers to spare for a second node
     switch (cb) {
         case 128: return nt == 1 ? launch_nt<AT, 128, 1>(p, n_blocks, st) : nt == 2 ? launch_nt<AT, 128, 2>(p, n_blocks, st) : launch_nt<AT, 128, 4>(p, n_blocks, st);
