@@ -124,6 +124,35 @@ def test_projection_step_wait_runs_out_and_the_cluster_still_meets(waitlib, act,
     assert_close(rig.states()[0], o_h, TOL_STATE, "node states after recovery")
 
 
+@pytest.mark.parametrize("width,d_model,d_inner,vocab", [(5, 64, 96, 104), (40, 416, 1216, 4800)])
+def test_block_generation_wait_runs_out_and_the_call_returns(waitlib, width, d_model, d_inner, vocab):
+    """The block products wait for one bulk copy of the activations: without it they store nothing, and nothing that
+    follows in the chain does (the LM head of 4800 columns waits for nothing but the kernel ahead: its logits are those
+    of whatever is in h)."""
+    from paper_2506_01206_b200.drafter import ToyDrafter
+    d = ToyDrafter(n_layers=2, d_model=d_model, d_inner=d_inner, dt_rank=8, vocab=vocab, max_nodes=width)
+    d.node_slot.copy_(torch.arange(1, width + 1, device="cuda"))
+    d.cache.ssm.fill_(3.0); d.cache.conv.fill_(3.0)
+    d._xz.fill_(7.0); d.y.fill_(7.0); d.logits.fill_(7.0)
+    with using(waitlib):
+        d.generation(0, width, use_graph=False)
+        torch.cuda.synchronize()
+    assert int(d.status.item()) == md.MDRAFT_DEV_WAIT_EXPIRED
+    for t, what in ((d._xz, "in_proj"), (d.y, "projection step")) + (() if vocab > 4736 else ((d.logits, "LM head"),)):
+        assert bool((t == 7.0).all()), f"{what}: a block that gave up must not have written results"
+    assert bool((d.cache.ssm == 3.0).all()) and bool((d.cache.conv == 3.0).all())
+    assert torch.equal(d._h, d.embed[d.tokens]), "out_proj: the residual is as the embedding left it"
+    d.status.zero_()
+    d.cache.ssm.zero_(); d.cache.conv.zero_()
+    d.generation(0, width, use_graph=False)
+    torch.cuda.synchronize()
+    assert int(d.status.item()) == 0
+    from test_gpu_block import TOL_LOGITS
+    from test_gpu_drafter import _replica_logits
+    conv0, h0 = d.cache.conv[:, 0].double().cpu().numpy(), d.cache.ssm[:, 0].double().cpu().numpy()
+    assert_close(d.logits[width - 1].double().cpu().numpy(), _replica_logits(d, [0], conv0, h0), TOL_LOGITS, "logits after recovery")
+
+
 def test_ssd_prefill_wait_runs_out_tensor_memory_is_freed_and_the_next_call_is_correct(waitlib):
     """The tensor-core kernels of the SSD encode allocate tensor memory before they wait for their copies: when the
     wait runs out they must still free it (a leak would stall later blocks on the same SM for good) and store no
