@@ -104,7 +104,7 @@ struct PrefillPlan {
 // against 26.0 us, 512 x 4096 27.5 against 31.0, 1536 x 2048 34.4 against 32.7 with A = powers and 41.7 against 42.5 with a
 // general A, 1536 x 32768 357 against 338 and 507 against 491: narrow while one wave of them takes chunks of at most
 // kNarrowChunk (kNarrowChunkGeneral) tokens.
-// Where one sequence is one or two channel blocks wide, chunks of less than a 128th of it (to the nearest 8 tokens) cost the carry scan
+// Where one sequence is one or two channel blocks wide, chunks of less than a 128th of it (to the nearest 8 tokens, beyond 40 to the next) cost the carry scan
 // more than they give the passes (3000 tokens x 64 / 128 / 192 channels: 16-token chunks 16.8 / 18.3 / 20.4 us, 24-token 15.7 / 16.8 /
 // 18.8; 4000 x 64 / 256: 16-token 20.1 / 25.4, 32-token 16.7 / 24.9), up to kOneBlockChunk tokens for one channel block, whose chunks then
 // have an SM each (5000 x 128: 32-token 23.1, 40-token 20.4; 6976 x 112, general A: 31.7, 56-token 28.1; 8000 x 64: 23.9, 64-token

@@ -14,12 +14,12 @@
 // A call in which every sequence fits one chunk runs the output pass only.
 //
 // Data movement.  One thread owns one channel and keeps its 16 state entries in registers as 8 packed pairs
-// (fma.rn.f32x2 / mul.rn.f32x2: one instruction per two entries).  A block of 128 or 512 channels walks its chunk in
+// (fma.rn.f32x2 / mul.rn.f32x2: one instruction per two entries).  A block of 128, 256 or 512 channels walks its chunk in
 // tiles of 16 (bf16) or 8 (fp32) tokens; the x / dt / z boxes (tile x 128 channels) and the B / C boxes of a tile
 // are brought into a ring of shared-memory stages by TMA (cp.async.bulk.tensor, one instruction per matrix and
 // tile, completion counted on an mbarrier), two tiles ahead of the arithmetic.  The block is warp-specialised: one extra
 // warp queues the copies, widens each landed B / C tile to fp32 (read afterwards as 128-bit broadcasts) and hands it
-// to the 4 or 16 channel warps through a "ready" mbarrier; each channel warp releases a stage through an "empty" mbarrier
+// to the 4, 8 or 16 channel warps through a "ready" mbarrier; each channel warp releases a stage through an "empty" mbarrier
 // when it is done, so the channel warps never wait for one another.  Every wait on an mbarrier is bounded: if
 // it runs out, the warp raises MDRAFT_DEV_WAIT_EXPIRED and stops; the copy warp first gives the copies it still
 // has in flight a bounded chance to land (they target this block's shared memory).
@@ -37,8 +37,8 @@ constexpr int kBoxCols = kPrefillThreads;  // channels of one TMA box (and of on
 constexpr int kStages = 3;              // shared-memory ring depth
 constexpr int kTileBytes = 4096;        // one staged x / dt / z box: kTT rows of kBoxCols activations
 constexpr int kBCBytes = 512;           // one staged B or C tile: kTT rows of 16 activations
-// A block covers SUB boxes of channels (SUB = 1: 128 channels, 4 channel warps; SUB = 4: 512 channels, 16 channel
-// warps that share the block's B / C tiles and advance tile by tile together).  Stage layout: x boxes, dt boxes,
+// A block covers SUB boxes of channels (SUB = 1: 128 channels, 4 channel warps; SUB = 2: 256 channels, 8 warps, unsplit sequences
+// only; SUB = 4: 512 channels, 16 channel warps, which share the block's B / C tiles and advance tile by tile together).  Stage layout: x boxes, dt boxes,
 // z boxes, B, C.
 __host__ __device__ constexpr int stage_bytes(int sub) { return 3 * sub * kTileBytes + 2 * kBCBytes; }
 __host__ __device__ constexpr int off_x(int) { return 0; }
@@ -47,7 +47,10 @@ __host__ __device__ constexpr int off_z(int sub) { return 2 * sub * kTileBytes; 
 __host__ __device__ constexpr int off_b(int sub) { return 3 * sub * kTileBytes; }
 __host__ __device__ constexpr int off_c(int sub) { return 3 * sub * kTileBytes + kBCBytes; }
 __host__ __device__ constexpr int smem_bytes(int sub) { return kStages * (stage_bytes(sub) + 2 * kBCBytes * 2); }  // + fp32 B, C
-constexpr int kFmaPairs = 1;            // pairs of decays per token computed on the FMA pipe when A is general (measured: 0 -> 43.8, 1 -> 42.5, 2 -> 43.0, 3 -> 45.6 us per 2048x1536 call)
+// Pairs of decays per token computed on the FMA pipe when A is general: the special-function unit is the busiest one there (63-68 % of a
+// one-layer pass's cycles, prologue included).  0 / 1 / 2 / 3 pairs: 39.8 / 37.7 / 38.0 / 40.3 us for 1777 x 1536, 44.8 / 42.9 / 42.6 / 45.7
+// for 2048, 502 / 481 / 482 / 516 for 32768, and in fp32 43.9 / 42.3 / 42.2 / 45.5 for three sequences of 2700 x 1000.
+constexpr int kFmaPairs = 1;
 // Tokens whose state-independent part is computed together, so that their special-function latencies overlap: 8 for A = powers
 // (4 instead: 642 against 610 us for 148 wide blocks of 2048 tokens, 250 against 226 us for blocks of 128 channels), 4 for a
 // general A, whose 16 exponentials a token keep the unit busy (8: 870 against 828 us).
@@ -129,11 +132,13 @@ __device__ __forceinline__ void grid_release_dependents() { asm volatile("gridde
 // The usual case (kFast: conv, softplus, recurrence, gate) works in scaled quantities, which takes the constant factors of the
 // base-2 special functions out of the token loop: step sizes are kept times log2(e) (what lg2 gives) and the conv's sum times
 // -log2(e) (what its SiLU's exponential takes).  Both factors leave the product of step size, u and B again at no cost, so that the
-// state is never scaled and enters and leaves the registers bit for bit: with A = powers the SiLU's denominator is formed times
-// kSiluScale, by the multiply-add that would be the addition of 1, and u comes out times ln(2); a general A has no register to spare
-// for that constant (one sequence of 20821 x 264, fp32: 99.4 against 109 us), there B is widened times kInputScale.
-// (One layer of 32 packed sequences, 141650 tokens: 1492 -> 1389 us.)
+// state is never scaled and enters and leaves the registers bit for bit.  With bf16 activations and A = powers the SiLU's denominator is
+// formed times kSiluScale, by the multiply-add that would be the addition of 1, and u comes out times ln(2) (24 layers of 2048 x 1536 in
+// one call: 328.9 us, 337.6 with B scaled); a general A has no register to spare for that constant (one fp32 sequence of 20821 x 264:
+// 109 against 99.4 us) and fp32 gains nothing by it (8 layers of 5492 x 1608: 587 against 576), there B is widened times kInputScale.
+// (One layer of 32 packed sequences, 141650 tokens: 1492 -> 1254 us.)
 constexpr float kSiluScale = -kLog2e * kLog2e, kInputScale = -kLn2 * kLn2;
+template <typename AT, bool kPow> constexpr bool kScaleSilu = kPow && sizeof(AT) == 2;
 
 template <typename AT, bool kPow, bool kOut, bool kFast>
 struct ChannelScan {
@@ -160,7 +165,7 @@ struct ChannelScan {
         w[0] = wv.x * fu; w[1] = wv.y * fu; w[2] = wv.z * fu; w[3] = wv.w * fu;
         cb = L.conv_b ? __ldg(L.conv_b + d) * fu : 0.0f;
         dtb = L.dt_bias ? __ldg(L.dt_bias + d) * (kFast ? kLog2e : 1.0f) : 0.0f;
-        dsk = L.D ? __ldg(L.D + d) * (kFast ? (kPow ? kLog2e : -kLn2) : 1.0f) : 0.0f;
+        dsk = L.D ? __ldg(L.D + d) * (kFast ? (kScaleSilu<AT, kPow> ? kLog2e : -kLn2) : 1.0f) : 0.0f;
         sum_delta = 0.0f;
         flags = kFast ? (uint32_t)MDRAFT_DT_SOFTPLUS : L.flags;
 #pragma unroll
@@ -212,7 +217,7 @@ struct ChannelScan {
             acc = fmaf(w[2], win[2], acc);
             acc = fmaf(w[3], xv, acc);
             win[0] = win[1]; win[1] = win[2]; win[2] = xv;
-            e.u = !kFast ? silu(acc) : kPow ? acc * rcp(fmaf(ex2(acc), kSiluScale, kSiluScale)) : acc * rcp(1.0f + ex2(acc));
+            e.u = !kFast ? silu(acc) : kScaleSilu<AT, kPow> ? acc * rcp(fmaf(ex2(acc), kSiluScale, kSiluScale)) : acc * rcp(1.0f + ex2(acc));
         }
         e.delta = 0.f; e.du = 0.f; e.gate = 0.f;
         if (flags & MDRAFT_CONV_ONLY) return;
@@ -468,7 +473,7 @@ __global__ void __launch_bounds__(SUB * kBoxCols + 32, PER_SM) chunk_kernel(cons
                 const AT* rb = reinterpret_cast<const AT*>(s_stage[s] + off_b(SUB));
                 const AT* rc = reinterpret_cast<const AT*>(s_stage[s] + off_c(SUB));
                 for (int i = lane; i < rows * kN; i += 32) {
-                    (&sBf[s][0][0])[i] = Act<AT>::to_f32(rb[i]) * (kFast && !kPow ? kInputScale : 1.0f);
+                    (&sBf[s][0][0])[i] = Act<AT>::to_f32(rb[i]) * (kFast && !kScaleSilu<AT, kPow> ? kInputScale : 1.0f);
                     if (want_c) (&sCf[s][0][0])[i] = Act<AT>::to_f32(rc[i]);
                 }
             }
