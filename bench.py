@@ -9,7 +9,7 @@ workload (Mamba-130M: 24 layers, d_inner 1536, d_state 16; context 2048 tokens; 
 the per-phase throughputs (prefill token*channels/s, tree node-updates/s) are reported beside it.
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl reference]
-    python bench.py --profile-case prefill|tree|proj|ssd [sizes ...] (small runs of one kernel family for a profiler)
+    python bench.py --profile-case prefill|stack|tree|proj|ssd|generation [sizes ...] (small runs of one kernel family for a profiler)
 
 N > 1 (under torchrun) runs N independent replicas (the path has no exchange step): weak scaling.
 `--impl reference` times the fp64 CPU oracle on a bounded sample of the same workload.
@@ -354,21 +354,6 @@ def run_ours(args):
     split = kernel_split(stack, 3)
     split_general = kernel_split(stack_general, 2)
 
-    # ---- the output-pass kernel alone, replayed from a graph: the same 2048 rows given as 49 independent sequences of 42
-    # tokens are not split, so the call launches ONLY the output pass (one launch for all 24 layers).
-    n_ck = -(-T // 42)
-    cu_alone = i32(np.minimum(np.arange(n_ck + 1) * 42, T), dev)
-    alone_stack = DrafterStack(stack.layers, n_ck, T, n_ck, 42, 0, dev)
-    alone_slots = i32(np.arange(n_ck), dev)
-    assert alone_stack.prefill_launches_per_layer(T, n_ck, 42) == 1
-
-    def do_alone():
-        alone_stack.prefill(dev_pre, out_pre, cu_alone, 42, alone_slots, alone_slots)
-
-    ms_alone = time_graph(capture(do_alone), Kp, 3)
-    alone_stack.check_status()
-    output_pass_us = 1e3 * ms_alone / NL
-
     # ---- tree step on the batched-serving shape (32 sequences x 32-node trees): whole round and its widest level
     bt = BatchedTree(seed=rank)
     bt_layers = [upload_layer(p, w.cfg.act, md.MDRAFT_DT_SOFTPLUS | (md.MDRAFT_A_POWERS if is_pow else 0), dev) for p in w.params]
@@ -496,7 +481,7 @@ def run_ours(args):
         cfg4_lens = [int(v) for v in np.diff(gen.seq_lengths(gen.get_config(4)))]
         prefill_shapes = {
             "note": "whole prefill call (summary pass + carry scan + output pass) per layer; hbm_frac against the measured copy bandwidth; "
-                    "fp32_issue_frac = lane-operations per token*channel (82 as counted in DESIGN.md, 70 as the scope table estimated) x units / time / (148 x 128 x 1965 MHz)",
+                    "fp32_issue_frac = lane-operations per token*channel (82 counted from the formulas the kernels evaluate, 70 a rounder estimate) x units / time / (148 x 128 x 1965 MHz)",
             "long_context_32768_bf16": prefill_leg("bf16", [32768], 4, 5),
             "packed_batch_32_seqs_1k_8k_bf16": prefill_leg("bf16", cfg4_lens, 2, 3),
             "fp32_activations_2048": prefill_leg("f32", [2048], 8, 10),
@@ -632,12 +617,14 @@ def run_ours(args):
     launches = md.mdraft_prefill_stack_launches(stack.layers[0], NL, T, 1, T) + -(-NL // 32) * (len(levels) - 1) + 1
     alu_peak = SM_COUNT * FP32_LANES_PER_SM * SM_MAX_MHZ * 1e6  # fp32 lane-ops/s at the maximum SM clock
 
-    # dominant kernel: the output pass of the prefill (chunk_kernel<bf16, kOut>).  Algorithmic bytes of one layer's
-    # prefill over that kernel's own duration; the whole three-kernel call is quoted beside it.
+    # dominant kernel: the output pass of the prefill (chunk_kernel<bf16, kOut>), which takes all layers of the step's encode in
+    # one launch: every sequence is left whole, so it is the call's only kernel.  The three kernels of a call for one
+    # layer, which is cut into chunks, are quoted beside it.
     pb = w.prefill_bytes_per_layer()
-    scan_s = output_pass_us * 1e-6
-    call_s = ms_prefill * 1e-3 / NL
-    kname = "chunk_kernel<bf16, %s, output pass>" % ("structured A" if is_pow else "general A")
+    if md.mdraft_prefill_stack_launches(stack.layers[0], NL, T, 1, T) != 1:
+        raise RuntimeError("the step's encode is expected to be one launch")
+    scan_s = call_s = ms_prefill * 1e-3 / NL
+    kname = "chunk_kernel<bf16, 256-channel blocks, %s, output pass>" % ("structured A" if is_pow else "general A")
     lane_ops = ALU_LANE_OPS_PER_UNIT * T * D
     roofline = {
         # bf16 activations: 82 fp32 lane-ops against 8 bytes per token*channel put this kernel's ridge point far on
@@ -647,15 +634,14 @@ def run_ours(args):
         "unit": "T fp32 lane-op/s (one instruction on one lane; an FMA counts once)", "frac": lane_ops / scan_s / alu_peak,
         "traffic": ncu_traffic("prefill_output_pass")[0], "traffic_kernel": ncu_traffic("prefill_output_pass")[1],
         "peak_source": "148 SMs x 128 fp32 lanes x %.0f MHz (clocks.max.sm)" % SM_MAX_MHZ,
-        "algorithmic_lane_ops_per_launch": lane_ops, "algorithmic_bytes_per_launch": pb, "launch_us": output_pass_us,
-        "timed": "CUDA-graph replay of one launch of this kernel over 24 layers (the 2048 rows as 49 unsplit sequences of 42 tokens), time / 24",
-        "launch_us_between_events": split[2],
+        "algorithmic_lane_ops_per_launch": NL * lane_ops, "algorithmic_bytes_per_launch": NL * pb, "launch_us": 1e3 * ms_prefill,
+        "timed": "CUDA-graph replay of the step's own encode call: one launch of this kernel over the 24 layers",
         "hbm": {"achieved": pb / scan_s / 1e9, "peak": peak, "unit": "GB/s", "frac": pb / scan_s / 1e9 / peak, "peak_source": peak_src,
                 "frac_of_nominal_8000": pb / scan_s / 1e9 / 8000.0},
         "whole_prefill_call": {"us": call_s * 1e6, "achieved": pb / call_s / 1e9, "frac": pb / call_s / 1e9 / peak,
                                "alu_frac": lane_ops / call_s / alu_peak,
                                "summary_pass_us": split[0], "carry_scan_us": split[1], "output_pass_us": split[2],
-                               "timed": "call: CUDA-graph replay of the call over 24 layers, time / 24; per-kernel: CUDA events recorded by the library between the kernels of a call, launched eagerly with the host queued ahead (no overlap between the kernels, event gaps included)"},
+                               "timed": "call: CUDA-graph replay of the call over 24 layers, time / 24; the *_pass_us / carry_scan_us keys: the three kernels of a call for ONE layer (cut into chunks), CUDA events recorded by the library between them, launched eagerly with the host queued ahead (no overlap between the kernels, event gaps included)"},
     }
     tb = w.tree_bytes_per_layer()
     bt_round_bytes = sum(bt.level_bytes(a, b) for a, b in zip(bt.levels[:-1], bt.levels[1:]))
@@ -664,8 +650,8 @@ def run_ours(args):
         "bound": "hbm", "kernel": "tree_step_kernel<bf16>", "workload": "32 sequences x 32-node trees, widest level (%d nodes), 24 layers" % (hi - lo),
         "achieved": NL * bt_wide_bytes / (ms_bt_widest * 1e-3) / 1e9, "peak": peak, "unit": "GB/s",
         "frac": NL * bt_wide_bytes / (ms_bt_widest * 1e-3) / 1e9 / peak, "traffic": ncu_traffic("tree_step_widest_level")[0], "traffic_kernel": ncu_traffic("tree_step_widest_level")[1],
-        "algorithmic_bytes_per_launch": bt_wide_bytes, "launch_us": 1e3 * ms_bt_widest / NL,
-        "timed": "CUDA-graph replay of the level, one launch over 24 layers (distinct 110 MB pools), time / 24",
+        "algorithmic_bytes_per_launch": NL * bt_wide_bytes, "launch_us": 1e3 * ms_bt_widest,
+        "timed": "CUDA-graph replay of the level, one launch over the 24 layers (distinct 110 MB pools)",
         "whole_round": {"ms": ms_bt_round, "levels": [b - a for a, b in zip(bt.levels[:-1], bt.levels[1:])],
                         "node_updates_per_s": world * NL * bt.M / (ms_bt_round * 1e-3),
                         "hbm_frac": NL * bt_round_bytes / (ms_bt_round * 1e-3) / 1e9 / peak},
@@ -686,40 +672,37 @@ def run_ours(args):
         "note": "same workload with the A_POWERS hint withheld: one exponential per (token, channel, state)",
     }
 
-    # ---- context figure: drafting latency per round of a whole 130M-shaped block stack with real data dependence
-    # (split mode: conv step -> torch matmuls for the projections -> S6 step; projection step: one launch that does
-    # all of it; random weights, one CUDA graph per generation step), the quantity of the paper's Table 4.  Not part
-    # of `value`.
+    # ---- context figure: drafting latency per round of a whole 130M-shaped block stack with real data dependence (random
+    # weights, one CUDA graph per generation step), the quantity of the paper's Table 4.  Not part of `value`.  With bf16
+    # weights and levels of at most 64 nodes a generation runs in the library's block kernels whichever mode was asked for;
+    # the modes themselves (split: conv step -> torch matmuls for the projections -> S6 step; projection step: one
+    # launch does all of that) are what other types and wider levels run, and are timed with the block kernels off.
     drafter = None
     if rank == 0 and world == 1:
         from paper_2506_01206_b200.drafter import ToyDrafter
         drafter = {"unit": "ms per draft round (host launches and top-k between generation steps included)",
                    "paper_context": "6.62 (chain of 5) and 8.30 (tree (3,2,2,1,1)) on an RTX 4090, unit unstated, Mamba-130M drafter (paper Table 4)"}
-        for mode, fused in (("split_mode", False), ("projection_step", True)):
+
+        def round_ms(fn):
+            for _ in range(3):
+                fn()
+            torch.cuda.synchronize()
+            ts = []
+            for _ in range(10):
+                t0 = time.perf_counter()
+                fn()
+                torch.cuda.synchronize()
+                ts.append((time.perf_counter() - t0) * 1e3)
+            return statistics.median(ts)
+
+        for mode, fused, block in (("block_kernels", False, True), ("split_mode", False, False), ("projection_step", True, False)):
             td = ToyDrafter(max_nodes=64, seed=0, device=dev, fused=fused)
+            td.block_kernels = td.block_kernels and block
             drafter[mode] = {}
             for name, cfg_t in (("chain_5", (1, 1, 1, 1, 1)), ("tree_3_2_2_1_1", (3, 2, 2, 1, 1))):
-                for _ in range(3):
-                    td.draft_round(11, cfg_t)
-                torch.cuda.synchronize()
-                ts = []
-                for _ in range(10):
-                    t0 = time.perf_counter()
-                    td.draft_round(11, cfg_t)
-                    torch.cuda.synchronize()
-                    ts.append((time.perf_counter() - t0) * 1e3)
-                drafter[mode][name] = statistics.median(ts)
-                if fused:   # the same round as one replayed graph (one host launch per round)
-                    for _ in range(3):
-                        td.draft_round_one_graph(11, cfg_t)
-                    torch.cuda.synchronize()
-                    ts = []
-                    for _ in range(10):
-                        t0 = time.perf_counter()
-                        td.draft_round_one_graph(11, cfg_t)
-                        torch.cuda.synchronize()
-                        ts.append((time.perf_counter() - t0) * 1e3)
-                    drafter.setdefault("projection_step_one_graph_per_round", {})[name] = statistics.median(ts)
+                drafter[mode][name] = round_ms(lambda: td.draft_round(11, cfg_t))
+                if block:   # the same round as one replayed graph (one host launch per round)
+                    drafter.setdefault("block_kernels_one_graph_per_round", {})[name] = round_ms(lambda: td.draft_round_one_graph(11, cfg_t))
             if int(td.status.item()):
                 raise RuntimeError("device status bits set in the drafter leg")
             del td
@@ -770,21 +753,23 @@ def run_ours(args):
 def profile_case(what, sizes):
     """Small, self-contained runs of one kernel family for a profiler (ncu): few launches, well under 1 GB on the device,
     inputs larger than L2 across the layers so that DRAM counters still mean something.
-      prefill [tokens=2048] [layers=4] [reps=3] [fp32=0]   130M-shaped context encode, bf16 (or fp32) activations, structured A
+      prefill [tokens=2048] [layers=4] [reps=3] [fp32=0] [general=0]   130M-shaped context encode layer by layer, bf16 (or fp32) activations
+      stack   [tokens=2048] [layers=24] [reps=3]           the same, all layers in one call
       tree    [layers=4] [reps=2]                          one batched-serving draft round, 32 sequences x 32-node trees
       proj    [nodes=18] [layers=24] [reps=3]              one tree level through the step that forms dt, B, C itself
-      ssd     [tokens=2048] [layers=2] [reps=3]            Mamba-2 (SSD) context encode, 24 heads x 64 channels, 128 states"""
+      ssd     [tokens=2048] [layers=2] [reps=3]            Mamba-2 (SSD) context encode, 24 heads x 64 channels, 128 states
+      generation [nodes=18] [layers=24] [reps=3]           one generation of the drafter's block stack"""
     import torch
     import paper_2506_01206_b200 as md
     from paper_2506_01206_b200.device_inputs import i32, to_device, torch_act, upload_layer
     flags = md.MDRAFT_DT_SOFTPLUS | md.MDRAFT_A_POWERS
     status = torch.zeros(1, dtype=torch.int32, device="cuda")
     if what == "prefill":
-        tokens, n_layers, reps, fp32 = (list(sizes) + [2048, 4, 3, 0][len(sizes):])[:4]
+        tokens, n_layers, reps, fp32, general = (list(sizes) + [2048, 4, 3, 0, 0][len(sizes):])[:5]
         cfg = gen.get_config(1)
         act = "f32" if fp32 else cfg.act
         tdt, D = torch_act(act), cfg.d_inner
-        lays = [upload_layer(gen.layer_params(cfg, l), act, flags) for l in range(n_layers)]
+        lays = [upload_layer(gen.layer_params(cfg, l), act, md.MDRAFT_DT_SOFTPLUS if general else flags) for l in range(n_layers)]
         ins = [[to_device(a, tdt) for a in gen.prefill_inputs(cfg, l, tokens)] for l in range(n_layers)]
         outs = [torch.empty((tokens, D), dtype=tdt, device="cuda") for _ in range(n_layers)]
         cache = md.StateCache(n_layers, 1, D, act=tdt)
@@ -795,6 +780,28 @@ def profile_case(what, sizes):
                 md.mdraft_conv_scan_prefill(lays[l], cache, l, *ins[l], outs[l], None, tokens, None, slot, ws, 0, status)
         torch.cuda.synchronize()
         print("prefill: %d tokens x %d channels, %s, %d layers x %d, status %d" % (tokens, D, act, n_layers, reps, int(status.item())))
+    elif what == "stack":
+        from paper_2506_01206_b200.stack import DrafterStack
+        tokens, n_layers, reps = (list(sizes) + [2048, 24, 3][len(sizes):])[:3]
+        cfg = gen.get_config(1)
+        tdt, D = torch_act(cfg.act), cfg.d_inner
+        st = DrafterStack([upload_layer(gen.layer_params(cfg, l), cfg.act, flags) for l in range(n_layers)], 1, tokens, 1, tokens)
+        ins = [[to_device(a, tdt) for a in gen.prefill_inputs(cfg, l, tokens)] for l in range(n_layers)]
+        outs = [torch.empty((tokens, D), dtype=tdt, device="cuda") for _ in range(n_layers)]
+        for _ in range(reps):
+            st.prefill(ins, outs, None, tokens, None, i32([0]))
+        torch.cuda.synchronize()
+        st.check_status()
+        print("stack: %d tokens x %d channels, %d layers in one call x %d" % (tokens, D, n_layers, reps))
+    elif what == "generation":
+        from paper_2506_01206_b200.drafter import ToyDrafter
+        n_nodes, n_layers, reps = (list(sizes) + [18, 24, 3][len(sizes):])[:3]
+        td = ToyDrafter(n_layers=n_layers, max_nodes=n_nodes)
+        td.node_slot.copy_(i32(list(range(1, n_nodes + 1))))
+        for _ in range(reps):
+            td.generation(0, n_nodes, use_graph=False)
+        torch.cuda.synchronize()
+        print("generation: %d nodes, %d layers x %d, status %d" % (n_nodes, n_layers, reps, int(td.status.item())))
     elif what == "tree":
         n_layers, reps = (list(sizes) + [4, 2][len(sizes):])[:2]
         bt = BatchedTree(seed=0)
@@ -806,9 +813,9 @@ def profile_case(what, sizes):
         cache = md.StateCache(n_layers, bt.S + bt.M, D, act=tdt)
         cache.ssm.normal_()
         par, nod = i32(bt.parent), i32(bt.nodes)
-        for _ in range(reps):
-            for l in range(n_layers):
-                md.mdraft_tree_step(lays[l], cache, l, *ins[l], outs[l], par, nod, bt.levels, status)
+        for _ in range(reps):   # every level of all layers in one launch, as the round runs
+            if not md.mdraft_tree_step_stack(lays, range(n_layers), cache, ins, outs, par, nod, bt.levels, status):
+                raise RuntimeError("the layers did not run side by side")
         torch.cuda.synchronize()
         print("tree: %d nodes, levels %s, %d layers x %d, status %d" % (bt.M, np.diff(bt.levels).tolist(), n_layers, reps, int(status.item())))
     elif what == "ssd":
@@ -855,7 +862,7 @@ def main():
     ap.add_argument("--impl", default="ours", choices=["ours", "reference"])
     ap.add_argument("--no-cpu", action="store_true", help="skip the CPU-oracle baseline leg")
     ap.add_argument("--quick", action="store_true", help="skip the further prefill shapes (long context, packed batch, fp32)")
-    ap.add_argument("--profile-case", choices=["prefill", "tree", "proj", "ssd"], help="run one small kernel case for a profiler and exit")
+    ap.add_argument("--profile-case", choices=["prefill", "stack", "tree", "proj", "ssd", "generation"], help="run one small kernel case for a profiler and exit")
     ap.add_argument("sizes", nargs="*", type=int, help="sizes of the profile case (see profile_case)")
     args = ap.parse_args()
     if args.profile_case:
