@@ -540,7 +540,7 @@ def run_ours(args):
                                    "peak": tf_peak, "frac_issued": flops_issued / (ms_sp * 1e-3) / 1e12 / tf_peak},
                         "token_channels_per_s": T * D / (ms_sp * 1e-3),
                         "note": "HBM binds before the tensor cores at this shape (20.8 MB against 2.9 GFLOP per layer); the kernels are "
-                                "far from either: one 256-thread block per SM walks its phases one after another"},
+                                "far from either: blocks of 256 threads, three to an SM, walk phases that wait for one another"},
             "tree_step": {"bound": "hbm", "kernel": "ssd_step_kernel", "nodes": M, "levels": len(levels) - 1, "us_per_layer_round": ms_st * 1e3,
                           "algorithmic_bytes_per_layer_round": st_bytes, "achieved": st_bytes / (ms_st * 1e-3) / 1e9, "peak": peak_hbm, "unit": "GB/s",
                           "frac": st_bytes / (ms_st * 1e-3) / 1e9 / peak_hbm, "node_updates_per_s": M / (ms_st * 1e-3)},
