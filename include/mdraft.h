@@ -88,7 +88,9 @@ enum {
     MDRAFT_DEV_WAIT_EXPIRED = 4  /* a bounded on-chip wait ran out (results invalid)   */
 };
 
-/* Per-layer constants.  All arrays fp32, device, read-only, caller-owned. */
+/* Per-layer constants.  All arrays fp32, device, read-only, caller-owned.  The context encodes may start while the kernel
+ * ahead of them on the stream is finishing, and read these arrays (not their inputs, states or slots) without waiting for
+ * it: constants that a kernel has just written need a synchronisation, a copy or another kernel in between. */
 typedef struct {
     int32_t d_inner;        /* D */
     int32_t d_state;        /* N, must be 16 */
