@@ -83,3 +83,28 @@ def test_noalloc_prefill_refuses_problems_beyond_its_scratch():
     assert e.value.status == -4
     torch.cuda.synchronize()
     assert float(out.float().min()) == 7.0 and float(out.float().max()) == 7.0, "a refused call must launch nothing"
+
+
+def test_noalloc_prefill_of_a_batch_that_only_fewer_chunks_fit_equals_prefill_with_as_much_workspace():
+    lens = [130] + [9] * 7 + [10] * 12 + [8] * 11 + [24, 0]
+    S, T, Dn = len(lens), sum(lens), 1520
+    prob = parity.make_problem(parity.small_config(Dn, "bf16", S), lens, conv_bias=True, general_A=True)
+    lay, tdt, dev = _device_problem(prob)
+    cu, final = i32(prob.cu), i32(np.arange(S))
+    assert md.mdraft_prefill_workspace_bytes(lay, T, S, max(lens)) > md.NOALLOC_SCRATCH_BYTES
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    res = []
+    for scratch in (torch.empty(md.NOALLOC_SCRATCH_BYTES, dtype=torch.uint8, device="cuda"), None):
+        cache, out = md.StateCache(1, S, Dn, act=tdt), torch.full((T, Dn), float("nan"), dtype=tdt, device="cuda")
+        if scratch is None:
+            md.mdraft_conv_scan_prefill_noalloc(lay, cache, 0, *dev, out, cu, max(lens), None, final, 0, status)
+        else:
+            md.mdraft_conv_scan_prefill(lay, cache, 0, *dev, out, cu, max(lens), None, final, scratch, 0, status)
+        torch.cuda.synchronize()
+        res.append((out, cache.ssm, cache.conv))
+    assert int(status.item()) == 0
+    for a, b in zip(*res):
+        assert torch.equal(a, b)
+    o_out, _, o_h = oracle.prefill(oracle.layer_from_params(prob.params), prob.x, prob.z, prob.dt, prob.B, prob.C, prob.cu)
+    assert_close(res[1][0].float().cpu().numpy(), o_out, TOL["bf16"], "out against the oracle")
+    assert_close(res[1][1][0].cpu().numpy(), o_h, TOL_STATE, "SSM state against the oracle")
