@@ -11,6 +11,7 @@
 #include "commit.cuh"
 #include "common.cuh"
 #include "prefill.cuh"
+#include "prefill_cluster.cuh"
 #include "ssd.cuh"
 #include "tree_proj.cuh"
 #include "tree_step.cuh"
@@ -411,6 +412,59 @@ int run_prefill(const PrefillCall& call, const PrefillPlan& pl, int32_t n_layers
     return launch_prefill<ML>(b, act, pl.form, call.stream) == cudaSuccess ? MDRAFT_OK : MDRAFT_ERR_CUDA;
 }
 
+// The one-kernel form (csrc/prefill_cluster.cu) of a call, or blocks = 0 where the plan above is the faster one.  Measured over 900 calls of 1 to
+// 16 layers, 1 to 8 sequences of 10 to 4000 tokens, 64 to 1536 channels, fp32 and bf16, either A, under 17 forms each:
+//  - the one-kernel form takes kOne us and so much per block of a cluster, and per token of a chunk kLatency us plus kShare for every
+//    further warp on a scheduler (standard deviation 7 %);
+//  - the other takes kSplit + kSplitWork per token of work of a scheduler where it cuts sequences, kWhole + kWholeToken per token
+//    of the longest where it does not (15 %), so the one-kernel form has to promise 12 % less.
+// It wins where the work is small: 256 x 64 fp32 9.2 -> 6.4 us, 256 x 768 bf16 12.3 -> 8.1, 1024 x 128 to 256 0.76 of the time; in the mean over
+// those calls 16 % (12 of them lose 3 % or more).  It loses where the work fills the machine, since its clusters leave a seventh of the SMs out and
+// its channel groups are narrow: 1777 x 1536, general A, 35.5 against 41.4 at best, 4096 x 1536 52 against 77.
+ClusterForm cluster_form(const mdraft_layer* L, int n_layers, int T, int n_seq, int max_seqlen, const mdraft_prefill_opts* opts) {
+    if (one_at_a_time(L) || (opts && (opts->chunk_len > 0 || opts->block_channels || opts->event_after_chunk_state || opts->event_after_carry_scan))) return {0, 0};
+    constexpr double kOne = 4.1, kCluster = 0.6, kBlock = 0.13, kWarp = 0.15, kLatency[2] = {0.195, 0.275}, kShare[2] = {0.112, 0.167};
+    constexpr double kSplit = 11.1, kSplitSeqs = 0.7, kSplitWork[2] = {0.166, 0.239}, kWhole = 3.3, kWholeToken = 0.104, kMargin = 0.88;
+    const int general = !(L->flags & MDRAFT_A_POWERS), sms = sm_count();
+    const int64_t groups = (int64_t)n_layers * ((L->d_inner + kClusterCols - 1) / kClusterCols), clusters = groups * n_seq;
+    if (clusters > 8 * sms || (L->d_inner + kClusterCols - 1) / kClusterCols > 65535 || (int64_t)n_layers * n_seq > 65535) return {0, 0};
+    ClusterForm best = {0, 0};
+    double least = kSplit + (double)T * groups / (4 * sms) * kSplitWork[general] + (n_seq > 1 ? kSplitSeqs : 0.0);
+    const double blocks = (double)n_layers * n_seq * ((L->d_inner + kPrefillThreads - 1) / kPrefillThreads), rounds = 1.2 * blocks / sms;
+    const double whole = kWhole + max_seqlen * kWholeToken * (general ? kGeneralOne : 1.0) * (rounds > 1.0 ? rounds : 1.0);
+    least = kMargin * (whole < least ? whole : least);
+    auto weigh = [&](int c, int w) {
+        const int share = prefill_cluster_share(c, clusters);
+        if (share * w > 16) return;   // the warps of an SM, 128 registers a thread
+        const double busy = share * w > 4 ? share * w / 4.0 - 1.0 : 0.0;   // further warps on the fullest scheduler
+        const double t = kOne + (c > 1 ? kCluster : 0.0) + kBlock * c + kWarp * busy + prefill_cluster_chunk(max_seqlen, c * w, !general) * (kLatency[general] + kShare[general] * busy);
+        if (t < least) { least = t; best = {c, w}; }
+    };
+    weigh(1, 2);
+    for (int w = 4; w <= kClusterMaxWarps; w *= 2)
+        for (int c = 1; c <= kClusterMaxBlocks; ++c) weigh(c, w);
+    return best;
+}
+
+template <int ML>
+int run_prefill_cluster(const PrefillCall& call, const ClusterForm& form, int32_t n_layers, const mdraft_layer* layers, const int32_t* layer_index, const mdraft_io* io) {
+    ClusterBatch<ML> b;
+    ClusterArgs& a = b.c;
+    a.pool = PoolDev{};
+    a.ssm_layer_stride = a.conv_layer_stride = 0;
+    if (call.cache) {
+        a.pool = pool_dev(call.cache, layers->act, 0);
+        a.ssm_layer_stride = call.cache->ssm_layer_stride; a.conv_layer_stride = call.cache->conv_layer_stride;
+    }
+    a.n_layers = n_layers; a.d_inner = layers->d_inner; a.T = call.total_tokens; a.n_seq = call.n_seq;
+    a.cu = call.cu_seqlens; a.init_slot = call.init_slot; a.final_slot = call.final_slot; a.dev_status = call.dev_status;
+    for (int32_t i = 0; i < n_layers; ++i) {
+        const mdraft_io& v = io[i];
+        b.l[i] = {layer_dev(layers + i), layer_index[i], v.x, v.z, v.dt, v.B, v.C, v.out, v.ldx, v.ldz, v.lddt, v.ldb, v.ldc, v.ldo};
+    }
+    return launch_prefill_cluster<ML>(b, layers->act, form, call.stream) == cudaSuccess ? MDRAFT_OK : MDRAFT_ERR_CUDA;
+}
+
 __global__ void classify_A_kernel(const float* A, int D, int N, int32_t* res) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= D * N) return;
@@ -470,7 +524,8 @@ int32_t mdraft_prefill_stack_launches(const mdraft_layer* layer, int32_t n_layer
     if (max_seqlen > total_tokens) max_seqlen = total_tokens;
     int32_t n = 0;
     for_each_prefill_run(layer, n_layers, n_seq, [&](int32_t nl, int32_t times) {
-        n += times * (!plan_prefill(layer, nl, total_tokens, n_seq, max_seqlen, opts, kAnyWorkspace).form.chunked ? 1 : (layer->flags & MDRAFT_CONV_ONLY) ? 2 : 3);
+        const bool one = cluster_form(layer, nl, total_tokens, n_seq, max_seqlen, opts).blocks > 0 || !plan_prefill(layer, nl, total_tokens, n_seq, max_seqlen, opts, kAnyWorkspace).form.chunked;
+        n += times * (one ? 1 : (layer->flags & MDRAFT_CONV_ONLY) ? 2 : 3);
     });
     return n;
 }
@@ -528,6 +583,10 @@ int mdraft_conv_scan_prefill_stack(int32_t n_layers, const mdraft_layer* layers,
                     if (!workspace || workspace_bytes < pl.bytes) return MDRAFT_ERR_WORKSPACE;
                     if (reinterpret_cast<uintptr_t>(workspace) & 255u) return MDRAFT_ERR_MISALIGNED;
                 }
+            } else if (const ClusterForm cf = cluster_form(layers + l0, nl, plan_tokens, n_seq, max_seqlen, opts); cf.blocks > 0) {
+                const int r = nl == 1 ? run_prefill_cluster<1>(call, cf, nl, layers + l0, layer_index + l0, io + l0)
+                                      : run_prefill_cluster<kClusterMaxLayers>(call, cf, nl, layers + l0, layer_index + l0, io + l0);
+                if (r) return r;
             } else {
                 const int r = nl == 1 ? run_prefill<1>(call, pl, nl, layers + l0, layer_index + l0, io + l0)
                                       : run_prefill<kPrefillMaxLayers>(call, pl, nl, layers + l0, layer_index + l0, io + l0);

@@ -1,0 +1,80 @@
+"""The one-kernel form of the context encode (the chunks of a sequence are the warps of a thread-block cluster), where the default
+plan takes it: against the fp64 oracle, and against the three-kernel form of the same call.
+
+Tolerances: those of the other encodes (tests/parity.py).  The two forms differ by where they cut a sequence, and across a cut a state
+decays by the exponential of the summed step sizes instead of a product of one per token.  A token's factor for A = -n is good to n 2^-22
+(powers of one approximate exponential, whose error has the same sign in all of them) and some 1 / (n Delta) = 100 / n tokens count, so the two
+may be 100 * 2^-22 = 2.4e-5 apart; the largest of some 10^5 elements, taken relative to its value or the RMS, lies up to four times that
+out: 1e-4.  bf16 outputs are besides rounded once each, 2^-8 of the value at most apart when a tie falls, with the RMS floor 2^-7."""
+
+import numpy as np
+import pytest
+import torch
+
+import parity
+from parity import TOL, TOL_STATE, assert_close
+from test_gpu_parity_small import random_state, run_gpu_prefill, run_oracle_prefill
+
+pytestmark = pytest.mark.gpu
+
+import paper_2506_01206_b200 as md
+from paper_2506_01206_b200.device_inputs import i32, to_device, torch_act, upload_layer
+
+TOL_FORMS = 1e-4
+
+SHAPES = [   # act, D, lengths
+    ("f32", 8, [1]), ("bf16", 8, [3]), ("bf16", 32, [64]), ("f32", 64, [256]), ("bf16", 40, [65, 1, 0, 4, 257]), ("f32", 200, [33, 500]),
+    ("bf16", 768, [256]), ("bf16", 1536, [130]), ("f32", 1000, [17, 90]), ("bf16", 72, [511]), ("f32", 24, [2, 0, 1, 500]), ("bf16", 1496, [31, 32, 33])]
+
+
+@pytest.mark.parametrize("act,Dn,lens", SHAPES)
+@pytest.mark.parametrize("general_A", [False, True])
+def test_one_kernel_form_matches_oracle_and_the_general_form(act, Dn, lens, general_A):
+    cfg = parity.small_config(Dn, act, len(lens), cid=97)
+    prob = parity.make_problem(cfg, lens, conv_bias=True, general_A=general_A)
+    flags = md.MDRAFT_DT_SOFTPLUS | (0 if general_A else md.MDRAFT_A_POWERS)
+    lay = upload_layer(prob.params, act, flags)
+    assert md.mdraft_prefill_stack_launches(lay, 1, sum(lens), len(lens), max(lens)) == 1
+    ci, hi = random_state(cfg, len(lens), 7)
+    for init, strided, in_place in ((False, False, False), (True, True, False), (True, False, True)):
+        state = (ci, hi) if init else (None, None)
+        got = run_gpu_prefill(prob, flags, 0, *state, in_place=in_place, strided=strided)
+        o_out, o_conv, o_h = run_oracle_prefill(prob, flags, *state)
+        assert_close(got[0], o_out, TOL[act], "out")
+        assert_close(got[2], o_h, TOL_STATE, "final SSM state")
+        assert np.array_equal(got[1], o_conv)
+        other = run_gpu_prefill(prob, flags, 32, *state, in_place=in_place, strided=strided)
+        assert_close(got[0], other[0], TOL_FORMS if act == "f32" else 2 ** -7, "out, other form")
+        assert_close(got[2], other[2], TOL_FORMS, "state, other form")
+        assert np.array_equal(got[1], other[1])
+
+
+@pytest.mark.parametrize("act", ["f32", "bf16"])
+def test_one_kernel_form_of_a_stack_and_its_faults(act):
+    """Several layers in one launch; a sequence with a slot out of range and one with malformed offsets are left out alone."""
+    lens, Dn, NL = [50, 70, 20], 136, 3
+    tdt = torch_act(act)
+    probs = [parity.make_problem(parity.small_config(Dn, act, 3, cid=70 + l), lens) for l in range(NL)]
+    flags = md.MDRAFT_DT_SOFTPLUS | md.MDRAFT_A_POWERS
+    lays = [upload_layer(p.params, act, flags) for p in probs]
+    assert md.mdraft_prefill_stack_launches(lays[0], NL, sum(lens), 3, max(lens)) == 1
+    cache = md.StateCache(NL, 3, Dn, act=tdt)
+    cache.ssm.fill_(5.0)
+    out = torch.full((NL, sum(lens), Dn), 9.0, dtype=tdt, device="cuda")
+    ins = [tuple(to_device(a, tdt) for a in (p.x, p.z, p.dt, p.B, p.C)) for p in probs]
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    ws = torch.empty(max(256, md.mdraft_prefill_stack_workspace_bytes(lays[0], NL, sum(lens), 3, max(lens))), dtype=torch.uint8, device="cuda")
+    assert md.mdraft_conv_scan_prefill_stack(lays, range(NL), cache, ins, list(out), i32([0, 50, 120, 140]), max(lens), None, i32([0, 7, 2]), ws, status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == md.MDRAFT_DEV_BAD_SLOT
+    assert bool((out[:, 50:120] == 9.0).all()) and bool((cache.ssm[:, 1] == 5.0).all())
+    for l, p in enumerate(probs):
+        o_out, _, o_h = run_oracle_prefill(p, flags)
+        for s, (a, b) in ((0, (0, 50)), (2, (120, 140))):
+            assert_close(out[l, a:b].float().cpu().numpy(), o_out[a:b], TOL[act], f"layer {l} sequence {s}")
+            assert_close(cache.ssm[l, s].cpu().numpy(), o_h[s], TOL_STATE, f"layer {l} state {s}")
+    status.zero_(); out.fill_(9.0)
+    assert md.mdraft_conv_scan_prefill_stack(lays, range(NL), cache, ins, list(out), i32([0, 50, 200, 140]), max(lens), None, i32([0, 1, 2]), ws, status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == md.MDRAFT_DEV_BAD_SEQLENS
+    assert not bool((out[:, :50] == 9.0).all()) and bool((out[:, 50:] == 9.0).all())
