@@ -68,11 +68,13 @@ __global__ void __launch_bounds__(kTB) tree_step_kernel(const TreeArgs c, const 
     // Launched the ordinary way nothing runs ahead of this kernel: the wait costs nothing, and passing it first lets
     // every copy be requested at once.
     if (ordinary_launch) asm volatile("griddepcontrol.wait;" ::: "memory");
-    const TreeLayer& p = layers.l[ML == 1 ? 0 : blockIdx.z];
+    // Blocks start in grid order, so a level leaves its last layers' states in L2; every other level begins with those.
+    const bool flip = c.level_in_call & 1;
+    const TreeLayer& p = layers.l[ML == 1 ? 0 : flip ? gridDim.z - 1 - blockIdx.z : blockIdx.z];
     const int D = p.L.d_inner;
     const int node = c.lvl_begin + blockIdx.x;
     const int tid = threadIdx.x;
-    const int d0 = blockIdx.y * kTB;
+    const int d0 = (flip ? gridDim.y - 1 - blockIdx.y : blockIdx.y) * kTB;
     const int cols = min(kTB, D - d0);
     const int d = d0 + tid;
     const bool live = tid < cols;
