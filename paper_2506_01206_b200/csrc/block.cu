@@ -88,41 +88,38 @@ __device__ __forceinline__ void load_w(WFrag<kColTiles>& w, uint32_t w_rows, int
         ldmatrix_x4_trans(w.v[j][1], at + 16 * pitch);
     }
 }
-// acc += W^T a for the first `tiles` groups of 8 nodes.
-template <int kColTiles>
-__device__ __forceinline__ void multiply(float (&acc)[kColTiles][kNodeTiles][4], const WFrag<kColTiles>& w, const uint4 (&a)[kNodeTiles], int tiles) {
+// acc += W^T a for TILES groups of 8 nodes.
+template <int kColTiles, int TILES>
+__device__ __forceinline__ void multiply(float (&acc)[kColTiles][TILES][4], const WFrag<kColTiles>& w, const uint4 (&a)[TILES]) {
 #pragma unroll
-    for (int i = 0; i < kNodeTiles; ++i) {
-        if (i < tiles) {
+    for (int i = 0; i < TILES; ++i)
 #pragma unroll
-            for (int j = 0; j < kColTiles; ++j) {
-                mma16816(acc[j][i], w.v[j][0][0], w.v[j][0][1], w.v[j][0][2], w.v[j][0][3], a[i].x, a[i].y);
-                mma16816(acc[j][i], w.v[j][1][0], w.v[j][1][1], w.v[j][1][2], w.v[j][1][3], a[i].z, a[i].w);
-            }
+        for (int j = 0; j < kColTiles; ++j) {
+            mma16816(acc[j][i], w.v[j][0][0], w.v[j][0][1], w.v[j][0][2], w.v[j][0][3], a[i].x, a[i].y);
+            mma16816(acc[j][i], w.v[j][1][0], w.v[j][1][1], w.v[j][1][2], w.v[j][1][3], a[i].z, a[i].w);
         }
-    }
 }
 __device__ __forceinline__ float squares(const uint4& v, float acc) { return square_pair(v.w, square_pair(v.z, square_pair(v.y, square_pair(v.x, acc)))); }
 // A warp's share of the nodes' sums of squares, and of the block's result, into shared memory.
-__device__ __forceinline__ void put_squares(float* s_sq, const float (&sq)[kNodeTiles], int g, int t) {
+template <int TILES>
+__device__ __forceinline__ void put_squares(float* s_sq, const float (&sq)[TILES], int g, int t) {
 #pragma unroll
-    for (int i = 0; i < kNodeTiles; ++i) {
+    for (int i = 0; i < TILES; ++i) {
         float v = sq[i];
         v += __shfl_xor_sync(0xffffffffu, v, 1);
         v += __shfl_xor_sync(0xffffffffu, v, 2);
         if (t == 0) s_sq[i * 8 + g] = v;
     }
 }
-template <int kColTiles>
-__device__ __forceinline__ void put_part(float* part, const float (&acc)[kColTiles][kNodeTiles][4], int tiles, int g, int t) {
+template <int kColTiles, int TILES>
+__device__ __forceinline__ void put_part(float* part, const float (&acc)[kColTiles][TILES][4], int g, int t) {
     constexpr int kPitch = part_pitch(kColTiles * 16);
 #pragma unroll
-    for (int i = 0; i < kNodeTiles; ++i)
-        if (i < tiles)
+    for (int i = 0; i < TILES; ++i)
 #pragma unroll
-            for (int j = 0; j < kColTiles; ++j)
+        for (int j = 0; j < kColTiles; ++j)
 #pragma unroll
-                for (int e = 0; e < 4; ++e) part[(i * 8 + 2 * t + (e & 1)) * kPitch + j * 16 + (e >> 1) * 8 + g] = acc[j][i][e];
+            for (int e = 0; e < 4; ++e) part[(i * 8 + 2 * t + (e & 1)) * kPitch + j * 16 + (e >> 1) * 8 + g] = acc[j][i][e];
 }
 // The warps' shares added up in order, normalised, added to (add0: what the thread's first pair is added to), rounded, stored.
 template <int NT, int NW, bool NORM>
@@ -156,15 +153,15 @@ __host__ __device__ inline int rows_offset(int k, int nt, int nw) {   // W or th
     return ((w > part ? w : part) + 127) / 128 * 128;
 }
 
-// PRE: blocks of the contraction whose fragments of W a warp takes into registers before the wait.
-template <int NT, int NW, int PRE, bool NORM>
+// PRE: blocks of the contraction whose fragments of W a warp takes into registers before the wait.  TILES: groups of 8 nodes a block may have.
+template <int NT, int NW, int PRE, bool NORM, int TILES>
 __global__ void __launch_bounds__(NW * 32, PRE > 0 ? 0 : 2) small_linear_kernel(const SmallLinear p) {
     constexpr int kCols = NT / 16, kPitch = w_pitch(NT);
     extern __shared__ __align__(128) unsigned char s_w[];   // W as [k][NT], later the warps' partial results [NW][kRows][NT]; then the activations
     __shared__ float s_sq[NW][kRows];
     __shared__ __align__(8) uint64_t bar;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
-    const int n0 = blockIdx.x * NT, m0 = blockIdx.y * kRows, rows = min(kRows, p.m - m0), tiles = (rows + 7) / 8;
+    const int n0 = blockIdx.x * NT, m0 = blockIdx.y * kRows, rows = min(kRows, p.m - m0);
     grid_release_dependents();
     if (threadIdx.x == 0) {
         mbar_init(&bar, 1);
@@ -203,11 +200,11 @@ __global__ void __launch_bounds__(NW * 32, PRE > 0 ? 0 : 2) small_linear_kernel(
     }
     const bool ok = mbar_wait_bounded(&bar, 0u);
 
-    float acc[kCols][kNodeTiles][4] = {};
-    float sq[kNodeTiles] = {};
-    auto load_a = [&](uint4 (&a)[kNodeTiles], int kb) {
+    float acc[kCols][TILES][4] = {};
+    float sq[TILES] = {};
+    auto load_a = [&](uint4 (&a)[TILES], int kb) {
 #pragma unroll
-        for (int i = 0; i < kNodeTiles; ++i) {
+        for (int i = 0; i < TILES; ++i) {
             a[i] = make_uint4(0u, 0u, 0u, 0u);
             if (i * 8 + g < rows) a[i] = *reinterpret_cast<const uint4*>(s_a + (i * 8 + g) * p.k * 2 + kb * 64 + t * 16);
             if (NORM) sq[i] = squares(a[i], sq[i]);
@@ -216,21 +213,21 @@ __global__ void __launch_bounds__(NW * 32, PRE > 0 ? 0 : 2) small_linear_kernel(
 #pragma unroll
     for (int q = 0; q < PRE; ++q)
         if (warp + q * NW < kblocks) {
-            uint4 a[kNodeTiles];
+            uint4 a[TILES];
             load_a(a, warp + q * NW);
-            multiply<kCols>(acc, w[q], a, tiles);
+            multiply(acc, w[q], a);
         }
 #pragma unroll 1
     for (int kb = warp + PRE * NW; kb < kblocks; kb += NW) {
-        uint4 a[kNodeTiles];
+        uint4 a[TILES];
         load_a(a, kb);
         load_w<kCols>(w[0], smem_u32(s_w) + (uint32_t)(kb * 32 * kPitch), kPitch, lane);
-        multiply<kCols>(acc, w[0], a, tiles);
+        multiply(acc, w[0], a);
     }
     if (NORM) put_squares(s_sq[warp], sq, g, t);
     const bool all_ok = !__syncthreads_or(!ok);   // and nobody reads W any more
     float* const part = reinterpret_cast<float*>(s_w);
-    put_part<kCols>(part + warp * kRows * part_pitch(NT), acc, tiles, g, t);
+    put_part(part + warp * kRows * part_pitch(NT), acc, g, t);
     __syncthreads();
     if (all_ok) {
         finish<NT, NW, NORM>(p, part, s_sq, rows, m0, n0, add0);
@@ -245,12 +242,13 @@ __global__ void __launch_bounds__(NW * 32, PRE > 0 ? 0 : 2) small_linear_kernel(
 // one.  A warp's share of the contraction stays the same from tile to tile, so its activations stay in registers.
 constexpr int kWideNT = 32, kWideWarps = 8, kWideStages = 3, kWideBlocks = 4;   // kWideBlocks: blocks of 32 of the contraction a warp may hold
 
+template <int TILES>
 __global__ void __launch_bounds__(kWideWarps * 32, 1) wide_linear_kernel(const SmallLinear p) {
     constexpr int NW = kWideWarps, NT = kWideNT, kCols = NT / 16, kPitch = w_pitch(NT);
     extern __shared__ __align__(128) unsigned char s_w[];   // [kWideStages][k][NT], then the warps' partial results [NW][kRows][NT]
     __shared__ float s_sq[NW][kRows];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
-    const int m0 = blockIdx.y * kRows, rows = min(kRows, p.m - m0), node_tiles = (rows + 7) / 8;
+    const int m0 = blockIdx.y * kRows, rows = min(kRows, p.m - m0);
     const int kblocks = p.k / 32, tiles = (p.n + NT - 1) / NT, stage_bytes = p.k * kPitch;
     float* const part = reinterpret_cast<float*>(s_w + kWideStages * stage_bytes);
     grid_release_dependents();
@@ -272,12 +270,12 @@ __global__ void __launch_bounds__(kWideWarps * 32, 1) wide_linear_kernel(const S
 #pragma unroll
     for (int s = 0; s < kWideStages - 1; ++s) fetch(blockIdx.x + s * step, s);
     grid_wait();
-    uint4 a[kWideBlocks][kNodeTiles];
-    float sq[kNodeTiles] = {};
+    uint4 a[kWideBlocks][TILES];
+    float sq[TILES] = {};
 #pragma unroll
     for (int q = 0; q < kWideBlocks; ++q)
 #pragma unroll
-        for (int i = 0; i < kNodeTiles; ++i) {
+        for (int i = 0; i < TILES; ++i) {
             const int kb = warp + q * NW, row = i * 8 + g;
             a[q][i] = make_uint4(0u, 0u, 0u, 0u);
             if (kb < kblocks && row < rows) a[q][i] = *reinterpret_cast<const uint4*>(p.a + (size_t)(m0 + row) * p.k + kb * 32 + t * 8);
@@ -285,20 +283,20 @@ __global__ void __launch_bounds__(kWideWarps * 32, 1) wide_linear_kernel(const S
 #pragma unroll
     for (int q = 0; q < kWideBlocks; ++q)
 #pragma unroll
-        for (int i = 0; i < kNodeTiles; ++i) sq[i] = squares(a[q][i], sq[i]);
+        for (int i = 0; i < TILES; ++i) sq[i] = squares(a[q][i], sq[i]);
     put_squares(s_sq[warp], sq, g, t);
     int stage = 0;
     for (int tile = blockIdx.x; tile < tiles; tile += step) {
         asm volatile("cp.async.wait_group %0;" ::"n"(kWideStages - 2) : "memory");
         __syncwarp();
-        float acc[kCols][kNodeTiles][4] = {};
+        float acc[kCols][TILES][4] = {};
 #pragma unroll
         for (int q = 0; q < kWideBlocks; ++q) {
             const int kb = warp + q * NW;
             if (kb < kblocks) {
                 WFrag<kCols> w;
                 load_w<kCols>(w, smem_u32(s_w) + (uint32_t)(stage * stage_bytes + kb * 32 * kPitch), kPitch, lane);
-                multiply<kCols>(acc, w, a[q], node_tiles);
+                multiply(acc, w, a[q]);
             }
         }
         __syncwarp();
@@ -306,7 +304,7 @@ __global__ void __launch_bounds__(kWideWarps * 32, 1) wide_linear_kernel(const S
         fetch(tile + (kWideStages - 1) * step, ahead >= kWideStages ? ahead - kWideStages : ahead);
         if (++stage == kWideStages) stage = 0;
         __syncthreads();   // the partial results of the tile before have been read
-        put_part<kCols>(part + warp * kRows * part_pitch(NT), acc, node_tiles, g, t);
+        put_part(part + warp * kRows * part_pitch(NT), acc, g, t);
         __syncthreads();
         finish<NT, NW, true>(p, part, s_sq, rows, m0, tile * NT, __nv_bfloat162());
     }
@@ -323,11 +321,12 @@ __global__ void embed_kernel(const int64_t* tokens, const __nv_bfloat16* embed, 
 }
 
 constexpr int kMaxSmem = 224 * 1024;   // beside up to 2 KB of static shared memory
+constexpr int kSmemAlone = 116 * 1024; // more than half of an SM's
 
 template <auto kKernel>
 cudaError_t launch_chained(dim3 grid, int threads, int smem, const SmallLinear& p, cudaStream_t st) {
     if (smem > kMaxSmem) return cudaErrorInvalidValue;
-    const cudaError_t e = allow_smem<kKernel>(kMaxSmem);
+    const cudaError_t e = allow_smem<kKernel>(kMaxSmem, true);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
@@ -342,32 +341,59 @@ cudaError_t launch_chained(dim3 grid, int threads, int smem, const SmallLinear& 
     return cudaLaunchKernelEx(&cfg, kKernel, p);
 }
 
+template <int NT, int NW, int PRE, bool NORM, int TILES>
+cudaError_t launch_tiles(const SmallLinear& p, cudaStream_t st) {
+    const int rows = p.m < kRows ? p.m : kRows, need = rows_offset(p.k, NT, NW) + rows * p.k * 2;
+    return launch_chained<small_linear_kernel<NT, NW, PRE, NORM, TILES>>(dim3((p.n + NT - 1) / NT, (p.m + kRows - 1) / kRows), NW * 32,
+                                                                      p.alone && need < kSmemAlone ? kSmemAlone : need, p, st);
+}
+// A kernel for each number of node groups in one row tile, with the fragments of W ahead of the wait; one without them for two row tiles.
 template <int NT, int NW, int PRE, bool NORM>
 cudaError_t launch_tile(const SmallLinear& p, cudaStream_t st) {
-    const int rows = p.m < kRows ? p.m : kRows;
-    return launch_chained<small_linear_kernel<NT, NW, PRE, NORM>>(dim3((p.n + NT - 1) / NT, (p.m + kRows - 1) / kRows), NW * 32,
-                                                             rows_offset(p.k, NT, NW) + rows * p.k * 2, p, st);
+    switch (p.m <= kRows ? (p.m + 7) / 8 : 0) {
+        case 1: return launch_tiles<NT, NW, PRE, NORM, 1>(p, st);
+        case 2: return launch_tiles<NT, NW, PRE, NORM, 2>(p, st);
+        case 3: return launch_tiles<NT, NW, PRE, NORM, 3>(p, st);
+        case 4: return launch_tiles<NT, NW, PRE, NORM, 4>(p, st);
+        default: return launch_tiles<NT, NW, 0, NORM, kNodeTiles>(p, st);
+    }
 }
 
 }  // namespace
 
+// The kernels of the chain overlap: a product's blocks start wherever there is room, long before their turn, and fetch weights.  Where they gather
+// on a few SMs - two in_proj blocks, or one beside out_proj's - the chain waits for those.  With shared memory asked for so that in_proj's
+// blocks keep off one another, and from five nodes on off out_proj's, a generation of 1 / 4 / 8 / 16 / 18 / 24 / 32 nodes takes
+// 190 / 210 / 230 / 254 / 276 / 308 / 335 us; without 224 / 242 / 246 / 280 / 306 / 320 / 336.  Up to four nodes the two products'
+// blocks are better beside each other (apart 203 / 221 us).  Only where one wave holds them all.
+void keep_products_apart(int d_model, int d_inner, int n_nodes, bool& in_proj, bool& out_proj) {
+    const int sms = sm_count(), tile = 2 * d_inner <= 16 * sms ? 16 : 32, blocks = (2 * d_inner + tile - 1) / tile + (d_model + 15) / 16;
+    in_proj = n_nodes <= kRows && blocks <= sms;
+    out_proj = in_proj && n_nodes > 4;
+}
+
 cudaError_t launch_small_linear(const SmallLinear& p, cudaStream_t st) {
     const int sms = sm_count();
-    const bool one_tile = p.m <= kRows;
     // out_proj (the only product that is added to something and not normalised) has at most kBlockMaxModel columns: few blocks even
     // of the narrow tile.
     // Fragments of W in registers ahead of the wait while one row tile leaves room for the kernels of the chain beside each
     // other (18 nodes: 329 -> 304 us a generation); with two, the registers they take cost more (64 nodes: 486 -> 534 us).
-    if (p.eps < 0.0f) return one_tile ? launch_tile<16, 12, 4, false>(p, st) : launch_tile<16, 12, 0, false>(p, st);
+    if (p.eps < 0.0f) return launch_tile<16, 12, 4, false>(p, st);
     // Beyond one wave of 32-column tiles the persistent form, where the contraction fits its registers and shared memory.
     const int smem = kWideStages * p.k * w_pitch(kWideNT) + kWideWarps * kRows * part_pitch(kWideNT) * 4;
     if (p.n > 32 * sms && p.k <= kWideWarps * kWideBlocks * 32 && smem <= kMaxSmem) {
         const int tiles = (p.n + kWideNT - 1) / kWideNT, mt = (p.m + kRows - 1) / kRows, per_row = sms / mt;
-        return launch_chained<wide_linear_kernel>(dim3(tiles < per_row ? tiles : per_row, mt), kWideWarps * 32, smem, p, st);
+        const dim3 grid(tiles < per_row ? tiles : per_row, mt);
+        switch (mt > 1 ? kNodeTiles : (p.m + 7) / 8) {
+            case 1: return launch_chained<wide_linear_kernel<1>>(grid, kWideWarps * 32, smem, p, st);
+            case 2: return launch_chained<wide_linear_kernel<2>>(grid, kWideWarps * 32, smem, p, st);
+            case 3: return launch_chained<wide_linear_kernel<3>>(grid, kWideWarps * 32, smem, p, st);
+            default: return launch_chained<wide_linear_kernel<kNodeTiles>>(grid, kWideWarps * 32, smem, p, st);
+        }
     }
     // The narrow tile for a narrow n, whose blocks are few.
-    if (p.n <= 16 * sms) return one_tile ? launch_tile<16, 12, 4, true>(p, st) : launch_tile<16, 12, 0, true>(p, st);
-    return one_tile ? launch_tile<32, 12, 2, true>(p, st) : launch_tile<32, 12, 0, true>(p, st);
+    if (p.n <= 16 * sms) return launch_tile<16, 12, 4, true>(p, st);
+    return launch_tile<32, 12, 2, true>(p, st);
 }
 
 cudaError_t launch_embed(const int64_t* tokens, const __nv_bfloat16* embed, __nv_bfloat16* h, int m, int d, int vocab, int32_t* dev_status, cudaStream_t st) {

@@ -531,7 +531,7 @@ cudaError_t launch_nt(const TreeProjArgs& p, int n_blocks, cudaStream_t st) {
     at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.numAttrs = p.chained ? 2 : 1;
     const bool pow = p.L.flags & MDRAFT_A_POWERS;
-    const cudaError_t e = pow ? allow_smem<tree_proj_kernel<AT, CB, NT, true>>(kSmem) : allow_smem<tree_proj_kernel<AT, CB, NT, false>>(kSmem);
+    const cudaError_t e = pow ? allow_smem<tree_proj_kernel<AT, CB, NT, true>>(kSmem, true) : allow_smem<tree_proj_kernel<AT, CB, NT, false>>(kSmem, true);
     if (e != cudaSuccess) return e;
     return cudaLaunchKernelEx(&cfg, pow ? tree_proj_kernel<AT, CB, NT, true> : tree_proj_kernel<AT, CB, NT, false>, p);
 }
