@@ -418,6 +418,9 @@ __global__ void __launch_bounds__(SUB * kBoxCols + 32, PER_SM) chunk_kernel(cons
 // warp g takes kCarryPer consecutive chunks: it loads their summaries at once, folds them into one (P, q) pair,
 // publishes the pair, folds the pairs of the warps before it into its starting state, and then replays its own
 // chunks to write the state after each.  Rounds carry the running state forward past 48 chunks.
+// Registers count beyond the kernel itself: its blocks and the output pass's start as the summary pass leaves SMs, beside one another.  The
+// decays are formed twice instead of kept: 126 -> 104 registers, 1777 x 1536 (general A) 35.5 -> 35.1 us, three sequences of 700 to 1400 x
+// 1000 in fp32 46.3 -> 45.3.  (Held down to 64 or 48 registers it spills and loses 4 us; 10 to 16 warps of 3 or 4 chunks lose 0.5 to 3.)
 constexpr int kCarryGroups = 8, kCarryPer = 6;
 
 __device__ __forceinline__ float4 fold4(const float4& a, const float4& h, const float4& q) {
@@ -460,34 +463,39 @@ __global__ void __launch_bounds__(kCarryGroups * 32) carry_kernel(const __grid_c
     for (int base = 0; base < nsum; base += kCarryGroups * kCarryPer) {
         const int c0 = base + g * kCarryPer;
         const int cnt = min(kCarryPer, nsum - c0);  // may be <= 0
-        float4 q[kCarryPer], a[kCarryPer];
+        float4 q[kCarryPer];
+        float sd[kCarryPer];
         const float4* qp = wsq + (size_t)(first + c0) * per_chunk + col;
         const float* sp = at_bytes(p.ws_sd, ws_off) + (size_t)(first + c0) * D + dd;
 #pragma unroll
         for (int i = 0; i < kCarryPer; ++i) {
             q[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-            float sd = 0.0f;  // padding past nsum: decay 1, nothing added
-            if (i < cnt) { q[i] = qp[(size_t)i * per_chunk]; sd = sp[(size_t)i * D]; }
-            a[i] = make_float4(ex2(a2.x * sd), ex2(a2.y * sd), ex2(a2.z * sd), ex2(a2.w * sd));  // decay of the whole chunk
+            sd[i] = 0.0f;  // padding past nsum: decay 1, nothing added
+            if (i < cnt) { q[i] = qp[(size_t)i * per_chunk]; sd[i] = sp[(size_t)i * D]; }
         }
+        auto decay = [&](int i) { return make_float4(ex2(a2.x * sd[i]), ex2(a2.y * sd[i]), ex2(a2.z * sd[i]), ex2(a2.w * sd[i])); };  // of the whole chunk
         float4 Pg = make_float4(1.f, 1.f, 1.f, 1.f), qg = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
         for (int i = 0; i < kCarryPer; ++i) {
-            qg = fold4(a[i], qg, q[i]);
-            Pg.x *= a[i].x; Pg.y *= a[i].y; Pg.z *= a[i].z; Pg.w *= a[i].w;
+            const float4 a = decay(i);
+            qg = fold4(a, qg, q[i]);
+            Pg.x *= a.x; Pg.y *= a.y; Pg.z *= a.z; Pg.w *= a.w;
         }
         sP[g][lane] = Pg;
         sQ[g][lane] = qg;
         __syncthreads();
-        float4 h = carry;
-        for (int gg = 0; gg < g; ++gg) h = fold4(sP[gg][lane], h, sQ[gg][lane]);
-        float4 after = h;  // running state after the whole round, the same in every warp
-        for (int gg = g; gg < kCarryGroups; ++gg) after = fold4(sP[gg][lane], after, sQ[gg][lane]);
+        float4 h = carry, after = carry;  // state before this warp's chunks; after the whole round, the same in every warp
+#pragma unroll 2
+        for (int gg = 0; gg < kCarryGroups; ++gg) {
+            if (gg == g) h = after;
+            after = fold4(sP[gg][lane], after, sQ[gg][lane]);
+        }
         float4* op = wsq + (size_t)(first + c0) * per_chunk + col;
 #pragma unroll
         for (int i = 0; i < kCarryPer; ++i) {
+            asm volatile("" : "+f"(sd[i]));  // the decays are formed again: kept, they would cost 24 registers
             if (i < cnt) {
-                h = fold4(a[i], h, q[i]);
+                h = fold4(decay(i), h, q[i]);
                 if (live) op[(size_t)i * per_chunk] = h;
             }
         }
