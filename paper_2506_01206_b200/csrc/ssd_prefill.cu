@@ -41,8 +41,7 @@ namespace {
 constexpr int P = kSsdP, N = kSsdN, Q = kSsdQ;
 constexpr int kThreads = 256;                 // two warps per 32 accumulator lanes: warps w and w + 4 share rows 32 (w % 4) .. and split the columns
 constexpr int kRowsPerWarp = Q / (kThreads / 32);   // rows of the chunk a warp convolves and stores
-constexpr uint32_t kColBytes = Q * 16;        // one 8-wide column of core matrices over 128 rows: 2048 bytes
-constexpr uint32_t kXdColBytes = Q * 16 + 16; // the same for the thread-written Xd / Xw operand, padded against bank conflicts
+constexpr uint32_t kXdColBytes = Q * 16 + 16; // one 8-wide column of core matrices over 128 rows of the thread-written Xd / Xw operand, padded against bank conflicts
 constexpr uint32_t kHinColBytes = P * 16;     // H_in: 64 rows
 
 // ---------------------------------------------------------------- PTX helpers
@@ -177,12 +176,14 @@ __device__ __forceinline__ uint32_t pack_bf(float lo, float hi) {
 
 // ---------------------------------------------------------------- what both tensor-core kernels share
 // Per-row scalars of a chunk: step size and running log-decay.  Thread t = row t; rows past the chunk's end get a
-// step size of 0 (no decay, no input).  Leaves delta[t], cs[t] (natural log) and csl[t] = cs[t] * log2(e) in shared memory.
+// step size of 0 (no decay, no input).  Leaves delta[t], csl[t] = the running log-decay times log2(e), the chunk's whole log-decay and,
+// visible after the caller's next barrier, weight[t] = delta[t] exp(what the chunk decays by after row t) in shared memory.
 struct RowScalars {
     float delta[Q];
-    float cs[Q];
+    float weight[Q];
     float csl[Q];
     float warp_sum[4];
+    float decay;
 };
 
 __device__ __forceinline__ void row_scalars(RowScalars& rs, const SsdPrefillArgs& p, int head, int t0, int rows, float a_head, float dtb) {
@@ -207,10 +208,11 @@ __device__ __forceinline__ void row_scalars(RowScalars& rs, const SsdPrefillArgs
         for (int w = 0; w < warp; ++w) before += rs.warp_sum[w];
         la += before;
         rs.delta[t] = delta;
-        rs.cs[t] = la;
         rs.csl[t] = la * kLog2e;
+        if (t == Q - 1) rs.decay = la;
     }
     __syncthreads();
+    if (owner) rs.weight[t] = delta * ex2(rs.csl[Q - 1] - rs.csl[t]);
 }
 
 // The three rows before the chunk, as rows 0..2 of the extended x tile (rows 3.. are the TMA box): the sequence's own
@@ -235,7 +237,7 @@ __device__ __forceinline__ void load_rows(const __nv_bfloat16* xs_ext, uint32_t 
     for (int i = 0; i < kRowsPerWarp + 3; ++i) xr[i] = col[(r0 + i) * (P / 2)];
 }
 
-// Taps and bias of this lane's channel pair.
+// Taps and bias of this lane's channel pair, times -log2(e): what the exponential of the SiLU takes.
 struct Taps {
     float4 wa, wb;
     float ba, bb;
@@ -245,8 +247,13 @@ struct Taps {
         wb = __ldg(reinterpret_cast<const float4*>(L.conv_w + (size_t)(d + 1) * kW));
         ba = L.conv_b ? __ldg(L.conv_b + d) : 0.0f;
         bb = L.conv_b ? __ldg(L.conv_b + d + 1) : 0.0f;
+        wa.x *= -kLog2e; wa.y *= -kLog2e; wa.z *= -kLog2e; wa.w *= -kLog2e; ba *= -kLog2e;
+        wb.x *= -kLog2e; wb.y *= -kLog2e; wb.z *= -kLog2e; wb.w *= -kLog2e; bb *= -kLog2e;
     }
 };
+
+// SiLU of a sum that comes times -log2(e): the factor leaves by the denominator, in the multiply-add that would be the addition of 1.
+__device__ __forceinline__ float silu_scaled(float v) { return v * rcp(fmaf(ex2(v), -kLog2e, -kLog2e)); }
 
 // conv + SiLU of those rows; calls f(row, index in the warp, u_lo, u_hi).
 template <typename F>
@@ -262,7 +269,7 @@ __device__ __forceinline__ void conv_rows(const uint32_t (&xr)[kRowsPerWarp + 3]
         a = fmaf(wa.y, bf_lo(w1), a); b = fmaf(wb.y, bf_hi(w1), b);
         a = fmaf(wa.z, bf_lo(w2), a); b = fmaf(wb.z, bf_hi(w2), b);
         a = fmaf(wa.w, bf_lo(xv), a); b = fmaf(wb.w, bf_hi(xv), b);
-        f(r0 + i, i, silu(a), silu(b));
+        f(r0 + i, i, silu_scaled(a), silu_scaled(b));
     }
 }
 
@@ -327,10 +334,9 @@ __global__ void __launch_bounds__(kThreads, 3) ssd_chunk_state_kernel(const SsdP
     }
     __syncthreads();   // every thread holds its rows: the x tile may be overwritten
     if (ok) {
-        const float cs_end_l = sm.rs.csl[Q - 1];
         unsigned char* xd_g = reinterpret_cast<unsigned char*>(p.ws_xd) + ((size_t)cidx * H + head) * ((P / 8) * kXdColBytes);
         conv_rows(xr, taps, [&](int r, int, float ua, float ub) {
-            const float wgt = r < rows ? sm.rs.delta[r] * ex2(cs_end_l - sm.rs.csl[r]) : 0.0f;
+            const float wgt = sm.rs.weight[r];
             const float va = r < rows ? wgt * ua : 0.0f, vb = r < rows ? wgt * ub : 0.0f;
             const uint32_t hi = pack_bf(va, vb);
             const uint32_t lo = pack_bf(va - bf_lo(hi), vb - bf_hi(hi));
@@ -338,7 +344,7 @@ __global__ void __launch_bounds__(kThreads, 3) ssd_chunk_state_kernel(const SsdP
             *reinterpret_cast<uint32_t*>(sm.xw_hi + off) = hi;
             *reinterpret_cast<uint32_t*>(xw_lo + off) = lo;
             // Xd = Delta u goes straight to the workspace, in the layout of the chunk-scan kernel's operand
-            const float dl = r < rows ? sm.rs.delta[r] : 0.0f;
+            const float dl = sm.rs.delta[r];
             *reinterpret_cast<uint32_t*>(xd_g + off) = r < rows ? pack_bf(dl * ua, dl * ub) : 0u;
             if (r < rows) *reinterpret_cast<uint32_t*>(p.ws_u + (size_t)(ci.t0 + r) * p.L.d_inner + head * P + 2 * lane) = pack_bf(ua, ub);
         });
@@ -374,7 +380,7 @@ __global__ void __launch_bounds__(kThreads, 3) ssd_chunk_state_kernel(const SsdP
 #pragma unroll
             for (int j = 0; j < 32; ++j) dst[(size_t)(half * 32 + j) * N] = v[j];
         }
-        if (tid == 0) p.ws_decay[(size_t)cidx * H + head] = sm.rs.cs[Q - 1];
+        if (tid == 0) p.ws_decay[(size_t)cidx * H + head] = sm.rs.decay;
     } else if (tid == 0) {
         flag(p.dev_status, MDRAFT_DEV_WAIT_EXPIRED);
         if (!ok) mbar_wait_bounded(&sm.bar_tma, 0u);   // the copies target this block's shared memory: one more bounded chance
@@ -471,7 +477,8 @@ struct ScanSmem {
     uint32_t tmem_base;
 };
 constexpr int kZOffset = 2 * N * P * 2 - Q * P * 2;   // of the z box in region B, behind the y rows' last bytes
-static_assert(sizeof(float) * Q * (P + 1) <= N / 8 * Q * 16 + kZOffset, "the y staging rows must end before the z box");
+constexpr int kYPitch = P + 4;   // floats of a staged y row: written as 16 bytes by a lane per row, read as 8 bytes by a lane per channel pair, both without conflicts
+static_assert(sizeof(float) * Q * kYPitch <= N / 8 * Q * 16 + kZOffset, "the y staging rows must end before the z box");
 static_assert((P / 8) * kXdColBytes <= N / 8 * Q * 16 && 2 * N * P * 2 <= N / 8 * Q * 16, "re-used regions too small");
 static_assert(3 * (sizeof(ScanSmem) + 1024 + 1024) <= 227 * 1024, "three blocks per SM");
 
@@ -493,7 +500,7 @@ __global__ void __launch_bounds__(kThreads, 3) ssd_chunk_scan_kernel(const SsdPr
     unsigned char* const xd = sm.regA;
     __nv_bfloat16* const hin = reinterpret_cast<__nv_bfloat16*>(sm.regB);
     __nv_bfloat16* const zs = reinterpret_cast<__nv_bfloat16*>(sm.regB + kZOffset);
-    float (*const ystage)[P + 1] = reinterpret_cast<float (*)[P + 1]>(sm.regA);   // runs on into regB
+    float (*const ystage)[kYPitch] = reinterpret_cast<float (*)[kYPitch]>(sm.regA);   // runs on into regB
 
     if (tid == 0) {
         mbar_init(&sm.bar_cb, 1); mbar_init(&sm.bar_dec, 1); mbar_init(&sm.bar_in, 1); mbar_init(&sm.bar_late, 1);
@@ -575,17 +582,23 @@ __global__ void __launch_bounds__(kThreads, 3) ssd_chunk_scan_kernel(const SsdPr
         __syncwarp();
     }
     const bool dec_ok = g_ok && mbar_wait_bounded(&sm.bar_dec, 0u);
-    uint32_t packed[2][16];
     auto mask_block = [&](int cb, const float (&g)[32], uint32_t (&m)[16]) {
         const float my = sm.csl[row];
+        const float4* theirs = reinterpret_cast<const float4*>(sm.csl + cb * 32);
 #pragma unroll
-        for (int j = 0; j < 32; j += 2) {
-            const int s0 = cb * 32 + j;
-            const float m0 = s0 <= row ? g[j] * ex2(my - sm.csl[s0]) : 0.0f;
-            const float m1 = s0 + 1 <= row ? g[j + 1] * ex2(my - sm.csl[s0 + 1]) : 0.0f;
-            m[j >> 1] = pack_bf(m0, m1);
+        for (int j = 0; j < 32; j += 4) {
+            const float4 c = theirs[j >> 2];
+            float v[4] = {g[j] * ex2(my - c.x), g[j + 1] * ex2(my - c.y), g[j + 2] * ex2(my - c.z), g[j + 3] * ex2(my - c.w)};
+            if (cb == rb) {   // only the block on the diagonal has entries to its right; their exponentials may overflow, so they are replaced, not scaled
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    if (j + e > lane) v[e] = 0.0f;
+            }
+            m[j >> 1] = pack_bf(v[0], v[1]);
+            m[(j >> 1) + 1] = pack_bf(v[2], v[3]);
         }
     };
+    uint32_t packed[2][16];
 #pragma unroll
     for (int j = 0; j < 16; ++j) { packed[0][j] = 0u; packed[1][j] = 0u; }   // column blocks right of the warp's rows stay zero
     if (dec_ok) {
@@ -631,7 +644,8 @@ __global__ void __launch_bounds__(kThreads, 3) ssd_chunk_scan_kernel(const SsdPr
         float yi[32];
         tmem_ld32(tY + lanes + half * 32, yi);
 #pragma unroll
-        for (int j = 0; j < 32; ++j) ystage[row][half * 32 + j] = y[j] + yi[j];
+        for (int j = 0; j < 32; j += 4)
+            *reinterpret_cast<float4*>(&ystage[row][half * 32 + j]) = make_float4(y[j] + yi[j], y[j + 1] + yi[j + 1], y[j + 2] + yi[j + 2], y[j + 3] + yi[j + 3]);
     }
     const int d = head * P + 2 * lane;
     uint32_t uraw[kRowsPerWarp];   // skip term inputs of the warp's rows (u of this lane's channel pair, from kernel 1)
@@ -650,8 +664,9 @@ __global__ void __launch_bounds__(kThreads, 3) ssd_chunk_scan_kernel(const SsdPr
             const int r = warp * kRowsPerWarp + i;
             if (r < rows) {
                 const uint32_t zv = zc[r * (P / 2)];
-                const float oa = fmaf(da, bf_lo(uraw[i]), ystage[r][2 * lane]) * silu_gate(bf_lo(zv));
-                const float ob = fmaf(db, bf_hi(uraw[i]), ystage[r][2 * lane + 1]) * silu_gate(bf_hi(zv));
+                const float2 yv = *reinterpret_cast<const float2*>(&ystage[r][2 * lane]);
+                const float oa = fmaf(da, bf_lo(uraw[i]), yv.x) * silu_gate(bf_lo(zv));
+                const float ob = fmaf(db, bf_hi(uraw[i]), yv.y) * silu_gate(bf_hi(zv));
                 *reinterpret_cast<uint32_t*>(p.out + (size_t)(ci.t0 + r) * p.ldo + d) = pack_bf(oa, ob);
             }
         }
