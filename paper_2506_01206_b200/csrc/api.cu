@@ -717,13 +717,12 @@ int mdraft_block_generation(const mdraft_block_stack* stack, const mdraft_cache*
     typedef __nv_bfloat16 bf;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     bf *hb = static_cast<bf*>(h), *xzb = static_cast<bf*>(xz), *yb = static_cast<bf*>(y);
-    bool in_alone, out_alone;
-    keep_products_apart(M, D, n_nodes, in_alone, out_alone);
+    const ProductPlacement place = place_products(M, D, n_nodes);
     // The first kernel is an ordinary launch: everything ahead of the call is complete before a kernel of the call reads
     // a parent's state, which no other kernel of the call writes.  Each later kernel may start while the one ahead runs.
     cudaError_t e = launch_embed(tokens, static_cast<const bf*>(stack->embed), hb, n_nodes, M, stack->vocab, dev_status, st);
     for (int32_t l = 0; l < stack->n_layers && e == cudaSuccess; ++l) {
-        e = launch_small_linear({hb, static_cast<const bf*>(stack->W_in[l]), nullptr, xzb, 2 * (int64_t)D, 2 * (int64_t)D, n_nodes, 2 * D, M, dev_status, in_alone, stack->eps}, st);
+        e = launch_small_linear({hb, static_cast<const bf*>(stack->W_in[l]), nullptr, xzb, 2 * (int64_t)D, 2 * (int64_t)D, n_nodes, 2 * D, M, dev_status, false, place.in_alone, stack->eps}, st);
         if (e != cudaSuccess) break;
         TreeProjArgs a;
         a.L = layer_dev(stack->layers + l);
@@ -733,10 +732,10 @@ int mdraft_block_generation(const mdraft_block_stack* stack, const mdraft_cache*
         a.W_x = stack->W_x[l]; a.W_dt = stack->W_dt[l]; a.dt_rank = R; a.nodes_per_cluster = 0;
         a.parent_slot = parent_slot; a.node_slot = node_slot; a.n_nodes = n_nodes; a.chained = 1; a.dev_status = dev_status;
         if ((e = launch_tree_proj(a, MDRAFT_BF16, st)) != cudaSuccess) break;
-        e = launch_small_linear({yb, static_cast<const bf*>(stack->W_out[l]), hb, hb, M, M, n_nodes, M, D, dev_status, out_alone, -1.0f}, st);
+        e = launch_small_linear({yb, static_cast<const bf*>(stack->W_out[l]), hb, hb, M, M, n_nodes, M, D, dev_status, place.out_late, place.out_alone, -1.0f}, st);
     }
     if (e == cudaSuccess)
-        e = launch_small_linear({hb, static_cast<const bf*>(stack->W_lm), nullptr, static_cast<bf*>(logits), stack->vocab, ldl, n_nodes, stack->vocab, M, dev_status, false, stack->eps}, st);
+        e = launch_small_linear({hb, static_cast<const bf*>(stack->W_lm), nullptr, static_cast<bf*>(logits), stack->vocab, ldl, n_nodes, stack->vocab, M, dev_status, false, false, stack->eps}, st);
     return e == cudaSuccess ? MDRAFT_OK : MDRAFT_ERR_CUDA;
 }
 

@@ -21,6 +21,7 @@
 // out_proj) or a split contraction with an exchange between blocks, and its round trip through tensor memory costs more than
 // the few dependent mma of a warp here.
 #include "block.cuh"
+#include "tree_proj.cuh"
 
 namespace mdraft {
 
@@ -162,7 +163,7 @@ __global__ void __launch_bounds__(NW * 32, PRE > 0 ? 0 : 2) small_linear_kernel(
     __shared__ __align__(8) uint64_t bar;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
     const int n0 = blockIdx.x * NT, m0 = blockIdx.y * kRows, rows = min(kRows, p.m - m0);
-    grid_release_dependents();
+    if (!p.release_late) grid_release_dependents();
     if (threadIdx.x == 0) {
         mbar_init(&bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -188,6 +189,7 @@ __global__ void __launch_bounds__(NW * 32, PRE > 0 ? 0 : 2) small_linear_kernel(
     for (int q = 0; q < PRE; ++q)
         if (warp + q * NW < kblocks) load_w<kCols>(w[q], smem_u32(s_w) + (uint32_t)((warp + q * NW) * 32 * kPitch), kPitch, lane);
     grid_wait();   // the activations are the work of the kernel ahead
+    if (p.release_late) grid_release_dependents();
     if (threadIdx.x == 0) {
         mbar_expect_tx(&bar, (uint32_t)(rows * p.k * 2));
         bulk_load(s_a, p.a + (size_t)m0 * p.k, (uint32_t)(rows * p.k * 2), &bar);
@@ -366,10 +368,14 @@ cudaError_t launch_tile(const SmallLinear& p, cudaStream_t st) {
 // blocks keep off one another, and from five nodes on off out_proj's, a generation of 1 / 4 / 8 / 16 / 18 / 24 / 32 nodes takes
 // 190 / 210 / 230 / 254 / 276 / 308 / 335 us; without 224 / 242 / 246 / 280 / 306 / 320 / 336.  Up to four nodes the two products'
 // blocks are better beside each other (apart 203 / 221 us).  Only where one wave holds them all.
-void keep_products_apart(int d_model, int d_inner, int n_nodes, bool& in_proj, bool& out_proj) {
+// The next layer's in_proj starts some 10 us ahead of its turn, as soon as out_proj's blocks have started.  Where the projection step alone has a block for
+// about every SM, it is better held back until out_proj's own turn: 18 / 23 / 24 / 28 / 32 nodes 272 / 290 / 303 / 324 / 335 us, held back
+// 277 / 298 / 298 / 313 / 316.  (Beyond one row tile it makes no odds: 33 / 48 / 64 nodes 384 / 490 / 482 and 392 / 489 / 477.)
+ProductPlacement place_products(int d_model, int d_inner, int n_nodes) {
     const int sms = sm_count(), tile = 2 * d_inner <= 16 * sms ? 16 : 32, blocks = (2 * d_inner + tile - 1) / tile + (d_model + 15) / 16;
-    in_proj = n_nodes <= kRows && blocks <= sms;
-    out_proj = in_proj && n_nodes > 4;
+    const int cb = tree_proj_block_channels(d_inner), step_blocks = n_nodes * ((d_inner + cb - 1) / cb);
+    const bool one_tile = n_nodes <= kRows, apart = one_tile && blocks <= sms;
+    return {apart, apart && n_nodes > 4, one_tile && step_blocks * 20 >= sms * 19};
 }
 
 cudaError_t launch_small_linear(const SmallLinear& p, cudaStream_t st) {

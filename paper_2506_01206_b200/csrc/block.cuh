@@ -18,12 +18,15 @@ struct SmallLinear {
     int64_t ldw, ldo;          // rows of a are dense (k values)
     int m, n, k;
     int32_t* dev_status;
+    bool release_late;         // the next kernel may start only once this one's turn has come
     bool alone;                // no two blocks of such products on one SM (keep_products_apart)
     float eps;                 // >= 0: the sum is scaled by 1 / sqrt(mean_k a[m][k]^2 + eps); < 0: not
 };
 
-// Which of a block's products, for so many nodes, take an SM without another product's block: see the measurements at the definition.
-void keep_products_apart(int d_model, int d_inner, int n_nodes, bool& in_proj, bool& out_proj);
+// Which of a block's products, for so many nodes, take an SM without another product's block, and whether out_proj holds back the layer after it:
+// see the measurements at the definition.
+struct ProductPlacement { bool in_alone, out_alone, out_late; };
+ProductPlacement place_products(int d_model, int d_inner, int n_nodes);
 
 cudaError_t launch_small_linear(const SmallLinear& p, cudaStream_t st);
 
