@@ -328,18 +328,19 @@ constexpr int kSmemAlone = 116 * 1024; // more than half of an SM's
 template <auto kKernel>
 cudaError_t launch_chained(dim3 grid, int threads, int smem, const SmallLinear& p, cudaStream_t st) {
     if (smem > kMaxSmem) return cudaErrorInvalidValue;
-    const cudaError_t e = allow_smem<kKernel>(kMaxSmem, true);
+    const cudaError_t e = allow_smem<kKernel>(kMaxSmem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1] = most_shared_memory();
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, kKernel, p);
 }
 

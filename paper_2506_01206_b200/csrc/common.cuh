@@ -142,21 +142,27 @@ int sm_count();
 
 // A kernel that wants more dynamic shared memory than a launch gets by default has the limit raised once per device: it is a
 // property of the loaded function, and asking for it on every call costs host time.
-// most_shared: the SM's memory is split in favour of shared memory, as much as it goes.  Kernels of a chain that overlap ask for it alike, so that what
-// fits beside what depends on their needs alone: left to itself the driver picks a split for each kernel, and a block starts only on an SM that
-// has, or is free to take, its kernel's.
 template <auto kKernel>
-inline cudaError_t allow_smem(int bytes, bool most_shared = false) {
-    if (bytes <= 48 * 1024 && !most_shared) return cudaSuccess;
+inline cudaError_t allow_smem(int bytes) {
+    if (bytes <= 48 * 1024) return cudaSuccess;
     static std::atomic<uint64_t> done{0};  // bit = device
     int dev = 0;
     const cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 64 && (done.load(std::memory_order_acquire) >> dev & 1u)) return cudaSuccess;
-    cudaError_t f = most_shared ? cudaFuncSetAttribute(kKernel, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared) : cudaSuccess;
-    if (f == cudaSuccess && bytes > 48 * 1024) f = cudaFuncSetAttribute(kKernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    const cudaError_t f = cudaFuncSetAttribute(kKernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if (f == cudaSuccess && dev < 64) done.fetch_or(1ull << dev, std::memory_order_release);
     return f;
+}
+
+// For kernels of a chain that overlap: launched with the SM's memory split in favour of shared memory as far as it goes, so that what fits beside what
+// depends on their needs alone.  Left to itself the driver picks a split for each kernel, and a block starts only on an SM that has, or is
+// free to take, its kernel's.
+inline cudaLaunchAttribute most_shared_memory() {
+    cudaLaunchAttribute a = {};
+    a.id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    a.val.sharedMemCarveout = (unsigned)cudaSharedmemCarveoutMaxShared;
+    return a;
 }
 
 __device__ __forceinline__ void flag(int32_t* dev_status, int bit) {

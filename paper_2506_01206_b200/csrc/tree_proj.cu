@@ -521,7 +521,7 @@ cudaError_t launch_nt(const TreeProjArgs& p, int n_blocks, cudaStream_t st) {
     cfg.blockDim = dim3(CB, 1, 1);
     cfg.dynamicSmemBytes = kSmem;
     cfg.stream = st;
-    cudaLaunchAttribute at[2];
+    cudaLaunchAttribute at[3];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = 1;
     at[0].val.clusterDim.y = (unsigned)n_blocks;  // the blocks of one group of nodes
@@ -529,9 +529,10 @@ cudaError_t launch_nt(const TreeProjArgs& p, int n_blocks, cudaStream_t st) {
     cfg.attrs = at;
     at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.numAttrs = p.chained ? 2 : 1;
+    at[2] = most_shared_memory();   // alone the driver's own split is 2-4 % faster (18 nodes 5.7 against 5.95 us)
+    cfg.numAttrs = p.chained ? 3 : 1;
     const bool pow = p.L.flags & MDRAFT_A_POWERS;
-    const cudaError_t e = pow ? allow_smem<tree_proj_kernel<AT, CB, NT, true>>(kSmem, true) : allow_smem<tree_proj_kernel<AT, CB, NT, false>>(kSmem, true);
+    const cudaError_t e = pow ? allow_smem<tree_proj_kernel<AT, CB, NT, true>>(kSmem) : allow_smem<tree_proj_kernel<AT, CB, NT, false>>(kSmem);
     if (e != cudaSuccess) return e;
     return cudaLaunchKernelEx(&cfg, pow ? tree_proj_kernel<AT, CB, NT, true> : tree_proj_kernel<AT, CB, NT, false>, p);
 }
