@@ -149,7 +149,8 @@ typedef struct {
  *                of 128 channels (one of 512 where the width fills those) or are, for several sequences, at most 256
  *                tokens; less is MDRAFT_ERR_WORKSPACE.  Sequences that the library leaves whole need none, although
  *                the query for a single layer answers as if they were cut.  A chunk length given in `opts` is kept:
- *                it needs all that the query says
+ *                it needs all that the query says.  Small problems are encoded in one kernel that uses none of it; they are refused
+ *                all the same where the workspace would not serve the other form
  *   dev_status : device int32 or NULL (see mdraft_dev_status bits); never cleared by the library
  */
 size_t mdraft_prefill_workspace_bytes(const mdraft_layer *layer, int32_t total_tokens, int32_t n_seq,
