@@ -418,7 +418,8 @@ int run_prefill(const PrefillCall& call, const PrefillPlan& pl, int32_t n_layers
 //    further warp on a scheduler (standard deviation 7 %);
 //  - the other takes kSplit + kSplitWork per token of work of a scheduler where it cuts sequences, kWhole + kWholeToken per token
 //    of the longest where it does not (15 %), so the one-kernel form has to promise 12 % less, and 20 % from sixteen sequences on, which the narrow form with four blocks to an SM
-//    serves better than that (20 x 1508 x 64, general A: 32.7 us, in one kernel 37.9).
+//    serves better than that (20 x 1508 x 64, general A: 32.7 us, in one kernel 37.9), and 25 % where one layer's one sequence is long for its width (1500 x 1536: 26.8 us, in
+//    one kernel 29.6; 1300 x 1200 25.5 and 28.6; 3925 x 368 28.5 and 34.4).
 // It wins where the work is small: 256 x 64 fp32 9.2 -> 6.4 us, 256 x 768 bf16 12.3 -> 8.1, 1024 x 128 to 256 0.76 of the time; in the mean over
 // those calls 16 % (12 of them lose 3 % or more).  It loses where the work fills the machine, since its clusters leave a seventh of the SMs out and
 // its channel groups are narrow: 1777 x 1536, general A, 35.5 against 41.4 at best, 4096 x 1536 52 against 77.
@@ -426,12 +427,13 @@ ClusterForm cluster_form(const mdraft_layer* L, int n_layers, int T, int n_seq, 
     if (one_at_a_time(L) || (opts && (opts->chunk_len > 0 || opts->block_channels || opts->event_after_chunk_state || opts->event_after_carry_scan))) return {0, 0};
     constexpr double kOne = 4.1, kCluster = 0.6, kBlock = 0.13, kWarp = 0.15, kLatency[2] = {0.195, 0.275}, kShare[2] = {0.112, 0.167};
     constexpr double kSplit = 11.1, kSplitSeqs = 0.7, kSplitWork[2] = {0.166, 0.239}, kWhole = 3.3, kWholeToken = 0.104;
-    const double margin = n_seq < 16 ? 0.88 : 0.8;
     const int general = !(L->flags & MDRAFT_A_POWERS), sms = sm_count();
     const int64_t groups = (int64_t)n_layers * ((L->d_inner + kClusterCols - 1) / kClusterCols), clusters = groups * n_seq;
+    const double work = (double)T * groups / (4 * sms);
+    const double margin = n_seq >= 16 ? 0.8 : n_seq * n_layers == 1 && work > 75.0 ? 0.75 : 0.88;
     if (clusters > 8 * sms || (L->d_inner + kClusterCols - 1) / kClusterCols > 65535 || (int64_t)n_layers * n_seq > 65535) return {0, 0};
     ClusterForm best = {0, 0};
-    double least = kSplit + (double)T * groups / (4 * sms) * kSplitWork[general] + (n_seq > 1 ? kSplitSeqs : 0.0);
+    double least = kSplit + work * kSplitWork[general] + (n_seq > 1 ? kSplitSeqs : 0.0);
     const double blocks = (double)n_layers * n_seq * ((L->d_inner + kPrefillThreads - 1) / kPrefillThreads), rounds = 1.2 * blocks / sms;
     const double whole = kWhole + max_seqlen * kWholeToken * (general ? kGeneralOne : 1.0) * (rounds > 1.0 ? rounds : 1.0);
     least = margin * (whole < least ? whole : least);

@@ -419,8 +419,10 @@ __global__ void __launch_bounds__(SUB * kBoxCols + 32, PER_SM) chunk_kernel(cons
 // publishes the pair, folds the pairs of the warps before it into its starting state, and then replays its own
 // chunks to write the state after each.  Rounds carry the running state forward past 48 chunks.
 // Registers count beyond the kernel itself: its blocks and the output pass's start as the summary pass leaves SMs, beside one another.  The
-// decays are formed twice instead of kept: 126 -> 104 registers, 1777 x 1536 (general A) 35.5 -> 35.1 us, three sequences of 700 to 1400 x
-// 1000 in fp32 46.3 -> 45.3.  (Held down to 64 or 48 registers it spills and loses 4 us; 10 to 16 warps of 3 or 4 chunks lose 0.5 to 3.)
+// decays are formed twice instead of kept: 126 -> 104 registers, 1777 x 1536 (general A) 35.5 -> 35.2 us, 2048 x 1536 31.3 -> 31.1, three
+// sequences of 574 to 1300 x 1000 in fp32 38.1 -> 37.1.  (Without the 1 in the launch bounds the compiler takes 80: 35.2, 31.8 and 35.8.  Held down to 64 or
+// 48 it spills and loses 4 us; 10 to 16 warps of 3 or 4 chunks lose 0.5 to 3.  The fold over the warps unrolled by 2 costs 10 % where a call takes many
+// rounds, 12 sequences of up to 9532 x 80 79.0 -> 88.5 us; by 8 it costs the short calls 5 %.)
 constexpr int kCarryGroups = 8, kCarryPer = 6;
 
 __device__ __forceinline__ float4 fold4(const float4& a, const float4& h, const float4& q) {
@@ -428,7 +430,7 @@ __device__ __forceinline__ float4 fold4(const float4& a, const float4& h, const 
 }
 
 template <int ML>
-__global__ void __launch_bounds__(kCarryGroups * 32) carry_kernel(const __grid_constant__ PrefillBatch<ML> batch) {
+__global__ void __launch_bounds__(kCarryGroups * 32, 1) carry_kernel(const __grid_constant__ PrefillBatch<ML> batch) {
     const PrefillArgs& p = batch.c;
     __shared__ float4 sP[kCarryGroups][32];
     __shared__ float4 sQ[kCarryGroups][32];
@@ -485,7 +487,7 @@ __global__ void __launch_bounds__(kCarryGroups * 32) carry_kernel(const __grid_c
         sQ[g][lane] = qg;
         __syncthreads();
         float4 h = carry, after = carry;  // state before this warp's chunks; after the whole round, the same in every warp
-#pragma unroll 2
+#pragma unroll 4
         for (int gg = 0; gg < kCarryGroups; ++gg) {
             if (gg == g) h = after;
             after = fold4(sP[gg][lane], after, sQ[gg][lane]);
