@@ -142,6 +142,10 @@ typedef struct {
  *   init_slot  : n_seq int32 or NULL; slot holding each sequence's starting state, -1 / NULL = zero state
  *   final_slot : n_seq int32 or NULL; slot that receives the state after the last token, -1 / NULL = discard.
  *                init_slot[s] == final_slot[s] is allowed (encode a context in pieces).
+ *                Hazards (caller's duty): the sequences of a call run side by side, in any order.  No two may have the same
+ *                final_slot.  Any number may start from a slot that none of them stores to.  A sequence may start from
+ *                another's final_slot only where it is cut, which a chunk length in `opts` guarantees for sequences of more
+ *                tokens than that: it then starts from what the slot held before the call
  *   max_seqlen : an upper bound on the longest sequence (HOST value, used to size the launch)
  *   workspace  : device scratch, 256-byte aligned; contents need not be initialised and are garbage afterwards.
  *                mdraft_prefill_workspace_bytes(...) says how much the call would like.  With less it cuts the sequences
@@ -149,8 +153,9 @@ typedef struct {
  *                of 128 channels (one of 512 where the width fills those) or are, for several sequences, at most 256
  *                tokens; less is MDRAFT_ERR_WORKSPACE.  Sequences that the library leaves whole need none, although
  *                the query for a single layer answers as if they were cut.  A chunk length given in `opts` is kept:
- *                it needs all that the query says.  Small problems are encoded in one kernel that uses none of it; they are refused
- *                all the same where the workspace would not serve the other form
+ *                it needs all that the query says.  Small problems are encoded in one kernel that uses none of it, unless several
+ *                sequences with both starting and final slots would otherwise be cut; they are refused all the same where
+ *                the workspace would not serve the other form
  *   dev_status : device int32 or NULL (see mdraft_dev_status bits); never cleared by the library
  */
 size_t mdraft_prefill_workspace_bytes(const mdraft_layer *layer, int32_t total_tokens, int32_t n_seq,
@@ -182,7 +187,8 @@ typedef struct {
  * no pool layer may appear twice.
  *   workspace : as above; mdraft_prefill_stack_workspace_bytes answers for layers that share the flags of `layer`.  The
  *               launches of a call share it, so layers with different flags need the largest answer over their groups
- * mdraft_prefill_stack_launches: kernels such a call launches (for accounting).
+ * mdraft_prefill_stack_launches: kernels such a call launches (for accounting), if it is of one sequence or has no init_slot or
+ * no final_slot; with both, a batch that would be cut takes three (two under MDRAFT_CONV_ONLY) also where this says one.
  */
 size_t mdraft_prefill_stack_workspace_bytes(const mdraft_layer *layer, int32_t n_layers, int32_t total_tokens, int32_t n_seq,
                                             int32_t max_seqlen, const mdraft_prefill_opts *opts);

@@ -423,6 +423,10 @@ int run_prefill(const PrefillCall& call, const PrefillPlan& pl, int32_t n_layers
 // It wins where the work is small: 256 x 64 fp32 9.2 -> 6.4 us, 256 x 768 bf16 12.3 -> 8.1, 1024 x 128 to 256 0.76 of the time; in the mean over
 // those calls 16 % (12 of them lose 3 % or more).  It loses where the work fills the machine, since its clusters leave a seventh of the SMs out and
 // its channel groups are narrow: 1777 x 1536, general A, 35.5 against 41.4 at best, 4096 x 1536 52 against 77.
+// It is for calls whose sequences do not look at one another's slots: a cluster reads its starting slot when it comes to run, by when another
+// sequence's may have stored its final state, where the three kernels take the state and window that a cut sequence starts
+// from ahead of the pass that stores.  The slots are on the device, so where several sequences have both and the plan cuts them, the caller of
+// this function keeps the three kernels.
 ClusterForm cluster_form(const mdraft_layer* L, int n_layers, int T, int n_seq, int max_seqlen, const mdraft_prefill_opts* opts) {
     if (one_at_a_time(L) || (opts && (opts->chunk_len > 0 || opts->block_channels || opts->event_after_chunk_state || opts->event_after_carry_scan))) return {0, 0};
     constexpr double kOne = 4.1, kCluster = 0.6, kBlock = 0.13, kWarp = 0.15, kLatency[2] = {0.195, 0.275}, kShare[2] = {0.112, 0.167};
@@ -587,7 +591,10 @@ int mdraft_conv_scan_prefill_stack(int32_t n_layers, const mdraft_layer* layers,
                     if (!workspace || workspace_bytes < pl.bytes) return MDRAFT_ERR_WORKSPACE;
                     if (reinterpret_cast<uintptr_t>(workspace) & 255u) return MDRAFT_ERR_MISALIGNED;
                 }
-            } else if (const ClusterForm cf = cluster_form(layers + l0, nl, plan_tokens, n_seq, max_seqlen, opts); cf.blocks > 0) {
+            } else if (const ClusterForm cf = pl.form.chunked && n_seq > 1 && init_slot && final_slot
+                                                  ? ClusterForm{0, 0}  // one sequence may start from a slot that another stores to: see cluster_form
+                                                  : cluster_form(layers + l0, nl, plan_tokens, n_seq, max_seqlen, opts);
+                       cf.blocks > 0) {
                 const int r = nl == 1 ? run_prefill_cluster<1>(call, cf, nl, layers + l0, layer_index + l0, io + l0)
                                       : run_prefill_cluster<kClusterMaxLayers>(call, cf, nl, layers + l0, layer_index + l0, io + l0);
                 if (r) return r;

@@ -78,3 +78,41 @@ def test_one_kernel_form_of_a_stack_and_its_faults(act):
     torch.cuda.synchronize()
     assert int(status.item()) == md.MDRAFT_DEV_BAD_SEQLENS
     assert not bool((out[:, :50] == 9.0).all()) and bool((out[:, 50:] == 9.0).all())
+
+
+@pytest.mark.parametrize("act,Dn,n_layers,lens", [("bf16", 200, 1, [300, 290, 301, 257]), ("f32", 72, 2, [400, 333, 500])])
+def test_sequences_may_start_from_a_slot_that_one_of_them_stores_to(act, Dn, n_layers, lens):
+    """Several sequences continue from one prefix's slot and the first stores its state back there: all of them start from what the slot
+    held before the call.  Only sequences that are cut promise that, so the call takes the three kernels (bit for bit those of the
+    same plan's chunk length), although its size is one that a call without starting slots does in one."""
+    S, T, tdt = len(lens), sum(lens), torch_act(act)
+    probs = [parity.make_problem(parity.small_config(Dn, act, S, cid=60 + l), lens) for l in range(n_layers)]
+    flags = md.MDRAFT_DT_SOFTPLUS | md.MDRAFT_A_POWERS
+    lays = [upload_layer(p.params, act, flags) for p in probs]
+    assert md.mdraft_prefill_stack_launches(lays[0], n_layers, T, S, max(lens)) == 1
+    ci, hi = random_state(probs[0].cfg, 1, 7)
+    ins = [tuple(to_device(a, tdt) for a in (p.x, p.z, p.dt, p.B, p.C)) for p in probs]
+    init, final = i32([0] * S), i32(np.arange(S))
+    res = []
+    for chunk_len in (0, 16):
+        cache = md.StateCache(n_layers, S, Dn, act=tdt)
+        cache.ssm[:, 0], cache.conv[:, 0] = torch.from_numpy(np.asarray(hi[0], dtype=np.float32)).cuda(), to_device(ci[0], tdt)
+        outs = list(torch.full((n_layers, T, Dn), float("nan"), dtype=tdt, device="cuda"))
+        status = torch.zeros(1, dtype=torch.int32, device="cuda")
+        if chunk_len or n_layers == 1:
+            for l in range(n_layers):
+                ws = torch.empty(md.mdraft_prefill_workspace_bytes(lays[l], T, S, max(lens), chunk_len), dtype=torch.uint8, device="cuda")
+                md.mdraft_conv_scan_prefill(lays[l], cache, l, *ins[l], outs[l], i32(probs[0].cu), max(lens), init, final, ws, chunk_len, status)
+        else:
+            ws = torch.empty(md.mdraft_prefill_stack_workspace_bytes(lays[0], n_layers, T, S, max(lens)), dtype=torch.uint8, device="cuda")
+            assert md.mdraft_conv_scan_prefill_stack(lays, range(n_layers), cache, ins, outs, i32(probs[0].cu), max(lens), init, final, ws, status)
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0
+        res.append((torch.stack(outs), cache.ssm, cache.conv))
+    for a, b in zip(*res):
+        assert torch.equal(a, b)
+    for l, p in enumerate(probs):
+        o_out, o_conv, o_h = run_oracle_prefill(p, flags, np.repeat(ci[:1], S, 0), np.repeat(hi[:1], S, 0))
+        assert_close(res[0][0][l].float().cpu().numpy(), o_out, TOL[act], f"out of layer {l}")
+        assert_close(res[0][1][l].cpu().numpy(), o_h, TOL_STATE, f"states of layer {l}")
+        assert np.array_equal(res[0][2][l].float().cpu().numpy().astype(np.float64), o_conv)
