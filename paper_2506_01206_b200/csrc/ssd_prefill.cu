@@ -406,15 +406,13 @@ __global__ void __launch_bounds__(kPassThreads) ssd_state_passing_kernel(const S
     // after everything before the call had finished, so they are read before the wait below.
     int first, nck;
     seq_chunks(p.cu, p.n_seq, p.T, Q, s, first, nck);   // whole warps call this
-    // malformed offsets: the sequence has no chunk and is skipped
-    if (p.cu && blockIdx.x == 0 && threadIdx.x == 0) {
-        const int lo = __ldg(p.cu + s), hi = __ldg(p.cu + s + 1);
-        if (lo < 0 || hi < lo || hi > p.T) flag(p.dev_status, MDRAFT_DEV_BAD_SEQLENS);
-    }
+    int s0, len; bool bad;   // malformed offsets: the sequence has no chunk and leaves its final slot alone
+    seq_span(p.cu, p.n_seq, p.T, s, s0, len, bad);
+    if (bad && blockIdx.x == 0 && threadIdx.x == 0) flag(p.dev_status, MDRAFT_DEV_BAD_SEQLENS);
     const int islot = load_slot(p.init_slot, s), fslot = load_slot(p.final_slot, s);
     const bool slots_ok = islot < p.pool.n_slots && fslot < p.pool.n_slots;
     if (!slots_ok && blockIdx.x == 0 && threadIdx.x == 0) flag(p.dev_status, MDRAFT_DEV_BAD_SLOT);
-    const bool mine = slots_ok && idx < D * (N / 4);
+    const bool mine = slots_ok && !bad && idx < D * (N / 4);
     // consecutive lanes: the two halves of a unit, then consecutive channels of one head and one state group, so that the
     // 16-byte operand units a warp writes are contiguous (its 32-byte reads of the chunk states each fill a sector)
     const int sub = idx & 1, ch = (idx >> 1) % P, g = (idx / (2 * P)) % (N / 8), head = mine ? idx / (2 * P * (N / 8)) : 0, d = head * P + ch;

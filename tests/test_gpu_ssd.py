@@ -207,6 +207,26 @@ def test_ssd_bad_slots_are_flagged_not_followed():
     assert int(status.item()) & md.MDRAFT_DEV_BAD_SLOT
 
 
+@pytest.mark.parametrize("init", [None, [3, 4, 5]])
+def test_ssd_malformed_offsets_leave_output_and_slots_alone(init):
+    """The sequence whose offsets step back is a no-op: neither its output rows nor its final slot are written, whether it has a
+    starting slot or starts from zeros."""
+    cfg, prm, arrs, cu = make(128, [60, 140, 30])
+    lay = upload_ssd_layer(prm)
+    cache = ssd_cache(6, 128)
+    cache.ssm.fill_(5.0); cache.conv.fill_(5.0); cache.ssm[0, 3:].fill_(2.0); cache.conv[0, 3:].fill_(2.0)
+    dev = [to_device(a, BF) for a in arrs]
+    out = torch.full((230, 128), float("nan"), dtype=BF, device="cuda")
+    ws = torch.empty(md.mdraft_ssd_prefill_workspace_bytes(lay, 230, 3), dtype=torch.uint8, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    md.mdraft_ssd_prefill(lay, cache, 0, *dev, out, i32([0, 60, 40, 70]), None if init is None else i32(init), i32([0, 1, 2]), ws, status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == md.MDRAFT_DEV_BAD_SEQLENS
+    assert bool((cache.ssm[0, 1] == 5.0).all()) and bool((cache.conv[0, 1].float() == 5.0).all())
+    assert not bool((cache.ssm[0, 0] == 5.0).all()) and not bool((cache.ssm[0, 2] == 5.0).all())
+    assert not bool(out[:70].isnan().any()) and bool(out[70:].isnan().all())
+
+
 def _ssd_case(seed):
     g = np.random.default_rng(5000 + seed)
     Dn = int(g.choice([64, 128, 192, 320]))
