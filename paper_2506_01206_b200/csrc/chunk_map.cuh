@@ -16,6 +16,9 @@ struct ChunkInfo {
 
 // Chunks per sequence: ceil(len / Lc); a sequence whose cu_seqlens entries are out of order or out of range
 // gets none.  Global chunk ids number the chunks of sequence 0, then 1, ...  Called by whole warps.
+// Offsets in order make at most n_seq + T / Lc chunks, which is what grids and workspace are sized for (`bound`).  Offsets
+// that step back let sequences overlap and can make more ({0, T, 0, T} makes twice as many): a sequence whose chunks do not all lie below
+// the bound gets none either, so that no index leaves the workspace.
 __device__ __forceinline__ void seq_span(const int32_t* cu, int n_seq, int T, int s, int& a, int& len, bool& bad) {
     a = 0; len = 0; bad = false;
     if (!cu) {  // no offsets given: one sequence that is all T rows (nothing to look up in memory)
@@ -29,7 +32,7 @@ __device__ __forceinline__ void seq_span(const int32_t* cu, int n_seq, int T, in
     }
 }
 
-__device__ inline ChunkInfo find_chunk(const int32_t* cu, int n_seq, int T, int Lc, int cidx) {
+__device__ inline ChunkInfo find_chunk(const int32_t* cu, int n_seq, int T, int Lc, int bound, int cidx) {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     ChunkInfo ci;
@@ -51,9 +54,9 @@ __device__ inline ChunkInfo find_chunk(const int32_t* cu, int n_seq, int T, int 
             int l = __ffs(m) - 1;
             int first = base + __shfl_sync(full, incl, l) - __shfl_sync(full, nc, l);
             int sa = __shfl_sync(full, a, l), sl = __shfl_sync(full, len, l);
-            ci.seq = sb + l;
-            ci.k = cidx - first;
             ci.nck = __shfl_sync(full, nc, l);
+            ci.seq = first + ci.nck <= bound ? sb + l : -1;
+            ci.k = cidx - first;
             ci.s0 = sa;
             ci.t0 = sa + ci.k * Lc;
             ci.t1 = min(ci.t0 + Lc, sa + sl);
@@ -65,12 +68,12 @@ __device__ inline ChunkInfo find_chunk(const int32_t* cu, int n_seq, int T, int 
 }
 
 // First global chunk id and chunk count of sequence s.  Called by whole warps.
-__device__ inline void seq_chunks(const int32_t* cu, int n_seq, int T, int Lc, int s, int& first, int& nck) {
+__device__ inline void seq_chunks(const int32_t* cu, int n_seq, int T, int Lc, int bound, int s, int& first, int& nck) {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     int base = 0;
     first = 0; nck = 0;
-    for (int sb = 0; sb <= s; sb += 32) {
+    for (int sb = 0; sb <= s && base < bound; sb += 32) {
         int a, len; bool bad;
         seq_span(cu, n_seq, T, sb + lane, a, len, bad);
         int nc = (len + Lc - 1) / Lc;
@@ -84,6 +87,7 @@ __device__ inline void seq_chunks(const int32_t* cu, int n_seq, int T, int Lc, i
             int l = s - sb;
             nck = __shfl_sync(full, nc, l);
             first = base + __shfl_sync(full, incl, l) - nck;
+            if (first + nck > bound) nck = 0;
             return;
         }
         base += __shfl_sync(full, incl, 31);

@@ -23,6 +23,8 @@
 // when it is done, so the channel warps never wait for one another.  Every wait on an mbarrier is bounded: if
 // it runs out, the warp raises MDRAFT_DEV_WAIT_EXPIRED and stops; the copy warp first gives the copies it still
 // has in flight a bounded chance to land (they target this block's shared memory).
+#include <limits.h>
+
 #include <type_traits>
 
 #include "channel_scan.cuh"
@@ -229,7 +231,8 @@ __global__ void __launch_bounds__(SUB * kBoxCols + 32, PER_SM) chunk_kernel(cons
         }
     }
 
-    const ChunkInfo ci = kOut && SUB <= 2 && c.longest_first ? ranked_sequence(c.cu, c.n_seq, c.T, cidx) : find_chunk(c.cu, c.n_seq, c.T, c.chunk_len, cidx);
+    // (Blocks of 256 channels take unsplit sequences only: one chunk each, which always have room.)
+    const ChunkInfo ci = kOut && SUB <= 2 && c.longest_first ? ranked_sequence(c.cu, c.n_seq, c.T, cidx) : find_chunk(c.cu, c.n_seq, c.T, c.chunk_len, SUB == 2 ? INT_MAX : c.n_chunks_bound, cidx);
     if (ci.seq < 0) { if (kOut) grid_wait(); return; }
     if (!kOut) {
         // No summary is needed for an unsplit sequence or for a sequence's last chunk; in conv-only mode the only
@@ -447,7 +450,7 @@ __global__ void __launch_bounds__(kCarryGroups * 32, 1) carry_kernel(const __gri
     // Sequence offsets, slots and the starting state are inputs of the call: the summary pass ahead of this kernel
     // let it start only after everything before the call had finished, so they may be read before the wait below.
     int first, nck;
-    seq_chunks(p.cu, p.n_seq, p.T, p.chunk_len, s, first, nck);
+    seq_chunks(p.cu, p.n_seq, p.T, p.chunk_len, p.n_chunks_bound, s, first, nck);
     const int islot = load_slot(p.init_slot, s), fslot = load_slot(p.final_slot, s);
     const bool slots_ok = islot < p.pool.n_slots && fslot < p.pool.n_slots;
     float4 carry = make_float4(0.f, 0.f, 0.f, 0.f);

@@ -299,7 +299,7 @@ __global__ void __launch_bounds__(kThreads, 3) ssd_chunk_state_kernel(const SsdP
     // lets them read the call's inputs without a wait of their own.
     grid_wait();
     grid_release_dependents();
-    const ChunkInfo ci = find_chunk(p.cu, p.n_seq, p.T, Q, cidx);
+    const ChunkInfo ci = find_chunk(p.cu, p.n_seq, p.T, Q, p.n_chunks_bound, cidx);
     if (ci.seq < 0) return;
     const int islot = load_slot(p.init_slot, ci.seq), fslot = load_slot(p.final_slot, ci.seq);
     if (islot >= p.pool.n_slots || fslot >= p.pool.n_slots) return;   // reported by the state-passing kernel
@@ -405,14 +405,15 @@ __global__ void __launch_bounds__(kPassThreads) ssd_state_passing_kernel(const S
     // Sequence offsets, slots and the starting state are inputs of the call: the kernel ahead let this one start only
     // after everything before the call had finished, so they are read before the wait below.
     int first, nck;
-    seq_chunks(p.cu, p.n_seq, p.T, Q, s, first, nck);   // whole warps call this
+    seq_chunks(p.cu, p.n_seq, p.T, Q, p.n_chunks_bound, s, first, nck);   // whole warps call this
     int s0, len; bool bad;   // malformed offsets: the sequence has no chunk and leaves its final slot alone
     seq_span(p.cu, p.n_seq, p.T, s, s0, len, bad);
     if (bad && blockIdx.x == 0 && threadIdx.x == 0) flag(p.dev_status, MDRAFT_DEV_BAD_SEQLENS);
+    const bool left_out = bad || (len > 0 && nck == 0);
     const int islot = load_slot(p.init_slot, s), fslot = load_slot(p.final_slot, s);
     const bool slots_ok = islot < p.pool.n_slots && fslot < p.pool.n_slots;
     if (!slots_ok && blockIdx.x == 0 && threadIdx.x == 0) flag(p.dev_status, MDRAFT_DEV_BAD_SLOT);
-    const bool mine = slots_ok && !bad && idx < D * (N / 4);
+    const bool mine = slots_ok && !left_out && idx < D * (N / 4);
     // consecutive lanes: the two halves of a unit, then consecutive channels of one head and one state group, so that the
     // 16-byte operand units a warp writes are contiguous (its 32-byte reads of the chunk states each fill a sector)
     const int sub = idx & 1, ch = (idx >> 1) % P, g = (idx / (2 * P)) % (N / 8), head = mine ? idx / (2 * P * (N / 8)) : 0, d = head * P + ch;
@@ -488,7 +489,7 @@ __global__ void __launch_bounds__(kThreads, 3) ssd_chunk_scan_kernel(const SsdPr
     grid_release_dependents();
     // Offsets, slots and the C / B rows are inputs of the call (complete before its first kernel let the others start): the
     // look-ups and the copies of C and B run while the kernels ahead are still at work.
-    const ChunkInfo ci = find_chunk(p.cu, p.n_seq, p.T, Q, cidx);
+    const ChunkInfo ci = find_chunk(p.cu, p.n_seq, p.T, Q, p.n_chunks_bound, cidx);
     if (ci.seq < 0) { grid_wait(); return; }
     const int islot = load_slot(p.init_slot, ci.seq), fslot = load_slot(p.final_slot, ci.seq);
     if (islot >= p.pool.n_slots || fslot >= p.pool.n_slots) { grid_wait(); return; }

@@ -236,6 +236,30 @@ def test_prefill_flags_bad_sequence_lengths_and_slots():
     assert float(out[:10].abs().max()) > 0 and float(out[10:].abs().max()) == 0.0
 
 
+@pytest.mark.parametrize("powers", [False, True])
+def test_overlapping_sequences_stay_inside_the_workspace(powers):
+    """Offsets {0, T, 0, T} make two sequences of all T rows around a malformed one: twice the chunks that offsets in order can make.
+    The sequence whose chunks find no room is left out with its slot, and nothing beyond the workspace is written."""
+    T, Dn, act, chunk_len = 300, 136, "bf16", 16
+    prob = parity.make_problem(parity.small_config(Dn, act, 1), [T], general_A=not powers)
+    flags = md.MDRAFT_DT_SOFTPLUS | (md.MDRAFT_A_POWERS if powers else 0)
+    lay = upload_layer(prob.params, act, flags)
+    cache = md.StateCache(1, 3, Dn, act=torch.bfloat16)
+    cache.ssm.fill_(5.0)
+    dev = [to_device(a, torch.bfloat16) for a in (prob.x, prob.z, prob.dt, prob.B, prob.C)]
+    out = torch.full((T, Dn), float("nan"), dtype=torch.bfloat16, device="cuda")
+    need = md.mdraft_prefill_workspace_bytes(lay, T, 3, T, chunk_len)
+    ws = torch.full((2 * need,), 77, dtype=torch.uint8, device="cuda")   # the second half is not the call's
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    md.mdraft_conv_scan_prefill(lay, cache, 0, *dev, out, i32([0, T, 0, T]), T, None, i32([0, 1, 2]), ws[:need], chunk_len, status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == md.MDRAFT_DEV_BAD_SEQLENS
+    assert bool((ws[need:] == 77).all()) and bool((cache.ssm[0, 1:] == 5.0).all())
+    o_out, _, o_h = run_oracle_prefill(prob, flags)
+    assert_close(out.float().cpu().numpy(), o_out, TOL[act], "out")
+    assert_close(cache.ssm[0, :1].cpu().numpy(), o_h, TOL_STATE, "state")
+
+
 @pytest.mark.parametrize("act", ["f32", "bf16"])
 def test_batch_of_empty_sequences_moves_the_state_and_needs_no_workspace(act):
     """No tokens at all: every sequence's final state is its starting state, copied from slot to slot (zeros where

@@ -227,6 +227,26 @@ def test_ssd_malformed_offsets_leave_output_and_slots_alone(init):
     assert not bool(out[:70].isnan().any()) and bool(out[70:].isnan().all())
 
 
+def test_ssd_overlapping_sequences_stay_inside_the_workspace():
+    """Offsets {0, T, 0, T}: twice the chunks that offsets in order can make.  The sequence whose chunks find no room is left out with
+    its slot, and nothing beyond the workspace is written."""
+    T = 300
+    cfg, prm, arrs, cu = make(128, [T])
+    lay, cache, dev = upload_ssd_layer(prm), ssd_cache(3, 128), [to_device(a, BF) for a in arrs]
+    cache.ssm.fill_(5.0)
+    out = torch.full((T, 128), float("nan"), dtype=BF, device="cuda")
+    need = md.mdraft_ssd_prefill_workspace_bytes(lay, T, 3)
+    ws = torch.full((2 * need,), 77, dtype=torch.uint8, device="cuda")   # the second half is not the call's
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    md.mdraft_ssd_prefill(lay, cache, 0, *dev, out, i32([0, T, 0, T]), None, i32([0, 1, 2]), ws[:need], status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == md.MDRAFT_DEV_BAD_SEQLENS
+    assert bool((ws[need:] == 77).all()) and bool((cache.ssm[0, 1:] == 5.0).all())
+    o_out, _, o_h = oracle.ssd_prefill(oracle.ssd_layer_from_params(prm), *arrs)
+    assert_close(out.float().cpu().numpy(), o_out, TOL["bf16"], "out")
+    assert_close(cache.ssm[0, :1].cpu().numpy(), o_h, TOL_STATE, "state")
+
+
 def _ssd_case(seed):
     g = np.random.default_rng(5000 + seed)
     Dn = int(g.choice([64, 128, 192, 320]))
