@@ -397,7 +397,7 @@ typedef struct {
  *   x, z, out : (T, D) bf16, strides ldx, ldz, ldo          dt : (T, H) bf16, stride lddt (elements; any value >= H)
  *   B, C      : (T, 128) bf16, strides ldb, ldc (multiples of 8 elements, base 16-byte aligned)
  *   cu_seqlens, init_slot, final_slot, dev_status, stream: as in mdraft_conv_scan_prefill (cu_seqlens may be NULL
- *   for one sequence)
+ *   for one sequence), but no sequence may start from another's final_slot, however long it is
  *   workspace : device scratch of at least mdraft_ssd_prefill_workspace_bytes(...) bytes, 256-byte aligned
  */
 size_t mdraft_ssd_prefill_workspace_bytes(const mdraft_ssd_layer *layer, int32_t total_tokens, int32_t n_seq);

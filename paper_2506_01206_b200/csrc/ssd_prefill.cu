@@ -14,12 +14,12 @@
 //      cores (tcgen05.mma, bf16 operands, fp32 accumulator in tensor memory); Xw is split into a bf16 value and a bf16
 //      remainder (two products into one accumulator) so that the state keeps fp32-level accuracy.  What kernel 3 needs
 //      of this work is handed over through the workspace: Xd = Delta u already in operand layout, u, and the running
-//      log-decays of the chunk's rows; the sequence's last chunk also leaves the conv window.
+//      log-decays of the chunk's rows.
 //   2. ssd_state_passing: per (channel, 4 states) the chunk states of a sequence are chained in token order; every
 //      chunk's incoming state is left in the operand layout the next kernel wants, the final state goes to its slot.
 //   3. ssd_chunk_scan: per (head, chunk) G = C B^T (issued before the kernel's wait: inputs only), the causal decay mask applied
 //      to G on its way out of tensor memory and back into it as the operand of Y = (G o L) Xd; C H_in^T on the tensor cores;
-//      then skip term, gate and store.  It touches no x, dt or conv weight: with the masked G in tensor memory its shared
+//      then skip term, gate and store; the sequence's last chunk also leaves the conv window.  It touches no dt or conv weight, and x for that only: with the masked G in tensor memory its shared
 //      memory is two operand tiles, and three blocks share an SM (all blocks of a 2048-token layer in one wave).
 //
 // Operands live in shared memory in the tensor core's canonical un-swizzled layout: 16-byte units of 8 bf16 values,
@@ -324,14 +324,7 @@ __global__ void __launch_bounds__(kThreads, 3) ssd_chunk_state_kernel(const SsdP
 
     bool ok = mbar_wait_bounded(&sm.bar_tma, 0u);
     uint32_t xr[kRowsPerWarp + 3];
-    if (ok) {
-        load_rows(xs_ext, xr);
-        // the sequence's last chunk leaves the window: the last three raw inputs (extended rows rows .. rows + 2)
-        if (ci.k == ci.nck - 1 && fslot >= 0 && warp < 3) {
-            __nv_bfloat16* dc = static_cast<__nv_bfloat16*>(p.pool.conv) + (size_t)fslot * p.pool.conv_slot_stride + (size_t)warp * p.L.d_inner + head * P + 2 * lane;
-            *reinterpret_cast<uint32_t*>(dc) = reinterpret_cast<const uint32_t*>(xs_ext)[(rows + warp) * (P / 2) + lane];
-        }
-    }
+    if (ok) load_rows(xs_ext, xr);
     __syncthreads();   // every thread holds its rows: the x tile may be overwritten
     if (ok) {
         unsigned char* xd_g = reinterpret_cast<unsigned char*>(p.ws_xd) + ((size_t)cidx * H + head) * ((P / 8) * kXdColBytes);
@@ -480,6 +473,7 @@ constexpr int kYPitch = P + 4;   // floats of a staged y row: written as 16 byte
 static_assert(sizeof(float) * Q * kYPitch <= N / 8 * Q * 16 + kZOffset, "the y staging rows must end before the z box");
 static_assert((P / 8) * kXdColBytes <= N / 8 * Q * 16 && 2 * N * P * 2 <= N / 8 * Q * 16, "re-used regions too small");
 static_assert(3 * (sizeof(ScanSmem) + 1024 + 1024) <= 227 * 1024, "three blocks per SM");
+static_assert(kThreads / 32 == 8 && kW - 1 == 3, "the window's rows go to warps 5 to 7");
 
 __global__ void __launch_bounds__(kThreads, 3) ssd_chunk_scan_kernel(const SsdPrefillArgs p, const __grid_constant__ SsdMaps maps) {
     extern __shared__ __align__(1024) unsigned char s_raw[];
@@ -548,8 +542,21 @@ __global__ void __launch_bounds__(kThreads, 3) ssd_chunk_scan_kernel(const SsdPr
         if (cb1 <= rb) tmem_ld32(tG + lanes + cb1 * 32, g1);
         tc_fence_before();
     }
+    // The sequence's last chunk leaves the window: the last three raw inputs, with rows of the starting window where the sequence is
+    // shorter.  Fetched here, stored behind the wait: the first chunk's starting window may come from the same slot, and
+    // kernel 1 is done with it then.  (From kernel 2, whose threads wait for their chunk states, the store cost 2048 x 1536 tokens 1.7 us.)
+    uint32_t* win_to = nullptr;
+    uint32_t win = 0u;
+    if (warp > 4 && ci.k == ci.nck - 1 && fslot >= 0) {
+        const int j = warp - 5, t = ci.t1 - (kW - 1) + j, dw = head * P + 2 * lane, D = p.L.d_inner;
+        __nv_bfloat16* const conv = static_cast<__nv_bfloat16*>(p.pool.conv) + dw;
+        win_to = reinterpret_cast<uint32_t*>(conv + (size_t)fslot * p.pool.conv_slot_stride + (size_t)j * D);
+        if (t >= ci.s0) win = *reinterpret_cast<const uint32_t*>(p.x + (size_t)t * p.ldx + dw);
+        else if (islot >= 0) win = *reinterpret_cast<const uint32_t*>(conv + (size_t)islot * p.pool.conv_slot_stride + (size_t)(t - ci.s0 + kW - 1) * D);
+    }
     __syncthreads();
     grid_wait();   // the incoming states and the running decays are the work of the kernels just before
+    if (win_to) *win_to = win;
     if (g_ok && tid == 0) {   // G is complete: its B rows make room for the incoming state
         mbar_expect_tx(&sm.bar_dec, Q * 4);
         bulk_load(sm.csl, p.ws_csl + ch_head * Q, Q * 4, &sm.bar_dec);

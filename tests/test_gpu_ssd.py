@@ -99,6 +99,33 @@ def test_ssd_prefill_in_pieces_equals_whole():
     assert np.array_equal(b[2], whole[2]) and np.array_equal(b[1], whole[1])
 
 
+def test_ssd_prefill_in_place_equals_slot_to_slot():
+    """Starting and final slot the same: the first chunk reads the window that the call replaces.  Sequences of one chunk and several,
+    shorter than the window, and empty."""
+    lens = [300, 1, 0, 129, 2, 3, 128, 700]
+    cfg, prm, arrs, cu = make(192, lens)
+    S, T = len(lens), sum(lens)
+    lay, dev, status = upload_ssd_layer(prm), [to_device(a, BF) for a in arrs], torch.zeros(1, dtype=torch.int32, device="cuda")
+    ws = torch.empty(md.mdraft_ssd_prefill_workspace_bytes(lay, T, S), dtype=torch.uint8, device="cuda")
+    g = np.random.default_rng(8)
+    hi, ci = g.normal(size=(S, 192, N)).astype(np.float32), gen.round_to_act(g.normal(size=(S, 3, 192)).astype(np.float32), "bf16")
+    res = []
+    for final in (np.arange(S), np.arange(S, 2 * S)):
+        cache = ssd_cache(2 * S, 192)
+        cache.ssm[0, :S], cache.conv[0, :S] = torch.from_numpy(hi).cuda(), to_device(ci, BF)
+        out = torch.full((T, 192), float("nan"), dtype=BF, device="cuda")
+        md.mdraft_ssd_prefill(lay, cache, 0, *dev, out, i32(cu), i32(np.arange(S)), i32(final), ws, status)
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0
+        f = torch.from_numpy(final).cuda()
+        res.append((out, cache.ssm[0, f], cache.conv[0, f]))
+    assert all(torch.equal(a, b) for a, b in zip(*res))
+    o_out, o_conv, o_h = oracle.ssd_prefill(oracle.ssd_layer_from_params(prm), *arrs, cu_seqlens=cu, conv_init=ci, h_init=hi)
+    assert_close(res[0][0].float().cpu().numpy(), o_out, TOL["bf16"], "out")
+    assert_close(res[0][1].cpu().numpy(), o_h, TOL_STATE, "states")
+    assert np.array_equal(res[0][2].float().cpu().numpy().astype(np.float64), o_conv)
+
+
 def test_ssd_prefill_raw_step_size_and_zero_step_size():
     cfg, prm, arrs, cu = make(128, [200])
     x, z, dt, B, C = arrs
