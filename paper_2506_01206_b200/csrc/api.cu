@@ -412,17 +412,20 @@ int run_prefill(const PrefillCall& call, const PrefillPlan& pl, int32_t n_layers
     return launch_prefill<ML>(b, act, pl.form, call.stream) == cudaSuccess ? MDRAFT_OK : MDRAFT_ERR_CUDA;
 }
 
-// The one-kernel form (csrc/prefill_cluster.cu) of a call, or blocks = 0 where the plan above is the faster one.  Measured over 900 calls of 1 to
-// 16 layers, 1 to 8 sequences of 10 to 4000 tokens, 64 to 1536 channels, fp32 and bf16, either A, under 17 forms each:
+// The one-kernel form (csrc/prefill_cluster.cu) of a call, or blocks = 0 where the plan above is the faster one.  Both are estimated:
 //  - the one-kernel form takes kOne us and so much per block of a cluster, and per token of a chunk kLatency us plus kShare for every
-//    further warp on a scheduler (standard deviation 7 %);
+//    further warp on a scheduler; short chunks of one block or two some 0.1 us a token more where they fill the machine; and 1.05 of all that
+//    where clusters of three blocks and more fill SMs that they share: then some no longer fit beside the rest, most with another call's
+//    blocks ahead of them (36 clusters of 7 blocks, 1128 channels x 1178 tokens: 28.3 us alone, 31.5 in a row; estimated 24.7);
 //  - the other takes kSplit + kSplitWork per token of work of a scheduler where it cuts sequences, kWhole + kWholeToken per token
-//    of the longest where it does not (15 %), so the one-kernel form has to promise 12 % less, and 20 % from sixteen sequences on, which the narrow form with four blocks to an SM
-//    serves better than that (20 x 1508 x 64, general A: 32.7 us, in one kernel 37.9), and 25 % where one layer's one sequence is long for its width (1500 x 1536: 26.8 us, in
-//    one kernel 29.6; 1300 x 1200 25.5 and 28.6; 3925 x 368 28.5 and 34.4).
-// It wins where the work is small: 256 x 64 fp32 9.2 -> 6.4 us, 256 x 768 bf16 12.3 -> 8.1, 1024 x 128 to 256 0.76 of the time; in the mean over
-// those calls 16 % (12 of them lose 3 % or more).  It loses where the work fills the machine, since its clusters leave a seventh of the SMs out and
-// its channel groups are narrow: 1777 x 1536, general A, 35.5 against 41.4 at best, 4096 x 1536 52 against 77.
+//    of the longest where it does not.  That is good to 15 %, and high where a cut call fills an SM with blocks that finish together (24-token chunks of
+//    1174 x 1112 18.7 us, estimated 21.8): the one-kernel form has to promise 14 % less, and 17 or 20 % (general A) where the other cuts
+//    and has much work.
+// It wins where the work is small: 256 x 64 fp32 9.2 -> 6.4 us, 256 x 768 bf16 12.3 -> 8.1, 1024 x 128 to 256 0.76 of the time; over 5709 calls that the rule
+// gives to it (1 to 24 layers, 1 to 48 sequences of 2 to 4500 tokens, 32 to 1536 channels; eight calls in a graph, either way) it takes 0.765 of
+// the other's time in the mean, and 19 of them lose 3 to 11 %.  (A margin of 12 % alone, 20 from sixteen sequences and 25 for a single long one on, had 223 of 8727 lose
+// 3 to 45 %; the tighter ones leave 1.4 % of that sample's time unwon in other calls.)  It loses where the work fills the machine, since its clusters
+// leave a seventh of the SMs out and its channel groups are narrow: 1777 x 1536, general A, 35.5 against 41.4 at best, 4096 x 1536 52 against 77.
 // It is for calls whose sequences do not look at one another's slots: a cluster reads its starting slot when it comes to run, by when another
 // sequence's may have stored its final state, where the three kernels take the state and window that a cut sequence starts
 // from ahead of the pass that stores.  The slots are on the device, so where several sequences have both and the plan cuts them, the caller of
@@ -434,21 +437,23 @@ ClusterForm cluster_form(const mdraft_layer* L, int n_layers, int T, int n_seq, 
     const int general = !(L->flags & MDRAFT_A_POWERS), sms = sm_count();
     const int64_t groups = (int64_t)n_layers * ((L->d_inner + kClusterCols - 1) / kClusterCols), clusters = groups * n_seq;
     const double work = (double)T * groups / (4 * sms);
-    const double margin = n_seq >= 16 ? 0.8 : n_seq * n_layers == 1 && work > 75.0 ? 0.75 : 0.88;
     if (clusters > 8 * sms || (L->d_inner + kClusterCols - 1) / kClusterCols > 65535 || (int64_t)n_layers * n_seq > 65535) return {0, 0};
     ClusterForm best = {0, 0};
     double least = kSplit + work * kSplitWork[general] + (n_seq > 1 ? kSplitSeqs : 0.0);
     const double blocks = (double)n_layers * n_seq * ((L->d_inner + kPrefillThreads - 1) / kPrefillThreads), rounds = 1.2 * blocks / sms;
     const double whole = kWhole + max_seqlen * kWholeToken * (general ? kGeneralOne : 1.0) * (rounds > 1.0 ? rounds : 1.0);
-    least = margin * (whole < least ? whole : least);
+    least = whole < least ? 0.86 * whole : (work <= 40.0 ? 0.86 : general ? 0.8 : 0.83) * least;
     auto weigh = [&](int c, int w) {
         const int share = prefill_cluster_share(c, clusters);
         if (share * w > 16) return;   // the warps of an SM, 128 registers a thread
         const double busy = share * w > 4 ? share * w / 4.0 - 1.0 : 0.0;   // further warps on the fullest scheduler
-        const double t = kOne + (c > 1 ? kCluster : 0.0) + kBlock * c + kWarp * busy + prefill_cluster_chunk(max_seqlen, c * w, !general) * (kLatency[general] + kShare[general] * busy);
+        const double places = (double)clusters * c / (share * sms);            // of the SMs' room
+        const int chunk = prefill_cluster_chunk(max_seqlen, c * w, !general);
+        double t = kOne + (c > 1 ? kCluster : 0.0) + kBlock * c + kWarp * busy + chunk * (kLatency[general] + kShare[general] * busy);
+        if (c <= 2 && places > 0.4) t += 0.1 * (places - 0.4) * (chunk < 16 ? chunk : 16);
+        if (c >= 3 && share >= 2 && places > 0.72) t *= 1.05;
         if (t < least) { least = t; best = {c, w}; }
     };
-    weigh(1, 2);
     for (int w = 4; w <= kClusterMaxWarps; w *= 2)
         for (int c = 1; c <= kClusterMaxBlocks; ++c) weigh(c, w);
     return best;
@@ -483,6 +488,15 @@ __global__ void classify_A_kernel(const float* A, int D, int N, int32_t* res) {
 }
 
 }  // namespace
+
+// The form of a call's first launch where none of its sequences starts from a slot: 256 * blocks + warps of the one-kernel form, 0 for the plan's
+// own kernels.  For the tests, which have to know what they run; no part of the interface.
+extern "C" int32_t mdraft_internal_prefill_form(const mdraft_layer* layer, int32_t n_layers, int32_t total_tokens, int32_t n_seq, int32_t max_seqlen) {
+    if (check_layer(layer) != MDRAFT_OK || n_layers <= 0 || total_tokens <= 0 || n_seq <= 0 || max_seqlen <= 0) return 0;
+    const int32_t most = prefill_most_layers(n_seq);
+    const ClusterForm f = cluster_form(layer, n_layers < most ? n_layers : most, total_tokens, n_seq, max_seqlen < total_tokens ? max_seqlen : total_tokens, nullptr);
+    return f.blocks * 256 + f.warps;
+}
 
 size_t mdraft::prefill_scratch_bytes(const mdraft_layer* layer, int32_t total_tokens, int32_t n_seq, int32_t max_seqlen, const mdraft_prefill_opts* opts,
                                      size_t available) {

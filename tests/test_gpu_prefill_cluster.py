@@ -7,6 +7,8 @@ decays by the exponential of the summed step sizes instead of a product of one p
 may be 100 * 2^-22 = 2.4e-5 apart; the largest of some 10^5 elements, taken relative to its value or the RMS, lies up to four times that
 out: 1e-4.  bf16 outputs are besides rounded once each, 2^-8 of the value at most apart when a tie falls, with the RMS floor 2^-7."""
 
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -22,19 +24,30 @@ from paper_2506_01206_b200.device_inputs import i32, to_device, torch_act, uploa
 
 TOL_FORMS = 1e-4
 
-SHAPES = [   # act, D, lengths
-    ("f32", 8, [1]), ("bf16", 8, [3]), ("bf16", 32, [64]), ("f32", 64, [256]), ("bf16", 40, [65, 1, 0, 4, 257]), ("f32", 200, [33, 500]),
-    ("bf16", 768, [256]), ("bf16", 1536, [130]), ("f32", 1000, [17, 90]), ("bf16", 72, [511]), ("f32", 24, [2, 0, 1, 500]), ("bf16", 1496, [31, 32, 33])]
+# act, D, lengths, (blocks, warps) that the rule gives with A = powers and with a general A; (0, 0): so short that the output pass alone is as fast
+SHAPES = [
+    ("f32", 8, [1], (0, 0), (0, 0)), ("bf16", 8, [3], (0, 0), (0, 0)), ("bf16", 1496, [31, 32, 33], (0, 0), (0, 0)),
+    ("bf16", 32, [64], (4, 4), (4, 4)), ("f32", 64, [256], (8, 8), (8, 8)), ("bf16", 40, [65, 1, 0, 4, 257], (6, 4), (6, 4)),
+    ("f32", 200, [33, 500], (6, 8), (6, 8)), ("bf16", 768, [256], (4, 8), (4, 8)), ("bf16", 1536, [130], (5, 8), (5, 8)),
+    ("f32", 1000, [17, 90], (3, 8), (3, 8)), ("bf16", 72, [511], (8, 8), (8, 8)), ("f32", 24, [2, 0, 1, 500], (8, 8), (8, 8)),
+    ("bf16", 768, [64, 63, 1, 4], (1, 8), (1, 8)), ("f32", 768, [48, 3, 0, 47], (1, 4), (3, 4)), ("bf16", 768, [64, 2], (2, 8), (2, 8)),
+    ("f32", 136, [32, 32], (1, 8), (2, 4)), ("f32", 520, [300, 299], (7, 4), (7, 4))]
 
 
-@pytest.mark.parametrize("act,Dn,lens", SHAPES)
+def form(layer, n_layers, lens):
+    """(blocks, warps) of the one-kernel form that a call without starting slots takes, (0, 0) for the plan's own kernels."""
+    f = md.load_library().mdraft_internal_prefill_form(ctypes.byref(layer.c()), n_layers, sum(lens), len(lens), max(lens))
+    return f // 256, f % 256
+
+
+@pytest.mark.parametrize("act,Dn,lens,powers_form,general_form", SHAPES)
 @pytest.mark.parametrize("general_A", [False, True])
-def test_one_kernel_form_matches_oracle_and_the_general_form(act, Dn, lens, general_A):
+def test_one_kernel_form_matches_oracle_and_the_general_form(act, Dn, lens, powers_form, general_form, general_A):
     cfg = parity.small_config(Dn, act, len(lens), cid=97)
     prob = parity.make_problem(cfg, lens, conv_bias=True, general_A=general_A)
     flags = md.MDRAFT_DT_SOFTPLUS | (0 if general_A else md.MDRAFT_A_POWERS)
     lay = upload_layer(prob.params, act, flags)
-    assert md.mdraft_prefill_stack_launches(lay, 1, sum(lens), len(lens), max(lens)) == 1
+    assert form(lay, 1, lens) == (general_form if general_A else powers_form)
     ci, hi = random_state(cfg, len(lens), 7)
     for init, strided, in_place in ((False, False, False), (True, True, False), (True, False, True)):
         state = (ci, hi) if init else (None, None)
@@ -57,7 +70,7 @@ def test_one_kernel_form_of_a_stack_and_its_faults(act):
     probs = [parity.make_problem(parity.small_config(Dn, act, 3, cid=70 + l), lens) for l in range(NL)]
     flags = md.MDRAFT_DT_SOFTPLUS | md.MDRAFT_A_POWERS
     lays = [upload_layer(p.params, act, flags) for p in probs]
-    assert md.mdraft_prefill_stack_launches(lays[0], NL, sum(lens), 3, max(lens)) == 1
+    assert form(lays[0], NL, lens) == (5, 4)
     cache = md.StateCache(NL, 3, Dn, act=tdt)
     cache.ssm.fill_(5.0)
     out = torch.full((NL, sum(lens), Dn), 9.0, dtype=tdt, device="cuda")
@@ -89,7 +102,7 @@ def test_sequences_may_start_from_a_slot_that_one_of_them_stores_to(act, Dn, n_l
     probs = [parity.make_problem(parity.small_config(Dn, act, S, cid=60 + l), lens) for l in range(n_layers)]
     flags = md.MDRAFT_DT_SOFTPLUS | md.MDRAFT_A_POWERS
     lays = [upload_layer(p.params, act, flags) for p in probs]
-    assert md.mdraft_prefill_stack_launches(lays[0], n_layers, T, S, max(lens)) == 1
+    assert form(lays[0], n_layers, lens) != (0, 0)
     ci, hi = random_state(probs[0].cfg, 1, 7)
     ins = [tuple(to_device(a, tdt) for a in (p.x, p.z, p.dt, p.B, p.C)) for p in probs]
     init, final = i32([0] * S), i32(np.arange(S))
