@@ -299,8 +299,10 @@ __global__ void __launch_bounds__(kClusterMaxWarps * 32, 2) cluster_kernel(const
         if (blocks > 1) cluster_arrive();   // this block no longer reads its neighbours; nobody stores a final state before all have come here
         __syncthreads();
         const float before = my_sum[32 + lane];
+        // (A block's first chunk starts from what the block starts from: a decay over no tokens is 1 for every A, also for an infinite one.)
 #pragma unroll
-        for (int q = 0; q < kN / 4; ++q) cs.set_state(q, fold4(decay4(a4[q], before), share.start[q][lane], mine[q * 32 + lane]));
+        for (int q = 0; q < kN / 4; ++q)
+            cs.set_state(q, warp == 0 ? share.start[q][lane] : fold4(decay4(a4[q], before), share.start[q][lane], mine[q * 32 + lane]));
 #pragma unroll
         for (int j = 0; j < kW - 1; ++j) cs.win[j] = win0[j];
         __syncwarp();   // the summaries make way for the widened tiles

@@ -129,3 +129,24 @@ def test_sequences_may_start_from_a_slot_that_one_of_them_stores_to(act, Dn, n_l
         assert_close(res[0][0][l].float().cpu().numpy(), o_out, TOL[act], f"out of layer {l}")
         assert_close(res[0][1][l].cpu().numpy(), o_h, TOL_STATE, f"states of layer {l}")
         assert np.array_equal(res[0][2][l].float().cpu().numpy().astype(np.float64), o_conv)
+
+
+@pytest.mark.parametrize("act", ["f32", "bf16"])
+@pytest.mark.parametrize("general_A", [False, True])
+def test_an_infinite_A_forgets_and_nothing_else(act, general_A):
+    """-exp(A_log) of a large A_log is -inf: such a state is its last input alone.  In every form, also where a chunk's decay is formed from a sum of
+    step sizes (inf times the 0 of a sequence's first chunk is not a number)."""
+    Dn, lens = 136, [256]
+    prob = parity.make_problem(parity.small_config(Dn, act, 1, cid=97), lens, general_A=general_A)
+    prob.params.A[::3] = -np.inf
+    if general_A:
+        prob.params.A[1::3, 5] = -np.inf
+    flags = md.MDRAFT_DT_SOFTPLUS | (0 if general_A else md.MDRAFT_A_POWERS)
+    assert form(upload_layer(prob.params, act, flags), 1, lens) != (0, 0)
+    state = random_state(prob.cfg, 1, 7)
+    o_out, o_conv, o_h = run_oracle_prefill(prob, flags, *state)
+    for chunk_len in (0, 32, 4096):
+        got = run_gpu_prefill(prob, flags, chunk_len, *state)
+        assert_close(got[0], o_out, TOL[act], f"out, chunk_len {chunk_len}")
+        assert_close(got[2], o_h, TOL_STATE, f"final SSM state, chunk_len {chunk_len}")
+        assert np.array_equal(got[1], o_conv)
