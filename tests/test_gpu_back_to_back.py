@@ -13,6 +13,7 @@ import torch
 
 import gen
 import parity
+from test_gpu_prefill_cluster import form
 
 pytestmark = pytest.mark.gpu
 
@@ -115,6 +116,35 @@ def test_prefills_in_a_row_on_one_workspace(act, powers):
 
     def run_layer(l):
         md.mdraft_conv_scan_prefill(lays[l], cache, l, *ins[l], outs[l], cu_d, max_len, init, final, ws, chunk_len, status)
+
+    _check(run_layer, NL, lambda l: [outs[l], cache.ssm[l, S:], cache.conv[l, S:]])
+    assert int(status.item()) == 0
+
+
+@pytest.mark.parametrize("act", ["bf16", "f32"])
+@pytest.mark.parametrize("powers", [False, True])
+@pytest.mark.parametrize("lens,Dn", [([611], 264), ([150, 3, 77], 200)])
+def test_one_kernel_prefills_in_a_row(act, powers, lens, Dn):
+    """Calls in the one-kernel form behind one another and behind calls in three kernels, which share a workspace that the former do not use."""
+    NL, S, T, tdt = 6, len(lens), int(sum(lens)), torch_act(act)
+    flags = md.MDRAFT_DT_SOFTPLUS | (md.MDRAFT_A_POWERS if powers else 0)
+    cfg = gen.Config(96, "row", NL, Dn, 16, 4, act, S, (1, 1), "none", 0, 5)
+    probs = [parity.make_problem(cfg, lens, layer=l, conv_bias=True, general_A=not powers) for l in range(NL)]
+    lays = [upload_layer(pr.params, act, flags) for pr in probs]
+    assert form(lays[0], 1, lens) != (0, 0)
+    ins = [[to_device(a, tdt) for a in (pr.x, pr.z, pr.dt, pr.B, pr.C)] for pr in probs]
+    outs = [torch.empty((T, Dn), dtype=tdt, device="cuda") for _ in range(NL)]
+    cache = md.StateCache(NL, 2 * S, Dn, act=tdt)
+    g = np.random.default_rng(12)
+    cache.ssm[:, :S] = torch.from_numpy(g.normal(size=(NL, S, Dn, 16)).astype(np.float32)).cuda()
+    cache.conv[:, :S] = to_device(g.normal(size=(NL, S, 3, Dn)).astype(np.float32), tdt)
+    max_len, chunk_lens = max(lens), [0, 0, 48, 0, 48, 48]
+    ws = torch.empty(max(md.mdraft_prefill_workspace_bytes(lays[0], T, S, max_len, c) for c in (0, 48)), dtype=torch.uint8, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    cu_d, init, final = i32(probs[0].cu), i32(np.arange(S)) if S == 1 else None, i32(np.arange(S, 2 * S))
+
+    def run_layer(l):
+        md.mdraft_conv_scan_prefill(lays[l], cache, l, *ins[l], outs[l], cu_d, max_len, init, final, ws, chunk_lens[l], status)
 
     _check(run_layer, NL, lambda l: [outs[l], cache.ssm[l, S:], cache.conv[l, S:]])
     assert int(status.item()) == 0

@@ -21,6 +21,7 @@ import oracle
 import parity
 from parity import TOL, TOL_STATE, assert_close
 from test_gpu_parity_small import run_gpu_prefill, run_oracle_prefill
+from test_gpu_prefill_cluster import form
 from test_gpu_tree import TreeRig
 from test_gpu_tree_proj import ProjRig
 
@@ -99,6 +100,47 @@ def test_prefill_outside_the_recipe(regime, act, powers):
         assert_close(g_out, o_out, TOL[act], f"out, chunk_len {chunk_len}")
         assert_close(g_h, o_h, TOL_STATE, f"final SSM state, chunk_len {chunk_len}")
         assert np.array_equal(g_conv, o_conv)
+
+
+@pytest.mark.parametrize("regime", [r for r in REGIMES if r != "zero_dt"])   # the one-kernel form forms its step sizes by softplus
+@pytest.mark.parametrize("act", ["f32", "bf16"])
+@pytest.mark.parametrize("powers", [False, True])
+def test_one_kernel_prefill_outside_the_recipe(regime, act, powers):
+    g = np.random.default_rng(case_seed(regime, act, powers, 3))
+    for lens, have_state in (([150], True), ([150, 3, 77], False)):
+        prob = parity.make_problem(parity.small_config(200, act, len(lens), cid=93), lens, conv_bias=True, general_A=not powers)
+        shape_A(prob.params, regime, powers, g)
+        prob.dt, raw = shape_dt(prob.dt, prob.params, regime, act, g)
+        assert not raw
+        flags = flags_for(False, powers)
+        lay = upload_layer(prob.params, act, flags)
+        assert not powers or md.mdraft_classify_A(lay.A)[0], "the test's A must have the promised structure"
+        assert form(lay, 1, lens) != (0, 0)
+        h0, c0 = (g.normal(size=(1, 200, 16)).astype(np.float32), gen.round_to_act(g.normal(size=(1, 3, 200)).astype(np.float32), act)) if have_state else (None, None)
+        o_out, o_conv, o_h = run_oracle_prefill(prob, flags, c0, h0)
+        g_out, g_conv, g_h = run_gpu_prefill(prob, flags, 0, c0, h0)
+        assert_close(g_out, o_out, TOL[act], f"out, lengths {lens}")
+        assert_close(g_h, o_h, TOL_STATE, f"final SSM state, lengths {lens}")
+        assert np.array_equal(g_conv, o_conv)
+
+
+@pytest.mark.parametrize("act", ["f32", "bf16"])
+@pytest.mark.parametrize("powers", [False, True])
+def test_one_kernel_prefill_whose_softplus_underflows_leaves_the_state_bit_identical(act, powers):
+    """log(1 + exp(-200)) is 0 in fp32: the folds of the chunks' summaries give back what the slot held."""
+    g = np.random.default_rng(18)
+    prob = parity.make_problem(parity.small_config(136, act, 1, cid=93), [90], conv_bias=True, general_A=not powers)
+    shape_A(prob.params, "", powers, g)
+    prob.dt = gen.round_to_act(g.normal(size=prob.dt.shape).astype(np.float32), act)
+    prob.params.dt_bias[:] = -200.0
+    flags = flags_for(False, powers)
+    assert form(upload_layer(prob.params, act, flags), 1, [90]) != (0, 0)
+    h0 = g.normal(size=(1, 136, 16)).astype(np.float32)
+    c0 = gen.round_to_act(g.normal(size=(1, 3, 136)).astype(np.float32), act)
+    g_out, _, g_h = run_gpu_prefill(prob, flags, 0, c0, h0)
+    assert np.array_equal(g_h.astype(np.float32).view(np.uint32), h0.view(np.uint32)), "a zero step size must freeze the state exactly"
+    o_out, _, _ = run_oracle_prefill(prob, flags, c0, h0)
+    assert_close(g_out, o_out, TOL[act], "out = (C.h0 + D u) * SiLU(z)")
 
 
 @pytest.mark.parametrize("act", ["f32", "bf16"])

@@ -5,6 +5,7 @@ import numpy as np
 import pytest
 import torch
 
+import gen
 import oracle
 import parity
 from parity import TOL, TOL_STATE, assert_close
@@ -39,6 +40,32 @@ def test_stack_prefill_matches_oracle(n_layers, Dn, act, lens, general_A):
         assert_close(outs[l].float().cpu().numpy(), o_out, TOL[act], f"out of layer {l}")
         assert_close(stack.cache.ssm[l].cpu().numpy(), o_h, TOL_STATE, f"state of layer {l}")
         assert np.array_equal(stack.cache.conv[l].float().cpu().numpy().astype(np.float64), o_conv)
+
+
+@pytest.mark.parametrize("act", ["f32", "bf16"])
+def test_stack_prefill_of_a_general_A_in_three_kernels_matches_oracle(act):
+    """Too much work for the one-kernel form: the summary pass, the carry scan and the output pass over several layers."""
+    n_layers, Dn, lens = 3, 520, [1500, 0, 700]
+    probs, tdt = _problems(n_layers, Dn, act, lens, True)
+    lays = [upload_layer(p.params, act, md.MDRAFT_DT_SOFTPLUS) for p in probs]
+    T, S = sum(lens), len(lens)
+    assert md.mdraft_prefill_stack_launches(lays[0], n_layers, T, S, max(lens)) == 3
+    stack = DrafterStack(lays, 2 * S, T, S, max(lens))
+    g = np.random.default_rng(8)
+    h0 = g.normal(size=(n_layers, S, Dn, 16)).astype(np.float32)
+    c0 = gen.round_to_act(g.normal(size=(n_layers, S, 3, Dn)).astype(np.float32), act)
+    stack.cache.ssm[:, S:], stack.cache.conv[:, S:] = torch.from_numpy(h0).cuda(), to_device(c0, tdt)
+    ins = [tuple(to_device(a, tdt) for a in (p.x, p.z, p.dt, p.B, p.C)) for p in probs]
+    outs = list(torch.full((n_layers, T, Dn), float("nan"), dtype=tdt, device="cuda"))
+    assert md.mdraft_conv_scan_prefill_stack(lays, range(n_layers), stack.cache, ins, outs, i32(probs[0].cu), max(lens), i32(np.arange(S, 2 * S)), i32(np.arange(S)),
+                                             stack.workspace, stack.status)
+    torch.cuda.synchronize()
+    stack.check_status()
+    for l, p in enumerate(probs):
+        o_out, o_conv, o_h = oracle.prefill(oracle.layer_from_params(p.params), p.x, p.z, p.dt, p.B, p.C, p.cu, c0[l], h0[l])
+        assert_close(outs[l].float().cpu().numpy(), o_out, TOL[act], f"out of layer {l}")
+        assert_close(stack.cache.ssm[l, :S].cpu().numpy(), o_h, TOL_STATE, f"state of layer {l}")
+        assert np.array_equal(stack.cache.conv[l, :S].float().cpu().numpy().astype(np.float64), o_conv)
 
 
 def test_layers_whose_tensors_overlap_run_in_order():
