@@ -414,17 +414,19 @@ int run_prefill(const PrefillCall& call, const PrefillPlan& pl, int32_t n_layers
 
 // The one-kernel form (csrc/prefill_cluster.cu) of a call, or blocks = 0 where the plan above is the faster one.  Both are estimated:
 //  - the one-kernel form takes kOne us and so much per block of a cluster, and per token of a chunk kLatency us plus kShare for every
-//    further warp on a scheduler; short chunks of one block or two some 0.1 us a token more where they fill the machine; and 1.05 of all that
-//    where clusters of three blocks and more fill SMs that they share: then some no longer fit beside the rest, most with another call's
-//    blocks ahead of them (36 clusters of 7 blocks, 1128 channels x 1178 tokens: 28.3 us alone, 31.5 in a row; estimated 24.7);
+//    further warp on a scheduler; short chunks of one block or two some 0.1 us a token more where they fill the machine; and 5 or 10 % more
+//    where clusters of many or wide blocks fill SMs that they share: then some no longer fit beside the rest, most with another call's
+//    blocks ahead of them (36 clusters of 7 blocks of 8 warps, 1128 channels x 1178 tokens: 28.3 us alone, 31.5 in a row; 24.7 by the rest of the estimate);
 //  - the other takes kSplit + kSplitWork per token of work of a scheduler where it cuts sequences, kWhole + kWholeToken per token
 //    of the longest where it does not.  That is good to 15 %, and high where a cut call fills an SM with blocks that finish together (24-token chunks of
-//    1174 x 1112 18.7 us, estimated 21.8): the one-kernel form has to promise 14 % less, and 17 or 20 % (general A) where the other cuts
-//    and has much work.
-// It wins where the work is small: 256 x 64 fp32 9.2 -> 6.4 us, 256 x 768 bf16 12.3 -> 8.1, 1024 x 128 to 256 0.76 of the time; over 5709 calls that the rule
-// gives to it (1 to 24 layers, 1 to 48 sequences of 2 to 4500 tokens, 32 to 1536 channels; eight calls in a graph, either way) it takes 0.765 of
-// the other's time in the mean, and 19 of them lose 3 to 11 %.  (A margin of 12 % alone, 20 from sixteen sequences and 25 for a single long one on, had 223 of 8727 lose
-// 3 to 45 %; the tighter ones leave 1.4 % of that sample's time unwon in other calls.)  It loses where the work fills the machine, since its clusters
+//    1174 x 1112 18.7 us, estimated 21.8).
+// So the one-kernel form has to promise 12 % less; 16 where one layer with much work is cut (general A or fp32: of 94 such calls that promise 12 to 16 %, 29
+// lose 3 % and more replayed); 20 from sixteen sequences on, which the narrow form with four blocks to an SM serves better than estimated (20 x 1508 x 64, general A: 32.7 us, in
+// one kernel 37.9); 25 where one layer's one sequence is long for its width (1500 x 1536: 26.8 us, in one kernel 29.6; 3925 x 368 28.5 and 34.4).
+// It wins where the work is small: 256 x 64 fp32 9.2 -> 6.4 us, 256 x 768 bf16 12.3 -> 8.1, 1024 x 128 to 256 0.76 of the time; over 4935 calls that the rule
+// gives to it (1 to 24 layers, 1 to 48 sequences of 2 to 4500 tokens, 32 to 1536 channels) it takes 0.774 of the other's time in the mean replayed from a
+// graph and 0.725 called, and 37 lose 3 to 10 % replayed, 16 lose 3 to 9 % called.  (With the first, third and fourth margin and no crowding 223 of 8727 lost 3 to 45 %
+// replayed.  20 % wherever a cut call has much work, 14 elsewhere: 19 of 5709, but four times as many wins given up as losses saved.)  It loses where the work fills the machine, since its clusters
 // leave a seventh of the SMs out and its channel groups are narrow: 1777 x 1536, general A, 35.5 against 41.4 at best, 4096 x 1536 52 against 77.
 // It is for calls whose sequences do not look at one another's slots: a cluster reads its starting slot when it comes to run, by when another
 // sequence's may have stored its final state, where the three kernels take the state and window that a cut sequence starts
@@ -442,7 +444,8 @@ ClusterForm cluster_form(const mdraft_layer* L, int n_layers, int T, int n_seq, 
     double least = kSplit + work * kSplitWork[general] + (n_seq > 1 ? kSplitSeqs : 0.0);
     const double blocks = (double)n_layers * n_seq * ((L->d_inner + kPrefillThreads - 1) / kPrefillThreads), rounds = 1.2 * blocks / sms;
     const double whole = kWhole + max_seqlen * kWholeToken * (general ? kGeneralOne : 1.0) * (rounds > 1.0 ? rounds : 1.0);
-    least = whole < least ? 0.86 * whole : (work <= 40.0 ? 0.86 : general ? 0.8 : 0.83) * least;
+    const double margin = n_seq >= 16 ? 0.8 : n_seq * n_layers == 1 && work > 75.0 ? 0.75 : n_layers == 1 && (general || L->act == MDRAFT_F32) && work > 40.0 && least <= whole ? 0.84 : 0.88;
+    least = margin * (whole < least ? whole : least);
     auto weigh = [&](int c, int w) {
         const int share = prefill_cluster_share(c, clusters);
         if (share * w > 16) return;   // the warps of an SM, 128 registers a thread
@@ -451,7 +454,7 @@ ClusterForm cluster_form(const mdraft_layer* L, int n_layers, int T, int n_seq, 
         const int chunk = prefill_cluster_chunk(max_seqlen, c * w, !general);
         double t = kOne + (c > 1 ? kCluster : 0.0) + kBlock * c + kWarp * busy + chunk * (kLatency[general] + kShare[general] * busy);
         if (c <= 2 && places > 0.4) t += 0.1 * (places - 0.4) * (chunk < 16 ? chunk : 16);
-        if (c >= 3 && share >= 2 && places > 0.72) t *= 1.05;
+        if (c >= 3 && share >= 2 && places > 0.72) t *= 1.0 + 0.05 * ((c >= 6) + (w == 8));
         if (t < least) { least = t; best = {c, w}; }
     };
     for (int w = 4; w <= kClusterMaxWarps; w *= 2)
