@@ -191,6 +191,11 @@ struct ChannelScan {
     }
 };
 
+// a h + q, four states at once.
+__device__ __forceinline__ float4 fold4(const float4& a, const float4& h, const float4& q) {
+    return make_float4(fmaf(a.x, h.x, q.x), fmaf(a.y, h.y, q.y), fmaf(a.z, h.z, q.z), fmaf(a.w, h.w, q.w));
+}
+
 // Conv window at the start of a chunk: the W-1 rows before t0, taken from the sequence itself, or (chunk 0)
 // from `src_rows` = (W-1, D) activations, or zeros.
 template <typename AT>

@@ -165,6 +165,11 @@ inline cudaLaunchAttribute most_shared_memory() {
     return a;
 }
 
+__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+// Programmatic stream serialisation: the work of the kernels ahead is complete and visible; the next kernel may start.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_release_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 __device__ __forceinline__ void flag(int32_t* dev_status, int bit) {
     if (dev_status) atomicOr(dev_status, bit);
 }

@@ -53,8 +53,6 @@ __host__ __device__ constexpr int off_b(int sub) { return 3 * sub * kTileBytes; 
 __host__ __device__ constexpr int off_c(int sub) { return 3 * sub * kTileBytes + kBCBytes; }
 __host__ __device__ constexpr int smem_bytes(int sub) { return kStages * (stage_bytes(sub) + 2 * kBCBytes * 2); }  // + fp32 B, C
 // ---------------------------------------------------------------- mbarrier + bulk copy
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
 }
@@ -92,8 +90,6 @@ __device__ __forceinline__ void tma_box(void* dst, const CUtensorMap* map, int c
 // stream serialisation: a kernel may start while its predecessor is still running, and must pass grid_wait() before
 // it touches anything the predecessor (or a kernel before that) writes, or overwrites anything it reads.  Every block
 // passes grid_wait() on every path, so that a kernel's completion implies that of all its predecessors.
-__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_release_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <typename T>
 __device__ __forceinline__ T* at_bytes(T* p, int64_t off) { return reinterpret_cast<T*>(reinterpret_cast<char*>(p) + off); }  // T may be void
@@ -427,10 +423,6 @@ __global__ void __launch_bounds__(SUB * kBoxCols + 32, PER_SM) chunk_kernel(cons
 // 48 it spills and loses 4 us; 10 to 16 warps of 3 or 4 chunks lose 0.5 to 3.  The fold over the warps unrolled by 2 costs 10 % where a call takes many
 // rounds, 12 sequences of up to 9532 x 80 79.0 -> 88.5 us; by 8 it costs the short calls 5 %.)
 constexpr int kCarryGroups = 8, kCarryPer = 6;
-
-__device__ __forceinline__ float4 fold4(const float4& a, const float4& h, const float4& q) {
-    return make_float4(fmaf(a.x, h.x, q.x), fmaf(a.y, h.y, q.y), fmaf(a.z, h.z, q.z), fmaf(a.w, h.w, q.w));
-}
 
 template <int ML>
 __global__ void __launch_bounds__(kCarryGroups * 32, 1) carry_kernel(const __grid_constant__ PrefillBatch<ML> batch) {

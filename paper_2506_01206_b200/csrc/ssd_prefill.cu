@@ -45,7 +45,6 @@ constexpr uint32_t kXdColBytes = Q * 16 + 16; // one 8-wide column of core matri
 constexpr uint32_t kHinColBytes = P * 16;     // H_in: 64 rows
 
 // ---------------------------------------------------------------- PTX helpers
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
 }
@@ -155,8 +154,7 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
 // before the kernel ahead of them has finished.  A kernel passes grid_wait() before it touches anything a kernel ahead
 // of it writes, or overwrites anything one reads; every block passes it on every path, so that a kernel's completion
 // implies the completion of everything before it.
-__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_release_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
 // SiLU of the gate input with one special-function instruction instead of two: z sigmoid(z) = 0.5 z (1 + tanh(z / 2)); the
