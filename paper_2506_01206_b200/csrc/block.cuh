@@ -19,7 +19,7 @@ struct SmallLinear {
     int m, n, k;
     int32_t* dev_status;
     bool release_late;         // the next kernel may start only once this one's turn has come
-    bool alone;                // no two blocks of such products on one SM (keep_products_apart)
+    bool alone;                // no two blocks of such products on one SM (place_products)
     float eps;                 // >= 0: the sum is scaled by 1 / sqrt(mean_k a[m][k]^2 + eps); < 0: not
 };
 

@@ -7,10 +7,10 @@
 //   2. the warps of a block fold those in token order (a thread takes four states of a channel), the cluster meets at its
 //      hardware barrier, and every block folds the sums of the blocks before it out of their shared memory onto the starting state;
 //   3. every warp runs its chunk again from its incoming state and writes the outputs; the last chunk stores state and window.
-// Two kernels, their start-up and the trip of the summaries through memory fall away, and a call needs no workspace.
+// Two kernels, their start-up and the trip of the summaries through memory fall away, and a call uses no workspace.
 //
 // A warp works alone between the two meetings: it fetches its tiles of 16 (bf16) or 8 (fp32) tokens with 16-byte asynchronous
-// copies (four requests a lane and tile), one tile ahead, and widens B and C for itself.  No warp waits for another's copies,
+// copies (eight requests a lane and tile in the output pass; in the first four, and two more of half the lanes), one tile ahead, and widens B and C for itself.  No warp waits for another's copies,
 // there are no descriptors to encode, and rows need no more alignment than the 16 bytes the interface asks for.
 #include <type_traits>
 

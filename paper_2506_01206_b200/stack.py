@@ -28,7 +28,7 @@ class DrafterStack:
         self.workspace = torch.empty(max(self.ws_bytes, stacked, 256), dtype=torch.uint8, device=device)
         self.status = torch.zeros(1, dtype=torch.int32, device=device)
 
-    # number of kernels one layer's prefill call launches (chunk summary + carry scan + main scan, or the main scan alone)
+    # number of kernels one layer's prefill call launches: chunk summary + carry scan + main scan, the main scan alone, or a small problem's one kernel
     def prefill_launches_per_layer(self, total_tokens: int, n_seq: int, max_seqlen: int) -> int:
         if not self.chunk_len:
             return mb.mdraft_prefill_stack_launches(self.layers[0], 1, total_tokens, n_seq, max_seqlen)
