@@ -285,7 +285,10 @@ struct StateSmem {
 static_assert((Q + 3) * P * 2 >= (P / 8) * kXdColBytes, "the remainder operand must fit the x tile it replaces");
 static_assert(3 * (sizeof(StateSmem) + 1024 + 1024) <= 227 * 1024, "three blocks per SM");
 
-__global__ void __launch_bounds__(kThreads, 3) ssd_chunk_state_kernel(const SsdPrefillArgs p, const __grid_constant__ SsdMaps maps) {
+// 72 registers, not the 79 that the compiler takes when it may (no spill): two of these blocks and one of the state-passing kernel's (106 registers)
+// are then all the registers of an SM, so that a passing block can start beside them and not only where a third of them has left (10 heads x 4870
+// tokens 36.8 -> 30.8 us, 18 x 2048 25.0 -> 22.0, 6 x 6000 35.8 -> 28.8, 24 x 2048 28.3 -> 28.1).
+__global__ void __maxnreg__(72) ssd_chunk_state_kernel(const SsdPrefillArgs p, const __grid_constant__ SsdMaps maps) {
     extern __shared__ __align__(1024) unsigned char s_raw[];
     StateSmem& sm = *reinterpret_cast<StateSmem*>(s_raw + ((1024u - (smem_u32(s_raw) & 1023u)) & 1023u));   // the swizzled tile starts on a 1024-byte boundary
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
