@@ -708,7 +708,7 @@ int mdraft_tree_step_proj(const mdraft_layer* layer, const mdraft_cache* cache, 
     a.x = x; a.z = z; a.out = out;
     a.ldx = ldx; a.ldz = ldz; a.ldo = ldo;
     a.W_x = proj->W_x; a.W_dt = proj->W_dt; a.dt_rank = proj->dt_rank; a.nodes_per_cluster = proj->nodes_per_cluster;
-    a.parent_slot = parent_slot; a.node_slot = node_slot; a.n_nodes = n_nodes; a.chained = 0; a.dev_status = dev_status;
+    a.parent_slot = parent_slot; a.node_slot = node_slot; a.n_nodes = n_nodes; a.chained = 0; a.most_shared = false; a.dev_status = dev_status;
     if (launch_tree_proj(a, act, static_cast<cudaStream_t>(stream)) != cudaSuccess) return MDRAFT_ERR_CUDA;
     return MDRAFT_OK;
 }
@@ -756,7 +756,7 @@ int mdraft_block_generation(const mdraft_block_stack* stack, const mdraft_cache*
         a.x = xzb; a.z = xzb + D; a.out = yb;
         a.ldx = a.ldz = 2 * (int64_t)D; a.ldo = D;
         a.W_x = stack->W_x[l]; a.W_dt = stack->W_dt[l]; a.dt_rank = R; a.nodes_per_cluster = 0;
-        a.parent_slot = parent_slot; a.node_slot = node_slot; a.n_nodes = n_nodes; a.chained = 1; a.dev_status = dev_status;
+        a.parent_slot = parent_slot; a.node_slot = node_slot; a.n_nodes = n_nodes; a.chained = 1; a.most_shared = place.step_split; a.dev_status = dev_status;
         if ((e = launch_tree_proj(a, MDRAFT_BF16, st)) != cudaSuccess) break;
         e = launch_small_linear({yb, static_cast<const bf*>(stack->W_out[l]), hb, hb, M, M, n_nodes, M, D, dev_status, place.out_late, place.out_alone, -1.0f}, st);
     }

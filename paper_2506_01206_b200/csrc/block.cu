@@ -369,11 +369,15 @@ cudaError_t launch_tile(const SmallLinear& p, cudaStream_t st) {
 // The next layer's in_proj starts some 10 us ahead of its turn, as soon as out_proj's blocks have started.  Where the projection step alone has a block for
 // about every SM, it is better held back until out_proj's own turn: 18 / 23 / 24 / 28 / 32 nodes 272 / 290 / 303 / 324 / 335 us, held back
 // 277 / 298 / 298 / 313 / 316.  (Beyond one row tile it makes no odds: 33 / 48 / 64 nodes 384 / 490 / 482 and 392 / 489 / 477.)
+// The step's blocks want the products' split of an SM's memory only where one wave, or hardly more, holds the products' (4 / 23 nodes 223 / 287 us, with its own
+// 230 / 294; 16 layers of 640 / 1280 channels, 4 nodes: 131 and 142; 1024 / 1536 channels, 160 blocks, 8 / 18 / 23 nodes 293 / 362 / 384 and 302 / 374 / 383).  Where more products'
+// blocks share SMs it is in the way: 12 layers of 1152 / 1536, 168 blocks, at 8 / 23 / 28 nodes 155 / 210 / 223 us, with its own 155 / 203 / 217; of 1408 / 1280
+// at 8 / 18 / 23 / 28 nodes 176 / 217 / 234 / 253 and 174 / 204 / 229 / 243.
 ProductPlacement place_products(int d_model, int d_inner, int n_nodes) {
     const int sms = sm_count(), tile = 2 * d_inner <= 16 * sms ? 16 : 32, blocks = (2 * d_inner + tile - 1) / tile + (d_model + 15) / 16;
     const int cb = tree_proj_block_channels(d_inner), step_blocks = n_nodes * ((d_inner + cb - 1) / cb);
     const bool one_tile = n_nodes <= kRows, apart = one_tile && blocks <= sms;
-    return {apart, apart && n_nodes > 4, one_tile && step_blocks * 20 >= sms * 19};
+    return {apart, apart && n_nodes > 4, one_tile && step_blocks * 20 >= sms * 19, 10 * blocks <= 11 * sms};
 }
 
 cudaError_t launch_small_linear(const SmallLinear& p, cudaStream_t st) {

@@ -24,8 +24,8 @@ struct SmallLinear {
 };
 
 // Which of a block's products, for so many nodes, take an SM without another product's block, and whether out_proj holds back the layer after it:
-// see the measurements at the definition.
-struct ProductPlacement { bool in_alone, out_alone, out_late; };
+// see the measurements at the definition.  step_split: the projection step is launched with the products' split of an SM's memory.
+struct ProductPlacement { bool in_alone, out_alone, out_late, step_split; };
 ProductPlacement place_products(int d_model, int d_inner, int n_nodes);
 
 cudaError_t launch_small_linear(const SmallLinear& p, cudaStream_t st);

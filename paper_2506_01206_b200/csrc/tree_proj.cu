@@ -529,7 +529,7 @@ cudaError_t launch_nt(const TreeProjArgs& p, int n_blocks, cudaStream_t st) {
     at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[1].val.programmaticStreamSerializationAllowed = 1;
     at[2] = most_shared_memory();   // alone the driver's own split is 2-4 % faster (18 nodes 5.7 against 5.95 us)
-    cfg.numAttrs = p.chained ? 3 : 1;
+    cfg.numAttrs = !p.chained ? 1 : p.most_shared ? 3 : 2;
     const bool pow = p.L.flags & MDRAFT_A_POWERS;
     const cudaError_t e = pow ? allow_smem<tree_proj_kernel<AT, CB, NT, true>>(kSmem) : allow_smem<tree_proj_kernel<AT, CB, NT, false>>(kSmem);
     if (e != cudaSuccess) return e;

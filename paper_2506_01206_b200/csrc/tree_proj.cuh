@@ -21,6 +21,7 @@ struct TreeProjArgs {
     const int32_t *parent_slot, *node_slot;
     int n_nodes;
     int chained;       // 1: launched behind a kernel that releases it early; only x and z are that kernel's work
+    bool most_shared;  // chained: with the split of an SM's memory that the kernels around it ask for
     int32_t* dev_status;
 };
 
