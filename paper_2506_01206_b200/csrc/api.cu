@@ -420,12 +420,13 @@ int run_prefill(const PrefillCall& call, const PrefillPlan& pl, int32_t n_layers
 //  - the other takes kSplit + kSplitWork per token of work of a scheduler where it cuts sequences, kWhole + kWholeToken per token
 //    of the longest where it does not.  That is good to 15 %, and high where a cut call fills an SM with blocks that finish together (24-token chunks of
 //    1174 x 1112 18.7 us, estimated 21.8).
-// So the one-kernel form has to promise 12 % less; 16 where one layer with much work is cut (general A or fp32: of 94 such calls that promise 12 to 16 %, 29
-// lose 3 % and more replayed); 20 from sixteen sequences on, which the narrow form with four blocks to an SM serves better than estimated (20 x 1508 x 64, general A: 32.7 us, in
+// So the one-kernel form has to promise 12 % less; 8 over several layers with A = powers and little work (57 calls that promise 8 to 12 %: 0.90 of the time in
+// the mean, five lose 3 % and more); 16 where much work is cut (one layer, general A or fp32: of 94 such calls that promise 12 to 16 %, 29 lose 3 % and more; several
+// layers, general A: 12 of 36; 8 layers of 3098 x 1016, fp32, A = powers: 190 us, in one kernel 233); 20 from sixteen sequences on, which the narrow form with four blocks to an SM serves better than estimated (20 x 1508 x 64, general A: 32.7 us, in
 // one kernel 37.9); 25 where one layer's one sequence is long for its width (1500 x 1536: 26.8 us, in one kernel 29.6; 3925 x 368 28.5 and 34.4).
-// It wins where the work is small: 256 x 64 fp32 9.2 -> 6.4 us, 256 x 768 bf16 12.3 -> 8.1, 1024 x 128 to 256 0.76 of the time; over 4935 calls that the rule
-// gives to it (1 to 24 layers, 1 to 48 sequences of 2 to 4500 tokens, 32 to 1536 channels) it takes 0.774 of the other's time in the mean replayed from a
-// graph and 0.725 called, and 37 lose 3 to 10 % replayed, 16 lose 3 to 9 % called.  (With the first, third and fourth margin and no crowding 223 of 8727 lost 3 to 45 %
+// It wins where the work is small: 256 x 64 fp32 9.2 -> 6.4 us, 256 x 768 bf16 12.3 -> 8.1, 1024 x 128 to 256 0.76 of the time; over 5170 calls that the rule
+// gives to it (1 to 24 layers, 1 to 48 sequences of 2 to 5000 tokens, 32 to 1760 channels) it takes 0.78 of the other's time in the mean replayed from a
+// graph, where 70 lose 3 to 15 %, and 0.70 called one after another, where 12 of 3089 lose 3 to 11 %.  (With 12, 20 and 25 % alone and no crowding 223 of 8727 lost 3 to 45 %
 // replayed.  20 % wherever a cut call has much work, 14 elsewhere: 19 of 5709, but four times as many wins given up as losses saved.)  It loses where the work fills the machine, since its clusters
 // leave a seventh of the SMs out and its channel groups are narrow: 1777 x 1536, general A, 35.5 against 41.4 at best, 4096 x 1536 52 against 77.
 // It is for calls whose sequences do not look at one another's slots: a cluster reads its starting slot when it comes to run, by when another
@@ -444,7 +445,8 @@ ClusterForm cluster_form(const mdraft_layer* L, int n_layers, int T, int n_seq, 
     double least = kSplit + work * kSplitWork[general] + (n_seq > 1 ? kSplitSeqs : 0.0);
     const double blocks = (double)n_layers * n_seq * ((L->d_inner + kPrefillThreads - 1) / kPrefillThreads), rounds = 1.2 * blocks / sms;
     const double whole = kWhole + max_seqlen * kWholeToken * (general ? kGeneralOne : 1.0) * (rounds > 1.0 ? rounds : 1.0);
-    const double margin = n_seq >= 16 ? 0.8 : n_seq * n_layers == 1 && work > 75.0 ? 0.75 : n_layers == 1 && (general || L->act == MDRAFT_F32) && work > 40.0 && least <= whole ? 0.84 : 0.88;
+    const bool much = least <= whole && (n_layers > 1 ? work > (general ? 80.0 : 200.0) : work > 40.0 && (general || L->act == MDRAFT_F32));
+    const double margin = n_seq >= 16 ? 0.8 : n_seq * n_layers == 1 && work > 75.0 ? 0.75 : much ? 0.84 : n_layers > 1 && !general && work <= 120.0 ? 0.92 : 0.88;
     least = margin * (whole < least ? whole : least);
     auto weigh = [&](int c, int w) {
         const int share = prefill_cluster_share(c, clusters);
