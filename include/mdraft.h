@@ -153,9 +153,9 @@ typedef struct {
  *                of 128 channels (one of 512 where the width fills those) or are, for several sequences, at most 256
  *                tokens; less is MDRAFT_ERR_WORKSPACE.  Sequences that the library leaves whole need none, although
  *                the query for a single layer answers as if they were cut.  A chunk length given in `opts` is kept:
- *                it needs all that the query says.  Small problems are encoded in one kernel that uses none of it, unless several
- *                sequences with both starting and final slots would otherwise be cut; they are refused all the same where
- *                the workspace would not serve the other form
+ *                it needs all that the query says.  Small problems are encoded in one kernel that uses none of it, or, where several
+ *                sequences with both starting and final slots would otherwise be cut, passes their final states through
+ *                it; they are refused all the same where the workspace would not serve the other form
  *   dev_status : device int32 or NULL (see mdraft_dev_status bits); never cleared by the library
  */
 size_t mdraft_prefill_workspace_bytes(const mdraft_layer *layer, int32_t total_tokens, int32_t n_seq,
@@ -188,7 +188,7 @@ typedef struct {
  *   workspace : as above; mdraft_prefill_stack_workspace_bytes answers for layers that share the flags of `layer`.  The
  *               launches of a call share it, so layers with different flags need the largest answer over their groups
  * mdraft_prefill_stack_launches: kernels such a call launches (for accounting), if it is of one sequence or has no init_slot or
- * no final_slot; with both, a batch that would be cut takes three (two under MDRAFT_CONV_ONLY) also where this says one.
+ * no final_slot; with both, a batch that would be cut takes two or three also where this says one.
  */
 size_t mdraft_prefill_stack_workspace_bytes(const mdraft_layer *layer, int32_t n_layers, int32_t total_tokens, int32_t n_seq,
                                             int32_t max_seqlen, const mdraft_prefill_opts *opts);

@@ -429,14 +429,13 @@ int run_prefill(const PrefillCall& call, const PrefillPlan& pl, int32_t n_layers
 // graph, where 70 lose 3 to 15 %, and 0.70 called one after another, where 12 of 3089 lose 3 to 11 %.  (With 12, 20 and 25 % alone and no crowding 223 of 8727 lost 3 to 45 %
 // replayed.  20 % wherever a cut call has much work, 14 elsewhere: 19 of 5709, but four times as many wins given up as losses saved.)  It loses where the work fills the machine, since its clusters
 // leave a seventh of the SMs out and its channel groups are narrow: 1777 x 1536, general A, 35.5 against 41.4 at best, 4096 x 1536 52 against 77.
-// It is for calls whose sequences do not look at one another's slots: a cluster reads its starting slot when it comes to run, by when another
-// sequence's may have stored its final state, where the three kernels take the state and window that a cut sequence starts
-// from ahead of the pass that stores.  The slots are on the device, so where several sequences have both and the plan cuts them, the caller of
-// this function keeps the three kernels.
-ClusterForm cluster_form(const mdraft_layer* L, int n_layers, int T, int n_seq, int max_seqlen, const mdraft_prefill_opts* opts) {
+// A cluster reads its starting slot when it comes to run, by when another sequence's may have stored its final state, where the three kernels take the
+// state and window that a cut sequence starts from ahead of the pass that stores.  The slots are on the device, so where several sequences have both and
+// the plan cuts them (`shared`) the final states go through the workspace and a second kernel, for kDeliver us.
+ClusterForm cluster_form(const mdraft_layer* L, int n_layers, int T, int n_seq, int max_seqlen, const mdraft_prefill_opts* opts, bool shared = false) {
     if (one_at_a_time(L) || (opts && (opts->chunk_len > 0 || opts->block_channels || opts->event_after_chunk_state || opts->event_after_carry_scan))) return {0, 0};
     constexpr double kOne = 4.1, kCluster = 0.6, kBlock = 0.13, kWarp = 0.15, kLatency[2] = {0.195, 0.275}, kShare[2] = {0.112, 0.167};
-    constexpr double kSplit = 11.1, kSplitSeqs = 0.7, kSplitWork[2] = {0.166, 0.239}, kWhole = 3.3, kWholeToken = 0.104;
+    constexpr double kSplit = 11.1, kSplitSeqs = 0.7, kSplitWork[2] = {0.166, 0.239}, kWhole = 3.3, kWholeToken = 0.104, kDeliver = 1.7;
     const int general = !(L->flags & MDRAFT_A_POWERS), sms = sm_count();
     const int64_t groups = (int64_t)n_layers * ((L->d_inner + kClusterCols - 1) / kClusterCols), clusters = groups * n_seq;
     const double work = (double)T * groups / (4 * sms);
@@ -447,7 +446,7 @@ ClusterForm cluster_form(const mdraft_layer* L, int n_layers, int T, int n_seq, 
     const double whole = kWhole + max_seqlen * kWholeToken * (general ? kGeneralOne : 1.0) * (rounds > 1.0 ? rounds : 1.0);
     const bool much = least <= whole && (n_layers > 1 ? work > (general ? 80.0 : 200.0) : work > 40.0 && (general || L->act == MDRAFT_F32));
     const double margin = n_seq >= 16 ? 0.8 : n_seq * n_layers == 1 && work > 75.0 ? 0.75 : much ? 0.84 : n_layers > 1 && !general && work <= 120.0 ? 0.92 : 0.88;
-    least = margin * (whole < least ? whole : least);
+    least = margin * (whole < least ? whole : least) - (shared ? kDeliver : 0.0);
     auto weigh = [&](int c, int w) {
         const int share = prefill_cluster_share(c, clusters);
         if (share * w > 16) return;   // the warps of an SM, 128 registers a thread
@@ -465,7 +464,7 @@ ClusterForm cluster_form(const mdraft_layer* L, int n_layers, int T, int n_seq, 
 }
 
 template <int ML>
-int run_prefill_cluster(const PrefillCall& call, const ClusterForm& form, int32_t n_layers, const mdraft_layer* layers, const int32_t* layer_index, const mdraft_io* io) {
+int run_prefill_cluster(const PrefillCall& call, const ClusterForm& form, const PrefillPlan* through, int32_t n_layers, const mdraft_layer* layers, const int32_t* layer_index, const mdraft_io* io) {
     ClusterBatch<ML> b;
     ClusterArgs& a = b.c;
     a.pool = PoolDev{};
@@ -476,6 +475,9 @@ int run_prefill_cluster(const PrefillCall& call, const ClusterForm& form, int32_
     }
     a.n_layers = n_layers; a.d_inner = layers->d_inner; a.T = call.total_tokens; a.n_seq = call.n_seq;
     a.cu = call.cu_seqlens; a.init_slot = call.init_slot; a.final_slot = call.final_slot; a.dev_status = call.dev_status;
+    a.ws_state = through ? reinterpret_cast<float*>(call.workspace + through->off_h0) : nullptr;
+    a.ws_window = through ? call.workspace + through->off_conv : nullptr;
+    a.ws_layer_bytes = through ? (int64_t)through->layer_bytes : 0;
     for (int32_t i = 0; i < n_layers; ++i) {
         const mdraft_io& v = io[i];
         b.l[i] = {layer_dev(layers + i), layer_index[i], v.x, v.z, v.dt, v.B, v.C, v.out, v.ldx, v.ldz, v.lddt, v.ldb, v.ldc, v.ldo};
@@ -494,12 +496,13 @@ __global__ void classify_A_kernel(const float* A, int D, int N, int32_t* res) {
 
 }  // namespace
 
-// The form of a call's first launch where none of its sequences starts from a slot: 256 * blocks + warps of the one-kernel form, 0 for the plan's
-// own kernels.  For the tests, which have to know what they run; no part of the interface.
-extern "C" int32_t mdraft_internal_prefill_form(const mdraft_layer* layer, int32_t n_layers, int32_t total_tokens, int32_t n_seq, int32_t max_seqlen) {
+// The form of a call's first launch: 256 * blocks + warps of the one-kernel form, 0 for the plan's own kernels.  shared: the plan cuts its several sequences,
+// which have both starting and final slots.  For the tests, which have to know what they run; no part of the interface.
+extern "C" int32_t mdraft_internal_prefill_form(const mdraft_layer* layer, int32_t n_layers, int32_t total_tokens, int32_t n_seq, int32_t max_seqlen,
+                                                int32_t shared) {
     if (check_layer(layer) != MDRAFT_OK || n_layers <= 0 || total_tokens <= 0 || n_seq <= 0 || max_seqlen <= 0) return 0;
     const int32_t most = prefill_most_layers(n_seq);
-    const ClusterForm f = cluster_form(layer, n_layers < most ? n_layers : most, total_tokens, n_seq, max_seqlen < total_tokens ? max_seqlen : total_tokens, nullptr);
+    const ClusterForm f = cluster_form(layer, n_layers < most ? n_layers : most, total_tokens, n_seq, max_seqlen < total_tokens ? max_seqlen : total_tokens, nullptr, shared != 0);
     return f.blocks * 256 + f.warps;
 }
 
@@ -600,6 +603,8 @@ int mdraft_conv_scan_prefill_stack(int32_t n_layers, const mdraft_layer* layers,
 
     const PrefillCall call = {cache, total_tokens, n_seq, cu_seqlens, init_slot, final_slot, static_cast<char*>(workspace), opts, dev_status,
                         static_cast<cudaStream_t>(stream)};
+    // A sequence that is cut starts from what its slot held before the call, also where another stores there.
+    auto shared_slots = [&](const PrefillPlan& pl) { return pl.form.chunked && n_seq > 1 && init_slot && final_slot; };
     for (int pass = 0; pass < 2; ++pass)  // every launch is checked before the first is made
         for (int32_t l0 = 0; l0 < n_layers;) {
             const int32_t nl = run_length(n_layers - l0, layers + l0, prefill_most_layers(n_seq));
@@ -610,12 +615,10 @@ int mdraft_conv_scan_prefill_stack(int32_t n_layers, const mdraft_layer* layers,
                     if (!workspace || workspace_bytes < pl.bytes) return MDRAFT_ERR_WORKSPACE;
                     if (reinterpret_cast<uintptr_t>(workspace) & 255u) return MDRAFT_ERR_MISALIGNED;
                 }
-            } else if (const ClusterForm cf = pl.form.chunked && n_seq > 1 && init_slot && final_slot
-                                                  ? ClusterForm{0, 0}  // one sequence may start from a slot that another stores to: see cluster_form
-                                                  : cluster_form(layers + l0, nl, plan_tokens, n_seq, max_seqlen, opts);
-                       cf.blocks > 0) {
-                const int r = nl == 1 ? run_prefill_cluster<1>(call, cf, nl, layers + l0, layer_index + l0, io + l0)
-                                      : run_prefill_cluster<kClusterMaxLayers>(call, cf, nl, layers + l0, layer_index + l0, io + l0);
+            } else if (const ClusterForm cf = cluster_form(layers + l0, nl, plan_tokens, n_seq, max_seqlen, opts, shared_slots(pl)); cf.blocks > 0) {
+                const PrefillPlan* through = shared_slots(pl) ? &pl : nullptr;
+                const int r = nl == 1 ? run_prefill_cluster<1>(call, cf, through, nl, layers + l0, layer_index + l0, io + l0)
+                                      : run_prefill_cluster<kClusterMaxLayers>(call, cf, through, nl, layers + l0, layer_index + l0, io + l0);
                 if (r) return r;
             } else {
                 const int r = nl == 1 ? run_prefill<1>(call, pl, nl, layers + l0, layer_index + l0, io + l0)

@@ -7,7 +7,8 @@
 //   2. the warps of a block fold those in token order (a thread takes four states of a channel), the cluster meets at its
 //      hardware barrier, and every block folds the sums of the blocks before it out of their shared memory onto the starting state;
 //   3. every warp runs its chunk again from its incoming state and writes the outputs; the last chunk stores state and window.
-// Two kernels, their start-up and the trip of the summaries through memory fall away, and a call uses no workspace.
+// Two kernels, their start-up and the trip of the summaries through memory fall away, and a call uses no workspace, unless one of its
+// sequences might start from a slot that another stores to: then the final states wait there until all clusters have run.
 //
 // A warp works alone between the two meetings: it fetches its tiles of 16 (bf16) or 8 (fp32) tokens with 16-byte asynchronous
 // copies (eight requests a lane and tile in the output pass; in the first four, and two more of half the lanes), one tile ahead, and widens B and C for itself.  No warp waits for another's copies,
@@ -123,8 +124,13 @@ __global__ void __launch_bounds__(kClusterMaxWarps * 32, 2) cluster_kernel(const
     AT* const conv = static_cast<AT*>(c.pool.conv) + p.layer_index * c.conv_layer_stride;
     const float4* const h_init = islot >= 0 ? reinterpret_cast<const float4*>(ssm + (size_t)islot * c.pool.ssm_slot_stride + (size_t)d * kN) : nullptr;
     const AT* const w_init = islot >= 0 ? conv + (size_t)islot * c.pool.conv_slot_stride : nullptr;
-    float4* const h_final = fslot >= 0 ? reinterpret_cast<float4*>(ssm + (size_t)fslot * c.pool.ssm_slot_stride + (size_t)d * kN) : nullptr;
-    AT* const w_final = fslot >= 0 ? conv + (size_t)fslot * c.pool.conv_slot_stride : nullptr;
+    float4* h_final = fslot >= 0 ? reinterpret_cast<float4*>(ssm + (size_t)fslot * c.pool.ssm_slot_stride + (size_t)d * kN) : nullptr;
+    AT* w_final = fslot >= 0 ? conv + (size_t)fslot * c.pool.conv_slot_stride : nullptr;
+    if (c.ws_state) {
+        const int64_t off = (ML == 1 ? 0 : blockIdx.z / c.n_seq) * c.ws_layer_bytes;
+        h_final = reinterpret_cast<float4*>(reinterpret_cast<char*>(c.ws_state) + off) + ((size_t)seq * D + d) * (kN / 4);
+        w_final = reinterpret_cast<AT*>(static_cast<char*>(c.ws_window) + off) + (size_t)seq * (kW - 1) * D;
+    }
     if (len == 0) {   // the final state is the starting state
         if (rank == 0 && warp == 0 && live && fslot >= 0 && fslot != islot) {
             for (int q = 0; q < kN / 4; ++q) h_final[q] = h_init ? h_init[q] : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -319,6 +325,47 @@ __global__ void __launch_bounds__(kClusterMaxWarps * 32, 2) cluster_kernel(const
     }
 }
 
+// Final states and windows from the workspace to their slots: a thread takes four states and, of the first threads, a piece of 16 bytes of the window.
+// It adds 1.3 to 1.9 us to a call, a launch behind the clusters and a trip through L2 (two sequences of 111 tokens x 472 channels, fp32: 7.4 us with the
+// states stored by the clusters, 9.0 so, 14.7 in three kernels; 22 of 64 x 168: 10.4, 12.3, 19.1).
+constexpr int kDeliverThreads = 256;
+
+template <typename AT, int ML>
+__global__ void __launch_bounds__(kDeliverThreads) deliver_kernel(const __grid_constant__ ClusterBatch<ML> batch) {
+    const ClusterArgs& c = batch.c;
+    const int seq = blockIdx.y, layer = ML == 1 ? 0 : blockIdx.z, D = c.d_inner;
+    grid_release_dependents();
+    grid_wait();
+    int s0, len; bool bad;
+    seq_span(c.cu, c.n_seq, c.T, seq, s0, len, bad);
+    const int islot = load_slot(c.init_slot, seq), fslot = load_slot(c.final_slot, seq);
+    if (bad || islot >= c.pool.n_slots || fslot >= c.pool.n_slots || fslot < 0 || (len == 0 && fslot == islot)) return;   // nothing has been left for it
+    const int i = blockIdx.x * kDeliverThreads + threadIdx.x, index = batch.l[layer].layer_index;
+    const int64_t off = layer * c.ws_layer_bytes;
+    if (i < D * (kN / 4)) {
+        const float4* from = reinterpret_cast<const float4*>(reinterpret_cast<const char*>(c.ws_state) + off) + (size_t)seq * D * (kN / 4);
+        reinterpret_cast<float4*>(c.pool.ssm + index * c.ssm_layer_stride + (size_t)fslot * c.pool.ssm_slot_stride)[i] = from[i];
+    }
+    if (i < (kW - 1) * D * (int)sizeof(AT) / 16) {   // the width is a multiple of 8
+        const uint4* from = reinterpret_cast<const uint4*>(static_cast<const char*>(c.ws_window) + off + (size_t)seq * (kW - 1) * D * sizeof(AT));
+        reinterpret_cast<uint4*>(static_cast<AT*>(c.pool.conv) + index * c.conv_layer_stride + (size_t)fslot * c.pool.conv_slot_stride)[i] = from[i];
+    }
+}
+
+template <typename AT, int ML>
+cudaError_t launch_deliver(const ClusterBatch<ML>& b, cudaStream_t st) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((b.c.d_inner * (kN / 4) + kDeliverThreads - 1) / kDeliverThreads, b.c.n_seq, b.c.n_layers);
+    cfg.blockDim = dim3(kDeliverThreads);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, deliver_kernel<AT, ML>, b);
+}
+
 template <typename AT, bool kPow, int ML>
 cudaError_t launch_typed(const ClusterBatch<ML>& b, const ClusterForm& form, cudaStream_t st) {
     const int smem = (int)sizeof(BlockShare) + form.warps * kWarpBytes;
@@ -341,7 +388,8 @@ cudaError_t launch_typed(const ClusterBatch<ML>& b, const ClusterForm& form, cud
     at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, cluster_kernel<AT, kPow, ML>, b);
+    const cudaError_t l = cudaLaunchKernelEx(&cfg, cluster_kernel<AT, kPow, ML>, b);
+    return l == cudaSuccess && b.c.ws_state ? launch_deliver<AT>(b, st) : l;
 }
 
 }  // namespace

@@ -16,6 +16,11 @@ struct ClusterArgs {
     int64_t ssm_layer_stride, conv_layer_stride;
     int n_layers, d_inner, T, n_seq;
     const int32_t *cu, *init_slot, *final_slot;
+    // Where set, final states and windows go here and to their slots by a kernel of its own behind all the clusters: every sequence then starts from what
+    // its slot held before the call, whichever sequence stores there.  Per layer ws_layer_bytes on; rows as in a slot, one per sequence.
+    float* ws_state;
+    void* ws_window;
+    int64_t ws_layer_bytes;
     int32_t* dev_status;
 };
 

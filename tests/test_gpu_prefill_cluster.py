@@ -34,9 +34,10 @@ SHAPES = [
     ("f32", 136, [32, 32], (1, 8), (2, 4)), ("f32", 520, [300, 299], (7, 4), (7, 4))]
 
 
-def form(layer, n_layers, lens):
-    """(blocks, warps) of the one-kernel form that a call without starting slots takes, (0, 0) for the plan's own kernels."""
-    f = md.load_library().mdraft_internal_prefill_form(ctypes.byref(layer.c()), n_layers, sum(lens), len(lens), max(lens))
+def form(layer, n_layers, lens, shared=False):
+    """(blocks, warps) of the one-kernel form that a call takes, (0, 0) for the plan's own kernels; shared: several sequences that would be cut have
+    both starting and final slots."""
+    f = md.load_library().mdraft_internal_prefill_form(ctypes.byref(layer.c()), n_layers, sum(lens), len(lens), max(lens), int(shared))
     return f // 256, f % 256
 
 
@@ -93,35 +94,33 @@ def test_one_kernel_form_of_a_stack_and_its_faults(act):
     assert not bool((out[:, :50] == 9.0).all()) and bool((out[:, 50:] == 9.0).all())
 
 
-@pytest.mark.parametrize("act,Dn,n_layers,lens", [("bf16", 200, 1, [300, 290, 301, 257]), ("f32", 72, 2, [400, 333, 500])])
-def test_sequences_may_start_from_a_slot_that_one_of_them_stores_to(act, Dn, n_layers, lens):
+@pytest.mark.parametrize("act,Dn,n_layers,lens,in_one", [
+    ("bf16", 200, 1, [150, 0, 140, 1, 90], True), ("f32", 72, 2, [400, 333, 0, 500], True), ("bf16", 520, 2, [900, 850, 700], False)])
+def test_sequences_may_start_from_a_slot_that_one_of_them_stores_to(act, Dn, n_layers, lens, in_one):
     """Several sequences continue from one prefix's slot and the first stores its state back there: all of them start from what the slot
-    held before the call.  Only sequences that are cut promise that, so the call takes the three kernels (bit for bit those of the
-    same plan's chunk length), although its size is one that a call without starting slots does in one."""
+    held before the call, bit for bit as from a slot that nobody stores to.  (The one-kernel form delivers the final states by a second kernel then.)"""
     S, T, tdt = len(lens), sum(lens), torch_act(act)
     probs = [parity.make_problem(parity.small_config(Dn, act, S, cid=60 + l), lens) for l in range(n_layers)]
     flags = md.MDRAFT_DT_SOFTPLUS | md.MDRAFT_A_POWERS
     lays = [upload_layer(p.params, act, flags) for p in probs]
-    assert form(lays[0], n_layers, lens) != (0, 0)
+    assert (form(lays[0], n_layers, lens, shared=True) != (0, 0)) == in_one
     ci, hi = random_state(probs[0].cfg, 1, 7)
     ins = [tuple(to_device(a, tdt) for a in (p.x, p.z, p.dt, p.B, p.C)) for p in probs]
-    init, final = i32([0] * S), i32(np.arange(S))
+    ws = torch.empty(md.mdraft_prefill_stack_workspace_bytes(lays[0], n_layers, T, S, max(lens)), dtype=torch.uint8, device="cuda")
     res = []
-    for chunk_len in (0, 16):
-        cache = md.StateCache(n_layers, S, Dn, act=tdt)
-        cache.ssm[:, 0], cache.conv[:, 0] = torch.from_numpy(np.asarray(hi[0], dtype=np.float32)).cuda(), to_device(ci[0], tdt)
+    for start in (0, S):
+        cache = md.StateCache(n_layers, S + 1, Dn, act=tdt)
+        cache.ssm.fill_(float("nan")); cache.conv.fill_(float("nan"))
+        cache.ssm[:, start], cache.conv[:, start] = torch.from_numpy(np.asarray(hi[0], dtype=np.float32)).cuda(), to_device(ci[0], tdt)
         outs = list(torch.full((n_layers, T, Dn), float("nan"), dtype=tdt, device="cuda"))
         status = torch.zeros(1, dtype=torch.int32, device="cuda")
-        if chunk_len or n_layers == 1:
-            for l in range(n_layers):
-                ws = torch.empty(md.mdraft_prefill_workspace_bytes(lays[l], T, S, max(lens), chunk_len), dtype=torch.uint8, device="cuda")
-                md.mdraft_conv_scan_prefill(lays[l], cache, l, *ins[l], outs[l], i32(probs[0].cu), max(lens), init, final, ws, chunk_len, status)
+        if n_layers == 1:
+            md.mdraft_conv_scan_prefill(lays[0], cache, 0, *ins[0], outs[0], i32(probs[0].cu), max(lens), i32([start] * S), i32(np.arange(S)), ws, 0, status)
         else:
-            ws = torch.empty(md.mdraft_prefill_stack_workspace_bytes(lays[0], n_layers, T, S, max(lens)), dtype=torch.uint8, device="cuda")
-            assert md.mdraft_conv_scan_prefill_stack(lays, range(n_layers), cache, ins, outs, i32(probs[0].cu), max(lens), init, final, ws, status)
+            assert md.mdraft_conv_scan_prefill_stack(lays, range(n_layers), cache, ins, outs, i32(probs[0].cu), max(lens), i32([start] * S), i32(np.arange(S)), ws, status)
         torch.cuda.synchronize()
         assert int(status.item()) == 0
-        res.append((torch.stack(outs), cache.ssm, cache.conv))
+        res.append((torch.stack(outs), cache.ssm[:, :S], cache.conv[:, :S]))
     for a, b in zip(*res):
         assert torch.equal(a, b)
     for l, p in enumerate(probs):
