@@ -123,15 +123,16 @@ def test_prefills_in_a_row_on_one_workspace(act, powers):
 
 @pytest.mark.parametrize("act", ["bf16", "f32"])
 @pytest.mark.parametrize("powers", [False, True])
-@pytest.mark.parametrize("lens,Dn", [([611], 264), ([150, 3, 77], 200)])
-def test_one_kernel_prefills_in_a_row(act, powers, lens, Dn):
-    """Calls in the one-kernel form behind one another and behind calls in three kernels, which share a workspace that the former do not use."""
+@pytest.mark.parametrize("lens,Dn,have_state", [([611], 264, True), ([150, 3, 77], 200, False), ([150, 0, 140, 90], 200, True)])
+def test_one_kernel_prefills_in_a_row(act, powers, lens, Dn, have_state):
+    """Calls in the one-kernel form behind one another and behind calls in three kernels, which share a workspace; the former use it for final states
+    where several sequences start from slots."""
     NL, S, T, tdt = 6, len(lens), int(sum(lens)), torch_act(act)
     flags = md.MDRAFT_DT_SOFTPLUS | (md.MDRAFT_A_POWERS if powers else 0)
     cfg = gen.Config(96, "row", NL, Dn, 16, 4, act, S, (1, 1), "none", 0, 5)
     probs = [parity.make_problem(cfg, lens, layer=l, conv_bias=True, general_A=not powers) for l in range(NL)]
     lays = [upload_layer(pr.params, act, flags) for pr in probs]
-    assert form(lays[0], 1, lens) != (0, 0)
+    assert form(lays[0], 1, lens, shared=have_state and S > 1) != (0, 0)
     ins = [[to_device(a, tdt) for a in (pr.x, pr.z, pr.dt, pr.B, pr.C)] for pr in probs]
     outs = [torch.empty((T, Dn), dtype=tdt, device="cuda") for _ in range(NL)]
     cache = md.StateCache(NL, 2 * S, Dn, act=tdt)
@@ -141,7 +142,7 @@ def test_one_kernel_prefills_in_a_row(act, powers, lens, Dn):
     max_len, chunk_lens = max(lens), [0, 0, 48, 0, 48, 48]
     ws = torch.empty(max(md.mdraft_prefill_workspace_bytes(lays[0], T, S, max_len, c) for c in (0, 48)), dtype=torch.uint8, device="cuda")
     status = torch.zeros(1, dtype=torch.int32, device="cuda")
-    cu_d, init, final = i32(probs[0].cu), i32(np.arange(S)) if S == 1 else None, i32(np.arange(S, 2 * S))
+    cu_d, init, final = i32(probs[0].cu), i32(np.arange(S)) if have_state else None, i32(np.arange(S, 2 * S))
 
     def run_layer(l):
         md.mdraft_conv_scan_prefill(lays[l], cache, l, *ins[l], outs[l], cu_d, max_len, init, final, ws, chunk_lens[l], status)
